@@ -195,13 +195,13 @@ static void plan_free(ffrg_ctx *ctx, Plan *pl) {
   double *arrs[] = {pl->rad_x, pl->rad_w, pl->a1_x, pl->a1_w, pl->a2_x, pl->a2_w, pl->psi_x, pl->psi_w,
                     pl->radF, pl->radq, pl->partial, pl->radD, pl->gpart, pl->ext_pd, pl->psi_s, pl->jrows};
   for (double *p : arrs) dev_free(ctx, p, 0);
+  dev_free(ctx, pl->tab64, 0);
   dev_free(ctx, pl->tab32, 0);
   dev_free(ctx, pl->radq32, 0);
   dev_free(ctx, pl->work_ctr, 0);
   dev_free(ctx, pl->ext_done, 0);
   dev_free(ctx, pl->kconst, 0);
   dev_free(ctx, pl->radF32, 0);
-  dev_free(ctx, pl->tabc, 0);
   dev_free(ctx, pl->kbuf, 0);
   delete pl;
 }
@@ -233,12 +233,12 @@ void plan_geometry(Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td) 
   // FP32 layout: (value, difference) node pairs; finite T: (Z, lambda) node
   // pairs per stack row plus one zero pair (same bytes as single values)
   // D4_FULL: compact [Z row 0 | lambda4 row 0 | lambda3 rows] in both precisions
+  // FP64 layout: one double2 per value (finite T: Z and lambda of a node side by side)
   pl->n_va = pb->model == FFRG_MODEL_D4_FULL ? pb->n_va : 1;
   pl->n_vb = pb->model == FFRG_MODEL_D4_FULL ? pb->n_vb : 1;
-  pl->tabc_count = pb->model == FFRG_MODEL_D4_FULL ? (2 + pl->n_va * pl->n_vb) * td->n_pts : 0;
-  pl->tab32_count = pb->model == FFRG_MODEL_FINITE_T ? td->n_stack * td->n_pts + 1
-                    : pl->tabc_count                 ? pl->tabc_count
-                                                     : pl->tab_count;
+  const int compact = pb->model == FFRG_MODEL_D4_FULL ? (2 + pl->n_va * pl->n_vb) * td->n_pts : pl->tab_count;
+  pl->tab32_count = pb->model == FFRG_MODEL_FINITE_T ? td->n_stack * td->n_pts + 1 : compact;
+  pl->tab64_count = pb->model == FFRG_MODEL_FINITE_T ? 2 * td->n_stack * td->n_pts : compact;
   int outer_total, rows_per_outer;
   if (is_d4(pb->model)) {
     pl->jb = pl->na2;
@@ -305,7 +305,8 @@ void plan_geometry(Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td) 
   auto al16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
   const size_t ang = (size_t)pl->na1 * 3 + (size_t)pl->na2 * 2;
   const size_t ang32 = ang + (size_t)4 * ((pl->na2 + 1) / 2);   // + second-angle node pairs
-  pl->smem64 = al16((size_t)(pl->tabc_count ? pl->tabc_count : pl->tab_count) * 8) + al16(ang * 8);
+  pl->smem64g = sizeof(FxTables) + al16(ang * 8);
+  pl->smem64 = pl->smem64g + (size_t)pl->tab64_count * sizeof(double2);
   // D4_FULL, mixed: lambda3 as cell polynomials (two float4 per (a, b, S0)
   // cell) after the Z and lambda4 line rows, when that fits in shared memory
   pl->l3cell = 0;
@@ -317,7 +318,32 @@ void plan_geometry(Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td) 
     }
   }
   pl->smem32 = al16((size_t)pl->tab32_count * 8) + al16(ang32 * 4);
-  pl->smem64g = al16(ang * 8);
+}
+
+void plan_grid(Plan *pl, const ffrg_table_desc *td) {
+  if (pl->fg_lo == td->x_min && pl->fg_hi == td->x_max) return;
+  pl->fg_ok = fx_grid(td->n_pts, td->x_min, td->x_max, &pl->fg);
+  pl->fg_lo = td->x_min;
+  pl->fg_hi = td->x_max;
+}
+
+// The tables of the fixed-point functions: built once per process, uploaded
+// once per device into a fixed device array (so that callers that may not
+// allocate can use them).
+static __device__ __align__(16) FxTables g_fx;
+
+const FxTables *fx_device_tables(int device) {
+  static std::mutex mu;
+  static std::map<int, const FxTables *> ptr;
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = ptr.find(device);
+  if (it != ptr.end()) return it->second;
+  std::vector<FxTables> host(1);
+  fx_build_tables(host.data());
+  void *p = nullptr;
+  if (cudaGetSymbolAddress(&p, g_fx) != cudaSuccess) return nullptr;
+  if (cudaMemcpy(p, host.data(), sizeof(FxTables), cudaMemcpyHostToDevice) != cudaSuccess) return nullptr;
+  return ptr[device] = (const FxTables *)p;
 }
 
 int get_plan(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc *td, Plan **out) {
@@ -330,11 +356,13 @@ int get_plan(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc *td, P
   auto it = ctx->plans.find(key);
   if (it != ctx->plans.end()) {
     *out = it->second;
+    plan_grid(it->second, td);
     return FFRG_OK;
   }
   Plan *pl = new Plan();  // value-initialised: pointers null, counts zero
   pl->key = key;
   plan_geometry(pl, pb, td);
+  plan_grid(pl, td);
 
   int st = FFRG_OK;
   std::vector<double> x(pl->nr), w(pl->nr);
@@ -369,7 +397,13 @@ int get_plan(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc *td, P
   if (!st) st = set_cuda_error(ctx, cudaMemset(pl->work_ctr, 0, 5 * sizeof(unsigned)), "cudaMemset(counters)");
   if (!st) st = dev_alloc(ctx, (void **)&pl->ext_done, (size_t)pl->n_ext * sizeof(unsigned));
   if (!st) st = dev_alloc(ctx, (void **)&pl->kconst, kKConstBytes);
-  if (!st && pl->tabc_count) st = dev_alloc(ctx, (void **)&pl->tabc, (size_t)pl->tabc_count * sizeof(double));
+  // FP64 line-form tables in global memory: finite T (long to build in every
+  // CTA), and tables that do not fit in shared memory.  The former can do without.
+  const bool too_big = pl->smem64 > kMaxDynSmemBytes && pb->model != FFRG_MODEL_FINITE_T_4D;
+  if (!st && (pb->model == FFRG_MODEL_FINITE_T || too_big)) {
+    st = dev_alloc(ctx, (void **)&pl->tab64, (size_t)pl->tab64_count * sizeof(double2));
+    if (st == FFRG_ENOMEM && !too_big) st = FFRG_OK;
+  }
   if (!st && pl->kbuf_count) st = dev_alloc(ctx, (void **)&pl->kbuf, pl->kbuf_count * sizeof(double));
   if (!st) st = dev_alloc(ctx, (void **)&pl->ext_pd, (size_t)pl->n_ext_p * sizeof(double));
   if (!st) st = dev_alloc(ctx, (void **)&pl->psi_s, (size_t)npsi * sizeof(double));
@@ -410,11 +444,10 @@ void fill_args(const Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td
   a.n_items = pl->fn_items;
   a.jb = pl->fjb;
   a.tab32_count = pl->tab32_count;
-  a.tabc_count = pl->tabc_count;
+  a.tab64_count = pl->tab64_count;
   a.n_va = pl->n_va;
   a.n_vb = pl->n_vb;
   a.l3cell = pl->l3cell;
-  a.tabc = pl->tabc;
   a.kbuf = pl->kbuf;
   a.k = k;
   a.m2_over_k2 = pb->m2_over_k2;
@@ -445,6 +478,9 @@ void fill_args(const Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td
   }
   a.twopiT = 2.0 * kPi * pb->T;
   a.sum_w2 = pl->sum_w2;
+  a.fg = pl->fg;
+  a.fg_ok = pl->fg_ok;
+  a.tab64 = pl->tab64;
   // FP32 scale constants of this k on the host (the kernels use them unless a
   // flow stage sets k_dev or m2_dev later); every field they read is set above
   a.kc_host = kconst_f32(a, k, a.m2_over_k2 * k * k + a.m2_shift);
@@ -524,7 +560,7 @@ int ffrg_destroy(ffrg_ctx *ctx) {
     cudaFree(pl->ext_done);
     cudaFree(pl->kconst);
     cudaFree(pl->radF32);
-    cudaFree(pl->tabc);
+    cudaFree(pl->tab64);
     cudaFree(pl->kbuf);
     delete pl;
   }

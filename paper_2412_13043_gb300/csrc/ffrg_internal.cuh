@@ -16,10 +16,12 @@
 #include <vector>
 
 #include "../../include/ffrg.h"
+#include "ffrg_fx.cuh"
 
 namespace ffrg {
 
 constexpr int kThreads = 256;          // threads per CTA of the RHS kernels
+constexpr int kThreads64 = 512;        // threads per CTA of the FP64 main kernels (one CTA per SM)
 constexpr int kThreadsWide = 1024;     // the D4_FULL mixed kernel with lambda3 cells: one CTA per SM
 constexpr size_t kMaxDynSmemBytes = 227 * 1024;   // dynamic shared memory of one block
 constexpr unsigned kStatusNonFinite = 1u;
@@ -49,6 +51,20 @@ struct KConst {
   T isy;  // 1/sy
 };
 
+// FP64: table coordinates in fixed point (ffrg_fx.cuh).  FxOff: offset of a
+// coordinate taken in y = sy s^2 of S0^2 = (sum of c squares)/c.
+struct FxOff {
+  int64_t v;
+  int c;
+};
+template <>
+struct KConst<double> {
+  double k2, inv_k2, m2, sy, som, isy, twopiT, sw2;
+  FxOff uy1, uy2, uy3, uy4;
+  int slow;             // the grid or k lies outside fixed point: coordinates by FP64 logarithms
+  const FxTables *us;   // staged tables (logarithms in the grid's units)
+};
+
 struct RhsArgs {
   int model, reg;
   int nr, na1, na2;
@@ -56,7 +72,7 @@ struct RhsArgs {
   int stat, nfreq;  // loop statistics (ffrg_statistics) and frequency rows: 2N+1 (bosonic), 2N+2 (fermionic)
   int n_tables, n_stack, n_pts, tab_count;
   int tab32_count; // float2 entries of the FP32 table layout
-  int tabc_count;  // D4_FULL: doubles of the compact FP64 tables (0 otherwise)
+  int tab64_count; // double2 entries of the FP64 table layout
   int n_va, n_vb;  // D4_FULL: vertex nodes in the shape variables a, b
   int l3cell;      // D4_FULL, mixed: lambda3 as FP32 cell polynomials (one 1024-thread CTA per SM)
   int cr;          // rows per work item (d=4: outer rows)
@@ -79,8 +95,13 @@ struct RhsArgs {
   double sum_w2;               // sum of the second-angle weights (D4)
   KConst<float> kc_host;       // FP32 scale constants from the host (valid when kc_host_ok, k_dev and m2_dev null)
   int kc_host_ok;
+  int fp64;                    // precision of this RHS (what the precompute kernel writes)
+  FxGrid fg;                   // the table grid in fixed point (FP64 kernels)
+  int fg_ok;
+  const FxTables *fx;          // device tables of the fixed-point functions
   const double *tab;           // FP64 tables [n_tables][n_stack][n_pts]
-  double *tabc;                // D4_FULL: compact FP64 tables [Z row | lambda4 row | lambda3 rows] (precompute)
+  double2 *tab64;              // FP64 tables in line form (tab64_entry), written by the precompute kernel; null:
+                               // the FP64 main kernels build them in shared memory
   void *kbuf;                  // FINITE_T: K[j][ip][r], j < N + n_ext_ang, in the kernel precision (main kernel)
   float2 *tab32;               // FP32 tables (rows in line form, or finite-T (Z, lambda) pairs), precompute kernel
   const double *rad_x, *rad_w; // unit-interval GL rule on [0, 1]
@@ -504,15 +525,19 @@ struct Plan {
   int fjb;                        // angle nodes per forward row (D3 / FINITE_T)
   int fcr64, fn_chunks64, fn_items64, fjb64;  // the same for the FP64 forward kernels
   int tab32_count;                // float2 entries of the FP32 table layout
-  int tabc_count, n_va, n_vb;     // D4_FULL: compact FP64 table doubles, vertex nodes
+  int tab64_count;                // double2 entries of the FP64 table layout
+  FxGrid fg;                      // the grid in fixed point, of the descriptor last seen
+  int fg_ok;
+  double fg_lo, fg_hi;
+  int n_va, n_vb;                 // D4_FULL: vertex nodes
   int l3cell;                     // D4_FULL: the FP32 lambda3 cell layout fits in shared memory
-  double *tabc;
+  double2 *tab64;
   size_t kbuf_count;              // FINITE_T: entries of K (N + n_ext_ang) x n_ext_p x n_rad
   double *kbuf;
   int grid64, grid32;       // persistent grids (FP64 / mixed kernels)
   int grid_single;          // finite T, mixed: grid of the single-launch RHS (-1: not available)
   size_t smem64, smem32;    // dynamic shared memory bytes
-  size_t smem64g;           // FP64 kernels with tables in global memory: angle rules only
+  size_t smem64g;           // FP64 kernels with tables in global memory: the rest
   double *rad_x, *rad_w, *a1_x, *a1_w, *a2_x, *a2_w, *psi_x, *psi_w;
   double sum_w2;
   double *radF, *radq, *partial, *ext_pd, *psi_s;
@@ -530,6 +555,8 @@ struct Plan {
 // Shape and launch geometry of a plan (no allocation): sizes from the problem
 // and the table descriptor, and the grouping of angular rows into work items.
 void plan_geometry(Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td);
+// The plan's fixed-point grid for the descriptor's x_min and x_max.
+void plan_grid(Plan *pl, const ffrg_table_desc *td);
 
 // Raise a kernel's dynamic shared-memory limit to at least `bytes` (never
 // lowers it: plans of different sizes share the kernel).
@@ -615,6 +642,9 @@ void fill_args(const Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td
                RhsArgs &a);
 int host_gauss_legendre(int n, double a, double b, double *x, double *w);
 int host_gauss_chebyshev2(int n, double *x, double *w);
+// device address of the fixed-point tables on the current device (uploaded on
+// the first call there); null on a CUDA error
+const FxTables *fx_device_tables(int device);
 
 // kernels launched from several translation units (ffrg_rhs.cu)
 int launch_rhs(ffrg_ctx *ctx, const Plan *pl, const RhsArgs &a, int precision, cudaStream_t s);

@@ -21,11 +21,12 @@
 
 namespace ffrg {
 
-constexpr size_t kNoallocScratchBytes = size_t(4) << 20;  // 4 MiB
+constexpr size_t kNoallocScratchBytes = size_t(4) << 20;  // 4 MiB: what the problems may need
+constexpr size_t kNoallocTab64Bytes = size_t(480) << 10;  // and the FP64 line-form tables
 constexpr int kNoallocMaxDevices = 64;
 
 // Shared by every call of ffrg_rhs_noalloc on a device; keeps the last call's contents.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes + kNoallocTab64Bytes];
 
 static std::mutex g_noalloc_mu;
 static unsigned char *g_noalloc_ptr[kNoallocMaxDevices];  // device address per device
@@ -118,12 +119,20 @@ extern "C" int ffrg_rhs_noalloc(const ffrg_problem *pb, const ffrg_table_desc *t
   pl.psi_s = sc.take<double>(npsi);
   pl.partial = sc.take<double>(std::max(pl.fn_items, pl.fn_items64));
   pl.tab32 = sc.take<float2>((size_t)pl.tab32_count);
-  if (pl.tabc_count) pl.tabc = sc.take<double>((size_t)pl.tabc_count);
   if (pl.kbuf_count) pl.kbuf = sc.take<double>(pl.kbuf_count);
   if (sc.used > kNoallocScratchBytes) return FFRG_EINVAL;  // problem needs more than the 4 MiB scratch
 
-  const size_t smem = precision == FFRG_MIXED ? pl.smem32 : pl.smem64;
-  if (smem > 227 * 1024) return FFRG_EINVAL;
+  // the tables must fit in shared memory as plain values (FP64 line form: twice as large, in global memory when
+  // it does not fit), so that line-form tables need at most 2 x 227 KB behind the scratch
+  const size_t values = (size_t)(pb->model == FFRG_MODEL_D4_FULL ? pl.tab64_count : pl.tab_count) * sizeof(double);
+  const size_t rules = ((size_t)pl.na1 * 3 + (size_t)pl.na2 * 2) * sizeof(double);
+  if (precision == FFRG_MIXED ? pl.smem32 > kMaxDynSmemBytes
+                              : ((values + 15) & ~(size_t)15) + ((rules + 15) & ~(size_t)15) > kMaxDynSmemBytes)
+    return FFRG_EINVAL;
+  if (precision == FFRG_FP64 && pb->model != FFRG_MODEL_FINITE_T_4D &&
+      (pb->model == FFRG_MODEL_FINITE_T || pl.smem64 > kMaxDynSmemBytes))
+    pl.tab64 = sc.take<double2>((size_t)pl.tab64_count);
+  plan_grid(&pl, td);
 
   cudaStream_t s = (cudaStream_t)stream;
   const size_t db = sizeof(double);

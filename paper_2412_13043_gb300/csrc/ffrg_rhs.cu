@@ -99,10 +99,12 @@ __device__ __noinline__ float pole_ftk(const RhsArgs *a, int ip, int jk, int r, 
 
 // Scale-dependent constants of one RHS in the kernel precision, computed once
 // per RHS by the precompute kernel into a small device block (RhsArgs::kconst)
-// that every CTA of the main kernel loads.  us/uo: table coordinate
-// (divided by n-1 in FP32); plim = -2 m^2 (near-pole test).  The kernels pass
+// that every CTA of the main kernel loads.  FP32 us/uo: table coordinate
+// divided by n-1; plim = -2 m^2 (near-pole test).  The kernels pass
 // squared momenta to the propagator as y = sy s^2 and omega^2 as som omega^2:
-// FP64 sy = som = 1; FP32 sy = log2(e)/k^2 (the regulator's exp2 argument)
+// FP64 sy = som = 1/k^2 with the Z table pre-scaled by k^2, so that y is the
+// regulator's argument (sy = 1 for the full vertex, whose shape variables
+// need s^2 itself); FP32 sy = log2(e)/k^2 (the regulator's exp2 argument)
 // and som = 1/(k^2 ln 2), with the FP32 Z table pre-scaled by k^2 ln 2
 // (see reg_g).
 // uy1..uy4: offsets of table coordinates taken in y of S0^2 = (sum of c
@@ -132,16 +134,22 @@ __device__ __forceinline__ KConst<double> make_kconst<double>(const RhsArgs &a) 
   c.k2 = kd * kd;
   c.inv_k2 = 1.0 / c.k2;
   c.m2 = m2d;
-  c.plim = -2.0 * m2d;
-  c.us = a.u_scale;
-  c.uo = a.u_off;
-  c.sy = 1.0;
-  c.som = 1.0;
-  c.isy = 1.0;
-  c.uy1 = a.uoc[0];
-  c.uy2 = a.uoc[1];
-  c.uy3 = a.uoc[2];
-  c.uy4 = a.uoc[3];
+  const bool full = a.model == FFRG_MODEL_D4_FULL;
+  c.sy = full ? 1.0 : c.inv_k2;
+  c.som = c.inv_k2;
+  c.isy = full ? 1.0 : c.k2;
+  c.slow = !a.fg_ok || !(kd > 0x1p-30) || !(kd < 0x1p30);
+  // coordinate of y = sy s^2: u_scale ln(y) + u_off + u_scale ln(1/sy)
+  int64_t off = a.fg.uo;
+  if (!full && !c.slow) {
+    const int hi = fx_clamp_hi(fx_bits(c.k2));
+    off += fx_log(fx_scaled(a.fx->log[fx_log_index(hi)], a.fg), a.fg, hi, (uint32_t)fx_bits(c.k2));
+  }
+  c.uy1 = {off - a.fg.uc[0], 1};
+  c.uy2 = {off - a.fg.uc[1], 2};
+  c.uy3 = {off - a.fg.uc[2], 3};
+  c.uy4 = {off - a.fg.uc[3], 4};
+  c.us = nullptr;
   c.twopiT = a.twopiT;
   c.sw2 = a.sum_w2;
   return c;
@@ -155,7 +163,64 @@ __device__ __forceinline__ KConst<float> load_kconst<float>(const RhsArgs &a) {
 }
 template <>
 __device__ __forceinline__ KConst<double> load_kconst<double>(const RhsArgs &a) {
-  return ((const KConstPair *)a.kconst)->d;
+  KConst<double> c = ((const KConstPair *)a.kconst)->d;
+  c.uy1.c = 1, c.uy2.c = 2, c.uy3.c = 3, c.uy4.c = 4;
+  return c;
+}
+
+// FP64 tables in line form: a node holds (T_i - d_i, d_i), d_i the difference
+// to the next node (0 at a row end), so that the interpolant is one FMA with
+// the weight 1 + w in [1, 2) of fx_node.  Layout: as the tables (D4_FULL: rows
+// Z | lambda4 | lambda3 rows; finite T: [row][node][Z, lambda]).  Z rows carry
+// k^2.  Entry i:
+__device__ __forceinline__ double2 tab64_entry(const RhsArgs &a, int i, double k2) {
+  const int np = a.n_pts, zn = a.n_stack * np;
+  size_t src;
+  int col;
+  bool z;
+  if (a.model == FFRG_MODEL_FINITE_T) {
+    z = !(i & 1);
+    src = (size_t)(i >> 1) + (z ? 0 : zn);
+    col = (i >> 1) % np;
+  } else {
+    const int row = i / np;
+    col = i - row * np;
+    z = row < (a.model == FFRG_MODEL_D4_FULL ? 1 : a.n_stack);
+    src = i;
+    if (a.model == FFRG_MODEL_D4_FULL) src = col + (row == 0 ? (size_t)0 : row == 1 ? (size_t)2 * zn : (size_t)zn + (size_t)(row - 2) * np);
+  }
+  const double f = z ? k2 : 1.0, v = f * a.tab[src];
+  const double d = col == np - 1 ? 0.0 : f * a.tab[src + 1] - v;
+  return make_double2(v - d, d);
+}
+
+// Node and weight of the coordinate of y (FP64 lookups): fixed point, or an
+// FP64 logarithm when the grid or k lies outside its range.
+__device__ __noinline__ void slow_node(const RhsArgs *a, double s2, int c, int &i, double &w1) {
+  double w;
+  lerp_pos(s2, a->u_scale, a->uoc[c - 1], a->n_pts, i, w);
+  w1 = 1.0 + w;
+}
+__device__ __forceinline__ void node_of(const RhsArgs &a, const KConst<double> &kc, double y, FxOff o, int &i,
+                                        double &w1) {
+  if (kc.slow) slow_node(&a, y * kc.isy, o.c, i, w1);   // uniform
+  else fx_node(a.fg, fx_log(kc.us->log, a.fg, y) + o.v, i, w1);
+}
+__device__ __forceinline__ double line64(double2 t, double w1) { return fma(t.y, w1, t.x); }
+
+// what a table lookup takes besides its row, argument and offset: the FP32
+// coordinate scale, or the FP64 argument block and constants
+struct Look64 {
+  const RhsArgs &a;
+  const KConst<double> &kc;
+};
+__device__ __forceinline__ float look_scale(const RhsArgs &, const KConst<float> &kc) { return kc.us; }
+__device__ __forceinline__ Look64 look_scale(const RhsArgs &a, const KConst<double> &kc) { return {a, kc}; }
+__device__ __forceinline__ double look(const double2 *row, double y, Look64 us, FxOff o, int) {
+  int i;
+  double w1;
+  node_of(us.a, us.kc, y, o, i, w1);
+  return line64(row[i], w1);
 }
 
 // FP32 regulator in propagator form.  With x = s^2/k^2 the kinetic part of the
@@ -182,14 +247,19 @@ __device__ __forceinline__ float reg_g(int reg, float y) {
 
 // Inverse propagator in the kernel precision from the table value Zs, the
 // scaled momentum y = sy s^2 and om2s = som omega^2 (FP64: Z, s^2, omega^2).
+// FP64: Z (s^2 + k^2 r) = Z k^2 h(x), h(x) = x + r(x) = x/(1 - e^{-x}) from the
+// fixed-point tables (flat shape: max(1, x)), Z table pre-scaled by k^2.
 // The FP32 version switches to FP64 when m^2 cancels more than half of
 // Z (omega^2 + s^2 + k^2 r), i.e. P < -2 m^2: close to the convexity pole.
 // `pole` is only evaluated on that rare branch.  POLE = false drops the test;
 // callers use it only when m^2 >= 0 and no Z < 0, where P >= 0 >= -2 m^2.
 template <bool POLE = true, typename Pole>
-__device__ __forceinline__ double inv_prop(const RhsArgs &a, double Z, double y, double om2s,
+__device__ __forceinline__ double inv_prop(const RhsArgs &a, double Zk, double y, double om2s,
                                            const KConst<double> &kc, Pole &&) {
-  return 1.0 / prop_den(a.reg, Z, om2s, y, kc.m2, kc.k2, kc.inv_k2);
+  const double x = a.model == FFRG_MODEL_D4_FULL ? y * kc.inv_k2 : y;   // sy s^2 = x otherwise
+  double h = a.reg == FFRG_REG_LITIM ? (x < 1.0 ? 1.0 : x) : fx_h(*kc.us, x);
+  if (a.model == FFRG_MODEL_FINITE_T) h += om2s;
+  return fx_rcp(fma(Zk, h, kc.m2));
 }
 
 template <bool POLE = true, typename Pole>
@@ -213,6 +283,10 @@ template <>
 struct MinBlocks<float> {
   static constexpr int value = 4;
 };
+// threads per CTA: FP64 one CTA of 512 threads per SM (128 registers; the
+// staged function tables once per SM)
+template <typename T>
+constexpr int kMainThreads = sizeof(T) == 8 ? kThreads64 : kThreads;
 
 // ---------------------------------------------------------------------------
 // 1. precompute kernel
@@ -350,10 +424,10 @@ __device__ __forceinline__ void precompute_body(const RhsArgs &a) {
   const int tid0 = ((blockIdx.x + gridDim.x - first_free) % gridDim.x) * blockDim.x + threadIdx.x;
   // the main kernel runs after this one (stream order)
   if (tid0 == 0 && a.work_ctr) *a.work_ctr = 0u;
-  if (a.kconst && (tid0 == 0 || tid0 == 32)) {  // two warps, in parallel
+  if (a.kconst && tid0 == 32) {
     KConstPair *kp = (KConstPair *)a.kconst;
-    if (tid0 == 0) kp->f = make_kconst<float>(a);
-    else kp->d = make_kconst<double>(a);
+    if (a.fp64) kp->d = make_kconst<double>(a);
+    else kp->f = make_kconst<float>(a);
   }
   precompute_radial(a, blockIdx.x, gridDim.x);
   // radial nodes q_r = qmax k x_r
@@ -370,21 +444,20 @@ __device__ __forceinline__ void precompute_body(const RhsArgs &a) {
   // with weight 0).
   const double kh = k2 * 0.6931471805599453094;
   const int z_count = a.n_stack * a.n_pts;
-  if (a.model == FFRG_MODEL_D4_FULL) {
-    // compact rows [Z row 0 | lambda4 row 0 | lambda3 rows]: FP64 copy and FP32
-    // pairs (with lambda3 cells: the two line rows only)
+  if (a.fp64) {
+    if (a.tab64)
+      for (int i = tid0; i < a.tab64_count; i += stride) a.tab64[i] = tab64_entry(a, i, k2);
+  } else if (a.model == FFRG_MODEL_D4_FULL) {
+    // compact rows [Z row 0 | lambda4 row 0 | lambda3 rows] (with lambda3 cells: the two line rows only)
     const int np = a.n_pts, ns = a.n_stack;
-    const int n_line = a.l3cell ? 2 * np : a.tabc_count;
-    for (int i = tid0; i < a.tabc_count; i += stride) {
+    const int n_line = a.l3cell ? 2 * np : a.tab64_count;
+    for (int i = tid0; i < n_line; i += stride) {
       const int row = i / np, col = i - row * np;
       const size_t src = row == 0 ? (size_t)col : row == 1 ? (size_t)2 * ns * np + col : ((size_t)ns + row - 2) * np + col;
       const double f = row == 0 ? kh : 1.0;
       const double v = a.tab[src];
-      a.tabc[i] = v;
-      if (i < n_line) {
-        const double d = col == np - 1 ? 0.0 : f * (a.tab[src + 1] - v);
-        a.tab32[i] = make_float2((float)(f * v - col * d), (float)((np - 1) * d));
-      }
+      const double d = col == np - 1 ? 0.0 : f * (a.tab[src + 1] - v);
+      a.tab32[i] = make_float2((float)(f * v - col * d), (float)((np - 1) * d));
     }
     if (a.l3cell) {
       // Cell (ia, ib, is) of lambda3 on the (a, b, S0) grid: the trilinear
@@ -454,13 +527,13 @@ __global__ void __launch_bounds__(kThreads) precompute_kernel(RhsArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// shared-memory layout of the main kernels: tables (FP64 values, or FP32 node
-// pairs), then the second-angle (node, weight) pairs and the first-angle
+// shared-memory layout of the main kernels: (FP64: the fixed-point function
+// tables,) tables (FP64 or FP32 node pairs), then the second-angle (node, weight) pairs and the first-angle
 // nodes, sines and weights
 // ---------------------------------------------------------------------------
 template <typename T>
 struct TabOf {
-  using type = double;
+  using type = double2;
 };
 template <>
 struct TabOf<float> {
@@ -478,7 +551,7 @@ struct Pair2<float> {
 template <typename T>
 __device__ __forceinline__ const typename TabOf<T>::type *table_src(const RhsArgs &a);
 template <>
-__device__ __forceinline__ const double *table_src<double>(const RhsArgs &a) { return a.tabc ? a.tabc : a.tab; }
+__device__ __forceinline__ const double2 *table_src<double>(const RhsArgs &a) { return a.tab64; }
 template <>
 __device__ __forceinline__ const float2 *table_src<float>(const RhsArgs &a) { return a.tab32; }
 
@@ -490,14 +563,15 @@ struct SmemLayout {
   float4 *cw4;  // FP32 kernels: second-angle nodes in pairs (x_2j, x_2j+1, w_2j, w_2j+1)
   P2 *cw2;
   T *c1, *s1, *w1;
-  // table entries in shared memory: FP64 values, or the FP32 layout
-  static __device__ int entries(const RhsArgs &a) {
-    return sizeof(T) == 4 ? a.tab32_count : (a.tabc_count ? a.tabc_count : a.tab_count);
-  }
+  FxTables *fx;
+  // table entries in shared memory
+  static __device__ int entries(const RhsArgs &a) { return sizeof(T) == 4 ? a.tab32_count : a.tab64_count; }
   // FP64 kernels whose tables exceed shared memory read them in place (L2)
   static __device__ bool in_global(const RhsArgs &a) { return sizeof(T) == 8 && a.tab_global; }
   __device__ SmemLayout(unsigned char *base, const RhsArgs &a) {
     const bool g = in_global(a);
+    fx = (FxTables *)base;
+    if (sizeof(T) == 8) base += sizeof(FxTables);
     tab = g ? const_cast<Tab *>(table_src<T>(a)) : (Tab *)base;
     size_t off = g ? 0 : ((size_t)entries(a) * sizeof(Tab) + 15) & ~(size_t)15;
     cw4 = (float4 *)(base + off);
@@ -509,12 +583,9 @@ struct SmemLayout {
   }
 };
 
-__device__ __forceinline__ double table_value(double v) { return v; }
-__device__ __forceinline__ float table_value(float2 v) { return v.x; }
-
 // handle of the table row that starts `off` entries into the staged tables:
-// an FP64 pointer, or an FP32 line row (Row32)
-__device__ __forceinline__ const double *tab_row(const SmemLayout<double> &S, int off) { return S.tab + off; }
+// an FP64 line row, or an FP32 one (Row32)
+__device__ __forceinline__ const double2 *tab_row(const SmemLayout<double> &S, int off) { return S.tab + off; }
 __device__ __forceinline__ Row32 tab_row(const SmemLayout<float> &S, int off) { return row32(S.tab + off); }
 
 // angle rules into shared memory in the kernel precision.  S1 = false skips
@@ -548,17 +619,35 @@ template <typename T>
 __device__ bool main_prologue(const RhsArgs &a, SmemLayout<T> &S, uint64_t *bar) {
   bool ok = true;
   stage_angles<T>(a, S);   // rules of the plan: not written by the precompute kernel
+  if constexpr (sizeof(T) == 8) {
+    // the function tables (logarithms in the grid's units), and line-form
+    // tables that the precompute kernel does not write
+    for (int j = threadIdx.x; j < kFxLog; j += blockDim.x) S.fx->log[j] = fx_scaled(a.fx->log[j], a.fg);
+    constexpr int kRest = (int)((sizeof(FxTables) - sizeof(a.fx->log)) / 16);
+    for (int j = threadIdx.x; j < kRest; j += blockDim.x)
+      ((int4 *)(S.fx->log + kFxLog))[j] = ((const int4 *)(a.fx->log + kFxLog))[j];
+    if (!a.tab64) {
+      const double k = scale_k(a), k2 = k * k;
+      for (int i = threadIdx.x; i < SmemLayout<T>::entries(a); i += blockDim.x) S.tab[i] = tab64_entry(a, i, k2);
+    }
+  }
   // launched as a programmatic dependent of the precompute kernel: wait here
   // for its writes (FP32 tables, radial factors, constants, counters)
   pdl_wait();
-  if (!SmemLayout<T>::in_global(a))   // uniform over the block
+  if (!SmemLayout<T>::in_global(a) && (sizeof(T) == 4 || a.tab64))   // uniform over the block
     ok = stage_to_smem<typename TabOf<T>::type>(S.tab, table_src<T>(a), SmemLayout<T>::entries(a), bar, a.status);
   __syncthreads();
   return ok;
 }
 
 // ---------------------------------------------------------------------------
-// 2. main kernels.  Work items are warp-sized: external point e x a chunk of
+// 2. main kernels.  FP64 (d=4 vertex workload, 1281 x 131072 terms): the FP64
+// pipe bounds a term at 134 instructions (three logarithms, an exponential,
+// two divisions, clamps and conversions), 41.5 ms; with those functions in
+// fixed point on the integer pipe (ffrg_fx.cuh) a term has 11 FP64
+// instructions (arguments, interpolations, products) and about 150 clocks of
+// integer work, which overlap: 4.04 ms.
+// Work items are warp-sized: external point e x a chunk of
 // `cr` outer rows (d=3: radial nodes; finite T: (Matsubara n, radial node)
 // pairs; d=4: (radial node, first-angle node) pairs).  Lane l takes rows
 // l, l+32, ... of its item and loops over the remaining angle nodes of each
@@ -749,7 +838,9 @@ __device__ __forceinline__ float ftk_row_x2(const SmemLayout<float> &S, const KC
 template <typename T, bool POLE>
 __device__ __forceinline__ RowAcc<T> d3_witem(const RhsArgs &a, const RhsArgs *sa, const SmemLayout<T> &S,
                                            const KConst<T> &kc, int e, int c, int lane) {
-  const T us = kc.us, uy1 = kc.uy1, sy = kc.sy;
+  const auto us = look_scale(a, kc);
+  const auto uy1 = kc.uy1;
+  const T sy = kc.sy;
   const int np = a.n_pts, na1 = a.na1, jb = a.jb, nblk = (na1 + jb - 1) / jb;
   const auto Zt = tab_row(S, 0);
   const T p = (T)((e < a.n_ext_p) ? a.ext_pd[e] : 0.0);
@@ -773,15 +864,22 @@ __device__ __forceinline__ RowAcc<T> d3_witem(const RhsArgs &a, const RhsArgs *s
   return acc;
 }
 
-// finite-T lookups of Z and lambda at stack row srow: FP64 tables [table][row][pt];
-// FP32 (Z, lambda) node pairs [row][pt] (+ one zero pair)
-__device__ __forceinline__ void zl_lookup(const double *tab, const RhsArgs &a, int srow, int i0, double w, double &Z,
-                                          double &L) {
-  Z = lerp_at(tab + (size_t)srow * a.n_pts, i0, w);
-  L = lerp_at(tab + ((size_t)a.n_stack + srow) * a.n_pts, i0, w);
+// finite-T lookups of Z and lambda at y in stack row srow: FP64 line-form
+// entries [row][pt][Z, lambda]; FP32 (Z, lambda) node pairs [row][pt] (+ one zero pair)
+__device__ __forceinline__ void zl_lookup(const double2 *tab, const RhsArgs &a, const KConst<double> &kc, int srow,
+                                          double y, double &Z, double &L) {
+  int i;
+  double w1;
+  node_of(a, kc, y, kc.uy1, i, w1);
+  const double2 *e = tab + 2 * ((size_t)srow * a.n_pts + i);
+  Z = line64(e[0], w1);
+  L = line64(e[1], w1);
 }
-__device__ __forceinline__ void zl_lookup(const float2 *tab, const RhsArgs &a, int srow, int i0, float w, float &Z,
-                                          float &L) {
+__device__ __forceinline__ void zl_lookup(const float2 *tab, const RhsArgs &a, const KConst<float> &kc, int srow,
+                                          float y, float &Z, float &L) {
+  int i0;
+  float w;
+  lerp_pos(y, kc.us, kc.uy1, a.n_pts, i0, w);
   const float2 *row = tab + (size_t)srow * a.n_pts;
   const float2 v0 = row[i0], v1 = row[i0 + 1];
   Z = fmaf(w, v1.x - v0.x, v0.x);
@@ -802,7 +900,7 @@ template <typename T, bool POLE>
 __device__ __forceinline__ void ftk_rows(const RhsArgs &a, const RhsArgs *sa, const SmemLayout<T> &S,
                                          const KConst<T> &kc, int outer, int c, int lane,
                                          const T *q_loc = nullptr, const T *p_loc = nullptr) {
-  const T us = kc.us, uy1 = kc.uy1, sy = kc.sy;
+  const T sy = kc.sy;
   const int np = a.n_pts, na1 = a.na1, nr = a.nr;
   const int jk = outer / a.n_ext_p, ip = outer - jk * a.n_ext_p;
   const int srow = min(jk, a.n_stack - 1);
@@ -820,10 +918,8 @@ __device__ __forceinline__ void ftk_rows(const RhsArgs &a, const RhsArgs *sa, co
     if constexpr (sizeof(T) == 4 && !POLE) rs = ftk_row_x2(S, kc, S.tab + (size_t)srow * np, np, na1, om2s, by, ty);
     else for (int j = 0; j < na1; ++j) {
       const T y = fma(ty, S.c1[j], by);
-      int i0;
-      T w, Z, Lv;
-      lerp_pos(y, us, uy1, np, i0, w);
-      zl_lookup(S.tab, a, srow, i0, w, Z, Lv);
+      T Z, Lv;
+      zl_lookup(S.tab, a, kc, srow, y, Z, Lv);
       auto pole = [&]() { return pole_ftk(sa, ip, jk, r, j); };
       rs = fma(S.w1[j] * Lv, inv_prop<POLE>(a, Z, y, om2s, kc, pole), rs);
     }
@@ -920,10 +1016,15 @@ __device__ __forceinline__ void shape_pos(float v, int m, int &i, float &w) {
   i = min((int)u, m - 2);
   w = u - (float)i;
 }
+// FP64: differences and squares rounded separately (no contraction with the
+// products that feed them), so that s3 - s1 - s2 cancels the rounded squares
+// that s2 was formed from
 __device__ __forceinline__ double shape_a(double s1, double s2, double s3) {
-  return (s3 - s1 - s2) / (2.0 * sqrt(s1 * s2));
+  return __dsub_rn(__dsub_rn(s3, s1), s2) * fx_rcp(2.0 * sqrt(s1 * s2));
 }
-__device__ __forceinline__ double shape_b(double s1, double s2) { return (s1 - s2) / (s1 + s2); }
+__device__ __forceinline__ double square(double v) { return __dmul_rn(v, v); }
+__device__ __forceinline__ float square(float v) { return v * v; }
+__device__ __forceinline__ double shape_b(double s1, double s2) { return (s1 - s2) * fx_rcp(s1 + s2); }
 __device__ __forceinline__ float shape_b(float s1, float s2) { return (s1 - s2) * hw_rcp(s1 + s2); }
 // cosine between q and -(q + p) at |q+p|^2 = A2: (s3-s1-s2)/(2 sqrt(s1 s2)) in
 // FP64; -(q + p c1)/|q + p| in FP32 (q.(q+p) = q (q + p c1), no cancellation)
@@ -948,19 +1049,20 @@ __device__ __forceinline__ float lam3_full(const RhsArgs &a, Row32 L3, float y3,
   const float v10 = line_at(row32_at(r00, da), ps), v11 = line_at(row32_at(r00, da + db), ps);
   return (1.0f - wa) * ((1.0f - wb) * v00 + wb * v01) + wa * ((1.0f - wb) * v10 + wb * v11);
 }
-template <typename T, typename Tab>
-__device__ __forceinline__ T lam3_full(const RhsArgs &a, const Tab *L3, T y3, T us, T uy3, T va, T vb) {
+__device__ __forceinline__ double lam3_full(const RhsArgs &a, const double2 *L3, double y3, Look64 us, FxOff uy3,
+                                            double va, double vb) {
   const int np = a.n_pts, na = a.n_va, nb = a.n_vb;
   int i0, ia, ib;
-  T w, wa, wb;
-  lerp_pos(y3, us, uy3, np, i0, w);
+  double w1, wa, wb;
+  node_of(us.a, us.kc, y3, uy3, i0, w1);
   shape_pos(va, na, ia, wa);
   shape_pos(vb, nb, ib, wb);
-  const Tab *r00 = L3 + (size_t)(ia * nb + ib) * np;
+  const double2 *r00 = L3 + (size_t)(ia * nb + ib) * np + i0;
   const int db = nb > 1 ? np : 0, da = na > 1 ? nb * np : 0;
-  const T v00 = lerp_at(r00, i0, w), v01 = lerp_at(r00 + db, i0, w);
-  const T v10 = lerp_at(r00 + da, i0, w), v11 = lerp_at(r00 + da + db, i0, w);
-  return ((T)1 - wa) * (((T)1 - wb) * v00 + wb * v01) + wa * (((T)1 - wb) * v10 + wb * v11);
+  const double v00 = line64(r00[0], w1), v01 = line64(r00[db], w1);
+  const double v10 = line64(r00[da], w1), v11 = line64(r00[da + db], w1);
+  const double v0 = fma(wb, v01 - v00, v00), v1 = fma(wb, v11 - v10, v10);
+  return fma(wa, v1 - v0, v0);
 }
 
 // lambda3 from the FP32 cell polynomials: the cell index from the three
@@ -1158,7 +1260,8 @@ __device__ __forceinline__ float tp_full_cell_x2(const RhsArgs &a, const SmemLay
 template <typename T, bool POLE, bool FULL = false, bool CELL = false>
 __device__ __forceinline__ RowAcc<T> d4_witem(const RhsArgs &a, const RhsArgs *sa, const SmemLayout<T> &S,
                                            const KConst<T> &kc, int e, int c, int lane) {
-  const T us = kc.us, sy = kc.sy;
+  const auto us = look_scale(a, kc);
+  const T sy = kc.sy;
   const int np = a.n_pts, np_ = a.n_ext_p, npsi = a.n_ext_ang, na1 = a.na1;
   const auto Zt = tab_row(S, 0), L3 = tab_row(S, (FULL ? 2 : 1) * np), L4 = tab_row(S, (FULL ? 1 : 2) * np);
   int block, ip, jp = 0;
@@ -1174,7 +1277,7 @@ __device__ __forceinline__ RowAcc<T> d4_witem(const RhsArgs &a, const RhsArgs *s
     ip = e - np_ - 1 - np_ * npsi;
   }
   const double pd = (block == 0 && ip == np_) ? 0.0 : a.ext_pd[ip];
-  const T p = (T)pd, p2 = p * p;
+  const T p = (T)pd, p2 = square(p);
   const T cpsi = (T)(block == 1 ? a.psi_x[jp] : 1.0), spsi = (T)(block == 1 ? a.psi_s[jp] : 0.0);
   const T C2 = (T)2 * p2 * ((T)1 + cpsi);
   const int o0 = c * a.cr, o1 = min(o0 + a.cr, a.nr);
@@ -1183,7 +1286,7 @@ __device__ __forceinline__ RowAcc<T> d4_witem(const RhsArgs &a, const RhsArgs *s
   RowAcc<T> acc;
   int r = o0 + lane / na1, ia = lane % na1;
   for (int row = lane; row < rows; row += 32) {
-    const T q = radial_q<T>(a, r), q2 = q * q, qp = q * p, c1 = S.c1[ia];
+    const T q = radial_q<T>(a, r), q2 = square(q), qp = q * p, c1 = S.c1[ia];
     const T A2 = q2 + p2 + (T)2 * qp * c1;   // >= 0 up to rounding; lookups clamp
     const T Ay = A2 * sy;
     const T ZA = look(Zt, Ay, us, kc.uy1, np);
@@ -1203,7 +1306,7 @@ __device__ __forceinline__ RowAcc<T> d4_witem(const RhsArgs &a, const RhsArgs *s
       const T l4 = look(L4, (q2 + A2 + (T)2 * p2) * sy, us, kc.uy4, np);
       v = kc.sw2 * GA * l4 * l4;
     } else {
-      const T uy1 = kc.uy1, uy3 = kc.uy3;
+      const auto uy1 = kc.uy1, uy3 = kc.uy3;
       T la;
       if constexpr (CELL)
         la = lam3_cell(cell32(a, S), (q2 + A2 + p2) * sy, us, uy3, va_shape_a(q, p, c1, q2, A2, p2),
@@ -1293,16 +1396,19 @@ __device__ __forceinline__ double warp_sum(double v) {
 // 0, every stack row).  Block-wide: every thread of the CTA must call it.
 // FP32 line rows do not hold node values, so the FP32 d=3 / d=4 kernels take
 // the signs from the FP64 tables, where the Z rows come first (the FP32 value
-// is the FP64 one times k^2 ln 2 > 0, rounded: the same sign).
-template <typename T>
-__device__ __forceinline__ bool pole_possible(const RhsArgs &a, const SmemLayout<T> &S, const KConst<T> &kc) {
+// is the FP64 one times k^2 ln 2 > 0, rounded: the same sign).  FP64 kernels
+// have no near-pole path.
+__device__ __forceinline__ bool pole_possible(const RhsArgs &a, const SmemLayout<double> &, const KConst<double> &) {
+  return false;
+}
+__device__ __forceinline__ bool pole_possible(const RhsArgs &a, const SmemLayout<float> &S, const KConst<float> &kc) {
   int neg = 0;
   const int nz = (a.model == FFRG_MODEL_D4_FULL ? 1 : a.n_stack) * a.n_pts;
-  if (sizeof(T) == 4 && a.model != FFRG_MODEL_FINITE_T)
+  if (a.model != FFRG_MODEL_FINITE_T)
     for (int i = threadIdx.x; i < nz; i += blockDim.x) neg |= a.tab[i] < 0.0;
   else
-    for (int i = threadIdx.x; i < nz; i += blockDim.x) neg |= table_value(S.tab[i]) < (T)0;
-  return __syncthreads_or(neg) || kc.m2 < (T)0;
+    for (int i = threadIdx.x; i < nz; i += blockDim.x) neg |= S.tab[i].x < 0.0f;
+  return __syncthreads_or(neg) || kc.m2 < 0.0f;
 }
 
 // Output of external point e from the sum s of its partials: diagram
@@ -1361,7 +1467,7 @@ __device__ __forceinline__ void item_loop(const RhsArgs &a, const RhsArgs *sa, c
 }
 
 template <int MODEL, typename T>
-__global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) rhs_main(RhsArgs a) {
+__global__ void __launch_bounds__(kMainThreads<T>, MinBlocks<T>::value) rhs_main(RhsArgs a) {
   if (skipped(a)) {   // wait all the same: this kernel completes after its precompute
     pdl_wait();
     return;
@@ -1372,8 +1478,9 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) rhs_main(RhsArg
   if (threadIdx.x == 0) sa = a;
   SmemLayout<T> S(smem, a);
   if (!main_prologue<T>(a, S, &bar)) return;
-  const KConst<T> kc = load_kconst<T>(a);
-  const bool pole = pole_possible<T>(a, S, kc);
+  KConst<T> kc = load_kconst<T>(a);
+  if constexpr (sizeof(T) == 8) kc.us = S.fx;
+  const bool pole = pole_possible(a, S, kc);
   if constexpr (MODEL == FFRG_MODEL_FINITE_T) {
     // K rows: items (stack row, |p|) x chunk of radial nodes from the counter
     const int lane = threadIdx.x & 31;
@@ -1383,11 +1490,11 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) rhs_main(RhsArg
       d = __shfl_sync(0xffffffffu, d, 0);
       if (d >= a.n_items) break;
       const int outer = d / a.n_chunks, c = d - outer * a.n_chunks;
-      if (pole) ftk_rows<T, true>(a, &sa, S, kc, outer, c, lane);
+      if (sizeof(T) == 4 && pole) ftk_rows<T, true>(a, &sa, S, kc, outer, c, lane);
       else ftk_rows<T, false>(a, &sa, S, kc, outer, c, lane);
     }
   } else {
-    if (pole) item_loop<MODEL, T, true>(a, &sa, S, kc);
+    if (sizeof(T) == 4 && pole) item_loop<MODEL, T, true>(a, &sa, S, kc);
     else item_loop<MODEL, T, false>(a, &sa, S, kc);
   }
 }
@@ -1406,7 +1513,7 @@ __global__ void __launch_bounds__(kThreadsWide, 1) rhs_main_cell(RhsArgs a) {
   SmemLayout<float> S(smem, a);
   if (!main_prologue<float>(a, S, &bar)) return;
   const KConst<float> kc = load_kconst<float>(a);
-  const bool pole = pole_possible<float>(a, S, kc);
+  const bool pole = pole_possible(a, S, kc);
   if (pole) item_loop<kModelD4FullCell, float, true>(a, &sa, S, kc);
   else item_loop<kModelD4FullCell, float, false>(a, &sa, S, kc);
 }
@@ -1629,7 +1736,11 @@ int precompute_blocks(const RhsArgs &a, int cap) {
   return std::max(1, std::min(n_rt * n_nb + (flat + kThreads - 1) / kThreads, cap));
 }
 
-int launch_precompute(ffrg_ctx *ctx, const RhsArgs &a, cudaStream_t s) {
+int launch_precompute(ffrg_ctx *ctx, const RhsArgs &a_in, cudaStream_t s) {
+  RhsArgs a = a_in;   // radial factors only: no kernel-precision tables or constants
+  a.fp64 = 1;
+  a.tab64 = nullptr;
+  a.kconst = nullptr;
   precompute_kernel<<<precompute_blocks(a, 4 * ctx->num_sms), kThreads, 0, s>>>(a);
   return set_cuda_error(ctx, cudaGetLastError(), "precompute launch");
 }
@@ -1644,7 +1755,10 @@ int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int 
   Plan *pl = const_cast<Plan *>(pl_c);
   const bool mixed = precision == FFRG_MIXED;
   RhsArgs a = a_in;  // forward geometry of this precision
+  a.fp64 = !mixed;
   if (!mixed) {
+    a.fx = fx_device_tables(ctx->device);
+    if (!a.fx) return set_cuda_error(ctx, cudaGetLastError(), "function tables");
     a.cr = pl->fcr64;
     a.n_chunks = pl->fn_chunks64;
     a.n_items = pl->fn_items64;
@@ -1657,6 +1771,10 @@ int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int 
   if (!mixed && smem > kMaxDynSmem) {   // FP64 tables beyond shared memory: read from L2
     a.tab_global = 1;
     smem = pl->smem64g;
+    if (!a.tab64) {
+      ctx->last_error = "plan without FP64 line-form tables";
+      return FFRG_ENOMEM;
+    }
   }
   void (*kern)(RhsArgs) = nullptr;
   switch (a.model) {
@@ -1669,7 +1787,7 @@ int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int 
     break;
   default: kern = mixed ? rhs_main<FFRG_MODEL_FINITE_T, float> : rhs_main<FFRG_MODEL_FINITE_T, double>; break;
   }
-  int threads = kThreads;
+  int threads = mixed ? kThreads : kThreads64;
   if (mixed && a.model == FFRG_MODEL_D4_FULL && a.l3cell) {
     kern = rhs_main_cell;
     threads = kThreadsWide;
@@ -1795,7 +1913,7 @@ __global__ void __launch_bounds__(kThreads, 4)
     stage_angles<float>(sa, S);
     __syncthreads();
     const KConst<float> kc = load_kconst<float>(sa);
-    const bool pole = pole_possible<float>(sa, S, kc);
+    const bool pole = pole_possible(sa, S, kc);
     for (int g = lo + warp; g < hi; g += nw) {
       const int item = g - start[f];
       const int e = item / sa.n_chunks, c = item - e * sa.n_chunks;

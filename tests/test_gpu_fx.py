@@ -1,0 +1,53 @@
+"""FP64 right-hand sides at the edges of the fixed-point functions: grids and scales beyond their range (FP64
+logarithms instead), the smallest tables, tables too large for shared memory, the flat regulator's kink, and
+mass terms near the propagator pole; against the CPU oracle at the FP64 bar of the other tests."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import ffrg_inputs as fi
+import oracle
+from gpu_common import gpu_context
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = gpu_context()
+    yield c
+    c.close()
+
+
+def _grid(wl, lo, hi):
+    wl.problem = dataclasses.replace(wl.problem, x_min=lo, x_max=hi, p_min=lo, p_max=hi)
+    return wl
+
+
+CASES = {
+    "k above fixed point": lambda: (fi.make_d3(seed=1, n_ext_p=5, n_rad=16, n_ang=8), 3e9),
+    "k below fixed point": lambda: (fi.make_d3(seed=2, n_ext_p=5, n_rad=16, n_ang=8), 2e-10),
+    "grid below fixed point": lambda: (_grid(fi.make_d3(seed=3, n_ext_p=5, n_rad=16, n_ang=8), 1e-20, 10.0), 0.3),
+    "two nodes": lambda: (fi.make_d3(seed=4, n_pts=2, n_ext_p=3, n_rad=9, n_ang=5), 1.0),
+    "tables in global memory": lambda: (fi.make_d4(seed=5, n_pts=4000, n_ext_ang=1, n_rad=2, n_ang1=2, n_ang2=2), 1.0),
+    "finite T tables in global memory": lambda: (fi.make_finite_t(seed=6, N=40, T=0.02, n_pts=160, n_ext_p=2, n_rad=8,
+                                                                  n_ang=5), 0.7),
+    "flat regulator": lambda: (fi.make_d3(seed=7, n_ext_p=9, n_rad=31, n_ang=11, regulator=fi.REG_LITIM), 1.0),
+    "near the pole": lambda: (fi.make_d3(seed=8, n_ext_p=9, n_rad=16, n_ang=8, m2_over_k2=-0.97), 0.5),
+    # the shape variables cancel the squares of legs 1e5 apart in length (an error of u p / q unless both sides
+    # round the squares alike)
+    "full vertex, small k": lambda: (fi.make_d4_full(seed=9, n_pts=12, n_va=3, n_vb=2, n_ext_ang=2, n_rad=8, n_ang1=6,
+                                                     n_ang2=4), 1e-4),
+}
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_fp64_at_the_edges(ctx, case):
+    import paper_2412_13043_gb300 as ffrg
+    wl, k = CASES[case]()
+    tabs = ctx.tables(wl.problem, wl.tables)
+    got = ctx.rhs(wl.problem, tabs, k, precision=ffrg.FP64).cpu().numpy()
+    tabs.free()
+    ref = oracle.rhs(wl.problem, wl.tables, k)
+    assert np.max(np.abs(got - ref) / np.abs(ref)) < 1e-12
