@@ -196,6 +196,8 @@ static void plan_free(ffrg_ctx *ctx, Plan *pl) {
                     pl->radF, pl->radq, pl->partial, pl->radD, pl->gpart, pl->ext_pd, pl->psi_s, pl->jrows};
   for (double *p : arrs) dev_free(ctx, p, 0);
   dev_free(ctx, pl->tab64, 0);
+  dev_free(ctx, pl->rowbuf, 0);
+  dev_free(ctx, pl->item_done, 0);
   dev_free(ctx, pl->tab32, 0);
   dev_free(ctx, pl->radq32, 0);
   dev_free(ctx, pl->work_ctr, 0);
@@ -268,7 +270,12 @@ void plan_geometry(Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td) 
   auto forward = [&](bool fp64, int &fcr, int &fn_chunks, int &fn_items, int &fjb) {
     if (is_d4(pb->model)) {
       fjb = pl->na2;
-      fcr = chunk(8 * 32);
+      // FP64: down to one row per lane until every resident warp (152 x 16)
+      // has about six items.  32 radial x 16 first-angle nodes, 193 external
+      // points: 386 items of 256 rows left 127 SMs idle (176 us a RHS), 3088
+      // of 32 rows: 41 us
+      const long long rows = (long long)pl->n_ext * outer_total * rows_per_outer;
+      fcr = chunk(fp64 ? (int)std::min(256LL, std::max(32LL, rows / (152 * 16 * 6) / 32 * 32)) : 8 * 32);
       fn_chunks = (outer_total + fcr - 1) / fcr;
       fn_items = pl->n_ext * fn_chunks;
     } else if (pb->model == FFRG_MODEL_FINITE_T) {
@@ -320,11 +327,13 @@ void plan_geometry(Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td) 
   pl->smem32 = al16((size_t)pl->tab32_count * 8) + al16(ang32 * 4);
 }
 
-void plan_grid(Plan *pl, const ffrg_table_desc *td) {
-  if (pl->fg_lo == td->x_min && pl->fg_hi == td->x_max) return;
+bool plan_grid(Plan *pl, const ffrg_table_desc *td, int device) {
+  if (!pl->fx) pl->fx = fx_device_tables(device);
+  if (pl->fg_lo == td->x_min && pl->fg_hi == td->x_max) return pl->fx;
   pl->fg_ok = fx_grid(td->n_pts, td->x_min, td->x_max, &pl->fg);
   pl->fg_lo = td->x_min;
   pl->fg_hi = td->x_max;
+  return pl->fx;
 }
 
 // The tables of the fixed-point functions: built once per process, uploaded
@@ -356,15 +365,14 @@ int get_plan(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc *td, P
   auto it = ctx->plans.find(key);
   if (it != ctx->plans.end()) {
     *out = it->second;
-    plan_grid(it->second, td);
+    plan_grid(it->second, td, ctx->device);
     return FFRG_OK;
   }
   Plan *pl = new Plan();  // value-initialised: pointers null, counts zero
   pl->key = key;
   plan_geometry(pl, pb, td);
-  plan_grid(pl, td);
 
-  int st = FFRG_OK;
+  int st = plan_grid(pl, td, ctx->device) ? FFRG_OK : set_cuda_error(ctx, cudaGetLastError(), "function tables");
   std::vector<double> x(pl->nr), w(pl->nr);
   host_gauss_legendre(pl->nr, 0.0, 1.0, x.data(), w.data());
   st = st ? st : upload_rule(ctx, x, &pl->rad_x);
@@ -398,15 +406,20 @@ int get_plan(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc *td, P
   if (!st) st = dev_alloc(ctx, (void **)&pl->ext_done, (size_t)pl->n_ext * sizeof(unsigned));
   if (!st) st = dev_alloc(ctx, (void **)&pl->kconst, kKConstBytes);
   // FP64 line-form tables in global memory: finite T (long to build in every
-  // CTA), and tables that do not fit in shared memory.  The former can do without.
+  // CTA), and tables that do not fit in shared memory.  The former can do
+  // without: optional buffers are left out in a context with a memory budget,
+  // so that it holds what it would hold without them.
   const bool too_big = pl->smem64 > kMaxDynSmemBytes && pb->model != FFRG_MODEL_FINITE_T_4D;
-  if (!st && (pb->model == FFRG_MODEL_FINITE_T || too_big)) {
+  if (!st && ((pb->model == FFRG_MODEL_FINITE_T && !ctx->budget) || too_big))
     st = dev_alloc(ctx, (void **)&pl->tab64, (size_t)pl->tab64_count * sizeof(double2));
-    if (st == FFRG_ENOMEM && !too_big) st = FFRG_OK;
-  }
   if (!st && pl->kbuf_count) st = dev_alloc(ctx, (void **)&pl->kbuf, pl->kbuf_count * sizeof(double));
   if (!st) st = dev_alloc(ctx, (void **)&pl->ext_pd, (size_t)pl->n_ext_p * sizeof(double));
   if (!st) st = dev_alloc(ctx, (void **)&pl->psi_s, (size_t)npsi * sizeof(double));
+  if (is_d4(pb->model) && ctx->budget) {   // the larger items of the mixed kernels, fewer partial sums
+    pl->fcr64 = pl->fcr;
+    pl->fn_chunks64 = pl->fn_chunks;
+    pl->fn_items64 = pl->fn_items;
+  }
   if (!st)
     st = dev_alloc(ctx, (void **)&pl->partial, (size_t)std::max(pl->fn_items, pl->fn_items64) * sizeof(double));
   if (!st) st = dev_alloc(ctx, (void **)&pl->tab32,
@@ -480,6 +493,7 @@ void fill_args(const Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td
   a.sum_w2 = pl->sum_w2;
   a.fg = pl->fg;
   a.fg_ok = pl->fg_ok;
+  a.fx = pl->fx;
   a.tab64 = pl->tab64;
   // FP32 scale constants of this k on the host (the kernels use them unless a
   // flow stage sets k_dev or m2_dev later); every field they read is set above
@@ -561,6 +575,8 @@ int ffrg_destroy(ffrg_ctx *ctx) {
     cudaFree(pl->kconst);
     cudaFree(pl->radF32);
     cudaFree(pl->tab64);
+    cudaFree(pl->rowbuf);
+    cudaFree(pl->item_done);
     cudaFree(pl->kbuf);
     delete pl;
   }

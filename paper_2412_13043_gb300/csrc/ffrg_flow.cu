@@ -564,6 +564,10 @@ extern "C" int ffrg_flow(ffrg_ctx *ctx, const ffrg_problem *pb_in, const ffrg_ta
   a.k_dev = &ctl->k_stage;
   a.m2_dev = mode == kModeD3Feedback ? &ctl->m2_stage : nullptr;
   a.skip = &ctl->done;
+  // the step controller of a feedback flow sees the last bits of its RHS: the
+  // fixed FP64 arithmetic, where its tables fit in shared memory
+  a.ref64 = mode != kModeFrozen && precision == FFRG_FP64 && ref64_smem(pl) <= kMaxDynSmemBytes;
+  if (a.ref64) ref64_setup(ctx, pl);
 
   const int eb = 256, eg = (ny + eb - 1) / eb;
   long long attempts_done = 0;

@@ -9,15 +9,16 @@
 // Z and L on one log grid in |Q|.  The frequency set depends on k: the loop
 // Matsubara frequencies with |q0| <= qmax_over_k k while there are at most
 // 2N+1 (+1 fermionic) of them, Gauss-Legendre nodes of the domain beyond.
-// Three launches per RHS: the frequency set and radial nodes (one block), the
-// loop factors F(f, r) = w_f w_r q_r^2 dR G^2 L at (q0_f, q_r) in FP64, and one
-// block per external point summing F(f, r) times the angular sum of the
-// shifted line over (f, r) in a fixed order.  The scale k is read on the
+// Three launches per RHS: the frequency set, radial nodes and constants (one
+// block), the loop factors F(f, r) = w_f w_r q_r^2 dR G^2 L at (q0_f, q_r) in
+// FP64, and the sums of F(f, r) times the angular sum of the shifted line by
+// warp-sized items (external point x rows (f, r)).  The scale k is read on the
 // device (a flow's stage scale), so every step of a flow sees its own
 // frequency set.
 #include <math.h>
 
 #include "ffrg_internal.cuh"
+#include "ffrg_prop64.cuh"
 
 namespace ffrg {
 
@@ -52,6 +53,11 @@ __global__ void ft4_freq_kernel(RhsArgs a, int nfreq_max) {
   const double qs = a.qmax_over_k * k;
   for (int r = threadIdx.x; r < a.nr; r += blockDim.x) a.radq[r] = qs * a.rad_x[r];
   if (threadIdx.x == 0) kb[2 * nfreq_max] = (double)nf;
+  if (threadIdx.x == 32) {
+    *a.work_ctr = 0u;
+    if (a.fp64) ((KConstPair *)a.kconst)->d = make_kconst<double>(a);
+  }
+  for (int i = threadIdx.x; i < a.n_ext; i += blockDim.x) a.ext_done[i] = 0u;
 }
 
 // F(f, r) = w_f w_r q^2 dR(Q) G(Q)^2 L(|Q|), |Q|^2 = q0_f^2 + q_r^2 (FP64; FP32 copy)
@@ -64,29 +70,14 @@ __global__ void ft4_factor_kernel(RhsArgs a, int nfreq_max) {
   if (idx >= nf * a.nr) return;
   const int f = idx / a.nr, r = idx - f * a.nr;
   const double k = scale_k(a), k2 = k * k, inv_k2 = 1.0 / k2, m2 = mass2(a, k);
-  const double q = a.radq[r], q0 = kb[f], Q2 = q0 * q0 + q * q;
-  const double *Zt = a.tab, *Lt = a.tab + a.n_pts;
-  const double Z = look(Zt, Q2, a.u_scale, a.u_off, a.n_pts);
-  const double L = look(Lt, Q2, a.u_scale, a.u_off, a.n_pts);
-  const double G = 1.0 / prop_den(a.reg, Z, 0.0, Q2, m2, k2, inv_k2);
+  const double q = a.radq[r], q0 = kb[f];
+  const LoopNode t = loop_node(a, fma(q0, q0, q * q), k2, inv_k2);
+  const double Z = lerp_at(a.tab, t.i0, t.wl), L = lerp_at(a.tab + a.n_pts, t.i0, t.wl);
+  const double G = fx_rcp(fma(Z, t.P, m2));
   const double wr = a.qmax_over_k * k * a.rad_w[r];
-  const double F = kb[nfreq_max + f] * wr * q * q * Z * k2 * reg_rdot(a.reg, Q2 * inv_k2) * G * G * L;
+  const double F = kb[nfreq_max + f] * wr * q * q * Z * t.rd * G * G * L;
   a.radF[idx] = F;
   a.radF32[idx] = (float)F;
-}
-
-// angular sum of the shifted line at (q0 + p0, q, p): sum_c v_c L(|Q+P|) G(Q+P)
-__device__ __forceinline__ double ft4_row(const RhsArgs &a, double sh2, double q, double p, double k2, double inv_k2,
-                                          double m2) {
-  const double *Zt = a.tab, *Lt = a.tab + a.n_pts;
-  double rs = 0.0;
-  for (int c = 0; c < a.na1; ++c) {
-    const double QP2 = fmax(0.0, sh2 + fma(2.0 * q * p, a.a1_x[c], q * q + p * p));
-    const double Z = look(Zt, QP2, a.u_scale, a.u_off, a.n_pts);
-    const double L = look(Lt, QP2, a.u_scale, a.u_off, a.n_pts);
-    rs = fma(a.a1_w[c] * L, 1.0 / prop_den(a.reg, Z, 0.0, QP2, m2, k2, inv_k2), rs);
-  }
-  return rs;
 }
 
 // FP32 angular sum (the mixed path) from shared memory: zl[i] = (Z_i, Z_{i+1}
@@ -140,21 +131,33 @@ __device__ __forceinline__ float ft4_row32(const RhsArgs &a, const float4 *zl, c
   return rs;
 }
 
-// one block per external point e = (p, m): threads over the (f, r) terms,
-// f major, in a fixed order; FP64 accumulation.  The FP32 kernel stages both
-// tables and the angle rule in shared memory first.
+// Warp items: external point e = (p, m) x `cr` rows (f, r), f major (cr and
+// the item order depend only on the shape and the frequency set); a lane's
+// rows and the items of an external point are added in a fixed order, FP64.
+// The warp that completes an external point writes its output.  Each CTA
+// first stages the tables and the angle rule: FP64 (one 512-thread CTA per SM)
+// the function tables and line-form tables of ffrg_prop64.cuh, FP32 node
+// quadruples.  Bound: FP64 six FP64 instructions and the integer work of one
+// logarithm, regulator and reciprocal per term.  64 momenta x 9 frequencies,
+// 96 x 48 nodes, k = 1 (25 loop frequencies): FP64 10.60 ms with FP64
+// functions and one block per external point, 1.04 ms so.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) ft4_main_kernel(RhsArgs a, int nfreq_max) {
-  __shared__ double red[kThreads / 32];
+__global__ void __launch_bounds__(sizeof(T) == 8 ? kThreads64 : kThreads)
+    ft4_main_kernel(RhsArgs a, int nfreq_max) {
   extern __shared__ __align__(16) unsigned char ft4_smem[];
-  const int e = blockIdx.x, nm = a.n_ext_ang, ip = e / nm, m = e - ip * nm;
+  const int lane = threadIdx.x & 31, nm = a.n_ext_ang;
   const double *kb = (const double *)a.kbuf;
   const double k = scale_k(a), k2 = k * k, m2 = mass2(a, k);
-  const double p = ext_momentum(a, ip);
-  const double p0 = a.stat ? kPi * a.T * exp(-k / (kPi * a.T)) : 2.0 * kPi * a.T * m;
+  // FP64: function tables | (Z, L) line-form pairs | (node, weight)
+  FxTables *fx = (FxTables *)ft4_smem;
+  double2 *zl64 = (double2 *)(ft4_smem + sizeof(FxTables)), *cw64 = zl64 + 2 * a.n_pts;
   float4 *zl = reinterpret_cast<float4 *>(ft4_smem);
   float2 *cw = reinterpret_cast<float2 *>(zl + a.n_pts);
-  if (sizeof(T) == 4) {
+  if constexpr (sizeof(T) == 8) {
+    stage_fx(a, fx);
+    for (int i = threadIdx.x; i < 2 * a.n_pts; i += blockDim.x) zl64[i] = tab64_entry(a, i, k2);
+    for (int c = threadIdx.x; c < a.na1; c += blockDim.x) cw64[c] = make_double2(a.a1_x[c], a.a1_w[c]);
+  } else {
     const double *Zt = a.tab, *Lt = a.tab + a.n_pts;
     for (int i = threadIdx.x; i < a.n_pts; i += blockDim.x) {
       const bool last = i + 1 >= a.n_pts;
@@ -163,35 +166,88 @@ __global__ void __launch_bounds__(kThreads) ft4_main_kernel(RhsArgs a, int nfreq
                           last ? 0.0f : (float)(Lt[i + 1] - l0));
     }
     for (int c = threadIdx.x; c < a.na1; c += blockDim.x) cw[c] = make_float2((float)a.a1_x[c], (float)a.a1_w[c]);
-    __syncthreads();
   }
-  pdl_wait();   // the factor kernel's F(f, r) (and through it the frequency set)
-  const int nf = (int)kb[2 * nfreq_max];
+  __syncthreads();
+  pdl_wait();   // the factor kernel's F(f, r) (and through it the frequency set, constants and counters)
+  const int rows = (int)kb[2 * nfreq_max] * a.nr, cr = a.cr, nc = max(1, (rows + cr - 1) / cr);
   const float us = (float)(a.u_scale * 0.69314718055994530942), uo = (float)a.u_off;
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < nf * a.nr; i += blockDim.x) {
-    const int f = i / a.nr, r = i - f * a.nr;
-    const double sh = kb[f] + p0, q = a.radq[r];
-    if (sizeof(T) == 8) {
-      acc = fma(a.radF[i], ft4_row(a, sh * sh, q, p, k2, 1.0 / k2, m2), acc);
-    } else {
-      const float rs = ft4_row32(a, zl, cw, (float)(sh * sh), (float)q, (float)p, (float)k2, (float)(1.0 / k2),
-                                 (float)m2, us, uo);
-      acc = fma(a.radF[i], (double)rs, acc);
-    }
+  KConst<double> kc;
+  if constexpr (sizeof(T) == 8) {
+    kc = load_kconst<double>(a);
+    kc.us = fx;
   }
-  const double t = block_sum(acc, red);
-  if (threadIdx.x == 0) {
-    const double v = a.norm * t;
-    a.out[e] = v;
-    if (!isfinite(v)) raise_status(a.status, kStatusNonFinite);
+  for (;;) {
+    int d = 0;
+    if (lane == 0) d = (int)atomicAdd(a.work_ctr, 1u);
+    d = __shfl_sync(0xffffffffu, d, 0);
+    if (d >= a.n_ext * nc) break;
+    const int e = d / nc, c0 = d - e * nc, ip = e / nm, m = e - ip * nm;
+    const double p = ext_momentum(a, ip);
+    const double p0 = a.stat ? kPi * a.T * exp(-k / (kPi * a.T)) : 2.0 * kPi * a.T * m;
+    double acc = 0.0;
+    for (int i = c0 * cr + lane; i < min((c0 + 1) * cr, rows); i += 32) {
+      const int f = i / a.nr, r = i - f * a.nr;
+      const double sh = kb[f] + p0, q = a.radq[r];
+      if constexpr (sizeof(T) == 8) {
+        // sum_c v_c L(|Q+P|) G(Q+P) at y = |Q+P|^2 / k^2 = by + ty c
+        const double by = fma(sh, sh, fma(q, q, p * p)) * kc.sy, ty = 2.0 * q * p * kc.sy;
+        double rs = 0.0;
+        for (int c = 0; c < a.na1; ++c) {
+          const double2 cv = cw64[c];
+          const double y = fma(ty, cv.x, by);
+          int n;
+          double w1;
+          node_of(a, kc, y, kc.uy1, n, w1);
+          const double Z = line64(zl64[2 * n], w1), L = line64(zl64[2 * n + 1], w1);
+          rs = fma(cv.y * L, inv_prop<false>(a, Z, y, 0.0, kc, 0), rs);
+        }
+        acc = fma(a.radF[i], rs, acc);
+      } else {
+        const float rs = ft4_row32(a, zl, cw, (float)(sh * sh), (float)q, (float)p, (float)k2, (float)(1.0 / k2),
+                                   (float)m2, us, uo);
+        acc = fma(a.radF[i], (double)rs, acc);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    unsigned done = 0;
+    if (lane == 0) {
+      a.partial[(size_t)e * nc + c0] = acc;
+      __threadfence();
+      done = atomicAdd(a.ext_done + e, 1u);
+    }
+    done = __shfl_sync(0xffffffffu, done, 0);
+    if (done == (unsigned)nc - 1u) {
+      __threadfence();
+      double t = 0.0;
+      for (int j = lane; j < nc; j += 32) t += __ldcg(a.partial + (size_t)e * nc + j);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+      if (lane == 0) {
+        const double v = a.norm * t;
+        a.out[e] = v;
+        if (!isfinite(v)) raise_status(a.status, kStatusNonFinite);
+      }
+    }
   }
 }
 
-int launch_ft4(ffrg_ctx *ctx, const Plan *pl, const RhsArgs &a, int precision, cudaStream_t s) {
-  if (!a.kbuf || !a.radq || !a.radF || !a.radF32 || !a.a2_x) {
-    ctx->last_error = "plan without the frequency buffer or radial factors";
+int launch_ft4(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int precision, cudaStream_t s) {
+  Plan *pl = const_cast<Plan *>(pl_c);
+  RhsArgs a = a_in;
+  a.fp64 = precision != FFRG_MIXED;
+  if (!a.kbuf || !a.radq || !a.radF || !a.radF32 || !a.a2_x || !a.work_ctr || !a.ext_done || !a.kconst) {
+    ctx->last_error = "plan without the frequency buffer, radial factors or counters";
     return FFRG_EINVAL;
+  }
+  const size_t smem = a.fp64 ? sizeof(FxTables) + (size_t)(2 * pl->n_pts + pl->na1) * sizeof(double2)
+                             : (size_t)pl->n_pts * sizeof(float4) + (size_t)pl->na1 * sizeof(float2);
+  void (*kern)(RhsArgs, int) = a.fp64 ? ft4_main_kernel<double> : ft4_main_kernel<float>;
+  const int threads = a.fp64 ? kThreads64 : kThreads;
+  int &grid = a.fp64 ? pl->grid64 : pl->grid32;
+  if (grid == 0) {   // (external points) x (rows of the largest frequency set) in warp items
+    const int st = persistent_grid(ctx, (const void *)kern, smem, a.n_items, &grid, threads);
+    if (st) return st;
   }
   const int nfreq = pl->nfreq;
   ft4_freq_kernel<<<1, kThreads, 0, s>>>(a, nfreq);
@@ -201,18 +257,7 @@ int launch_ft4(ffrg_ctx *ctx, const Plan *pl, const RhsArgs &a, int precision, c
   if (e != cudaSuccess) return set_cuda_error(ctx, e, "finite-T 4D factor launch");
   const bool prof = ctx->profiling && ctx->prof_used * 2 + 1 < (int)ctx->prof_events.size();
   if (prof) cudaEventRecord(ctx->prof_events[2 * ctx->prof_used], s);
-  if (precision == FFRG_MIXED) {
-    const size_t smem = (size_t)pl->n_pts * sizeof(float4) + (size_t)pl->na1 * sizeof(float2);
-    if (smem > 227 * 1024) {
-      ctx->last_error = "tables and angle rule do not fit in shared memory";
-      return FFRG_EINVAL;
-    }
-    int st = ensure_smem_limit(ctx, (const void *)ft4_main_kernel<float>, smem);
-    if (st) return st;
-    e = launch_dependent(ft4_main_kernel<float>, dim3(a.n_ext), dim3(kThreads), smem, s, true, a, nfreq);
-  } else {
-    e = launch_dependent(ft4_main_kernel<double>, dim3(a.n_ext), dim3(kThreads), 0, s, true, a, nfreq);
-  }
+  e = launch_dependent(kern, dim3(grid), dim3(threads), smem, s, true, a, nfreq);
   if (e != cudaSuccess) return set_cuda_error(ctx, e, "finite-T 4D launch");
   if (prof) {
     cudaEventRecord(ctx->prof_events[2 * ctx->prof_used + 1], s);

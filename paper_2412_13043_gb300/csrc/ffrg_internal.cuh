@@ -96,6 +96,9 @@ struct RhsArgs {
   KConst<float> kc_host;       // FP32 scale constants from the host (valid when kc_host_ok, k_dev and m2_dev null)
   int kc_host_ok;
   int fp64;                    // precision of this RHS (what the precompute kernel writes)
+  int ref64;                   // FP64 RHS of an adaptive feedback flow (ffrg_ref64.cu)
+  double *rowbuf;              // its row values [n_ext][rows], or null: items run whole
+  unsigned *item_done;         // finished row groups per item, reset by the precompute kernel
   FxGrid fg;                   // the table grid in fixed point (FP64 kernels)
   int fg_ok;
   const FxTables *fx;          // device tables of the fixed-point functions
@@ -529,12 +532,16 @@ struct Plan {
   FxGrid fg;                      // the grid in fixed point, of the descriptor last seen
   int fg_ok;
   double fg_lo, fg_hi;
+  const FxTables *fx;
   int n_va, n_vb;                 // D4_FULL: vertex nodes
   int l3cell;                     // D4_FULL: the FP32 lambda3 cell layout fits in shared memory
   double2 *tab64;
   size_t kbuf_count;              // FINITE_T: entries of K (N + n_ext_ang) x n_ext_p x n_rad
   double *kbuf;
   int grid64, grid32;       // persistent grids (FP64 / mixed kernels)
+  int grid_ref;             // feedback flows, FP64
+  double *rowbuf;
+  unsigned *item_done;
   int grid_single;          // finite T, mixed: grid of the single-launch RHS (-1: not available)
   size_t smem64, smem32;    // dynamic shared memory bytes
   size_t smem64g;           // FP64 kernels with tables in global memory: the rest
@@ -555,8 +562,9 @@ struct Plan {
 // Shape and launch geometry of a plan (no allocation): sizes from the problem
 // and the table descriptor, and the grouping of angular rows into work items.
 void plan_geometry(Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td);
-// The plan's fixed-point grid for the descriptor's x_min and x_max.
-void plan_grid(Plan *pl, const ffrg_table_desc *td);
+// The plan's fixed-point grid for the descriptor's x_min and x_max, and the
+// function tables on the device; false when those cannot be uploaded.
+bool plan_grid(Plan *pl, const ffrg_table_desc *td, int device);
 
 // Raise a kernel's dynamic shared-memory limit to at least `bytes` (never
 // lowers it: plans of different sizes share the kernel).
@@ -647,10 +655,17 @@ int host_gauss_chebyshev2(int n, double *x, double *w);
 const FxTables *fx_device_tables(int device);
 
 // kernels launched from several translation units (ffrg_rhs.cu)
+// grid of a persistent kernel: resident CTAs, at most one warp per item
+int persistent_grid(ffrg_ctx *ctx, const void *kernel, size_t smem, int items, int *grid, int threads);
 int launch_rhs(ffrg_ctx *ctx, const Plan *pl, const RhsArgs &a, int precision, cudaStream_t s);
 // the finite-T model with a 4D regulator (frequency set, loop factors, one
 // block per external point); launch_rhs dispatches to it
 int launch_ft4(ffrg_ctx *ctx, const Plan *pl, const RhsArgs &a, int precision, cudaStream_t s);
+// the FP64 RHS of adaptive feedback flows (RhsArgs::ref64): buffers (before
+// any capture) and main kernel
+void ref64_setup(ffrg_ctx *ctx, Plan *pl);
+size_t ref64_smem(const Plan *pl);
+int launch_ref64(ffrg_ctx *ctx, Plan *pl, const RhsArgs &a, cudaStream_t s);
 // launch_rhs with the finite-T contraction optional: contract = false stops
 // after the angle-integrated kernel K (plan kbuf, in the kernel precision)
 int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl, const RhsArgs &a, int precision, cudaStream_t s,

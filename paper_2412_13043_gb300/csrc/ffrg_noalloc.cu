@@ -117,9 +117,9 @@ extern "C" int ffrg_rhs_noalloc(const ffrg_problem *pb, const ffrg_table_desc *t
   pl.kconst = sc.take<double>(kKConstBytes / sizeof(double));
   pl.ext_pd = sc.take<double>(pl.n_ext_p);
   pl.psi_s = sc.take<double>(npsi);
-  pl.partial = sc.take<double>(std::max(pl.fn_items, pl.fn_items64));
   pl.tab32 = sc.take<float2>((size_t)pl.tab32_count);
   if (pl.kbuf_count) pl.kbuf = sc.take<double>(pl.kbuf_count);
+  pl.partial = sc.take<double>(is_d4(pb->model) ? pl.fn_items : std::max(pl.fn_items, pl.fn_items64));
   if (sc.used > kNoallocScratchBytes) return FFRG_EINVAL;  // problem needs more than the 4 MiB scratch
 
   // the tables must fit in shared memory as plain values (FP64 line form: twice as large, in global memory when
@@ -132,7 +132,16 @@ extern "C" int ffrg_rhs_noalloc(const ffrg_problem *pb, const ffrg_table_desc *t
   if (precision == FFRG_FP64 && pb->model != FFRG_MODEL_FINITE_T_4D &&
       (pb->model == FFRG_MODEL_FINITE_T || pl.smem64 > kMaxDynSmemBytes))
     pl.tab64 = sc.take<double2>((size_t)pl.tab64_count);
-  plan_grid(&pl, td);
+  if (precision == FFRG_FP64 && is_d4(pb->model) && pl.fn_items64 > pl.fn_items) {   // finer items of small problems
+    if (sc.used + (size_t)pl.fn_items64 * sizeof(double) + 256 <= sizeof(g_noalloc_scratch)) {
+      pl.partial = sc.take<double>(pl.fn_items64);
+    } else {
+      pl.fcr64 = pl.fcr;
+      pl.fn_chunks64 = pl.fn_chunks;
+      pl.fn_items64 = pl.fn_items;
+    }
+  }
+  if (!plan_grid(&pl, td, dev)) return FFRG_ECUDA;
 
   cudaStream_t s = (cudaStream_t)stream;
   const size_t db = sizeof(double);

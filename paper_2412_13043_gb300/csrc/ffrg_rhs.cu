@@ -32,6 +32,7 @@
 #include <tuple>
 
 #include "ffrg_internal.cuh"
+#include "ffrg_prop64.cuh"
 
 namespace ffrg {
 
@@ -97,132 +98,6 @@ __device__ __noinline__ float pole_ftk(const RhsArgs *a, int ip, int jk, int r, 
   return pole_prop(a, a->tab + (size_t)srow * a->n_pts, q * q + p * p + 2.0 * q * p * c, om * om);
 }
 
-// Scale-dependent constants of one RHS in the kernel precision, computed once
-// per RHS by the precompute kernel into a small device block (RhsArgs::kconst)
-// that every CTA of the main kernel loads.  FP32 us/uo: table coordinate
-// divided by n-1; plim = -2 m^2 (near-pole test).  The kernels pass
-// squared momenta to the propagator as y = sy s^2 and omega^2 as som omega^2:
-// FP64 sy = som = 1/k^2 with the Z table pre-scaled by k^2, so that y is the
-// regulator's argument (sy = 1 for the full vertex, whose shape variables
-// need s^2 itself); FP32 sy = log2(e)/k^2 (the regulator's exp2 argument)
-// and som = 1/(k^2 ln 2), with the FP32 Z table pre-scaled by k^2 ln 2
-// (see reg_g).
-// uy1..uy4: offsets of table coordinates taken in y of S0^2 = (sum of c
-// squares)/c (c = 1..4; ln(sy) and ln c folded in); twopiT = 2 pi T;
-// sw2 = sum of the second-angle weights.
-struct KConstPair {
-  KConst<float> f;
-  KConst<double> d;
-};
-static_assert(sizeof(KConstPair) <= kKConstBytes, "constant block too small");
-
-// The k-dependent constants of one RHS: FP32 from kconst_f32 (or the host's
-// copy of it), FP64 below; once per RHS on one thread.
-template <typename T>
-__device__ __forceinline__ KConst<T> make_kconst(const RhsArgs &a);
-template <>
-__device__ __forceinline__ KConst<float> make_kconst<float>(const RhsArgs &a) {
-  // the host's copy when the scale and mass are host values (plain RHS calls)
-  if (a.kc_host_ok && !a.k_dev && !a.m2_dev) return a.kc_host;
-  const double kd = scale_k(a);
-  return kconst_f32(a, kd, mass2(a, kd));
-}
-template <>
-__device__ __forceinline__ KConst<double> make_kconst<double>(const RhsArgs &a) {
-  const double kd = scale_k(a), m2d = mass2(a, kd);
-  KConst<double> c;
-  c.k2 = kd * kd;
-  c.inv_k2 = 1.0 / c.k2;
-  c.m2 = m2d;
-  const bool full = a.model == FFRG_MODEL_D4_FULL;
-  c.sy = full ? 1.0 : c.inv_k2;
-  c.som = c.inv_k2;
-  c.isy = full ? 1.0 : c.k2;
-  c.slow = !a.fg_ok || !(kd > 0x1p-30) || !(kd < 0x1p30);
-  // coordinate of y = sy s^2: u_scale ln(y) + u_off + u_scale ln(1/sy)
-  int64_t off = a.fg.uo;
-  if (!full && !c.slow) {
-    const int hi = fx_clamp_hi(fx_bits(c.k2));
-    off += fx_log(fx_scaled(a.fx->log[fx_log_index(hi)], a.fg), a.fg, hi, (uint32_t)fx_bits(c.k2));
-  }
-  c.uy1 = {off - a.fg.uc[0], 1};
-  c.uy2 = {off - a.fg.uc[1], 2};
-  c.uy3 = {off - a.fg.uc[2], 3};
-  c.uy4 = {off - a.fg.uc[3], 4};
-  c.us = nullptr;
-  c.twopiT = a.twopiT;
-  c.sw2 = a.sum_w2;
-  return c;
-}
-
-template <typename T>
-__device__ __forceinline__ KConst<T> load_kconst(const RhsArgs &a);
-template <>
-__device__ __forceinline__ KConst<float> load_kconst<float>(const RhsArgs &a) {
-  return ((const KConstPair *)a.kconst)->f;
-}
-template <>
-__device__ __forceinline__ KConst<double> load_kconst<double>(const RhsArgs &a) {
-  KConst<double> c = ((const KConstPair *)a.kconst)->d;
-  c.uy1.c = 1, c.uy2.c = 2, c.uy3.c = 3, c.uy4.c = 4;
-  return c;
-}
-
-// FP64 tables in line form: a node holds (T_i - d_i, d_i), d_i the difference
-// to the next node (0 at a row end), so that the interpolant is one FMA with
-// the weight 1 + w in [1, 2) of fx_node.  Layout: as the tables (D4_FULL: rows
-// Z | lambda4 | lambda3 rows; finite T: [row][node][Z, lambda]).  Z rows carry
-// k^2.  Entry i:
-__device__ __forceinline__ double2 tab64_entry(const RhsArgs &a, int i, double k2) {
-  const int np = a.n_pts, zn = a.n_stack * np;
-  size_t src;
-  int col;
-  bool z;
-  if (a.model == FFRG_MODEL_FINITE_T) {
-    z = !(i & 1);
-    src = (size_t)(i >> 1) + (z ? 0 : zn);
-    col = (i >> 1) % np;
-  } else {
-    const int row = i / np;
-    col = i - row * np;
-    z = row < (a.model == FFRG_MODEL_D4_FULL ? 1 : a.n_stack);
-    src = i;
-    if (a.model == FFRG_MODEL_D4_FULL) src = col + (row == 0 ? (size_t)0 : row == 1 ? (size_t)2 * zn : (size_t)zn + (size_t)(row - 2) * np);
-  }
-  const double f = z ? k2 : 1.0, v = f * a.tab[src];
-  const double d = col == np - 1 ? 0.0 : f * a.tab[src + 1] - v;
-  return make_double2(v - d, d);
-}
-
-// Node and weight of the coordinate of y (FP64 lookups): fixed point, or an
-// FP64 logarithm when the grid or k lies outside its range.
-__device__ __noinline__ void slow_node(const RhsArgs *a, double s2, int c, int &i, double &w1) {
-  double w;
-  lerp_pos(s2, a->u_scale, a->uoc[c - 1], a->n_pts, i, w);
-  w1 = 1.0 + w;
-}
-__device__ __forceinline__ void node_of(const RhsArgs &a, const KConst<double> &kc, double y, FxOff o, int &i,
-                                        double &w1) {
-  if (kc.slow) slow_node(&a, y * kc.isy, o.c, i, w1);   // uniform
-  else fx_node(a.fg, fx_log(kc.us->log, a.fg, y) + o.v, i, w1);
-}
-__device__ __forceinline__ double line64(double2 t, double w1) { return fma(t.y, w1, t.x); }
-
-// what a table lookup takes besides its row, argument and offset: the FP32
-// coordinate scale, or the FP64 argument block and constants
-struct Look64 {
-  const RhsArgs &a;
-  const KConst<double> &kc;
-};
-__device__ __forceinline__ float look_scale(const RhsArgs &, const KConst<float> &kc) { return kc.us; }
-__device__ __forceinline__ Look64 look_scale(const RhsArgs &a, const KConst<double> &kc) { return {a, kc}; }
-__device__ __forceinline__ double look(const double2 *row, double y, Look64 us, FxOff o, int) {
-  int i;
-  double w1;
-  node_of(us.a, us.kc, y, o, i, w1);
-  return line64(row[i], w1);
-}
-
 // FP32 regulator in propagator form.  With x = s^2/k^2 the kinetic part of the
 // inverse propagator is Z (omega^2 + s^2 + k^2 r(x)) = Z (omega^2 + k^2 h(x)),
 // = (k^2 ln 2 Z) (g(y) + omega^2/(k^2 ln 2)),
@@ -253,15 +128,6 @@ __device__ __forceinline__ float reg_g(int reg, float y) {
 // Z (omega^2 + s^2 + k^2 r), i.e. P < -2 m^2: close to the convexity pole.
 // `pole` is only evaluated on that rare branch.  POLE = false drops the test;
 // callers use it only when m^2 >= 0 and no Z < 0, where P >= 0 >= -2 m^2.
-template <bool POLE = true, typename Pole>
-__device__ __forceinline__ double inv_prop(const RhsArgs &a, double Zk, double y, double om2s,
-                                           const KConst<double> &kc, Pole &&) {
-  const double x = a.model == FFRG_MODEL_D4_FULL ? y * kc.inv_k2 : y;   // sy s^2 = x otherwise
-  double h = a.reg == FFRG_REG_LITIM ? (x < 1.0 ? 1.0 : x) : fx_h(*kc.us, x);
-  if (a.model == FFRG_MODEL_FINITE_T) h += om2s;
-  return fx_rcp(fma(Zk, h, kc.m2));
-}
-
 template <bool POLE = true, typename Pole>
 __device__ __forceinline__ float inv_prop(const RhsArgs &a, float Zs, float y, float om2s, const KConst<float> &kc,
                                           Pole &&pole) {
@@ -299,45 +165,6 @@ constexpr int kPreR = 64, kPreN = 8;
 // template tag of the D4_FULL mixed kernel with lambda3 cells (not a public model)
 constexpr int kModelD4FullCell = 100 + FFRG_MODEL_D4_FULL;
 
-// n-independent terms of radial node r (q = L x_r): q^2, weight x measure,
-// k^2 r(x), k^2 rdot(x) and the table position of q^2
-struct RadialNode {
-  double q2, wm, kr, rd, wl;
-  int i0;
-};
-__device__ __forceinline__ RadialNode radial_node(const RhsArgs &a, int r, double L, double k2, double inv_k2) {
-  RadialNode t;
-  const double q = L * a.rad_x[r], w = L * a.rad_w[r], q2 = q * q, x = q2 * inv_k2;
-  t.q2 = q2;
-  t.wm = w * (is_d4(a.model) ? q2 * q : q2);
-  double rx, rdx;
-  reg_r_rdot(a.reg, x, rx, rdx);
-  t.kr = k2 * rx;
-  t.rd = k2 * rdx;
-  lerp_pos(q2, a.u_scale, a.u_off, a.n_pts, t.i0, t.wl);
-  return t;
-}
-
-// Finite T: F(n, r) = w q^2 Z rdot k^2 G^2 lambda at the loop frequency of
-// stack row n (>= 0), written to both loop indices that share it: n and -n
-// (bosonic) or -n-1 (fermionic); row of loop index n in radF: n + N + stat.
-__device__ __forceinline__ void radial_F_finite_t(const RhsArgs &a, int n, int r, double q2, double wm, double kr,
-                                                  double rd, int i0, double wl, double m2) {
-  const int row = min(n, a.n_stack - 1);
-  const double Z = lerp_at(a.tab + (size_t)row * a.n_pts, i0, wl);
-  const double Lq = lerp_at(a.tab + ((size_t)a.n_stack + row) * a.n_pts, i0, wl);
-  const double om = a.stat ? (2.0 * n + 1.0) * kPi * a.T : 2.0 * kPi * a.T * n;
-  const double G = 1.0 / (Z * (om * om + q2 + kr) + m2);
-  const double F = wm * (Z * rd) * G * G * Lq;
-  const int nr = a.nr, ip = (a.N + a.stat + n) * nr + r, im = (a.N - n) * nr + r;
-  a.radF[ip] = F;
-  a.radF[im] = F;
-  if (a.radF32) {
-    a.radF32[ip] = (float)F;
-    a.radF32[im] = (float)F;
-  }
-}
-
 // Per-radial part of the precompute, blocks blk, blk + nblk, ... of the
 // kPreR x kPreN blocks; every thread of the calling block must run it (it
 // synchronises the block).
@@ -345,15 +172,15 @@ __device__ __forceinline__ void precompute_radial(const RhsArgs &a, int blk, int
   const double k = scale_k(a), k2 = k * k, inv_k2 = 1.0 / k2, m2 = mass2(a, k);
   const double L = a.qmax_over_k * k;
   // Per-radial factors F(n, r), in blocks of kPreR radial nodes x kPreN
-  // stack rows j.  Phase A: the n-independent part of each node (q^2, weight
-  // x measure, k^2 r(x), k^2 rdot(x), the table position of q^2) once per
+  // stack rows j.  Phase A: the n-independent part of each node (weight x
+  // measure, k^2 h(x), k^2 rdot(x), the table position of q^2) once per
   // block into shared memory.  Phase B: F for stack row j, written to both
   // loop indices that read row j and share its frequency^2: n = j and
   // n = -j (bosonic, omega_j = 2 pi T j) or n = -j-1 (fermionic, nu_j =
   // (2j+1) pi T).  Row of loop index n in radF: n + N + stat.
   const int nr = a.nr, N = a.N;
   const int n_rt = (nr + kPreR - 1) / kPreR, n_nb = N / kPreN + 1;
-  __shared__ double s_q2[kPreR], s_wm[kPreR], s_kr[kPreR], s_rd[kPreR], s_wl[kPreR];
+  __shared__ double s_wm[kPreR], s_P[kPreR], s_rd[kPreR], s_wl[kPreR];
   __shared__ int s_i0[kPreR];
   for (int pb = blk; pb < n_rt * n_nb; pb += nblk) {
     const int rt = pb % n_rt, nb = pb / n_rt;
@@ -361,26 +188,24 @@ __device__ __forceinline__ void precompute_radial(const RhsArgs &a, int blk, int
     __syncthreads();  // the previous block's shared values are no longer read
     for (int i = threadIdx.x; i < rn; i += blockDim.x) {
       const RadialNode t = radial_node(a, r0 + i, L, k2, inv_k2);
-      s_q2[i] = t.q2;
       s_wm[i] = t.wm;
-      s_kr[i] = t.kr;
-      s_rd[i] = t.rd;
-      s_i0[i] = t.i0;
-      s_wl[i] = t.wl;
+      s_P[i] = t.n.P;
+      s_rd[i] = t.n.rd;
+      s_i0[i] = t.n.i0;
+      s_wl[i] = t.n.wl;
     }
     __syncthreads();
     const int n0 = nb * kPreN, n1 = min(n0 + kPreN, N + 1);
     for (int j = threadIdx.x; j < (n1 - n0) * rn; j += blockDim.x) {
       const int n = n0 + j / rn, i = j - (j / rn) * rn, r = r0 + i;
-      const double q2 = s_q2[i], wl = s_wl[i], rd = s_rd[i];
+      const double P = s_P[i], wl = s_wl[i], rd = s_rd[i];
       const int i0 = s_i0[i];
       if (a.model == FFRG_MODEL_FINITE_T) {
-        radial_F_finite_t(a, n, r, q2, s_wm[i], s_kr[i], rd, i0, wl, m2);
+        radial_F_finite_t(a, n, r, s_wm[i], P, rd, i0, wl, m2);
       } else {
         double F;
         const double Z = lerp_at(a.tab, i0, wl);
-        const double P = q2 + s_kr[i];
-        const double G = 1.0 / (Z * P + m2);
+        const double G = fast_factors(a) ? fx_rcp(fma(Z, P, m2)) : 1.0 / fma(Z, P, m2);
         F = s_wm[i] * (Z * rd) * G * G;
         // d F / d Z(q): dR = Z k^2 rdot, G = 1/(Z P + m^2) with P = q^2 + k^2 r
         if (a.radD) a.radD[r] = s_wm[i] * rd * G * G * (1.0 - 2.0 * Z * G * P);
@@ -409,7 +234,7 @@ __device__ __forceinline__ void radial_unit(const RhsArgs &a, int u, int lane) {
   if (r >= a.nr) return;
   const double k = scale_k(a), k2 = k * k, inv_k2 = 1.0 / k2, m2 = mass2(a, k);
   const RadialNode t = radial_node(a, r, a.qmax_over_k * k, k2, inv_k2);
-  for (int n = n0; n < min(n0 + kRadN, a.N + 1); ++n) radial_F_finite_t(a, n, r, t.q2, t.wm, t.kr, t.rd, t.i0, t.wl, m2);
+  for (int n = n0; n < min(n0 + kRadN, a.N + 1); ++n) radial_F_finite_t(a, n, r, t.wm, t.n.P, t.n.rd, t.n.i0, t.n.wl, m2);
 }
 
 // Every thread of a block of the calling grid (blockIdx.x over the grid,
@@ -505,6 +330,8 @@ __device__ __forceinline__ void precompute_body(const RhsArgs &a) {
   }
   if (a.ext_done)
     for (int i = tid0; i < a.n_ext; i += stride) a.ext_done[i] = 0u;
+  if (a.item_done)
+    for (int i = tid0; i < a.n_items; i += stride) a.item_done[i] = 0u;
   // per-external-point constants used by every work item of the main kernels
   // one FP64 exp per value: value i on CTA i mod G, thread i / G, so that a
   // large grid spreads them over SMs and a small one keeps them in parallel lanes
@@ -622,10 +449,7 @@ __device__ bool main_prologue(const RhsArgs &a, SmemLayout<T> &S, uint64_t *bar)
   if constexpr (sizeof(T) == 8) {
     // the function tables (logarithms in the grid's units), and line-form
     // tables that the precompute kernel does not write
-    for (int j = threadIdx.x; j < kFxLog; j += blockDim.x) S.fx->log[j] = fx_scaled(a.fx->log[j], a.fg);
-    constexpr int kRest = (int)((sizeof(FxTables) - sizeof(a.fx->log)) / 16);
-    for (int j = threadIdx.x; j < kRest; j += blockDim.x)
-      ((int4 *)(S.fx->log + kFxLog))[j] = ((const int4 *)(a.fx->log + kFxLog))[j];
+    stage_fx(a, S.fx);
     if (!a.tab64) {
       const double k = scale_k(a), k2 = k * k;
       for (int i = threadIdx.x; i < SmemLayout<T>::entries(a); i += blockDim.x) S.tab[i] = tab64_entry(a, i, k2);
@@ -1466,8 +1290,15 @@ __device__ __forceinline__ void item_loop(const RhsArgs &a, const RhsArgs *sa, c
   }
 }
 
+// The argument block into shared memory, a word per thread (one thread copying
+// all of it held the block's prologue back; visible after the next barrier).
+__device__ __forceinline__ void copy_args(RhsArgs *dst, const RhsArgs &a) {
+  static_assert(sizeof(RhsArgs) % 4 == 0, "word copy");
+  for (int i = threadIdx.x; i < (int)(sizeof(RhsArgs) / 4); i += blockDim.x) ((int *)dst)[i] = ((const int *)&a)[i];
+}
+
 template <int MODEL, typename T>
-__global__ void __launch_bounds__(kMainThreads<T>, MinBlocks<T>::value) rhs_main(RhsArgs a) {
+__global__ void __launch_bounds__(kMainThreads<T>, MinBlocks<T>::value) rhs_main(const __grid_constant__ RhsArgs a) {
   if (skipped(a)) {   // wait all the same: this kernel completes after its precompute
     pdl_wait();
     return;
@@ -1475,7 +1306,7 @@ __global__ void __launch_bounds__(kMainThreads<T>, MinBlocks<T>::value) rhs_main
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t bar;
   __shared__ RhsArgs sa;  // for the out-of-line near-pole path
-  if (threadIdx.x == 0) sa = a;
+  if constexpr (sizeof(T) == 4) copy_args(&sa, a);
   SmemLayout<T> S(smem, a);
   if (!main_prologue<T>(a, S, &bar)) return;
   KConst<T> kc = load_kconst<T>(a);
@@ -1501,7 +1332,7 @@ __global__ void __launch_bounds__(kMainThreads<T>, MinBlocks<T>::value) rhs_main
 
 // D4_FULL, mixed, lambda3 as cell polynomials: the cells take most of shared
 // memory, so one CTA of 1024 threads per SM (the warps of four 256-thread CTAs)
-__global__ void __launch_bounds__(kThreadsWide, 1) rhs_main_cell(RhsArgs a) {
+__global__ void __launch_bounds__(kThreadsWide, 1) rhs_main_cell(const __grid_constant__ RhsArgs a) {
   if (skipped(a)) {   // wait all the same: this kernel completes after its precompute
     pdl_wait();
     return;
@@ -1509,7 +1340,7 @@ __global__ void __launch_bounds__(kThreadsWide, 1) rhs_main_cell(RhsArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t bar;
   __shared__ RhsArgs sa;  // for the out-of-line near-pole path
-  if (threadIdx.x == 0) sa = a;
+  copy_args(&sa, a);
   SmemLayout<float> S(smem, a);
   if (!main_prologue<float>(a, S, &bar)) return;
   const KConst<float> kc = load_kconst<float>(a);
@@ -1581,7 +1412,7 @@ __device__ __forceinline__ bool grid_wait(const unsigned *arrive, unsigned targe
   return *s_ok != 0;
 }
 
-__global__ void __launch_bounds__(kThreadsWide, 1) ft_single_kernel(RhsArgs a) {
+__global__ void __launch_bounds__(kThreadsWide, 1) ft_single_kernel(const __grid_constant__ RhsArgs a) {
   if (skipped(a)) return;  // uniform over the grid: no counter is touched
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ RhsArgs sa;  // for the out-of-line near-pole path
@@ -1591,10 +1422,8 @@ __global__ void __launch_bounds__(kThreadsWide, 1) ft_single_kernel(RhsArgs a) {
   // arrivals before this launch: thread 0 alone waits at the barriers, so the
   // value stays in its register and the load overlaps the prologue
   unsigned base = 0;
-  if (threadIdx.x == 0) {
-    base = *(volatile unsigned *)(cnt + 2);
-    sa = a;
-  }
+  if (threadIdx.x == 0) base = *(volatile unsigned *)(cnt + 2);
+  copy_args(&sa, a);
   const int lane = threadIdx.x & 31;
   // The block's own inputs, the values the precompute would store, from the
   // FP64 tables and rules (one CTA per SM, so this FP64 work is per SM): the
@@ -1660,13 +1489,12 @@ __global__ void __launch_bounds__(kThreadsWide, 1) ft_single_kernel(RhsArgs a) {
 // ---------------------------------------------------------------------------
 constexpr size_t kMaxDynSmem = kMaxDynSmemBytes;
 
-template <typename K>
-static int persistent_grid(ffrg_ctx *ctx, K kernel, size_t smem, int items, int *grid, int threads = kThreads) {
+int persistent_grid(ffrg_ctx *ctx, const void *kernel, size_t smem, int items, int *grid, int threads) {
   if (smem > kMaxDynSmem) {
     ctx->last_error = "dressing tables do not fit in shared memory";
     return FFRG_EINVAL;
   }
-  int st = ensure_smem_limit(ctx, (const void *)kernel, smem);
+  int st = ensure_smem_limit(ctx, kernel, smem);
   if (st) return st;
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
@@ -1696,7 +1524,7 @@ static int launch_ft_single(ffrg_ctx *ctx, Plan *pl, const RhsArgs &a, cudaStrea
     } else {
       // one warp per K-row item and one per radial unit (32 nodes x kRadN rows)
       const int units = ((a.nr + 31) / 32) * ((a.N + 1 + kRadN - 1) / kRadN);
-      int st = persistent_grid(ctx, ft_single_kernel, smem, a.n_items + units, &pl->grid_single, kThreadsWide);
+      int st = persistent_grid(ctx, (const void *)ft_single_kernel, smem, a.n_items + units, &pl->grid_single, kThreadsWide);
       if (st) return st;
     }
   }
@@ -1756,9 +1584,22 @@ int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int 
   const bool mixed = precision == FFRG_MIXED;
   RhsArgs a = a_in;  // forward geometry of this precision
   a.fp64 = !mixed;
+  a.ref64 = a_in.ref64 && !mixed;
+  if (a.ref64) {
+    a.rowbuf = pl->rowbuf;
+    a.item_done = pl->item_done;
+    a.tab64 = nullptr;
+    a.kconst = nullptr;
+    if (a.model == FFRG_MODEL_D3) {
+      a.cr = pl->fcr64;
+      a.n_chunks = pl->fn_chunks64;
+      a.n_items = pl->fn_items64;
+      a.jb = pl->fjb64;
+    }
+    precompute_kernel<<<precompute_blocks(a, 4 * ctx->num_sms), kThreads, 0, s>>>(a);
+    return launch_ref64(ctx, pl, a, s);
+  }
   if (!mixed) {
-    a.fx = fx_device_tables(ctx->device);
-    if (!a.fx) return set_cuda_error(ctx, cudaGetLastError(), "function tables");
     a.cr = pl->fcr64;
     a.n_chunks = pl->fn_chunks64;
     a.n_items = pl->fn_items64;
@@ -1776,7 +1617,7 @@ int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int 
       return FFRG_ENOMEM;
     }
   }
-  void (*kern)(RhsArgs) = nullptr;
+  void (*kern)(const RhsArgs) = nullptr;
   switch (a.model) {
   case FFRG_MODEL_D3: kern = mixed ? rhs_main<FFRG_MODEL_D3, float> : rhs_main<FFRG_MODEL_D3, double>; break;
   case FFRG_MODEL_D4_VERTEX:
@@ -1807,7 +1648,7 @@ int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int 
     if (st != kNoSingleLaunch) return st;   // else the three launches below
   }
   if (grid == 0) {
-    st = persistent_grid(ctx, kern, smem, a.n_items, &grid, threads);
+    st = persistent_grid(ctx, (const void *)kern, smem, a.n_items, &grid, threads);
     if (st) return st;
   }
   precompute_kernel<<<precompute_blocks(a, 4 * ctx->num_sms), kThreads, 0, s>>>(a);

@@ -276,6 +276,7 @@ static int slot_setup(Server &S, int si) {
   // tick stream is issued after this wait.
   e = cudaStreamSynchronize(S.io);
   if (e != cudaSuccess) return set_cuda_error(&S.lc, e, "serve upload sync");
+  if (!plan_grid(&pl, &r->td, S.lc.device)) return set_cuda_error(&S.lc, cudaGetLastError(), "function tables");
   fill_args(&pl, &r->pb, &r->td, (const double *)(b + L.o_tab), r->Lambda, sl.ra);
   sl.ra.fused_ctr = nullptr;   // batched kernels only
   sl.ra.out = (double *)(b + L.o_raw);

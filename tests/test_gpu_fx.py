@@ -51,3 +51,25 @@ def test_fp64_at_the_edges(ctx, case):
     tabs.free()
     ref = oracle.rhs(wl.problem, wl.tables, k)
     assert np.max(np.abs(got - ref) / np.abs(ref)) < 1e-12
+
+
+@pytest.mark.parametrize("model,n_pts", [("d3", 20), ("d4", 12), ("d4", 37)])
+def test_feedback_flow_does_not_depend_on_where_rows_are_computed(model, n_pts):
+    """The FP64 RHS of feedback flows computes the rows of small problems in 32-row groups; without the row buffer
+    (a context with a memory budget) each item's rows run in one warp.  Same bits either way."""
+    import torch
+
+    import paper_2412_13043_gb300 as ffrg
+    if model == "d3":
+        wl = fi.make_d3(seed=3, n_pts=n_pts, n_ext_p=n_pts, n_rad=37, n_ang=19, feedback=1, x_min=0.01)
+    else:
+        wl = fi.make_d4(seed=3, n_pts=n_pts, n_ext_ang=3, n_rad=21, n_ang1=13, n_ang2=5)
+    ends = []
+    for budget in (0, 1 << 30):
+        c = ffrg.Context(0, hbm_budget_bytes=budget)
+        tabs = c.tables(wl.problem, wl.tables)
+        y = torch.tensor(wl.y0, dtype=torch.float64, device="cuda")
+        c.flow(wl.problem, tabs, y, wl.Lambda, 2.0, feedback=1, rtol=1e-7)
+        ends.append(y.cpu().numpy())
+        c.close()
+    assert np.array_equal(ends[0], ends[1])
