@@ -8,292 +8,286 @@
 // Z(q) dependence of the per-radial factor F (regulator derivative and
 // G(q)^2) enters through dF/dZ(q) times the angular row sum.
 //
-// Determinism: no floating-point atomics.  Each warp accumulates into its own
-// shared-memory copy of the gradient, lanes taking turns in a fixed order;
-// warps are then summed in a fixed order into one partial per CTA, and a
+// Determinism: no floating-point atomics.  Each warp owns C copies of the
+// gradient in shared memory, one per group of 32/C lanes' turn (C a power of
+// two that the launch picks, adjoint_setup): lanes of one turn add to
+// different copies at once, the 32/C turns follow in a fixed order.  The
+// copies are then summed in a fixed order into one partial per CTA, and a
 // second kernel sums the CTA partials in a fixed order.  Results are
 // reproducible run to run for a given GPU (the persistent grid size fixes
-// which items each CTA owns).
+// which rows each warp owns).
+//
+// Bound: the FP64 pipe (16 clocks a warp instruction).  A d=4 inner term has
+// 17 FP64 instructions of value and derivatives, with the fixed-point
+// functions of ffrg_prop64.cuh, and three lookups to scatter, 2 + 4 x 16/C
+// each.  A turn costs a warp's two FP64 adds however few lanes take part, so
+// one lane per turn (C = 1) took longer than the evaluation.  96 points x 4
+// angles, 96 x 48 x 16 nodes: 25.05 ms a VJP with FP64 functions and C = 1,
+// 3.1 ms so (C = 16).
 #include <math.h>
 
 #include <algorithm>
 
 #include "ffrg_internal.cuh"
+#include "ffrg_prop64.cuh"
 
 namespace ffrg {
 
-constexpr int kAdjThreads = 256;
+constexpr int kAdjMaxWarps = 8;
+constexpr int kLam4Copies = 1;   // lambda4 takes part in the one-loop rows of the d=4 blocks only
 
 struct AdjArgs {
   RhsArgs a;
   const double *gbar;  // [n_ext]
   double *gpart;       // [grid][tab_count]
   double *jrows;       // Jacobian mode: one gradient row per work item [n_items][tab_count]
+  int lc;              // log2 of the copies of Z and lambda3
+  int n_wide;          // gradient entries with 2^lc copies (the rest: kLam4Copies)
 };
 
-// Jacobian mode: clear the warp-private gradients before a work item ...
-__device__ __forceinline__ void jac_item_begin(const AdjArgs &A, double *grad) {
-  if (!A.jrows) return;
-  __syncthreads();
-  const int nw = blockDim.x >> 5;
-  for (int i = threadIdx.x; i < nw * A.a.tab_count; i += blockDim.x) grad[i] = 0.0;
-  __syncthreads();
+// doubles of one warp's gradient copies
+__host__ __device__ inline int adj_warp_doubles(const AdjArgs &A) {
+  return (A.n_wide << A.lc) + (A.a.tab_count - A.n_wide) * kLam4Copies;
 }
 
-// ... and sum them (warps in order) into the item's row after it.
-__device__ __forceinline__ void jac_item_end(const AdjArgs &A, const double *grad, int item) {
-  if (!A.jrows) return;
-  __syncthreads();
-  const int nw = blockDim.x >> 5, T = A.a.tab_count;
-  for (int i = threadIdx.x; i < T; i += blockDim.x) {
-    double s = 0.0;
-    for (int w = 0; w < nw; ++w) s += grad[(size_t)w * T + i];
-    A.jrows[(size_t)item * T + i] = s;
-  }
-}
-
-// lanes add in turn: lane 0 first, lane 31 last
-__device__ __forceinline__ void warp_scatter2(double *g, int i0, double v0, double v1, int lane) {
-  for (int l = 0; l < 32; ++l) {
-    if (lane == l && (v0 != 0.0 || v1 != 0.0)) {
-      g[i0] += v0;
-      g[i0 + 1] += v1;
-    }
-    __syncwarp();
-  }
-}
-
-struct LerpPos {
-  int i0;
-  double w;
-};
-
-__device__ __forceinline__ LerpPos pos_of(const RhsArgs &a, double s2) {
-  LerpPos p;
-  lerp_pos(s2, a.u_scale, a.u_off, a.n_pts, p.i0, p.w);
-  return p;
-}
-__device__ __forceinline__ double val_at(const double *t, LerpPos p) { return lerp_at(t, p.i0, p.w); }
-
-// shared memory: tables | angle rules (c1, s1, w1, c2, w2) | per-warp gradients
+// shared memory: function tables | line-form tables | angle rules | per-warp gradient copies
 struct AdjSmem {
-  double *tab, *c1, *s1, *w1, *c2, *w2, *grad;
+  FxTables *fx;
+  double2 *tab, *cw2;
+  double *c1, *s1, *w1, *grad;
   __device__ AdjSmem(unsigned char *base, const RhsArgs &a) {
-    size_t off = ((size_t)a.tab_count * 8 + 15) & ~(size_t)15;
-    tab = (double *)base;
-    c1 = (double *)(base + off);
+    fx = (FxTables *)base;
+    tab = (double2 *)(base + sizeof(FxTables));
+    cw2 = tab + a.tab_count;
+    c1 = (double *)(cw2 + a.na2);
     s1 = c1 + a.na1;
     w1 = s1 + a.na1;
-    c2 = w1 + a.na1;
-    w2 = c2 + a.na2;
-    off += (((size_t)(3 * a.na1 + 2 * a.na2)) * 8 + 15) & ~(size_t)15;
-    grad = (double *)(base + off);
+    grad = w1 + a.na1;
   }
 };
 
-__device__ bool adj_prologue(const RhsArgs &a, AdjSmem &S, uint64_t *bar) {
-  bool ok = stage_to_smem<double>(S.tab, a.tab, a.tab_count, bar, a.status);
+__device__ __forceinline__ void adj_prologue(const AdjArgs &A, AdjSmem &S) {
+  const RhsArgs &a = A.a;
+  const double k = scale_k(a), k2 = k * k;
+  stage_fx(a, S.fx);
+  for (int i = threadIdx.x; i < a.tab_count; i += blockDim.x) S.tab[i] = tab64_entry(a, i, k2);
   for (int i = threadIdx.x; i < a.na1; i += blockDim.x) {
     double c = a.a1_x[i];
     S.c1[i] = c;
     S.s1[i] = sqrt(fmax(0.0, 1.0 - c * c));
     S.w1[i] = a.a1_w[i];
   }
-  for (int i = threadIdx.x; i < a.na2; i += blockDim.x) {
-    S.c2[i] = a.a2_x[i];
-    S.w2[i] = a.a2_w[i];
-  }
-  const int nw = blockDim.x >> 5;
-  for (int i = threadIdx.x; i < nw * a.tab_count; i += blockDim.x) S.grad[i] = 0.0;
+  for (int i = threadIdx.x; i < a.na2; i += blockDim.x) S.cw2[i] = make_double2(a.a2_x[i], a.a2_w[i]);
+  const int all = (int)(blockDim.x >> 5) * adj_warp_doubles(A);
+  for (int i = threadIdx.x; i < all; i += blockDim.x) S.grad[i] = 0.0;
   __syncthreads();
-  return ok;
 }
 
-__device__ void adj_epilogue(const AdjArgs &A, AdjSmem &S) {
-  if (A.jrows) return;
-  __syncthreads();
+// Block-wide: the sum of all warps' copies per table value (fixed order:
+// warps, then copies starting at the value's own index, which spreads the
+// threads over banks) into dst; the copies are cleared.  Z values carry k^2.
+__device__ __forceinline__ void adj_collect(const AdjArgs &A, AdjSmem &S, double k2, double *dst) {
   const RhsArgs &a = A.a;
-  const int nw = blockDim.x >> 5;
+  __syncthreads();
+  const int nw = blockDim.x >> 5, per = adj_warp_doubles(A), C = 1 << A.lc;
   for (int i = threadIdx.x; i < a.tab_count; i += blockDim.x) {
+    const bool wide = i < A.n_wide;
+    const int n = wide ? C : kLam4Copies;
+    double *g = S.grad + (wide ? i << A.lc : (A.n_wide << A.lc) + (i - A.n_wide) * kLam4Copies);
     double s = 0.0;
-    for (int w = 0; w < nw; ++w) s += S.grad[(size_t)w * a.tab_count + i];
-    A.gpart[(size_t)blockIdx.x * a.tab_count + i] = s;
+    for (int w = 0; w < nw; ++w)
+      for (int c = 0; c < n; ++c) {
+        double &v = g[(size_t)w * per + ((c + i) & (n - 1))];
+        s += v;
+        v = 0.0;
+      }
+    dst[i] = i < a.n_pts ? k2 * s : s;
+  }
+  __syncthreads();
+}
+
+// A lookup's node, kept inside the row (the last node as weight 1 of the cell
+// before it), and its value
+struct AdjPos {
+  int i;
+  double w1;
+};
+__device__ __forceinline__ AdjPos adj_pos(const RhsArgs &a, const KConst<double> &kc, double y, FxOff o) {
+  AdjPos p;
+  node_of(a, kc, y, o, p.i, p.w1);
+  if (p.i == a.n_pts - 1) {
+    p.i -= 1;
+    p.w1 = 2.0;
+  }
+  return p;
+}
+__device__ __forceinline__ double adj_val(const double2 *row, AdjPos p) { return line64(row[p.i], p.w1); }
+
+// add c (1 - w) and c w to entries j + p.i and + 1, in turns of 2^lc lanes
+__device__ __forceinline__ void adj_scatter(double *g, int lc, int j, AdjPos p, double c, bool valid, int lane) {
+  const double v1 = fma(c, p.w1, -c), v0 = c - v1;
+  double *e = g + (((j + p.i) << lc) + (lane & ((1 << lc) - 1)));
+  const int turn = lane >> lc;
+  for (int t = 0; t < (32 >> lc); ++t) {
+    if (t == turn && valid) {
+      e[0] += v0;
+      e[1 << lc] += v1;
+    }
+    __syncwarp();
   }
 }
 
-// Z coefficient of the propagator denominator: Z P + m^2, P = s^2 + k^2 r(s^2/k^2)
-__device__ __forceinline__ double zcoef(int reg, double s2, double k2, double inv_k2) {
-  return s2 + k2 * reg_r(reg, s2 * inv_k2);
+// regulator form h at y = x
+__device__ __forceinline__ double adj_h(const RhsArgs &a, const KConst<double> &kc, double x) {
+  return a.reg == FFRG_REG_LITIM ? (x < 1.0 ? 1.0 : x) : fx_h(*kc.us, x);
 }
 
 // ---------------------------------------------------------------------------
-// d = 3:  term = F_r w_j G(s)
+// d = 3:  term = F_r w_j G(s); row = (radial node, block of jb angle nodes)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kAdjThreads) d3_adjoint(AdjArgs A) {
+__device__ __forceinline__ void d3_adjoint_rows(const AdjArgs &A, const AdjSmem &S, const KConst<double> &kc, double *g,
+                                                int e, int row, bool valid, int lane) {
   const RhsArgs &a = A.a;
-  extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ uint64_t bar;
-  AdjSmem S(smem, a);
-  if (!adj_prologue(a, S, &bar)) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double *g = S.grad + (size_t)warp * a.tab_count;
-  const double k = scale_k(a), k2 = k * k, inv_k2 = 1.0 / k2, m2 = mass2(a, k);
   const int nblk = (a.na1 + a.jb - 1) / a.jb;
-  for (int item = blockIdx.x; item < a.n_items; item += gridDim.x) {
-    const int e = item / a.n_chunks, c = item - e * a.n_chunks;
-    const double p = (e < a.n_ext_p) ? ext_momentum(a, e) : 0.0;
-    const double gn = (A.jrows ? 1.0 : A.gbar[e]) * a.norm;
-    jac_item_begin(A, S.grad);
-    const int o0 = c * a.cr, o1 = min(o0 + a.cr, a.nr);
-    const int rows = (o1 - o0) * nblk;
-    for (int base = warp * 32; base < rows; base += blockDim.x) {
-      const int row = base + lane;
-      const bool valid = row < rows;
-      const int o = valid ? o0 + row / nblk : o0;
-      const int jb0 = valid ? (row % nblk) * a.jb : 0, jb1 = valid ? min(jb0 + a.jb, a.na1) : 0;
-      const double q = a.radq[o], F = a.radF[o], dF = a.radD[o];
-      double vrow = 0.0;
-      for (int jj = 0; jj < a.jb; ++jj) {
-        const int j = jb0 + jj;
-        double c0 = 0.0, c1 = 0.0;
-        int i0 = 0;
-        if (j < jb1) {
-          const double s2 = fmax(q * q + p * p + 2.0 * q * p * S.c1[j], 0.0);
-          const LerpPos ps = pos_of(a, s2);
-          const double Z = val_at(S.tab, ps), P = zcoef(a.reg, s2, k2, inv_k2);
-          const double G = 1.0 / (Z * P + m2);
-          vrow += S.w1[j] * G;
-          const double cz = gn * F * S.w1[j] * (-G * G * P);
-          i0 = ps.i0;
-          c0 = (1.0 - ps.w) * cz;
-          c1 = ps.w * cz;
-        }
-        warp_scatter2(g, i0, c0, c1, lane);
-      }
-      double q0 = 0.0, q1 = 0.0;
-      int iq = 0;
-      if (valid) {
-        const LerpPos pq = pos_of(a, q * q);
-        const double cq = gn * dF * vrow;
-        iq = pq.i0;
-        q0 = (1.0 - pq.w) * cq;
-        q1 = pq.w * cq;
-      }
-      warp_scatter2(g, iq, q0, q1, lane);
-    }
-    jac_item_end(A, S.grad, item);
+  const double p = (e < a.n_ext_p) ? a.ext_pd[e] : 0.0;
+  const double gn = (A.jrows ? 1.0 : A.gbar[e]) * a.norm;
+  if (!valid) row = 0;
+  const int o = row / nblk, j0 = (row - o * nblk) * a.jb;
+  const double q = a.radq[o], gF = gn * a.radF[o], dF = a.radD[o];
+  const double by = fma(q, q, p * p) * kc.sy, ty = 2.0 * q * p * kc.sy;
+  double vrow = 0.0;
+  for (int jj = 0; jj < a.jb; ++jj) {
+    const bool on = valid && j0 + jj < a.na1;
+    const int j = on ? j0 + jj : 0;
+    const double y = fma(ty, S.c1[j], by);
+    const AdjPos ps = adj_pos(a, kc, y, kc.uy1);
+    const double h = adj_h(a, kc, y), G = fx_rcp(fma(adj_val(S.tab, ps), h, kc.m2));
+    const double wG = on ? S.w1[j] * G : 0.0;
+    vrow += wG;
+    adj_scatter(g, A.lc, 0, ps, -gF * wG * (G * h), on, lane);
   }
-  adj_epilogue(A, S);
+  adj_scatter(g, A.lc, 0, adj_pos(a, kc, q * q * kc.sy, kc.uy1), gn * dF * vrow * kc.inv_k2, valid, lane);
 }
 
 // ---------------------------------------------------------------------------
-// d = 4 vertex expansion (tables Z | lambda3 | lambda4 at offsets 0 | n | 2n)
+// d = 4 vertex expansion (tables Z | lambda3 | lambda4 at offsets 0 | n | 2n);
+// row = (radial node, first-angle node)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kAdjThreads) d4_adjoint(AdjArgs A) {
+__device__ __forceinline__ void d4_adjoint_rows(const AdjArgs &A, const AdjSmem &S, const KConst<double> &kc, double *g,
+                                                int e, int row, bool valid, int lane) {
+  const RhsArgs &a = A.a;
+  const int np = a.n_pts, np_ = a.n_ext_p, npsi = a.n_ext_ang, lc = A.lc;
+  const double2 *Zt = S.tab, *L3 = S.tab + np, *L4 = S.tab + 2 * np;
+  double *g4 = g + (A.n_wide << lc);
+  int block, ip, jp = 0;
+  if (e <= np_) {
+    block = 0;
+    ip = e;
+  } else if (e < np_ + 1 + np_ * npsi) {
+    block = 1;
+    ip = (e - np_ - 1) / npsi;
+    jp = (e - np_ - 1) - ip * npsi;
+  } else {
+    block = 2;
+    ip = e - np_ - 1 - np_ * npsi;
+  }
+  const double p = (block == 0 && ip == np_) ? 0.0 : a.ext_pd[ip], p2 = p * p, sy = kc.sy, sw2 = kc.sw2;
+  const double coef = block == 1 ? 3.0 : (block == 2 ? 1.5 : 1.0);
+  const double gn = (A.jrows ? 1.0 : A.gbar[e]) * a.norm * coef;
+  if (!valid) row = 0;
+  const int r = row / a.na1, ia = row - r * a.na1;
+  const double q = a.radq[r], dF = a.radD[r], q2 = q * q, qp = q * p, c1 = S.c1[ia], w1 = S.w1[ia];
+  const double A2 = fma(2.0 * qp, c1, q2 + p2), Ay = A2 * sy;
+  const AdjPos pA = adj_pos(a, kc, Ay, kc.uy1);
+  const double hA = adj_h(a, kc, Ay), GA = fx_rcp(fma(adj_val(Zt, pA), hA, kc.m2));
+  const double GPA = -GA * (GA * hA);        // d GA / d Z(A) / k^2
+  const double gF = gn * a.radF[r] * w1;     // d(out)/d(row value) x gbar
+  double v;                                  // row value (without F w1)
+  if (block == 0) {
+    const AdjPos p4 = adj_pos(a, kc, (q2 + p2) * sy, kc.uy2), p3 = adj_pos(a, kc, (q2 + A2 + p2) * sy, kc.uy3);
+    const double l4 = adj_val(L4, p4), l3 = adj_val(L3, p3), gs = gF * sw2;
+    v = sw2 * fma(l3 * l3, GA, -0.5 * l4);
+    adj_scatter(g4, 0, 0, p4, -0.5 * gs, valid, lane);
+    adj_scatter(g, lc, np, p3, gs * 2.0 * l3 * GA, valid, lane);
+    adj_scatter(g, lc, 0, pA, gs * l3 * l3 * GPA, valid, lane);
+  } else if (block == 2) {
+    const AdjPos p4 = adj_pos(a, kc, (q2 + A2 + 2.0 * p2) * sy, kc.uy4);
+    const double l4 = adj_val(L4, p4), gs = gF * sw2;
+    v = sw2 * GA * l4 * l4;
+    adj_scatter(g4, 0, 0, p4, gs * 2.0 * GA * l4, valid, lane);
+    adj_scatter(g, lc, 0, pA, gs * l4 * l4 * GPA, valid, lane);
+  } else {
+    const double cpsi = a.psi_x[jp], spsi = a.psi_s[jp], C2 = 2.0 * p2 * (1.0 + cpsi);
+    const AdjPos pa = adj_pos(a, kc, (q2 + A2 + p2) * sy, kc.uy3);
+    const double la = adj_val(L3, pa);
+    const double base = q2 + p2, t1 = 2.0 * qp * cpsi * c1, t2 = 2.0 * qp * spsi * S.s1[ia];
+    const double by = base * sy, b0 = (base - t1) * sy, t2y = t2 * sy, sab = (A2 + C2) * sy;
+    const double gFA = gF * GA * la;         // common factor of the inner terms
+    double rs = 0.0;
+    for (int b = 0; b < a.na2; ++b) {
+      const double2 cw = S.cw2[b];
+      const double By = fma(-t2y, cw.x, b0);
+      const AdjPos pB = adj_pos(a, kc, By, kc.uy1), pb = adj_pos(a, kc, by + By, kc.uy3),
+                   pc = adj_pos(a, kc, sab + By, kc.uy3);
+      const double h = adj_h(a, kc, By), GB = fx_rcp(fma(adj_val(Zt, pB), h, kc.m2));
+      const double lb = adj_val(L3, pb), lc_ = adj_val(L3, pc);
+      const double wG = cw.y * GB, t = gFA * wG, cb = t * lc_;
+      rs = fma(wG * lb, lc_, rs);
+      adj_scatter(g, lc, np, pb, cb, valid, lane);
+      adj_scatter(g, lc, np, pc, t * lb, valid, lane);
+      adj_scatter(g, lc, 0, pB, -(cb * lb) * (GB * h), valid, lane);
+    }
+    v = GA * la * rs;
+    adj_scatter(g, lc, 0, pA, gF * GPA * la * rs, valid, lane);
+    adj_scatter(g, lc, np, pa, gF * GA * rs, valid, lane);
+  }
+  // Z(q) through F = w q^3 dR(q) G(q)^2
+  adj_scatter(g, lc, 0, adj_pos(a, kc, q2 * sy, kc.uy1), gn * dF * w1 * v * kc.inv_k2, valid, lane);
+}
+
+// VJP: warps take units of 32 rows of an external point (d=4: three-point
+// block first) in a fixed stride.  Jacobian: CTAs take items (external point x
+// chunk), the warps of a CTA its units, and each item's gradient is collected
+// into its row.
+template <int MODEL>
+__global__ void __launch_bounds__(32 * kAdjMaxWarps) adjoint_kernel(AdjArgs A) {
   const RhsArgs &a = A.a;
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ uint64_t bar;
   AdjSmem S(smem, a);
-  if (!adj_prologue(a, S, &bar)) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double *g = S.grad + (size_t)warp * a.tab_count;
-  const double k = scale_k(a), k2 = k * k, inv_k2 = 1.0 / k2, m2 = mass2(a, k);
-  const int np = a.n_pts, np_ = a.n_ext_p, npsi = a.n_ext_ang;
-  const double *Zt = S.tab, *L3 = S.tab + np, *L4 = S.tab + 2 * np;
-  const int oZ = 0, o3 = np, o4 = 2 * np;
-  const double third = 1.0 / 3.0, sw2 = a.sum_w2;
-  for (int item = blockIdx.x; item < a.n_items; item += gridDim.x) {
-    const int e = item / a.n_chunks, c = item - e * a.n_chunks;
-    int block, ip, jp = 0;
-    if (e <= np_) {
-      block = 0;
-      ip = e;
-    } else if (e < np_ + 1 + np_ * npsi) {
-      block = 1;
-      ip = (e - np_ - 1) / npsi;
-      jp = (e - np_ - 1) - ip * npsi;
-    } else {
-      block = 2;
-      ip = e - np_ - 1 - np_ * npsi;
-    }
-    const double p = (block == 0 && ip == np_) ? 0.0 : ext_momentum(a, ip);
-    const double cpsi = block == 1 ? a.psi_x[jp] : 1.0, spsi = sqrt(fmax(0.0, 1.0 - cpsi * cpsi));
-    const double p2 = p * p, C2 = 2.0 * p2 * (1.0 + cpsi);
-    const double coef = block == 1 ? 3.0 : (block == 2 ? 1.5 : 1.0);
-    const double gn = (A.jrows ? 1.0 : A.gbar[e]) * a.norm * coef;
-    jac_item_begin(A, S.grad);
-    const int o0 = c * a.cr, o1 = min(o0 + a.cr, a.nr);
-    const int rows = (o1 - o0) * a.na1;
-    for (int base = warp * 32; base < rows; base += blockDim.x) {
-      const int row = base + lane;
-      const bool valid = row < rows;
-      const int r = valid ? o0 + row / a.na1 : o0, ia = valid ? row % a.na1 : 0;
-      const double q = a.radq[r], F = a.radF[r], dF = a.radD[r];
-      const double q2 = q * q, qp = q * p, c1 = S.c1[ia], w1 = S.w1[ia];
-      const double A2 = fmax(q2 + p2 + 2.0 * qp * c1, 0.0);
-      const LerpPos pA = pos_of(a, A2);
-      const double ZA = val_at(Zt, pA), PA = zcoef(a.reg, A2, k2, inv_k2);
-      const double GA = 1.0 / (ZA * PA + m2);
-      const double gF = valid ? gn * F * w1 : 0.0;  // d(out)/d(row value) x gbar
-      double v = 0.0;                               // row value (without F w1)
-      if (block == 0) {
-        const LerpPos p4 = pos_of(a, (q2 + p2) * 0.5), p3 = pos_of(a, (q2 + A2 + p2) * third);
-        const double l4 = val_at(L4, p4), l3 = val_at(L3, p3);
-        v = sw2 * (-0.5 * l4 + l3 * l3 * GA);
-        double c4 = gF * sw2 * (-0.5), c3 = gF * sw2 * 2.0 * l3 * GA, cA = gF * sw2 * l3 * l3 * (-GA * GA * PA);
-        warp_scatter2(g, o4 + p4.i0, (1.0 - p4.w) * c4, p4.w * c4, lane);
-        warp_scatter2(g, o3 + p3.i0, (1.0 - p3.w) * c3, p3.w * c3, lane);
-        warp_scatter2(g, oZ + pA.i0, (1.0 - pA.w) * cA, pA.w * cA, lane);
-      } else if (block == 2) {
-        const LerpPos p4 = pos_of(a, (q2 + A2 + 2.0 * p2) * 0.25);
-        const double l4 = val_at(L4, p4);
-        v = sw2 * GA * l4 * l4;
-        double c4 = gF * sw2 * 2.0 * GA * l4, cA = gF * sw2 * l4 * l4 * (-GA * GA * PA);
-        warp_scatter2(g, o4 + p4.i0, (1.0 - p4.w) * c4, p4.w * c4, lane);
-        warp_scatter2(g, oZ + pA.i0, (1.0 - pA.w) * cA, pA.w * cA, lane);
-      } else {
-        const LerpPos pa = pos_of(a, (q2 + A2 + p2) * third);
-        const double la = val_at(L3, pa);
-        const double basev = q2 + p2, t1 = 2.0 * qp * cpsi * c1, t2 = 2.0 * qp * spsi * S.s1[ia];
-        const double sab = A2 + C2;
-        const double gFA = gF * GA * la;  // common factor of the inner terms
-        double rs = 0.0;
-        for (int b = 0; b < a.na2; ++b) {
-          const double B2 = fmax(basev - t1 - t2 * S.c2[b], 0.0);
-          const LerpPos pB = pos_of(a, B2), pb = pos_of(a, (basev + B2) * third), pc = pos_of(a, (sab + B2) * third);
-          const double ZB = val_at(Zt, pB), PB = zcoef(a.reg, B2, k2, inv_k2);
-          const double GB = 1.0 / (ZB * PB + m2);
-          const double lb = val_at(L3, pb), lc = val_at(L3, pc);
-          const double w2 = S.w2[b];
-          rs += w2 * GB * lb * lc;
-          const double cB = gFA * w2 * (-GB * GB * PB) * lb * lc;
-          const double cb = gFA * w2 * GB * lc, cc = gFA * w2 * GB * lb;
-          warp_scatter2(g, oZ + pB.i0, (1.0 - pB.w) * cB, pB.w * cB, lane);
-          warp_scatter2(g, o3 + pb.i0, (1.0 - pb.w) * cb, pb.w * cb, lane);
-          warp_scatter2(g, o3 + pc.i0, (1.0 - pc.w) * cc, pc.w * cc, lane);
-        }
-        v = GA * la * rs;
-        const double cA = gF * (-GA * GA * PA) * la * rs, ca = gF * GA * rs;
-        warp_scatter2(g, oZ + pA.i0, (1.0 - pA.w) * cA, pA.w * cA, lane);
-        warp_scatter2(g, o3 + pa.i0, (1.0 - pa.w) * ca, pa.w * ca, lane);
-      }
-      // Z(q) through F = w q^3 dR(q) G(q)^2
-      const LerpPos pq = pos_of(a, q2);
-      const double cq = valid ? gn * dF * w1 * v : 0.0;
-      warp_scatter2(g, oZ + pq.i0, (1.0 - pq.w) * cq, pq.w * cq, lane);
-    }
-    jac_item_end(A, S.grad, item);
+  adj_prologue(A, S);
+  KConst<double> kc = load_kconst<double>(a);
+  kc.us = S.fx;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  double *g = S.grad + (size_t)warp * adj_warp_doubles(A);
+  const int rows = MODEL == FFRG_MODEL_D3 ? a.nr * ((a.na1 + a.jb - 1) / a.jb) : a.nr * a.na1;
+  auto unit = [&](int e, int row, int end) {
+    if constexpr (MODEL == FFRG_MODEL_D3) d3_adjoint_rows(A, S, kc, g, e, row, row < end, lane);
+    else d4_adjoint_rows(A, S, kc, g, e, row, row < end, lane);
+  };
+  if (!A.jrows) {
+    const int per = (rows + 31) / 32, rot = MODEL == FFRG_MODEL_D3 ? 0 : a.n_ext_p + 1;
+    for (int u = warp * gridDim.x + blockIdx.x; u < a.n_ext * per; u += nw * gridDim.x)
+      unit((u / per + rot) % a.n_ext, (u % per) * 32 + lane, rows);
+    adj_collect(A, S, kc.k2, A.gpart + (size_t)blockIdx.x * a.tab_count);
+    return;
   }
-  adj_epilogue(A, S);
+  const int irows = rows / a.nr * a.cr;
+  for (int item = blockIdx.x; item < a.n_items; item += gridDim.x) {
+    const int e = item / a.n_chunks, c = item - e * a.n_chunks, end = min((c + 1) * irows, rows);
+    for (int row = c * irows + warp * 32; row < end; row += nw * 32) unit(e, row + lane, end);
+    adj_collect(A, S, kc.k2, A.jrows + (size_t)item * a.tab_count);
+  }
 }
 
-// fixed-order sum of the CTA partials
+// fixed-order sum of the CTA partials: a warp per table value, lanes strided, then the warp tree
 __global__ void adj_reduce_kernel(const double *gpart, int grid, int count, double *tbar) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (i >= count) return;
   double s = 0.0;
-  for (int b = 0; b < grid; ++b) s += gpart[(size_t)b * count + i];
-  tbar[i] = s;
+  for (int b = lane; b < grid; b += 32) s += gpart[(size_t)b * count + i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (lane == 0) tbar[i] = s;
 }
 
 }  // namespace ffrg
@@ -312,29 +306,62 @@ __global__ void jac_reduce_kernel(const double *jrows, int n_ext, int n_chunks, 
   J[idx] = s;
 }
 
-// Launch geometry, shared memory and scratch of the adjoint kernels of a plan.
-static int adjoint_setup(ffrg_ctx *ctx, Plan *pl, int model, void (**kern_out)(AdjArgs)) {
-  void (*kern)(AdjArgs) = model == FFRG_MODEL_D3 ? d3_adjoint : d4_adjoint;
+// Launch geometry, shared memory and scratch of the adjoint kernels of a plan,
+// and A's share of it.  Copies C and warps: the pair with the least FP64 work
+// per inner term, 17 + 3 (2 + 4 x 16/C) instructions of 16 clocks on one pipe
+// that one warp per SMSP keeps about half busy and two almost full, among
+// those whose gradients fit (96 points: C = 16 with 6 warps).
+static int adjoint_setup(ffrg_ctx *ctx, Plan *pl, AdjArgs &A, void (**kern_out)(AdjArgs)) {
+  void (*kern)(AdjArgs) =
+      pl->model == FFRG_MODEL_D3 ? adjoint_kernel<FFRG_MODEL_D3> : adjoint_kernel<FFRG_MODEL_D4_VERTEX>;
   *kern_out = kern;
-  if (pl->adj_grid) return FFRG_OK;
-  const int nw = kAdjThreads / 32;
-  size_t smem = (((size_t)pl->tab_count * 8 + 15) & ~(size_t)15) +
-                ((((size_t)(3 * pl->na1 + 2 * pl->na2)) * 8 + 15) & ~(size_t)15) + (size_t)nw * pl->tab_count * 8;
-  if (smem > 200 * 1024) {
+  // tables up to what eight warps with one copy each hold in 200 KB
+  const size_t limit = (((size_t)pl->tab_count * 8 + 15) & ~(size_t)15) +
+                       ((((size_t)(3 * pl->na1 + 2 * pl->na2)) * 8 + 15) & ~(size_t)15) +
+                       (size_t)kAdjMaxWarps * pl->tab_count * 8;
+  if (limit > 200 * 1024) {
     ctx->last_error = "adjoint: tables too large for per-warp shared-memory gradients";
     return FFRG_EINVAL;
   }
+  A.a.tab_count = pl->tab_count;
+  A.n_wide = (pl->model == FFRG_MODEL_D3 ? 1 : 2) * pl->n_pts;
+  if (pl->adj_grid) {
+    A.lc = pl->adj_lc;
+    return FFRG_OK;
+  }
+  const size_t fixed = sizeof(FxTables) + (size_t)pl->tab_count * 16 + ((size_t)3 * pl->na1 + 2 * (size_t)pl->na2) * 8;
+  int lc = 0, nw = 0;
+  double best = 0.0;
+  for (int l = 0; l <= 5; ++l) {
+    A.lc = l;
+    const size_t per = (size_t)adj_warp_doubles(A) * 8;
+    const int w = fixed + per > kMaxDynSmemBytes ? 0 : (int)std::min<size_t>(kAdjMaxWarps, (kMaxDynSmemBytes - fixed) / per);
+    const double rate = std::min(1.0, 0.13 * w) / (17.0 + 3.0 * (2.0 + 64.0 / (1 << l)));
+    if (w >= 1 && rate > best) {
+      best = rate;
+      lc = l;
+      nw = w;
+    }
+  }
+  if (nw == 0) {
+    ctx->last_error = "adjoint: tables too large for per-warp shared-memory gradients";
+    return FFRG_EINVAL;
+  }
+  A.lc = lc;
+  const size_t smem = fixed + (size_t)nw * adj_warp_doubles(A) * 8;
   int st = ensure_smem_limit(ctx, (const void *)kern, smem);
   if (st) return st;
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kAdjThreads, smem);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * nw, smem);
   if (e != cudaSuccess || per_sm < 1) return set_cuda_error(ctx, e ? e : cudaErrorInvalidConfiguration, "occupancy");
-  int grid = std::max(1, std::min(pl->n_items, per_sm * ctx->num_sms));
+  const int grid = std::max(1, std::min(pl->n_items, per_sm * ctx->num_sms));
   st = dev_alloc(ctx, (void **)&pl->radD, (size_t)pl->nr * pl->nfreq * sizeof(double));
   if (!st) st = dev_alloc(ctx, (void **)&pl->gpart, (size_t)grid * pl->tab_count * sizeof(double));
   if (st) return st;
   pl->adj_smem = smem;
   pl->adj_grid = grid;
+  pl->adj_lc = lc;
+  pl->adj_threads = 32 * nw;
   return FFRG_OK;
 }
 
@@ -347,15 +374,15 @@ int launch_jacobian(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc
   Plan *pl = nullptr;
   st = get_plan(ctx, pb, td, &pl);
   if (st) return st;
+  AdjArgs A;
+  memset(&A, 0, sizeof(A));
   void (*kern)(AdjArgs) = nullptr;
-  st = adjoint_setup(ctx, pl, pb->model, &kern);
+  st = adjoint_setup(ctx, pl, A, &kern);
   if (st) return st;
   if (!pl->jrows) {
     st = dev_alloc(ctx, (void **)&pl->jrows, (size_t)pl->n_items * pl->tab_count * sizeof(double));
     if (st) return st;
   }
-  AdjArgs A;
-  memset(&A, 0, sizeof(A));
   fill_args(pl, pb, td, tab, k, A.a);
   A.a.status = ctx->status_dev;
   A.a.cr = pl->cr;  // block-sized work items
@@ -366,7 +393,7 @@ int launch_jacobian(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc
   A.jrows = pl->jrows;
   st = launch_precompute(ctx, A.a, s);
   if (st) return st;
-  kern<<<pl->adj_grid, kAdjThreads, pl->adj_smem, s>>>(A);
+  kern<<<pl->adj_grid, pl->adj_threads, pl->adj_smem, s>>>(A);
   const size_t tot = (size_t)pl->n_ext * pl->tab_count;
   jac_reduce_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(pl->jrows, pl->n_ext, pl->n_chunks, pl->tab_count, J);
   return set_cuda_error(ctx, cudaGetLastError(), "jacobian launch");
@@ -394,11 +421,11 @@ extern "C" int ffrg_rhs_adjoint(ffrg_ctx *ctx, const ffrg_problem *pb, const ffr
   st = get_plan(ctx, pb, &tables->desc, &pl);
   if (st) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  void (*kern)(AdjArgs) = nullptr;
-  st = adjoint_setup(ctx, pl, pb->model, &kern);
-  if (st) return st;
   AdjArgs A;
   memset(&A, 0, sizeof(A));
+  void (*kern)(AdjArgs) = nullptr;
+  st = adjoint_setup(ctx, pl, A, &kern);
+  if (st) return st;
   fill_args(pl, pb, &tables->desc, tables->dev, k, A.a);
   A.a.status = ctx->status_dev;
   A.a.cr = pl->cr;  // block-sized work items
@@ -410,7 +437,7 @@ extern "C" int ffrg_rhs_adjoint(ffrg_ctx *ctx, const ffrg_problem *pb, const ffr
   A.gpart = pl->gpart;
   st = launch_precompute(ctx, A.a, s);
   if (st) return st;
-  kern<<<pl->adj_grid, kAdjThreads, pl->adj_smem, s>>>(A);
-  adj_reduce_kernel<<<(pl->tab_count + 255) / 256, 256, 0, s>>>(pl->gpart, pl->adj_grid, pl->tab_count, tbar_dev);
+  kern<<<pl->adj_grid, pl->adj_threads, pl->adj_smem, s>>>(A);
+  adj_reduce_kernel<<<(pl->tab_count + 7) / 8, 256, 0, s>>>(pl->gpart, pl->adj_grid, pl->tab_count, tbar_dev);
   return set_cuda_error(ctx, cudaGetLastError(), "adjoint launch");
 }

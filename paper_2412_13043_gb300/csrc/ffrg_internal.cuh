@@ -554,7 +554,7 @@ struct Plan {
   float2 *tab32;
   double *radD, *gpart;     // adjoint scratch (allocated on first use)
   double *jrows;            // Jacobian rows per work item (allocated on first use)
-  int adj_grid;
+  int adj_grid, adj_lc, adj_threads;   // adjoint kernels: CTAs, log2 of gradient copies per warp, threads
   size_t adj_smem;
   std::vector<double> psi_w_host;
 };

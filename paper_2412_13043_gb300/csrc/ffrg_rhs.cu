@@ -1568,7 +1568,6 @@ int launch_precompute(ffrg_ctx *ctx, const RhsArgs &a_in, cudaStream_t s) {
   RhsArgs a = a_in;   // radial factors only: no kernel-precision tables or constants
   a.fp64 = 1;
   a.tab64 = nullptr;
-  a.kconst = nullptr;
   precompute_kernel<<<precompute_blocks(a, 4 * ctx->num_sms), kThreads, 0, s>>>(a);
   return set_cuda_error(ctx, cudaGetLastError(), "precompute launch");
 }
