@@ -190,21 +190,82 @@ static int upload_rule(ffrg_ctx *ctx, const std::vector<double> &h, double **d) 
   return set_cuda_error(ctx, e, "cudaMemcpy(rule)");
 }
 
+// Scratch of one RHS in flight (the rest of a plan is shared by its stages).
+static int plan_scratch(ffrg_ctx *ctx, Plan *pl, bool want_tab64) {
+  const size_t nF = (size_t)pl->nr * pl->nfreq;
+  int st = dev_alloc(ctx, (void **)&pl->radF, nF * sizeof(double));
+  if (!st) st = dev_alloc(ctx, (void **)&pl->radF32, nF * sizeof(float));
+  if (!st) st = dev_alloc(ctx, (void **)&pl->radq, pl->nr * sizeof(double));
+  if (!st) st = dev_alloc(ctx, (void **)&pl->radq32, pl->nr * sizeof(float));
+  // work_ctr[0]: item counter of the main kernels; [1..4]: grid counters of
+  // the finite-T mixed single-launch RHS (all zero at the start)
+  if (!st) st = dev_alloc(ctx, (void **)&pl->work_ctr, 5 * sizeof(unsigned));
+  if (!st) st = set_cuda_error(ctx, cudaMemset(pl->work_ctr, 0, 5 * sizeof(unsigned)), "cudaMemset(counters)");
+  if (!st) st = dev_alloc(ctx, (void **)&pl->ext_done, (size_t)pl->n_ext * sizeof(unsigned));
+  if (!st) st = dev_alloc(ctx, (void **)&pl->kconst, kKConstBytes);
+  if (!st && want_tab64) st = dev_alloc(ctx, (void **)&pl->tab64, (size_t)pl->tab64_count * sizeof(double2));
+  if (!st && pl->kbuf_count) st = dev_alloc(ctx, (void **)&pl->kbuf, pl->kbuf_count * sizeof(double));
+  if (!st) st = dev_alloc(ctx, (void **)&pl->ext_pd, (size_t)pl->n_ext_p * sizeof(double));
+  if (!st) st = dev_alloc(ctx, (void **)&pl->psi_s, (size_t)std::max(1, pl->n_ext_ang) * sizeof(double));
+  if (!st)
+    st = dev_alloc(ctx, (void **)&pl->partial, (size_t)std::max(pl->fn_items, pl->fn_items64) * sizeof(double));
+  if (!st) st = dev_alloc(ctx, (void **)&pl->tab32,
+                          (size_t)std::max(pl->tab_count, pl->tab32_count) * sizeof(float2));
+  return st;
+}
+static void plan_scratch_free(ffrg_ctx *ctx, Plan *pl) {
+  void *arrs[] = {pl->radF, pl->radF32, pl->radq, pl->radq32, pl->work_ctr, pl->ext_done, pl->kconst,
+                  pl->tab64, pl->kbuf, pl->ext_pd, pl->psi_s, pl->partial, pl->tab32};
+  for (void *p : arrs) dev_free(ctx, p, 0);
+}
+static void plan_scratch_clear(Plan *pl) {
+  pl->radF = pl->radq = pl->kbuf = pl->ext_pd = pl->psi_s = pl->partial = nullptr;
+  pl->radF32 = pl->radq32 = nullptr;
+  pl->work_ctr = pl->ext_done = nullptr;
+  pl->kconst = nullptr;
+  pl->tab64 = nullptr;
+  pl->tab32 = nullptr;
+}
+
+bool stage_plans(ffrg_ctx *ctx, Plan *pl) {
+  if (pl->stage[0]) {
+    for (Plan *sp : pl->stage) {   // what the plan has learnt since
+      sp->fg = pl->fg, sp->fg_ok = pl->fg_ok, sp->fg_lo = pl->fg_lo, sp->fg_hi = pl->fg_hi;
+      sp->grid64 = pl->grid64, sp->grid32 = pl->grid32;
+    }
+    return true;
+  }
+  for (int i = 0; i < kStages - 1; ++i) {
+    Plan *sp = new Plan(*pl);
+    plan_scratch_clear(sp);
+    sp->radD = sp->gpart = sp->jrows = sp->rowbuf = nullptr;
+    sp->item_done = nullptr;
+    for (Plan *&q : sp->stage) q = nullptr;
+    pl->stage[i] = sp;
+    if (plan_scratch(ctx, sp, pl->tab64 != nullptr)) {
+      cudaGetLastError();
+      for (Plan *&q : pl->stage) {
+        if (q) plan_scratch_free(ctx, q);
+        delete q;
+        q = nullptr;
+      }
+      return false;
+    }
+  }
+  return true;
+}
+
 static void plan_free(ffrg_ctx *ctx, Plan *pl) {
   if (!pl) return;
-  double *arrs[] = {pl->rad_x, pl->rad_w, pl->a1_x, pl->a1_w, pl->a2_x, pl->a2_w, pl->psi_x, pl->psi_w,
-                    pl->radF, pl->radq, pl->partial, pl->radD, pl->gpart, pl->ext_pd, pl->psi_s, pl->jrows};
-  for (double *p : arrs) dev_free(ctx, p, 0);
-  dev_free(ctx, pl->tab64, 0);
-  dev_free(ctx, pl->rowbuf, 0);
-  dev_free(ctx, pl->item_done, 0);
-  dev_free(ctx, pl->tab32, 0);
-  dev_free(ctx, pl->radq32, 0);
-  dev_free(ctx, pl->work_ctr, 0);
-  dev_free(ctx, pl->ext_done, 0);
-  dev_free(ctx, pl->kconst, 0);
-  dev_free(ctx, pl->radF32, 0);
-  dev_free(ctx, pl->kbuf, 0);
+  for (Plan *sp : pl->stage)
+    if (sp) {
+      plan_scratch_free(ctx, sp);
+      delete sp;
+    }
+  plan_scratch_free(ctx, pl);
+  void *arrs[] = {pl->rad_x, pl->rad_w, pl->a1_x, pl->a1_w, pl->a2_x, pl->a2_w, pl->psi_x, pl->psi_w,
+                  pl->radD, pl->gpart, pl->jrows, pl->rowbuf, pl->item_done};
+  for (void *p : arrs) dev_free(ctx, p, 0);
   delete pl;
 }
 
@@ -394,36 +455,17 @@ int get_plan(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc *td, P
   pl->psi_w_host = wp;
   st = st ? st : upload_rule(ctx, xp, &pl->psi_x);
   st = st ? st : upload_rule(ctx, wp, &pl->psi_w);
-  size_t nF = (size_t)pl->nr * pl->nfreq;
-  if (!st) st = dev_alloc(ctx, (void **)&pl->radF, nF * sizeof(double));
-  if (!st) st = dev_alloc(ctx, (void **)&pl->radF32, nF * sizeof(float));
-  if (!st) st = dev_alloc(ctx, (void **)&pl->radq, pl->nr * sizeof(double));
-  if (!st) st = dev_alloc(ctx, (void **)&pl->radq32, pl->nr * sizeof(float));
-  // work_ctr[0]: item counter of the main kernels; [1..4]: grid counters of
-  // the finite-T mixed single-launch RHS (all zero at the start)
-  if (!st) st = dev_alloc(ctx, (void **)&pl->work_ctr, 5 * sizeof(unsigned));
-  if (!st) st = set_cuda_error(ctx, cudaMemset(pl->work_ctr, 0, 5 * sizeof(unsigned)), "cudaMemset(counters)");
-  if (!st) st = dev_alloc(ctx, (void **)&pl->ext_done, (size_t)pl->n_ext * sizeof(unsigned));
-  if (!st) st = dev_alloc(ctx, (void **)&pl->kconst, kKConstBytes);
-  // FP64 line-form tables in global memory: finite T (long to build in every
-  // CTA), and tables that do not fit in shared memory.  The former can do
-  // without: optional buffers are left out in a context with a memory budget,
-  // so that it holds what it would hold without them.
-  const bool too_big = pl->smem64 > kMaxDynSmemBytes && pb->model != FFRG_MODEL_FINITE_T_4D;
-  if (!st && ((pb->model == FFRG_MODEL_FINITE_T && !ctx->budget) || too_big))
-    st = dev_alloc(ctx, (void **)&pl->tab64, (size_t)pl->tab64_count * sizeof(double2));
-  if (!st && pl->kbuf_count) st = dev_alloc(ctx, (void **)&pl->kbuf, pl->kbuf_count * sizeof(double));
-  if (!st) st = dev_alloc(ctx, (void **)&pl->ext_pd, (size_t)pl->n_ext_p * sizeof(double));
-  if (!st) st = dev_alloc(ctx, (void **)&pl->psi_s, (size_t)npsi * sizeof(double));
   if (is_d4(pb->model) && ctx->budget) {   // the larger items of the mixed kernels, fewer partial sums
     pl->fcr64 = pl->fcr;
     pl->fn_chunks64 = pl->fn_chunks;
     pl->fn_items64 = pl->fn_items;
   }
-  if (!st)
-    st = dev_alloc(ctx, (void **)&pl->partial, (size_t)std::max(pl->fn_items, pl->fn_items64) * sizeof(double));
-  if (!st) st = dev_alloc(ctx, (void **)&pl->tab32,
-                          (size_t)std::max(pl->tab_count, pl->tab32_count) * sizeof(float2));
+  // FP64 line-form tables in global memory: finite T (long to build in every
+  // CTA), and tables that do not fit in shared memory.  The former can do
+  // without: optional buffers are left out in a context with a memory budget,
+  // so that it holds what it would hold without them.
+  const bool too_big = pl->smem64 > kMaxDynSmemBytes && pb->model != FFRG_MODEL_FINITE_T_4D;
+  if (!st) st = plan_scratch(ctx, pl, (pb->model == FFRG_MODEL_FINITE_T && !ctx->budget) || too_big);
   if (st) {
     plan_free(ctx, pl);
     return st;
@@ -565,20 +607,7 @@ int ffrg_destroy(ffrg_ctx *ctx) {
   cudaDeviceSynchronize();
   for (auto &kv : ctx->plans) {
     Plan *pl = kv.second;
-    double *arrs[] = {pl->rad_x, pl->rad_w, pl->a1_x, pl->a1_w, pl->a2_x, pl->a2_w, pl->psi_x, pl->psi_w,
-                      pl->radF, pl->radq, pl->partial, pl->radD, pl->gpart, pl->ext_pd, pl->psi_s, pl->jrows};
-    for (double *p : arrs) cudaFree(p);
-    cudaFree(pl->tab32);
-    cudaFree(pl->radq32);
-    cudaFree(pl->work_ctr);
-    cudaFree(pl->ext_done);
-    cudaFree(pl->kconst);
-    cudaFree(pl->radF32);
-    cudaFree(pl->tab64);
-    cudaFree(pl->rowbuf);
-    cudaFree(pl->item_done);
-    cudaFree(pl->kbuf);
-    delete pl;
+    plan_free(ctx, pl);
   }
   ctx->plans.clear();
   for (void *p : ctx->owned) cudaFree(p);
@@ -589,6 +618,10 @@ int ffrg_destroy(ffrg_ctx *ctx) {
   if (ctx->flow_host) cudaFreeHost(ctx->flow_host);
   if (ctx->flow_ev) cudaEventDestroy(ctx->flow_ev);
   if (ctx->flow_stream) cudaStreamDestroy(ctx->flow_stream);
+  for (cudaStream_t q : ctx->stage_stream)
+    if (q) cudaStreamDestroy(q);
+  for (cudaEvent_t q : ctx->stage_ev)
+    if (q) cudaEventDestroy(q);
   if (ctx->status_dev) cudaFree(ctx->status_dev);
   if (ctx->status_host) cudaFreeHost(ctx->status_host);
   delete ctx;

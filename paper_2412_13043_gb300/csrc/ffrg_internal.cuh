@@ -506,6 +506,10 @@ struct ffrg_ctx {
   size_t host_out_cap = 0;
   void *flow_host = nullptr;
   cudaStream_t flow_stream = nullptr;
+  // frozen flows: streams (beside flow_stream) of the stages of a step, their
+  // fork event and join events
+  cudaStream_t stage_stream[4] = {};
+  cudaEvent_t stage_ev[5] = {};
   cudaEvent_t flow_ev = nullptr;
   // ffrg_ft_states scratch (operand slices, exact pass sums, scales), grown on demand
   void *states_dev = nullptr;
@@ -539,6 +543,7 @@ struct Plan {
   size_t kbuf_count;              // FINITE_T: entries of K (N + n_ext_ang) x n_ext_p x n_rad
   double *kbuf;
   int grid64, grid32;       // persistent grids (FP64 / mixed kernels)
+  Plan *stage[4];           // frozen flows: the same plan with scratch of its own for further stages (or null)
   int grid_ref;             // feedback flows, FP64
   double *rowbuf;
   unsigned *item_done;
@@ -597,8 +602,10 @@ int batched_ctas_per_sm(ffrg_ctx *ctx, int model, size_t smem);
 int launch_rhs_batched(ffrg_ctx *ctx, const BatchList &bl, cudaStream_t s);
 
 // Device control block and argument block of one DP5(4) flow.
+constexpr int kStages = 5;   // distinct stage times of a DP5(4) step after its first (c_5 = c_6 = 1)
 struct FlowCtl {
   double t, dt, h, t0, t1, dt_min, dt_max, atol, rtol, end_tol, Lambda;
+  double k_stages[kStages];   // frozen flows: the scales of the next step's stages
   double k_stage, m2_stage, err;
   long long steps, rejects, max_steps;
   int last_rejected, done, status, accepted;
@@ -641,6 +648,9 @@ cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t s
 }
 
 // helpers implemented in ffrg_api.cu
+// kStages - 1 copies of a plan that share its rules but not its scratch; false
+// when there is no memory for them
+bool stage_plans(ffrg_ctx *ctx, Plan *pl);
 int set_cuda_error(ffrg_ctx *ctx, cudaError_t e, const char *what);
 int dev_alloc(ffrg_ctx *ctx, void **p, size_t bytes);
 void dev_free(ffrg_ctx *ctx, void *p, size_t bytes);
