@@ -59,48 +59,84 @@ void dev_free(ffrg_ctx *ctx, void *p, size_t bytes) {
   ctx->used = ctx->used >= bytes ? ctx->used - bytes : 0;
 }
 
-// Gauss-Legendre on [a,b].  Roots of P_n by Newton iteration in long double
-// starting from the asymptotic guess cos(pi (i - 1/4)/(n + 1/2)); P_n and P_n'
-// from the three-term recurrence (k+1) P_{k+1} = (2k+1) x P_k - k P_{k-1}.
+namespace {
+// Double-double numbers (hi + lo, |lo| <= ulp(hi)/2): Dekker's two-sum and
+// FMA products, about 104 bits.
+struct Dd {
+  double hi, lo;
+};
+inline Dd dd_fast(double a, double b) {
+  const double s = a + b;
+  return {s, b - (s - a)};
+}
+inline Dd dd_add(Dd a, Dd b) {
+  const double s = a.hi + b.hi, t = s - a.hi;
+  return dd_fast(s, ((a.hi - (s - t)) + (b.hi - t)) + (a.lo + b.lo));
+}
+inline Dd dd_mul(Dd a, Dd b) {
+  const double p = a.hi * b.hi;
+  return dd_fast(p, fma(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi));
+}
+inline Dd dd_div(Dd a, Dd b) {
+  const double q = a.hi / b.hi;
+  const Dd r = dd_add(a, dd_mul({-q, 0.0}, b));
+  const double q2 = r.hi / b.hi;
+  const Dd r2 = dd_add(r, dd_mul({-q2, 0.0}, b));
+  return dd_add(dd_fast(q, q2), {r2.hi / b.hi, 0.0});
+}
+}  // namespace
+
+// Gauss-Legendre on [a,b].  Roots of P_n by Newton iteration from the
+// asymptotic guess cos(pi (i - 1/4)/(n + 1/2)), P_n and P_n' from the
+// three-term recurrence P_{k+1} = z P_k + k/(k+1) (z P_k - P_{k-1}): in double
+// to convergence, then one step in double-double, whose dz ~ 1e-16 also carries
+// P_n' to the root by the Legendre equation (n > 1024: a second step, so that
+// the neglected n^6 dz^3 stays below 1e-18).  One extended pass per root
+// instead of five or six in long double, which is software quad precision on
+// Arm hosts: 128 nodes there 3.9 ms, 0.26 ms so.
 int host_gauss_legendre(int n, double a, double b, double *x, double *w) {
   if (n < 1 || n > kMaxNodes || !x || !w) return FFRG_EINVAL;
-  const long double pi = 3.141592653589793238462643383279502884L;
-  int half = (n + 1) / 2;
-  for (int i = 1; i <= half; ++i) {
-    long double z = cosl(pi * ((long double)i - 0.25L) / ((long double)n + 0.5L));
-    long double dp = 1.0L;
-    for (int it = 0; it < 60; ++it) {
-      long double pkm1 = 1.0L, pk = z;
-      for (int kk = 1; kk < n; ++kk) {
-        long double pkp1 = ((2.0L * kk + 1.0L) * z * pk - (long double)kk * pkm1) / (long double)(kk + 1);
-        pkm1 = pk;
-        pk = pkp1;
+  std::vector<Dd> ck(n);   // k/(k+1)
+  for (int k = 1; k < n; ++k) ck[k] = dd_div({(double)k, 0.0}, {(double)(k + 1), 0.0});
+  const long double mid = 0.5L * ((long double)a + (long double)b), hw = 0.5L * ((long double)b - (long double)a);
+  const double nn = (double)n * (n + 1.0);
+  for (int i = 1; i <= (n + 1) / 2; ++i) {
+    double z = cos(3.141592653589793238462643 * (i - 0.25) / (n + 0.5));
+    for (int it = 0; it < 20; ++it) {
+      double pm = 1.0, p = z;
+      for (int k = 1; k < n; ++k) {
+        const double t = z * p, pp = t + ck[k].hi * (t - pm);
+        pm = p;
+        p = pp;
       }
-      if (n == 1) { pk = z; pkm1 = 1.0L; }
-      dp = (long double)n * (pkm1 - z * pk) / (1.0L - z * z);
-      long double dz = pk / dp;
+      const double dz = p * (1.0 - z * z) / (n * (pm - z * p));
       z -= dz;
-      if (fabsl(dz) < 1e-19L) {
-        // derivative at the final iterate
-        pkm1 = 1.0L;
-        pk = z;
-        for (int kk = 1; kk < n; ++kk) {
-          long double pkp1 = ((2.0L * kk + 1.0L) * z * pk - (long double)kk * pkm1) / (long double)(kk + 1);
-          pkm1 = pk;
-          pk = pkp1;
-        }
-        if (n == 1) { pk = z; pkm1 = 1.0L; }
-        dp = (long double)n * (pkm1 - z * pk) / (1.0L - z * z);
-        break;
-      }
+      if (fabs(dz) < 1e-14) break;   // quadratic: the next step is below rounding
     }
-    long double wi = 2.0L / ((1.0L - z * z) * dp * dp);
-    long double mid = 0.5L * ((long double)a + (long double)b), hw = 0.5L * ((long double)b - (long double)a);
+    Dd zr = {z, 0.0}, q = {0.0, 0.0}, dp = {1.0, 0.0};
+    for (int pass = 0; pass < (n > 1024 ? 2 : 1); ++pass) {
+      z = zr.hi;
+      Dd pm = {1.0, 0.0}, p = {z, 0.0};
+      for (int k = 1; k < n; ++k) {
+        const Dd t = dd_mul({z, 0.0}, p), pp = dd_add(t, dd_mul(ck[k], dd_add(t, {-pm.hi, -pm.lo})));
+        pm = p;
+        p = pp;
+      }
+      const Dd q0 = dd_add({1.0, 0.0}, dd_mul({-z, 0.0}, {z, 0.0}));   // 1 - z^2
+      dp = dd_div(dd_mul({(double)n, 0.0}, dd_add(pm, dd_mul({-z, 0.0}, p))), q0);
+      const double dz = -p.hi / dp.hi;
+      zr = dd_add({z, 0.0}, {dz, 0.0});
+      // P_n'(z + dz): (1 - z^2) P'' = 2 z P' - n (n+1) P and its derivative
+      const double d2 = (2.0 * z * dp.hi - nn * p.hi) / q0.hi, d3 = (4.0 * z * d2 + (2.0 - nn) * dp.hi) / q0.hi;
+      dp = dd_add(dp, {dz * (d2 + 0.5 * dz * d3), 0.0});
+      q = dd_add({1.0, 0.0}, dd_mul({-zr.hi, -zr.lo}, zr));
+    }
+    const Dd wi = dd_div({2.0, 0.0}, dd_mul(q, dd_mul(dp, dp)));
+    const long double zl = (long double)zr.hi + zr.lo, wl = (long double)wi.hi + wi.lo;
     // i-th root counted from +1: goes to index n-i (ascending order)
-    x[n - i] = (double)(mid + hw * z);
-    x[i - 1] = (double)(mid - hw * z);
-    w[n - i] = (double)(hw * wi);
-    w[i - 1] = (double)(hw * wi);
+    x[n - i] = (double)(mid + hw * zl);
+    x[i - 1] = (double)(mid - hw * zl);
+    w[n - i] = w[i - 1] = (double)(hw * wl);
     if (2 * i - 1 == n) x[i - 1] = (double)mid;
   }
   return FFRG_OK;
