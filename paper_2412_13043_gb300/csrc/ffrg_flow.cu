@@ -124,11 +124,11 @@ __device__ __forceinline__ void decide_next_step(FlowCtl *c) {
 }
 
 // Scales of the next step's stages (frozen flows), one thread each.
-__device__ __forceinline__ void write_stage_scales(FlowCtl *c) {
-  const int s = threadIdx.x;
+__device__ __forceinline__ void write_stage_scale(FlowCtl *c, int s) {
   if (s < kStages && !*(volatile const int *)&c->done)
     c->k_stages[s] = c->Lambda * exp(-(*(volatile const double *)&c->t + kDpC[s + 1] * *(volatile const double *)&c->h));
 }
+__device__ __forceinline__ void write_stage_scales(FlowCtl *c) { write_stage_scale(c, threadIdx.x); }
 
 __global__ void flow_start_kernel(FlowCtl *c) {   // one block
   if (threadIdx.x == 0) decide_next_step(c);
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(1024) flow_control_kernel(FlowArgs f) { flow_c
 // End of a frozen step: the derivatives of all stages, the state of the last
 // one, then the control kernel's work and the next scales.  raw: the stages'
 // RHS, kStages x n_ext.
-__global__ void __launch_bounds__(1024) flow_frozen_control_kernel(FlowArgs f, const double *raw) {
+__device__ __forceinline__ void flow_frozen_control_body(const FlowArgs &f, const double *raw) {
   FlowCtl *c = f.ctl;
   if (*(volatile const int *)&c->done) return;
   const double h = c->h;
@@ -229,6 +229,12 @@ __global__ void __launch_bounds__(1024) flow_frozen_control_kernel(FlowArgs f, c
   flow_control_body(f);
   __syncthreads();
   write_stage_scales(c);
+}
+__global__ void __launch_bounds__(1024) flow_frozen_control_kernel(FlowArgs f, const double *raw) {
+  flow_frozen_control_body(f, raw);
+}
+__global__ void __launch_bounds__(1024) batched_flow_frozen_control_kernel(const FlowArgs *fa) {
+  flow_frozen_control_body(fa[blockIdx.x], fa[blockIdx.x].raw);
 }
 
 // ---------------------------------------------------------------------------
@@ -252,7 +258,10 @@ __global__ void __launch_bounds__(1024) batched_flow_control_kernel(const FlowAr
 
 __global__ void batched_flow_start_kernel(const FlowArgs *fa, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n && !fa[i].ctl->done) decide_next_step(fa[i].ctl);
+  if (i < n && !fa[i].ctl->done) {
+    decide_next_step(fa[i].ctl);
+    for (int s = 0; s < kStages; ++s) write_stage_scale(fa[i].ctl, s);
+  }
 }
 
 // First derivative (first-same-as-last stage 0) and the first step size.
@@ -280,6 +289,14 @@ int launch_flow_batched_step(ffrg_ctx *ctx, const FlowArgs *fa, int n, int max_n
     batched_flow_deriv_kernel<<<g, 256, 0, st>>>(fa, s);
   }
   batched_flow_control_kernel<<<n, 1024, 0, st>>>(fa);
+  return set_cuda_error(ctx, cudaGetLastError(), "batched flow step");
+}
+
+int launch_flow_batched_wide_step(ffrg_ctx *ctx, const FlowArgs *fa, int n, const BatchList &bl, cudaStream_t st) {
+  if (n == 0) return FFRG_OK;
+  int rc = launch_rhs_batched(ctx, bl, st);
+  if (rc) return rc;
+  batched_flow_frozen_control_kernel<<<n, 1024, 0, st>>>(fa);
   return set_cuda_error(ctx, cudaGetLastError(), "batched flow step");
 }
 

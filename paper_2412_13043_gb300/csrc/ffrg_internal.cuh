@@ -625,6 +625,10 @@ int launch_flow_batched_init(ffrg_ctx *ctx, const FlowArgs *fa, int n_flows, int
                              cudaStream_t s);
 int launch_flow_batched_step(ffrg_ctx *ctx, const FlowArgs *fa, int n_flows, int max_ny, const BatchList &bl,
                              cudaStream_t s);
+// The same step with the stages side by side: bl lists kStages descriptors per
+// flow, each writing its part of the flow's raw buffer (kStages x ny).
+int launch_flow_batched_wide_step(ffrg_ctx *ctx, const FlowArgs *fa, int n_flows, const BatchList &bl,
+                                  cudaStream_t s);
 
 // Launch `kern` on `s`; with `early`, as a programmatic dependent of the
 // kernel launched just before it (its CTAs may start while that kernel runs

@@ -54,7 +54,7 @@ struct ServeReq {
   ffrg_flow_stats stats{};
   double latency = 0.0;
   Clock::time_point t_submit;
-  size_t need = 0;   // device bytes while resident
+  size_t need = 0, need_wide = 0;   // device bytes while resident: one set of RHS scratch, and one per stage
   int ny = 0;
 };
 
@@ -62,9 +62,10 @@ struct ServeReq {
 struct SlotLayout {
   Plan pl;
   int ny, npsi;
-  size_t bytes;
+  int stages;   // sets of RHS scratch: kStages (a step's stages side by side), or 1
+  size_t bytes, stage_bytes;   // stage_bytes: one set of RHS scratch
   size_t o_tab, o_tab32, o_y, o_ys, o_K, o_raw, o_radF, o_radF32, o_radq, o_radq32, o_kc, o_extp, o_psis, o_part;
-  size_t o_kbuf;
+  size_t o_kbuf, o_stage;
   size_t o_rx, o_rw, o_a1x, o_a1w, o_a2x, o_a2w, o_psx, o_psw;
 };
 
@@ -74,7 +75,7 @@ static size_t seg(size_t &used, size_t bytes) {
   return off;
 }
 
-static void slot_layout(const ffrg_problem *pb, const ffrg_table_desc *td, SlotLayout &L) {
+static void slot_layout(const ffrg_problem *pb, const ffrg_table_desc *td, int stages, SlotLayout &L) {
   Plan &pl = L.pl;
   pl = Plan();
   plan_geometry(&pl, pb, td);
@@ -83,12 +84,23 @@ static void slot_layout(const ffrg_problem *pb, const ffrg_table_desc *td, SlotL
   L.npsi = std::max(1, pl.n_ext_ang);
   const size_t d = sizeof(double);
   size_t u = 0;
+  L.stages = stages;
   L.o_tab = seg(u, (size_t)pl.tab_count * d);
-  L.o_tab32 = seg(u, (size_t)pl.tab32_count * sizeof(float2));
   L.o_y = seg(u, (size_t)L.ny * d);
   L.o_ys = seg(u, (size_t)L.ny * d);
   L.o_K = seg(u, (size_t)7 * L.ny * d);
-  L.o_raw = seg(u, (size_t)pl.n_ext * d);
+  L.o_raw = seg(u, (size_t)pl.n_ext * d * stages);
+  L.o_rx = seg(u, (size_t)pl.nr * d);
+  L.o_rw = seg(u, (size_t)pl.nr * d);
+  L.o_a1x = seg(u, (size_t)pl.na1 * d);
+  L.o_a1w = seg(u, (size_t)pl.na1 * d);
+  L.o_a2x = seg(u, d);
+  L.o_a2w = seg(u, d);
+  L.o_psx = seg(u, (size_t)L.npsi * d);
+  L.o_psw = seg(u, (size_t)L.npsi * d);
+  // RHS scratch, `stages` times
+  L.o_stage = (u + 255) & ~(size_t)255;
+  L.o_tab32 = seg(u, (size_t)pl.tab32_count * sizeof(float2));
   L.o_radF = seg(u, (size_t)pl.nr * pl.nfreq * d);
   L.o_radq = seg(u, (size_t)pl.nr * d);
   L.o_radq32 = seg(u, (size_t)pl.nr * sizeof(float));
@@ -98,15 +110,8 @@ static void slot_layout(const ffrg_problem *pb, const ffrg_table_desc *td, SlotL
   L.o_extp = seg(u, (size_t)pl.n_ext_p * d);
   L.o_psis = seg(u, (size_t)L.npsi * d);
   L.o_part = seg(u, (size_t)pl.fn_items * d);
-  L.o_rx = seg(u, (size_t)pl.nr * d);
-  L.o_rw = seg(u, (size_t)pl.nr * d);
-  L.o_a1x = seg(u, (size_t)pl.na1 * d);
-  L.o_a1w = seg(u, (size_t)pl.na1 * d);
-  L.o_a2x = seg(u, d);
-  L.o_a2w = seg(u, d);
-  L.o_psx = seg(u, (size_t)L.npsi * d);
-  L.o_psw = seg(u, (size_t)L.npsi * d);
-  L.bytes = u;
+  L.stage_bytes = ((u + 255) & ~(size_t)255) - L.o_stage;
+  L.bytes = u + L.stage_bytes * (stages - 1);
 }
 
 // First-fit allocator over one device reservation; host bookkeeping only.
@@ -160,7 +165,7 @@ struct Slot {
   unsigned char *buf = nullptr;
   size_t cap = 0;
   SlotLayout L;
-  RhsArgs ra;
+  RhsArgs ra[kStages];   // ra[0] also takes the first derivative
   FlowArgs fa;
   bool fresh = false;    // admitted, first derivative not yet taken
   bool cooling = false;  // retired while a tick that still lists it is in flight
@@ -199,9 +204,9 @@ struct Server {
   FlowCtl *ctl_host = nullptr;        // pinned, kTickDepth snapshots of the control blocks
   cudaEvent_t tick_ev[kTickDepth] = {};  // end of the tick whose snapshot is in buffer b
   unsigned *status_dev = nullptr;
-  LaunchSet step_set, init_set;
-  unsigned char *stage_host = nullptr;  // pinned staging of descriptor uploads, two buffers
-  cudaEvent_t stage_ev[2] = {};         // end of the last upload from staging buffer 0 / 1
+  LaunchSet step_set, wide_set, init_set;   // flows stage by stage, flows with their stages side by side, new flows
+  unsigned char *stage_host = nullptr;  // pinned staging of descriptor uploads, four buffers
+  cudaEvent_t stage_ev[4] = {};         // end of the last upload from each staging buffer
   int stage_i = 0;
   size_t stage_bytes = 0;
   ffrg_serve_stats stats{};
@@ -233,16 +238,6 @@ static int slot_setup(Server &S, int si) {
   pl.a2_w = (double *)(b + L.o_a2w);
   pl.psi_x = (double *)(b + L.o_psx);
   pl.psi_w = (double *)(b + L.o_psw);
-  pl.radF = (double *)(b + L.o_radF);
-  pl.radq = (double *)(b + L.o_radq);
-  pl.radq32 = (float *)(b + L.o_radq32);
-  pl.radF32 = (float *)(b + L.o_radF32);
-  pl.kconst = b + L.o_kc;
-  pl.kbuf = pl.kbuf_count ? (double *)(b + L.o_kbuf) : nullptr;
-  pl.ext_pd = (double *)(b + L.o_extp);
-  pl.psi_s = (double *)(b + L.o_psis);
-  pl.partial = (double *)(b + L.o_part);
-  pl.tab32 = (float2 *)(b + L.o_tab32);
   struct Up { void *dst; const void *src; size_t n; } ups[] = {
       {b + L.o_tab, r->tab.data(), r->tab.size() * d}, {b + L.o_y, r->y0.data(), r->y0.size() * d},
       {pl.rad_x, rx.data(), rx.size() * d},           {pl.rad_w, rw.data(), rw.size() * d},
@@ -277,12 +272,26 @@ static int slot_setup(Server &S, int si) {
   e = cudaStreamSynchronize(S.io);
   if (e != cudaSuccess) return set_cuda_error(&S.lc, e, "serve upload sync");
   if (!plan_grid(&pl, &r->td, S.lc.device)) return set_cuda_error(&S.lc, cudaGetLastError(), "function tables");
-  fill_args(&pl, &r->pb, &r->td, (const double *)(b + L.o_tab), r->Lambda, sl.ra);
-  sl.ra.fused_ctr = nullptr;   // batched kernels only
-  sl.ra.out = (double *)(b + L.o_raw);
-  sl.ra.status = S.status_dev;
-  sl.ra.k_dev = &ctl->k_stage;
-  sl.ra.skip = &ctl->done;
+  for (int q = 0; q < L.stages; ++q) {
+    RhsArgs &ra = sl.ra[q];
+    unsigned char *bq = b + (size_t)q * L.stage_bytes;
+    pl.radF = (double *)(bq + L.o_radF);
+    pl.radq = (double *)(bq + L.o_radq);
+    pl.radq32 = (float *)(bq + L.o_radq32);
+    pl.radF32 = (float *)(bq + L.o_radF32);
+    pl.kconst = bq + L.o_kc;
+    pl.kbuf = pl.kbuf_count ? (double *)(bq + L.o_kbuf) : nullptr;
+    pl.ext_pd = (double *)(bq + L.o_extp);
+    pl.psi_s = (double *)(bq + L.o_psis);
+    pl.partial = (double *)(bq + L.o_part);
+    pl.tab32 = (float2 *)(bq + L.o_tab32);
+    fill_args(&pl, &r->pb, &r->td, (const double *)(b + L.o_tab), r->Lambda, ra);
+    ra.fused_ctr = nullptr;   // batched kernels only
+    ra.out = (double *)(b + L.o_raw) + (size_t)q * L.ny;
+    ra.status = S.status_dev;
+    ra.k_dev = L.stages == kStages ? &ctl->k_stages[q] : &ctl->k_stage;
+    ra.skip = &ctl->done;
+  }
   FlowArgs &f = sl.fa;
   memset(&f, 0, sizeof(f));
   f.ny = L.ny;
@@ -314,10 +323,12 @@ static size_t set_bytes_of(int cap) {
          sizeof(long long) * kMaxBatchGroups * (cap + 1);
 }
 
-// Upload the descriptors of the given slots as one compact launch set.
-static int build_set(Server &S, const std::vector<int> &ids, LaunchSet &ls) {
-  const int n = (int)ids.size(), cap = (int)S.slots.size();
-  ls.n = n;
+// Upload the descriptors of the given slots as one compact launch set, `per`
+// descriptors a flow (its stages, or one; first: the first derivative, at
+// the control block's stage scale).
+static int build_set(Server &S, const std::vector<int> &ids, int per, bool first, LaunchSet &ls) {
+  const int n_flows = (int)ids.size(), n = n_flows * per, cap = (int)S.slots.size() * kStages;
+  ls.n = n_flows;
   ls.max_ny = 0;
   BatchList &bl = ls.bl;
   bl = BatchList();
@@ -341,13 +352,14 @@ static int build_set(Server &S, const std::vector<int> &ids, LaunchSet &ls) {
     gcost(g)[0] = 0;
   }
   for (int i = 0; i < n; ++i) {
-    const Slot &sl = S.slots[ids[i]];
-    hd[i] = sl.ra;
-    hf[i] = sl.fa;
-    hl[i] = ids[i];
+    const Slot &sl = S.slots[ids[i / per]];
+    hd[i] = sl.ra[i % per];
+    if (first) hd[i].k_dev = &sl.fa.ctl->k_stage;
+    if (i % per == 0) hf[i / per] = sl.fa;
+    hl[i] = ids[i / per];
     ls.max_ny = std::max(ls.max_ny, sl.L.ny);
     bl.max_ext = std::max(bl.max_ext, sl.L.pl.n_ext);
-    bl.max_pre = std::max(bl.max_pre, precompute_blocks(sl.ra, 64));
+    bl.max_pre = std::max(bl.max_pre, precompute_blocks(sl.ra[0], 64));
     const size_t smem = smem32_of(sl.L.pl);
     const int occ = std::max(1, std::min(4, batched_ctas_per_sm(&S.lc, sl.L.pl.model, smem)));
     const int g = (sl.L.pl.model == FFRG_MODEL_D3 ? 0 : 4) + occ - 1;
@@ -364,7 +376,7 @@ static int build_set(Server &S, const std::vector<int> &ids, LaunchSet &ls) {
   e = cudaMemcpyAsync(ls.descs, stage, set_bytes_of(cap), cudaMemcpyHostToDevice, S.st);
   if (e == cudaSuccess) e = cudaEventRecord(S.stage_ev[S.stage_i], S.st);
   if (e != cudaSuccess) return set_cuda_error(&S.lc, e, "serve descriptor upload");
-  S.stage_i ^= 1;
+  S.stage_i = (S.stage_i + 1) & 3;
   int *dl = ls.lists;
   const long long *dc = (const long long *)(dl + list_ints(cap));
   bl.descs = ls.descs;
@@ -428,7 +440,7 @@ static int retire(Server &S, int si, const FlowCtl &c, int status) {
 static int admit(Server &S) {
   for (;;) {
     ServeReq *r = nullptr;
-    int si = -1;
+    int si = -1, stages = 1;
     {
       std::lock_guard<std::mutex> lock(S.mu);
       while (!S.queue.empty() && S.queue.front()->cancel) {
@@ -441,17 +453,22 @@ static int admit(Server &S) {
       for (int i = 0; i < (int)S.slots.size() && si < 0; ++i)
         if (!S.slots[i].req && !S.slots[i].cooling) si = i;
       if (si < 0) return FFRG_OK;
-      unsigned char *buf = S.arena.take(r->need);
+      // scratch for all stages of a step while it stays within a slot's
+      // share of the budget, so that as many flows are resident as without
+      const size_t wide = Arena::round(r->need_wide);
+      unsigned char *buf = wide <= S.arena.size / S.slots.size() ? S.arena.take(wide) : nullptr;
+      stages = buf ? kStages : 1;
+      if (!buf) buf = S.arena.take(r->need);
       if (!buf) return FFRG_OK;
       S.queue.pop_front();
       r->state = kResident;
       Slot &sl = S.slots[si];
       sl.req = r;
       sl.buf = buf;
-      sl.cap = r->need;
+      sl.cap = stages == kStages ? r->need_wide : r->need;
     }
     Slot &sl = S.slots[si];
-    slot_layout(&r->pb, &r->td, sl.L);
+    slot_layout(&r->pb, &r->td, stages, sl.L);
     int st = slot_setup(S, si);
     if (st) return st;
     std::lock_guard<std::mutex> lock(S.mu);
@@ -541,7 +558,7 @@ static void scheduler(Server *Sp) {
       if (S.slots[i].fresh) fresh.push_back(i);
     }
     if (!fresh.empty()) {
-      st = build_set(S, fresh, S.init_set);
+      st = build_set(S, fresh, 1, true, S.init_set);
       if (!st) st = launch_flow_batched_init(&S.lc, S.init_set.fa, S.init_set.n, S.init_set.max_ny, S.init_set.bl,
                                             S.st);
       if (st) break;
@@ -555,7 +572,10 @@ static void scheduler(Server *Sp) {
       continue;
     }
     if (changed) {
-      st = build_set(S, live, S.step_set);
+      std::vector<int> narrow, wide;
+      for (int i : live) (S.slots[i].L.stages == kStages ? wide : narrow).push_back(i);
+      st = build_set(S, narrow, 1, false, S.step_set);
+      if (!st) st = build_set(S, wide, kStages, false, S.wide_set);
       if (st) break;
       changed = false;
     }
@@ -563,7 +583,8 @@ static void scheduler(Server *Sp) {
     // the control blocks into this tick's host buffer
     const long long id = ++launched;
     const int b = (int)(id % kTickDepth);
-    st = launch_flow_batched_step(&S.lc, S.step_set.fa, S.step_set.n, S.step_set.max_ny, S.step_set.bl, S.st);
+    st = launch_flow_batched_wide_step(&S.lc, S.wide_set.fa, S.wide_set.n, S.wide_set.bl, S.st);
+    if (!st) st = launch_flow_batched_step(&S.lc, S.step_set.fa, S.step_set.n, S.step_set.max_ny, S.step_set.bl, S.st);
     if (st) break;
     cudaError_t e = cudaMemcpyAsync(S.ctl_host + (size_t)b * S.slots.size(), S.ctl_dev,
                                     sizeof(FlowCtl) * S.slots.size(), cudaMemcpyDeviceToHost, S.st);
@@ -616,33 +637,33 @@ extern "C" int ffrg_serve_start(ffrg_ctx *ctx, const ffrg_serve_opts *opts) {
   S->lc.server = nullptr;
   S->lc.profiling = 0;
   S->lc.prof_used = 0;
-  const int cap = opts->max_slots;
+  const int cap = opts->max_slots, dcap = cap * kStages;   // flows, descriptors of a launch set
   S->slots.resize(cap);
-  const size_t set_bytes = set_bytes_of(cap);
+  const size_t set_bytes = set_bytes_of(dcap);
   S->stage_bytes = set_bytes;
   cudaError_t e = cudaStreamCreateWithFlags(&S->st, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S->io, cudaStreamNonBlocking);
   for (int b = 0; b < kTickDepth; ++b)
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&S->tick_ev[b], cudaEventDisableTiming);
-  for (int b = 0; b < 2; ++b)
+  for (int b = 0; b < 4; ++b)
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&S->stage_ev[b], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMalloc((void **)&S->ctl_dev, sizeof(FlowCtl) * cap);
   if (e == cudaSuccess) e = cudaMemset(S->ctl_dev, 0, sizeof(FlowCtl) * cap);
   if (e == cudaSuccess) e = cudaMallocHost((void **)&S->ctl_host, sizeof(FlowCtl) * cap * kTickDepth);
   if (e == cudaSuccess) e = cudaMalloc((void **)&S->status_dev, 16);
   if (e == cudaSuccess) e = cudaMemset(S->status_dev, 0, 16);
-  if (e == cudaSuccess) e = cudaMallocHost((void **)&S->stage_host, set_bytes * 2);
+  if (e == cudaSuccess) e = cudaMallocHost((void **)&S->stage_host, set_bytes * 4);
   // the whole HBM budget of the resident flows, reserved once
   const size_t arena_bytes = S->opts.hbm_budget_bytes & ~(size_t)255;
   if (e == cudaSuccess) e = cudaMalloc((void **)&S->arena_mem, std::max<size_t>(arena_bytes, 256));
   if (e == cudaSuccess) S->arena.init(S->arena_mem, arena_bytes);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();  // the memsets above ran on the legacy stream
-  for (LaunchSet *ls : {&S->step_set, &S->init_set}) {
+  for (LaunchSet *ls : {&S->step_set, &S->wide_set, &S->init_set}) {
     unsigned char *blk = nullptr;
     if (e == cudaSuccess) e = cudaMalloc((void **)&blk, set_bytes);
     ls->descs = (RhsArgs *)blk;
-    ls->fa = (FlowArgs *)(blk + sizeof(RhsArgs) * cap);
-    ls->lists = (int *)(blk + (sizeof(RhsArgs) + sizeof(FlowArgs)) * cap);
+    ls->fa = (FlowArgs *)(blk + sizeof(RhsArgs) * dcap);
+    ls->lists = (int *)(blk + (sizeof(RhsArgs) + sizeof(FlowArgs)) * dcap);
   }
   if (e != cudaSuccess) {
     int st = set_cuda_error(ctx, e, "ffrg_serve_start");
@@ -652,10 +673,11 @@ extern "C" int ffrg_serve_start(ffrg_ctx *ctx, const ffrg_serve_opts *opts) {
     cudaFreeHost(S->stage_host);
     cudaFree(S->arena_mem);
     cudaFree(S->step_set.descs);
+    cudaFree(S->wide_set.descs);
     cudaFree(S->init_set.descs);
     for (int b = 0; b < kTickDepth; ++b)
       if (S->tick_ev[b]) cudaEventDestroy(S->tick_ev[b]);
-    for (int b = 0; b < 2; ++b)
+    for (int b = 0; b < 4; ++b)
       if (S->stage_ev[b]) cudaEventDestroy(S->stage_ev[b]);
     if (S->io) cudaStreamDestroy(S->io);
     if (S->st) cudaStreamDestroy(S->st);
@@ -680,7 +702,9 @@ extern "C" int ffrg_serve_submit(ffrg_ctx *ctx, const ffrg_problem *pb, const ff
       o->max_steps < 1)
     return FFRG_EINVAL;
   SlotLayout L;
-  slot_layout(pb, desc, L);
+  slot_layout(pb, desc, kStages, L);
+  const size_t need_wide = L.bytes;
+  slot_layout(pb, desc, 1, L);
   if (smem32_of(L.pl) > 227 * 1024) return FFRG_EINVAL;
   ServeReq *r = new ServeReq();
   r->pb = *pb;
@@ -690,6 +714,7 @@ extern "C" int ffrg_serve_submit(ffrg_ctx *ctx, const ffrg_problem *pb, const ff
   r->tab.assign(tables_host, tables_host + (size_t)L.pl.tab_count);
   r->y0.assign(y0_host, y0_host + L.ny);
   r->need = L.bytes;
+  r->need_wide = need_wide;
   r->ny = L.ny;
   std::lock_guard<std::mutex> lock(S->mu);
   if (S->stop) {
@@ -773,9 +798,10 @@ extern "C" int ffrg_serve_stop(ffrg_ctx *ctx) {
   cudaFree(S->status_dev);
   cudaFreeHost(S->stage_host);
   cudaFree(S->step_set.descs);
+  cudaFree(S->wide_set.descs);
   cudaFree(S->init_set.descs);
   for (int b = 0; b < kTickDepth; ++b) cudaEventDestroy(S->tick_ev[b]);
-  for (int b = 0; b < 2; ++b) cudaEventDestroy(S->stage_ev[b]);
+  for (int b = 0; b < 4; ++b) cudaEventDestroy(S->stage_ev[b]);
   cudaStreamDestroy(S->io);
   cudaStreamDestroy(S->st);
   const int fatal = S->fatal;
