@@ -376,14 +376,15 @@ void plan_geometry(Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td) 
       fn_chunks = (outer_total + fcr - 1) / fcr;
       fn_items = pl->n_ext * fn_chunks;
     } else if (pb->model == FFRG_MODEL_FINITE_T) {
-      // rows of K: (stack row j, |p|) x radial node, the whole angle rule per row
+      // rows of K: (stack row j, |p|, radial node) in memory order, the whole
+      // angle rule per row; an item is a multiple of 32 consecutive rows, so
+      // that lanes stay busy whatever n_rad is
       fjb = pl->na1;
-      const long long n_outer = (long long)(pl->N + pl->n_ext_ang) * pl->n_ext_p;
-      long long rpi = (n_outer * pl->nr + kTargetItems - 1) / kTargetItems;
-      rpi = std::min<long long>(std::max<long long>((rpi + 31) / 32 * 32, 32), 256);
-      fcr = (int)std::min<long long>(rpi, pl->nr);
-      fn_chunks = (pl->nr + fcr - 1) / fcr;
-      fn_items = (int)(n_outer * fn_chunks);
+      const long long rows = (long long)(pl->N + pl->n_ext_ang) * pl->n_ext_p * pl->nr;
+      long long rpi = (rows + kTargetItems - 1) / kTargetItems;
+      fcr = (int)std::min<long long>(std::max<long long>((rpi + 31) / 32 * 32, 32), 256);
+      fn_chunks = 1;
+      fn_items = (int)((rows + fcr - 1) / fcr);
     } else {
       const long long total_outer = (long long)pl->n_ext * outer_total;
       const long long kRowsWanted = 152LL * 2048;

@@ -595,7 +595,7 @@ struct BatchList {
   int n_flows;
   BatchGroup groups[kMaxBatchGroups];
   int n_groups;
-  int max_ext, max_pre;          // largest n_ext and precompute block count among the flows
+  int max_fin, max_pre;          // largest finalize and precompute block counts among the flows
 };
 // resident CTAs per SM of the serving main kernel of `model` with `smem` bytes
 int batched_ctas_per_sm(ffrg_ctx *ctx, int model, size_t smem);
@@ -685,6 +685,8 @@ int launch_ref64(ffrg_ctx *ctx, Plan *pl, const RhsArgs &a, cudaStream_t s);
 int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl, const RhsArgs &a, int precision, cudaStream_t s,
                       bool contract);
 int launch_precompute(ffrg_ctx *ctx, const RhsArgs &a, cudaStream_t s);
+// blocks of the finalize kernel for one flow
+int finalize_blocks(const RhsArgs &a);
 // blocks of the precompute kernel for one RHS (at most cap)
 int precompute_blocks(const RhsArgs &a, int cap);
 int launch_jacobian(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc *td, const double *tab, double k,

@@ -119,7 +119,13 @@ extern "C" int ffrg_rhs_noalloc(const ffrg_problem *pb, const ffrg_table_desc *t
   pl.psi_s = sc.take<double>(npsi);
   pl.tab32 = sc.take<float2>((size_t)pl.tab32_count);
   if (pl.kbuf_count) pl.kbuf = sc.take<double>(pl.kbuf_count);
-  pl.partial = sc.take<double>(is_d4(pb->model) ? pl.fn_items : std::max(pl.fn_items, pl.fn_items64));
+  // (finite T: no partial sums, but the same limit as when each K row's radial chunks had one)
+  size_t sums = is_d4(pb->model) ? pl.fn_items : std::max(pl.fn_items, pl.fn_items64);
+  if (pb->model == FFRG_MODEL_FINITE_T) {
+    const int cr = std::min(pl.fcr, pl.nr);
+    sums = (size_t)(pl.N + pl.n_ext_ang) * pl.n_ext_p * ((pl.nr + cr - 1) / cr);
+  }
+  pl.partial = sc.take<double>(sums);
   if (sc.used > kNoallocScratchBytes) return FFRG_EINVAL;  // problem needs more than the 4 MiB scratch
 
   // the tables must fit in shared memory as plain values (FP64 line form: twice as large, in global memory when

@@ -722,20 +722,24 @@ __device__ __forceinline__ void zl_lookup(const float2 *tab, const RhsArgs &a, c
 // instead of (2N+1) M angular sums per (p, r).
 template <typename T, bool POLE>
 __device__ __forceinline__ void ftk_rows(const RhsArgs &a, const RhsArgs *sa, const SmemLayout<T> &S,
-                                         const KConst<T> &kc, int outer, int c, int lane,
-                                         const T *q_loc = nullptr, const T *p_loc = nullptr) {
+                                         const KConst<T> &kc, int item, int lane, const T *q_loc = nullptr,
+                                         const T *p_loc = nullptr) {
   const T sy = kc.sy;
   const int np = a.n_pts, na1 = a.na1, nr = a.nr;
-  const int jk = outer / a.n_ext_p, ip = outer - jk * a.n_ext_p;
-  const int srow = min(jk, a.n_stack - 1);
-  const T om = kc.twopiT * ((T)jk + (T)(a.stat ? 0.5 : 0.0));   // omega_j or nu_j
-  const T om2s = om * om * kc.som;
-  // p and q from the precompute's arrays, or (q_loc, p_loc) from the block's
-  // own copies of the same values
-  const T p = p_loc ? p_loc[ip] : (T)a.ext_pd[ip];
-  T *K = (T *)a.kbuf + ((size_t)jk * a.n_ext_p + ip) * nr;
-  const int r0 = c * a.cr, r1 = min(r0 + a.cr, nr);
-  for (int r = r0 + lane; r < r1; r += 32) {
+  // first row of the item: (outer0, r0), outer = stack row x |p|
+  const long long R0 = (long long)item * a.cr;
+  const int outer0 = R0 >> 31 ? (int)(R0 / nr) : (int)R0 / nr, r0 = (int)(R0 - (long long)outer0 * nr);
+  const int n_outer = (a.N + a.n_ext_ang) * a.n_ext_p;
+  T *K = (T *)a.kbuf + R0;
+  for (int i = lane; i < a.cr; i += 32) {
+    const int outer = outer0 + (r0 + i) / nr, r = (r0 + i) % nr, jk = outer / a.n_ext_p, ip = outer - jk * a.n_ext_p;
+    if (outer >= n_outer) break;
+    const int srow = min(jk, a.n_stack - 1);
+    const T om = kc.twopiT * ((T)jk + (T)(a.stat ? 0.5 : 0.0));   // omega_j or nu_j
+    const T om2s = om * om * kc.som;
+    // p and q from the precompute's arrays, or (q_loc, p_loc) from the block's
+    // own copies of the same values
+    const T p = p_loc ? p_loc[ip] : (T)a.ext_pd[ip];
     const T q = q_loc ? q_loc[r] : radial_q<T>(a, r);
     const T by = fma(q, q, p * p) * sy, ty = (T)2 * q * p * sy;   // explicit FMAs, as in d3_witem
     T rs = 0;
@@ -747,7 +751,7 @@ __device__ __forceinline__ void ftk_rows(const RhsArgs &a, const RhsArgs *sa, co
       auto pole = [&]() { return pole_ftk(sa, ip, jk, r, j); };
       rs = fma(S.w1[j] * Lv, inv_prop<POLE>(a, Z, y, om2s, kc, pole), rs);
     }
-    K[r] = rs;
+    K[i] = rs;
   }
 }
 
@@ -1313,16 +1317,15 @@ __global__ void __launch_bounds__(kMainThreads<T>, MinBlocks<T>::value) rhs_main
   if constexpr (sizeof(T) == 8) kc.us = S.fx;
   const bool pole = pole_possible(a, S, kc);
   if constexpr (MODEL == FFRG_MODEL_FINITE_T) {
-    // K rows: items (stack row, |p|) x chunk of radial nodes from the counter
+    // K rows: items of consecutive rows (stack row, |p|, radial node) from the counter
     const int lane = threadIdx.x & 31;
     for (;;) {
       int d = 0;
       if (lane == 0) d = (int)atomicAdd(a.work_ctr, 1u);
       d = __shfl_sync(0xffffffffu, d, 0);
       if (d >= a.n_items) break;
-      const int outer = d / a.n_chunks, c = d - outer * a.n_chunks;
-      if (sizeof(T) == 4 && pole) ftk_rows<T, true>(a, &sa, S, kc, outer, c, lane);
-      else ftk_rows<T, false>(a, &sa, S, kc, outer, c, lane);
+      if (sizeof(T) == 4 && pole) ftk_rows<T, true>(a, &sa, S, kc, d, lane);
+      else ftk_rows<T, false>(a, &sa, S, kc, d, lane);
     }
   } else {
     if (sizeof(T) == 4 && pole) item_loop<MODEL, T, true>(a, &sa, S, kc);
@@ -1459,9 +1462,8 @@ __global__ void __launch_bounds__(kThreadsWide, 1) ft_single_kernel(const __grid
       if (lane == 0) d = (int)atomicAdd(cnt, 1u);
       d = __shfl_sync(0xffffffffu, d, 0);
       if (d >= a.n_items) break;
-      const int outer = d / a.n_chunks, c = d - outer * a.n_chunks;
-      if (pole) ftk_rows<float, true>(a, &sa, S, kc, outer, c, lane, q_loc, p_loc);
-      else ftk_rows<float, false>(a, &sa, S, kc, outer, c, lane, q_loc, p_loc);
+      if (pole) ftk_rows<float, true>(a, &sa, S, kc, d, lane, q_loc, p_loc);
+      else ftk_rows<float, false>(a, &sa, S, kc, d, lane, q_loc, p_loc);
     }
   grid_arrive(cnt + 1);
   ok = grid_wait(cnt + 1, base + gridDim.x, a.status, &s_ok) && ok;
@@ -1642,7 +1644,7 @@ int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int 
   // (k on the device: the FP32 constants would cost an FP64 chain per CTA)
   constexpr int kSingleLaunchItems = 152 * (kThreads / 32);
   if (mixed && a.model == FFRG_MODEL_FINITE_T && contract && a.fused_ctr && !a.k_dev && !a.m2_dev &&
-      a.n_items >= kSingleLaunchItems) {
+      (long long)a.n_items * a.cr >= 32LL * kSingleLaunchItems) {
     st = launch_ft_single(ctx, pl, a, s);
     if (st != kNoSingleLaunch) return st;   // else the three launches below
   }
@@ -1687,20 +1689,76 @@ __global__ void __launch_bounds__(kThreads) batched_precompute_kernel(const RhsA
   precompute_body(a);
 }
 
-// one block per external point blockIdx.x of flow blockIdx.y: finite T
-// contracts K (the same function as the single-flow kernel), d=3 sums the
-// item partials in warp 0
+// Outputs m0 .. m0 + kMTile - 1 of external momentum ip from K, by the block:
+// for each output the terms, order and accumulators of ft_contract, but the
+// radial factors and (through L1) the K rows that the outputs share are read
+// once.  One output at a time read 2 x (2N+1) n_rad values each from L2, which
+// bounded the kernel (48 flows x 5 stages of the serving mix: 300 us, so 173).
+constexpr int kMTile = 9;
+__device__ __forceinline__ void ft_contract_tile(const RhsArgs &a, int ip, int m0, double (*red)[kThreads / 32]) {
+  const int nm = min(a.n_ext_ang - m0, kMTile), nr = a.nr, n_lo = -a.N - a.stat;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kThreads / 32;
+  const float *K = (const float *)a.kbuf + (size_t)ip * nr;
+  const size_t row_step = (size_t)a.n_ext_p * nr;
+  auto krow = [&](int row, int m) { return K + (size_t)stack_index(a.stat, row + n_lo + m0 + m) * row_step; };
+  RowAcc<float> acc[kMTile];
+  int row = warp;
+  for (; row + 3 * nw < a.nfreq; row += 4 * nw) {
+    const int o = row * nr, dn = nw * nr;
+    for (int r = lane; r < nr; r += 32) {
+      const float f0 = a.radF32[o + r], f1 = a.radF32[o + dn + r], f2 = a.radF32[o + 2 * dn + r],
+                  f3 = a.radF32[o + 3 * dn + r];
+#pragma unroll
+      for (int m = 0; m < kMTile; ++m) {
+        if (m >= nm) break;
+        acc[m].add(f0, krow(row, m)[r]);
+        acc[m].add(f1, krow(row + nw, m)[r]);
+        acc[m].add(f2, krow(row + 2 * nw, m)[r]);
+        acc[m].add(f3, krow(row + 3 * nw, m)[r]);
+      }
+    }
+  }
+  for (; row < a.nfreq; row += nw)
+    for (int r = lane; r < nr; r += 32) {
+      const float f = a.radF32[row * nr + r];
+#pragma unroll
+      for (int m = 0; m < kMTile; ++m) {
+        if (m >= nm) break;
+        acc[m].add(f, krow(row, m)[r]);
+      }
+    }
+#pragma unroll
+  for (int m = 0; m < kMTile; ++m) {
+    if (m >= nm) break;
+    const double w = acc[m].item_sum();
+    if (lane == 0) red[m][warp] = w;
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < nm) {
+    double t = 0.0;
+    for (int j = 0; j < nw; ++j) t += red[threadIdx.x][j];
+    write_output(a, ip * a.n_ext_ang + m0 + threadIdx.x, t);
+  }
+}
+
+// blocks of one flow's finalize: finite T a tile of external frequencies of one momentum each, d=3 an output
+// per warp
+int finalize_blocks(const RhsArgs &a) {
+  return a.model == FFRG_MODEL_FINITE_T ? a.n_ext_p * ((a.n_ext_ang + kMTile - 1) / kMTile)
+                                        : (a.n_ext + kThreads / 32 - 1) / (kThreads / 32);
+}
 __global__ void __launch_bounds__(kThreads) batched_finalize_kernel(const RhsArgs *descs) {
-  __shared__ double red[kThreads / 32];
+  __shared__ double red[kMTile][kThreads / 32];
   const RhsArgs &a = descs[blockIdx.y];
-  const int e = blockIdx.x;
-  if (skipped(a) || e >= a.n_ext) return;   // uniform over the block
+  if (skipped(a)) return;   // uniform over the block
   if (a.model == FFRG_MODEL_FINITE_T) {
-    const double t = ft_contract<float>(a, e, red, threadIdx.x, blockDim.x, 0);
-    if (threadIdx.x == 0) write_output(a, e, t);
-  } else if (threadIdx.x < 32) {
-    const double t = sum_partials(a, e, threadIdx.x);
-    if (threadIdx.x == 0) write_output(a, e, t);
+    const int tiles = (a.n_ext_ang + kMTile - 1) / kMTile, ip = blockIdx.x / tiles;
+    if (ip < a.n_ext_p) ft_contract_tile(a, ip, (blockIdx.x - ip * tiles) * kMTile, red);
+  } else {
+    const int e = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (e >= a.n_ext) return;
+    const double t = sum_partials(a, e, lane);
+    if (lane == 0) write_output(a, e, t);
   }
 }
 
@@ -1750,16 +1808,16 @@ __global__ void __launch_bounds__(kThreads, 4)
     // the flow's FP32 tables by one bulk copy (up to ~150 KB for finite T)
     if (!stage_to_smem_phase<float2>(S.tab, sa.tab32, sa.tab32_count, &bar, parity, sa.status)) return;
     parity ^= 1u;
-    stage_angles<float>(sa, S);
+    stage_angles<float, false>(sa, S);   // d=3 and finite T: no sqrt(1 - c^2)
     __syncthreads();
     const KConst<float> kc = load_kconst<float>(sa);
     const bool pole = pole_possible(sa, S, kc);
     for (int g = lo + warp; g < hi; g += nw) {
       const int item = g - start[f];
       const int e = item / sa.n_chunks, c = item - e * sa.n_chunks;
-      if constexpr (MODEL == FFRG_MODEL_FINITE_T) {   // K rows (e: stack row x |p|)
-        if (pole) ftk_rows<float, true>(sa, &sa, S, kc, e, c, lane);
-        else ftk_rows<float, false>(sa, &sa, S, kc, e, c, lane);
+      if constexpr (MODEL == FFRG_MODEL_FINITE_T) {   // K rows
+        if (pole) ftk_rows<float, true>(sa, &sa, S, kc, item, lane);
+        else ftk_rows<float, false>(sa, &sa, S, kc, item, lane);
       } else {
         const double acc = pole ? witem<MODEL, float, true>(sa, &sa, S, kc, e, c, lane).item_sum()
                                 : witem<MODEL, float, false>(sa, &sa, S, kc, e, c, lane).item_sum();
@@ -1823,7 +1881,7 @@ int launch_rhs_batched(ffrg_ctx *ctx, const BatchList &bl, cudaStream_t s) {
                                   : launch_batched_main<FFRG_MODEL_FINITE_T>(ctx, bl.descs, G, s);
   }
   if (st) return st;
-  batched_finalize_kernel<<<dim3(std::max(1, bl.max_ext), bl.n_flows), kThreads, 0, s>>>(bl.descs);
+  batched_finalize_kernel<<<dim3(std::max(1, bl.max_fin), bl.n_flows), kThreads, 0, s>>>(bl.descs);
   return set_cuda_error(ctx, cudaGetLastError(), "batched rhs launch");
 }
 

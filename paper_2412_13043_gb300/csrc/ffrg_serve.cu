@@ -358,7 +358,7 @@ static int build_set(Server &S, const std::vector<int> &ids, int per, bool first
     if (i % per == 0) hf[i / per] = sl.fa;
     hl[i] = ids[i / per];
     ls.max_ny = std::max(ls.max_ny, sl.L.ny);
-    bl.max_ext = std::max(bl.max_ext, sl.L.pl.n_ext);
+    bl.max_fin = std::max(bl.max_fin, finalize_blocks(sl.ra[0]));
     bl.max_pre = std::max(bl.max_pre, precompute_blocks(sl.ra[0], 64));
     const size_t smem = smem32_of(sl.L.pl);
     const int occ = std::max(1, std::min(4, batched_ctas_per_sm(&S.lc, sl.L.pl.model, smem)));
