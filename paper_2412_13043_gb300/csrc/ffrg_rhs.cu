@@ -1684,6 +1684,7 @@ int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int 
 namespace ffrg {
 
 __global__ void __launch_bounds__(kThreads) batched_precompute_kernel(const RhsArgs *descs) {
+  pdl_trigger();   // the main kernel may become resident; it waits for this one's writes
   const RhsArgs &a = descs[blockIdx.y];
   if (skipped(a)) return;
   precompute_body(a);
@@ -1693,7 +1694,7 @@ __global__ void __launch_bounds__(kThreads) batched_precompute_kernel(const RhsA
 // for each output the terms, order and accumulators of ft_contract, but the
 // radial factors and (through L1) the K rows that the outputs share are read
 // once.  One output at a time read 2 x (2N+1) n_rad values each from L2, which
-// bounded the kernel (48 flows x 5 stages of the serving mix: 300 us, so 173).
+// bounded the kernel (48 flows x 5 stages of the serving mix: 300 us, so 136).
 constexpr int kMTile = 9;
 __device__ __forceinline__ void ft_contract_tile(const RhsArgs &a, int ip, int m0, double (*red)[kThreads / 32]) {
   const int nm = min(a.n_ext_ang - m0, kMTile), nr = a.nr, n_lo = -a.N - a.stat;
@@ -1747,7 +1748,7 @@ int finalize_blocks(const RhsArgs &a) {
   return a.model == FFRG_MODEL_FINITE_T ? a.n_ext_p * ((a.n_ext_ang + kMTile - 1) / kMTile)
                                         : (a.n_ext + kThreads / 32 - 1) / (kThreads / 32);
 }
-__global__ void __launch_bounds__(kThreads) batched_finalize_kernel(const RhsArgs *descs) {
+__global__ void __launch_bounds__(kThreads, 4) batched_finalize_kernel(const RhsArgs *descs) {
   __shared__ double red[kMTile][kThreads / 32];
   const RhsArgs &a = descs[blockIdx.y];
   if (skipped(a)) return;   // uniform over the block
@@ -1762,6 +1763,11 @@ __global__ void __launch_bounds__(kThreads) batched_finalize_kernel(const RhsArg
   }
 }
 
+// One persistent launch over all flows, whatever their model and table sizes:
+// one 1024-thread CTA per SM, so that 32 warps share one copy of a flow's
+// tables (with 256-thread CTAs the shared memory of large tables left 8 warps
+// an SM, and flows had to be launched in groups of equal occupancy one after
+// the other: four launches of 475 us together a tick of 48 serving flows, one of 410).
 // Each CTA takes a contiguous range of the combined item list holding an
 // equal share of the estimated cost (cost[f] is cumulative at the flow
 // boundaries, uniform per item within a flow), so that flows with longer
@@ -1778,12 +1784,10 @@ __device__ __forceinline__ int item_at_cost(const int *start, const long long *c
   return start[f] + (int)min((long long)items, (x - cost[f]) * items / w);
 }
 
-template <int MODEL>
-__global__ void __launch_bounds__(kThreads, 4)
-    batched_main_kernel(const RhsArgs *descs, const int *flows, const int *start, const long long *cost, int n_fl) {
+__global__ void __launch_bounds__(kThreadsWide, 1)
+    batched_main_kernel(const RhsArgs *descs, const int *start, const long long *cost, int n_fl) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ RhsArgs sa;
-  __shared__ int skip;
   __shared__ uint64_t bar;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   mbar_init_once(&bar);
@@ -1792,18 +1796,16 @@ __global__ void __launch_bounds__(kThreads, 4)
   const int g0 = blockIdx.x == 0 ? 0 : item_at_cost(start, cost, n_fl, W * blockIdx.x / gridDim.x);
   const int g1 = blockIdx.x + 1 == gridDim.x ? start[n_fl]
                                              : item_at_cost(start, cost, n_fl, W * (blockIdx.x + 1) / gridDim.x);
+  pdl_wait();   // the precompute kernel's tables, factors and constants
   int f = 0;
   while (f < n_fl && start[f + 1] <= g0) ++f;
   for (; f < n_fl && start[f] < g1; ++f) {
     const int lo = max(g0, start[f]), hi = min(g1, start[f + 1]);
     if (lo >= hi) continue;
     __syncthreads();  // the previous segment's tables are no longer read
-    if (threadIdx.x == 0) {
-      sa = descs[flows[f]];
-      skip = skipped(sa);
-    }
+    copy_args(&sa, descs[f]);
     __syncthreads();
-    if (skip) continue;
+    if (skipped(sa)) continue;   // uniform: the flag does not change while the kernel runs
     SmemLayout<float> S(smem, sa);
     // the flow's FP32 tables by one bulk copy (up to ~150 KB for finite T)
     if (!stage_to_smem_phase<float2>(S.tab, sa.tab32, sa.tab32_count, &bar, parity, sa.status)) return;
@@ -1812,75 +1814,31 @@ __global__ void __launch_bounds__(kThreads, 4)
     __syncthreads();
     const KConst<float> kc = load_kconst<float>(sa);
     const bool pole = pole_possible(sa, S, kc);
-    for (int g = lo + warp; g < hi; g += nw) {
-      const int item = g - start[f];
-      const int e = item / sa.n_chunks, c = item - e * sa.n_chunks;
-      if constexpr (MODEL == FFRG_MODEL_FINITE_T) {   // K rows
-        if (pole) ftk_rows<float, true>(sa, &sa, S, kc, item, lane);
-        else ftk_rows<float, false>(sa, &sa, S, kc, item, lane);
-      } else {
-        const double acc = pole ? witem<MODEL, float, true>(sa, &sa, S, kc, e, c, lane).item_sum()
-                                : witem<MODEL, float, false>(sa, &sa, S, kc, e, c, lane).item_sum();
+    if (sa.model == FFRG_MODEL_FINITE_T) {   // K rows
+      for (int g = lo + warp; g < hi; g += nw)
+        if (pole) ftk_rows<float, true>(sa, &sa, S, kc, g - start[f], lane);
+        else ftk_rows<float, false>(sa, &sa, S, kc, g - start[f], lane);
+    } else {
+      for (int g = lo + warp; g < hi; g += nw) {
+        const int item = g - start[f], e = item / sa.n_chunks, c = item - e * sa.n_chunks;
+        const double acc = pole ? witem<FFRG_MODEL_D3, float, true>(sa, &sa, S, kc, e, c, lane).item_sum()
+                                : witem<FFRG_MODEL_D3, float, false>(sa, &sa, S, kc, e, c, lane).item_sum();
         if (lane == 0) sa.partial[item] = acc;
       }
     }
   }
 }
 
-// resident CTAs per SM of the batched main kernel for a shared-memory size,
-// memoised per (model, bytes, device): the serving scheduler asks for every
-// flow of every launch set and every launch
-template <int MODEL>
-static int batched_occupancy(ffrg_ctx *ctx, size_t smem, int *per_sm) {
-  static std::mutex mu;
-  static std::map<std::tuple<int, size_t, int>, int> memo;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = memo.find({MODEL, smem, ctx->device});
-    if (it != memo.end()) {
-      *per_sm = it->second;
-      return FFRG_OK;
-    }
-  }
-  void (*kern)(const RhsArgs *, const int *, const int *, const long long *, int) = batched_main_kernel<MODEL>;
-  int st = ensure_smem_limit(ctx, (const void *)kern, smem);
-  if (st) return st;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, kThreads, smem);
-  if (e != cudaSuccess || *per_sm < 1) return set_cuda_error(ctx, e ? e : cudaErrorInvalidConfiguration, "occupancy");
-  std::lock_guard<std::mutex> lock(mu);
-  memo[{MODEL, smem, ctx->device}] = *per_sm;
-  return FFRG_OK;
-}
-
-int batched_ctas_per_sm(ffrg_ctx *ctx, int model, size_t smem) {
-  int per_sm = 1;
-  const int st = model == FFRG_MODEL_D3 ? batched_occupancy<FFRG_MODEL_D3>(ctx, smem, &per_sm)
-                                        : batched_occupancy<FFRG_MODEL_FINITE_T>(ctx, smem, &per_sm);
-  return st ? 1 : per_sm;
-}
-
-template <int MODEL>
-static int launch_batched_main(ffrg_ctx *ctx, const RhsArgs *descs, const BatchGroup &G, cudaStream_t s) {
-  if (G.n == 0 || G.items == 0) return FFRG_OK;
-  int per_sm = 0;
-  int st = batched_occupancy<MODEL>(ctx, G.smem, &per_sm);
-  if (st) return st;
-  const int ctas = (G.items + kThreads / 32 - 1) / (kThreads / 32);
-  const int grid = std::max(1, std::min(ctas, per_sm * ctx->num_sms));
-  batched_main_kernel<MODEL><<<grid, kThreads, G.smem, s>>>(descs, G.flows, G.start, G.cost, G.n);
-  return FFRG_OK;
-}
-
 int launch_rhs_batched(ffrg_ctx *ctx, const BatchList &bl, cudaStream_t s) {
   if (bl.n_flows == 0) return FFRG_OK;
-  batched_precompute_kernel<<<dim3(std::max(1, bl.max_pre), bl.n_flows), kThreads, 0, s>>>(bl.descs);
-  int st = FFRG_OK;
-  for (int g = 0; g < bl.n_groups && !st; ++g) {
-    const BatchGroup &G = bl.groups[g];
-    st = G.model == FFRG_MODEL_D3 ? launch_batched_main<FFRG_MODEL_D3>(ctx, bl.descs, G, s)
-                                  : launch_batched_main<FFRG_MODEL_FINITE_T>(ctx, bl.descs, G, s);
-  }
+  const int st = ensure_smem_limit(ctx, (const void *)batched_main_kernel, bl.smem);
   if (st) return st;
+  batched_precompute_kernel<<<dim3(std::max(1, bl.max_pre), bl.n_flows), kThreads, 0, s>>>(bl.descs);
+  constexpr int kWarps = kThreadsWide / 32;
+  const int grid = std::max(1, std::min((bl.items + kWarps - 1) / kWarps, ctx->num_sms));
+  const cudaError_t e = launch_dependent(batched_main_kernel, dim3(grid), dim3(kThreadsWide), bl.smem, s, true, bl.descs,
+                                         bl.start, bl.cost, bl.n_flows);
+  if (e != cudaSuccess) return set_cuda_error(ctx, e, "batched rhs launch");
   batched_finalize_kernel<<<dim3(std::max(1, bl.max_fin), bl.n_flows), kThreads, 0, s>>>(bl.descs);
   return set_cuda_error(ctx, cudaGetLastError(), "batched rhs launch");
 }

@@ -175,7 +175,6 @@ struct Slot {
 struct LaunchSet {
   RhsArgs *descs = nullptr;
   FlowArgs *fa = nullptr;
-  int *lists = nullptr;  // [all | d3 flows | d3 start | ft flows | ft start]
   BatchList bl{};
   int n = 0, max_ny = 0;
 };
@@ -314,13 +313,9 @@ static size_t smem32_of(const Plan &pl) {
   return pl.smem32;
 }
 
-// Launch set layout: descs | fa | lists (cap ints: all flows, then per group
-// cap flow indices and cap + 1 item offsets; padded to an even count so that
-// what follows is 8-byte aligned) | per group cap + 1 cost prefixes.
-static int list_ints(int cap) { return (cap + kMaxBatchGroups * (2 * cap + 1) + 1) & ~1; }
+// Launch set layout: descs | fa | cost prefixes (cap + 1) | item prefixes (cap + 1).
 static size_t set_bytes_of(int cap) {
-  return (sizeof(RhsArgs) + sizeof(FlowArgs)) * cap + sizeof(int) * list_ints(cap) +
-         sizeof(long long) * kMaxBatchGroups * (cap + 1);
+  return (sizeof(RhsArgs) + sizeof(FlowArgs)) * cap + (sizeof(long long) + sizeof(int)) * (cap + 1);
 }
 
 // Upload the descriptors of the given slots as one compact launch set, `per`
@@ -333,65 +328,44 @@ static int build_set(Server &S, const std::vector<int> &ids, int per, bool first
   BatchList &bl = ls.bl;
   bl = BatchList();
   if (n == 0) return FFRG_OK;
-  // host staging: descs | fa | lists | costs, in the staging buffer whose
-  // previous upload has ended (two buffers used in turn)
+  // host staging: in the staging buffer whose previous upload has ended (four
+  // buffers used in turn)
   unsigned char *stage = S.stage_host + (size_t)S.stage_i * S.stage_bytes;
   cudaError_t e = cudaEventSynchronize(S.stage_ev[S.stage_i]);
   if (e != cudaSuccess) return set_cuda_error(&S.lc, e, "serve staging wait");
   RhsArgs *hd = (RhsArgs *)stage;
   FlowArgs *hf = (FlowArgs *)(stage + sizeof(RhsArgs) * cap);
-  int *hl = (int *)(stage + (sizeof(RhsArgs) + sizeof(FlowArgs)) * cap);
-  long long *hc = (long long *)(hl + list_ints(cap));
-  int gn[kMaxBatchGroups] = {}, gitems[kMaxBatchGroups] = {};
-  size_t gsmem[kMaxBatchGroups] = {};
-  auto gflows = [&](int g) { return hl + cap + g * (2 * cap + 1); };
-  auto gstart = [&](int g) { return gflows(g) + cap; };
-  auto gcost = [&](int g) { return hc + (size_t)g * (cap + 1); };
-  for (int g = 0; g < kMaxBatchGroups; ++g) {
-    gstart(g)[0] = 0;
-    gcost(g)[0] = 0;
-  }
+  long long *hc = (long long *)(hf + cap);
+  int *hs = (int *)(hc + cap + 1);
+  hc[0] = 0;
+  hs[0] = 0;
+  // precompute blocks per descriptor: about two waves of the four resident on
+  // an SM.  A block is a chain of FP64 functions with little work, so 64 for
+  // each of 240 descriptors (25 waves) took 94 us a tick, 52 us so.
+  const int pre_cap = std::min(64, std::max(8, 2 * 4 * S.lc.num_sms / n));
   for (int i = 0; i < n; ++i) {
     const Slot &sl = S.slots[ids[i / per]];
     hd[i] = sl.ra[i % per];
     if (first) hd[i].k_dev = &sl.fa.ctl->k_stage;
     if (i % per == 0) hf[i / per] = sl.fa;
-    hl[i] = ids[i / per];
     ls.max_ny = std::max(ls.max_ny, sl.L.ny);
     bl.max_fin = std::max(bl.max_fin, finalize_blocks(sl.ra[0]));
-    bl.max_pre = std::max(bl.max_pre, precompute_blocks(sl.ra[0], 64));
-    const size_t smem = smem32_of(sl.L.pl);
-    const int occ = std::max(1, std::min(4, batched_ctas_per_sm(&S.lc, sl.L.pl.model, smem)));
-    const int g = (sl.L.pl.model == FFRG_MODEL_D3 ? 0 : 4) + occ - 1;
+    bl.max_pre = std::max(bl.max_pre, precompute_blocks(sl.ra[0], pre_cap));
+    bl.smem = std::max(bl.smem, smem32_of(sl.L.pl));
     // estimated cost of one item: rows x (angle nodes per row + per-row work)
-    const long long cost = (long long)sl.L.pl.fn_items * sl.L.pl.fcr * (sl.L.pl.fjb + 1);
-    const int k = gn[g]++;
-    gflows(g)[k] = i;
-    gitems[g] += sl.L.pl.fn_items;
-    gstart(g)[k + 1] = gitems[g];
-    gcost(g)[k + 1] = gcost(g)[k] + cost;
-    gsmem[g] = std::max(gsmem[g], smem);
+    hc[i + 1] = hc[i] + (long long)sl.L.pl.fn_items * sl.L.pl.fcr * (sl.L.pl.fjb + 1);
+    hs[i + 1] = hs[i] + sl.L.pl.fn_items;
   }
+  bl.items = hs[n];
   // stream order on the tick stream: after every tick that reads the old set
   e = cudaMemcpyAsync(ls.descs, stage, set_bytes_of(cap), cudaMemcpyHostToDevice, S.st);
   if (e == cudaSuccess) e = cudaEventRecord(S.stage_ev[S.stage_i], S.st);
   if (e != cudaSuccess) return set_cuda_error(&S.lc, e, "serve descriptor upload");
   S.stage_i = (S.stage_i + 1) & 3;
-  int *dl = ls.lists;
-  const long long *dc = (const long long *)(dl + list_ints(cap));
   bl.descs = ls.descs;
   bl.n_flows = n;
-  for (int g = 0; g < kMaxBatchGroups; ++g) {
-    if (gn[g] == 0) continue;
-    BatchGroup &G = bl.groups[bl.n_groups++];
-    G.model = g < 4 ? FFRG_MODEL_D3 : FFRG_MODEL_FINITE_T;
-    G.flows = dl + cap + g * (2 * cap + 1);
-    G.start = G.flows + cap;
-    G.cost = dc + (size_t)g * (cap + 1);
-    G.n = gn[g];
-    G.items = gitems[g];
-    G.smem = gsmem[g];
-  }
+  bl.cost = (const long long *)(ls.fa + cap);
+  bl.start = (const int *)(bl.cost + cap + 1);
   return FFRG_OK;
 }
 
@@ -663,7 +637,6 @@ extern "C" int ffrg_serve_start(ffrg_ctx *ctx, const ffrg_serve_opts *opts) {
     if (e == cudaSuccess) e = cudaMalloc((void **)&blk, set_bytes);
     ls->descs = (RhsArgs *)blk;
     ls->fa = (FlowArgs *)(blk + sizeof(RhsArgs) * dcap);
-    ls->lists = (int *)(blk + (sizeof(RhsArgs) + sizeof(FlowArgs)) * dcap);
   }
   if (e != cudaSuccess) {
     int st = set_cuda_error(ctx, e, "ffrg_serve_start");
