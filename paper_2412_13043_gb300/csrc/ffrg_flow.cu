@@ -136,8 +136,40 @@ __global__ void flow_start_kernel(FlowCtl *c) {   // one block
   write_stage_scales(c);
 }
 
+// Accept (returned) or reject the step of error norm err, and the next step
+// size (same controller as the CPU oracle).  One thread.
+__device__ __forceinline__ int step_control(FlowCtl *c, double err, int anybad) {
+  const double h = c->h;
+  c->err = err;
+  int acc = 0;
+  if (anybad) {
+    c->status = FFRG_ENONFINITE;
+    c->done = 1;
+  } else if (err <= 1.0) {
+    acc = 1;
+    c->t += h;
+    c->steps += 1;
+    double fac = (err == 0.0) ? 5.0 : 0.9 * pow(err, -0.2);
+    fac = fmin(fmax(fac, 0.2), 5.0);
+    if (c->last_rejected) fac = fmin(fac, 1.0);
+    c->last_rejected = 0;
+    c->dt = h * fac;
+  } else {
+    c->rejects += 1;
+    if (h <= c->dt_min) {
+      c->status = FFRG_ESTEP_UNDERFLOW;
+      c->done = 1;
+    } else {
+      c->dt = h * fmax(0.9 * pow(err, -0.2), 0.2);
+      c->last_rejected = 1;
+    }
+  }
+  c->dt = fmin(fmax(c->dt, c->dt_min), c->dt_max);
+  return acc;
+}
+
 // Error norm max_i |h sum_r E_r K_r,i| / (atol + rtol max(|y_i|, |y5_i|)),
-// accept / reject, step-size update (same controller as the CPU oracle).
+// accept / reject, step-size update.
 __device__ __forceinline__ void flow_control_body(const FlowArgs &f) {
   FlowCtl *c = f.ctl;
   __shared__ double red[32];
@@ -174,32 +206,7 @@ __device__ __forceinline__ void flow_control_body(const FlowArgs &f) {
       err = fmax(err, red[w]);
       anybad |= bad_s[w];
     }
-    c->err = err;
-    int acc = 0;
-    if (anybad) {
-      c->status = FFRG_ENONFINITE;
-      c->done = 1;
-    } else if (err <= 1.0) {
-      acc = 1;
-      c->t += h;
-      c->steps += 1;
-      double fac = (err == 0.0) ? 5.0 : 0.9 * pow(err, -0.2);
-      fac = fmin(fmax(fac, 0.2), 5.0);
-      if (c->last_rejected) fac = fmin(fac, 1.0);
-      c->last_rejected = 0;
-      c->dt = h * fac;
-    } else {
-      c->rejects += 1;
-      if (h <= c->dt_min) {
-        c->status = FFRG_ESTEP_UNDERFLOW;
-        c->done = 1;
-      } else {
-        c->dt = h * fmax(0.9 * pow(err, -0.2), 0.2);
-        c->last_rejected = 1;
-      }
-    }
-    c->dt = fmin(fmax(c->dt, c->dt_min), c->dt_max);
-    accept_s = acc;
+    accept_s = step_control(c, err, anybad);
   }
   __syncthreads();
   if (accept_s) {
@@ -214,27 +221,80 @@ __device__ __forceinline__ void flow_control_body(const FlowArgs &f) {
 
 __global__ void __launch_bounds__(1024) flow_control_kernel(FlowArgs f) { flow_control_body(f); }
 
-// End of a frozen step: the derivatives of all stages, the state of the last
-// one, then the control kernel's work and the next scales.  raw: the stages'
-// RHS, kStages x n_ext.
-__device__ __forceinline__ void flow_frozen_control_body(const FlowArgs &f, const double *raw) {
-  FlowCtl *c = f.ctl;
-  if (*(volatile const int *)&c->done) return;
-  const double h = c->h;
-  for (int i = threadIdx.x; i < f.ny; i += blockDim.x) {
-    for (int s = 1; s <= 6; ++s) f.K[(size_t)s * f.ny + i] = -raw[(size_t)min(s - 1, kStages - 1) * f.ny + i];
-    write_stage_state(f, 6, i, h);
+// End of a frozen step, one CTA: the derivatives of all stages, the state of
+// the last one, error norm, accept / reject and step size as in
+// flow_control_body, the next scales.  raw: the stages' RHS, kStages x n_ext.
+// Bound by its chain of dependent loads and FP64 operations, so the control
+// block is worked on in shared memory and the derivatives stay in registers
+// (15.0 us with both in global memory, 11.6 so).  snap: a copy of the
+// control block for the host (or null).
+__device__ __forceinline__ void copy_ctl(FlowCtl *dst, const FlowCtl *src) {
+  static_assert(sizeof(FlowCtl) % 8 == 0, "word copy");
+  for (int i = threadIdx.x; i < (int)(sizeof(FlowCtl) / 8); i += blockDim.x)
+    ((volatile long long *)dst)[i] = ((const volatile long long *)src)[i];
+}
+__device__ __forceinline__ void flow_frozen_control_body(const FlowArgs &f, const double *raw, FlowCtl *snap) {
+  __shared__ FlowCtl c;
+  __shared__ double red[32];
+  __shared__ int accept_s;
+  copy_ctl(&c, f.ctl);
+  __syncthreads();
+  if (c.done) {
+    if (snap) copy_ctl(snap, &c);
+    return;
+  }
+  const double h = c.h, atol = c.atol, rtol = c.rtol;
+  const int ny = f.ny, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double emax = 0.0;
+  int bad = 0;
+  for (int i = threadIdx.x; i < ny; i += blockDim.x) {
+    double K[7];
+    K[0] = f.K[i];
+#pragma unroll
+    for (int s = 1; s <= 6; ++s) K[s] = -raw[(size_t)min(s - 1, kStages - 1) * ny + i];
+    const double y = f.y[i];
+    double y5 = y, e = 0.0;
+#pragma unroll
+    for (int r = 0; r < 6; ++r) y5 += h * kDpA[6][r] * K[r];
+#pragma unroll
+    for (int r = 0; r < 7; ++r) e += kDpE[r] * K[r];
+    e *= h;
+    const double sc = atol + rtol * fmax(fabs(y), fabs(y5));
+    const double ei = fabs(e) / sc;
+    if (!isfinite(ei) || !isfinite(y5)) bad = 1;
+    else emax = fmax(emax, ei);
+    f.ys[i] = y5;
+    f.K[(size_t)6 * ny + i] = K[6];
+  }
+  for (int o = 16; o > 0; o >>= 1) emax = fmax(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+  if (lane == 0) red[warp] = emax;
+  const int anybad = __syncthreads_or(bad);
+  if (warp == 0) {
+    double err = lane < (int)(blockDim.x >> 5) ? red[lane] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) err = fmax(err, __shfl_xor_sync(0xffffffffu, err, o));
+    if (lane == 0) accept_s = step_control(&c, err, anybad);
   }
   __syncthreads();
-  flow_control_body(f);
+  if (accept_s)
+    for (int i = threadIdx.x; i < ny; i += blockDim.x) {
+      f.y[i] = f.ys[i];
+      f.K[i] = f.K[(size_t)6 * ny + i];  // first-same-as-last
+    }
+  if (threadIdx.x == 0 && !c.done) decide_next_step(&c);
   __syncthreads();
-  write_stage_scales(c);
+  write_stage_scales(&c);
+  __syncthreads();
+  copy_ctl(f.ctl, &c);
+  if (snap) copy_ctl(snap, &c);
 }
 __global__ void __launch_bounds__(1024) flow_frozen_control_kernel(FlowArgs f, const double *raw) {
-  flow_frozen_control_body(f, raw);
+  flow_frozen_control_body(f, raw, nullptr);
 }
-__global__ void __launch_bounds__(1024) batched_flow_frozen_control_kernel(const FlowArgs *fa) {
-  flow_frozen_control_body(fa[blockIdx.x], fa[blockIdx.x].raw);
+__global__ void __launch_bounds__(1024) batched_flow_frozen_control_kernel(const FlowArgs *fa, const FlowCtl *ctl0,
+                                                                           FlowCtl *snap) {
+  const FlowArgs f = fa[blockIdx.x];
+  pdl_wait();   // the stages' RHS
+  flow_frozen_control_body(f, f.raw, snap + (f.ctl - ctl0));
 }
 
 // ---------------------------------------------------------------------------
@@ -292,12 +352,13 @@ int launch_flow_batched_step(ffrg_ctx *ctx, const FlowArgs *fa, int n, int max_n
   return set_cuda_error(ctx, cudaGetLastError(), "batched flow step");
 }
 
-int launch_flow_batched_wide_step(ffrg_ctx *ctx, const FlowArgs *fa, int n, const BatchList &bl, cudaStream_t st) {
+int launch_flow_batched_wide_step(ffrg_ctx *ctx, const FlowArgs *fa, int n, const BatchList &bl, const FlowCtl *ctl0,
+                                  FlowCtl *snap, cudaStream_t st) {
   if (n == 0) return FFRG_OK;
   int rc = launch_rhs_batched(ctx, bl, st);
   if (rc) return rc;
-  batched_flow_frozen_control_kernel<<<n, 1024, 0, st>>>(fa);
-  return set_cuda_error(ctx, cudaGetLastError(), "batched flow step");
+  return set_cuda_error(ctx, launch_dependent(batched_flow_frozen_control_kernel, dim3(n), dim3(1024), 0, st, true, fa,
+                                              ctl0, snap), "batched flow step");
 }
 
 // ---------------------------------------------------------------------------

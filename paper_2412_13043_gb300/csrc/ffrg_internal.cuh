@@ -584,6 +584,7 @@ struct BatchList {
   const long long *cost;         // device: cumulative estimated cost at the flow boundaries (n_flows + 1)
   int n_flows, items;
   size_t smem;                   // largest shared-memory need (FP32 path)
+  bool fin_few;                  // small finalize tiles (few flows)
   int max_fin, max_pre;          // largest finalize and precompute block counts among the flows
 };
 int launch_rhs_batched(ffrg_ctx *ctx, const BatchList &bl, cudaStream_t s);
@@ -614,8 +615,10 @@ int launch_flow_batched_step(ffrg_ctx *ctx, const FlowArgs *fa, int n_flows, int
                              cudaStream_t s);
 // The same step with the stages side by side: bl lists kStages descriptors per
 // flow, each writing its part of the flow's raw buffer (kStages x ny).
+// ctl0: control block of slot 0; snap: host-visible copies of the control
+// blocks, by slot, written by the step's last kernel.
 int launch_flow_batched_wide_step(ffrg_ctx *ctx, const FlowArgs *fa, int n_flows, const BatchList &bl,
-                                  cudaStream_t s);
+                                  const FlowCtl *ctl0, FlowCtl *snap, cudaStream_t s);
 
 // Launch `kern` on `s`; with `early`, as a programmatic dependent of the
 // kernel launched just before it (its CTAs may start while that kernel runs
@@ -672,8 +675,8 @@ int launch_ref64(ffrg_ctx *ctx, Plan *pl, const RhsArgs &a, cudaStream_t s);
 int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl, const RhsArgs &a, int precision, cudaStream_t s,
                       bool contract);
 int launch_precompute(ffrg_ctx *ctx, const RhsArgs &a, cudaStream_t s);
-// blocks of the finalize kernel for one flow
-int finalize_blocks(const RhsArgs &a);
+// blocks of the finalize kernel for one flow (few: with small tiles)
+int finalize_blocks(const RhsArgs &a, bool few);
 // blocks of the precompute kernel for one RHS (at most cap)
 int precompute_blocks(const RhsArgs &a, int cap);
 int launch_jacobian(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc *td, const double *tab, double k,

@@ -1695,7 +1695,10 @@ __global__ void __launch_bounds__(kThreads) batched_precompute_kernel(const RhsA
 // radial factors and (through L1) the K rows that the outputs share are read
 // once.  One output at a time read 2 x (2N+1) n_rad values each from L2, which
 // bounded the kernel (48 flows x 5 stages of the serving mix: 300 us, so 136).
-constexpr int kMTile = 9;
+// kMTile frequencies a block; fewer (kMTileFew) when the blocks of all flows
+// do not fill the GPU, where the length of a block's chain counts.
+constexpr int kMTile = 9, kMTileFew = 3;
+template <int kMTile>
 __device__ __forceinline__ void ft_contract_tile(const RhsArgs &a, int ip, int m0, double (*red)[kThreads / 32]) {
   const int nm = min(a.n_ext_ang - m0, kMTile), nr = a.nr, n_lo = -a.N - a.stat;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kThreads / 32;
@@ -1744,17 +1747,21 @@ __device__ __forceinline__ void ft_contract_tile(const RhsArgs &a, int ip, int m
 
 // blocks of one flow's finalize: finite T a tile of external frequencies of one momentum each, d=3 an output
 // per warp
-int finalize_blocks(const RhsArgs &a) {
-  return a.model == FFRG_MODEL_FINITE_T ? a.n_ext_p * ((a.n_ext_ang + kMTile - 1) / kMTile)
+int finalize_blocks(const RhsArgs &a, bool few) {
+  const int tile = few ? kMTileFew : kMTile;
+  return a.model == FFRG_MODEL_FINITE_T ? a.n_ext_p * ((a.n_ext_ang + tile - 1) / tile)
                                         : (a.n_ext + kThreads / 32 - 1) / (kThreads / 32);
 }
+template <int kTile>
 __global__ void __launch_bounds__(kThreads, 4) batched_finalize_kernel(const RhsArgs *descs) {
-  __shared__ double red[kMTile][kThreads / 32];
+  __shared__ double red[kTile][kThreads / 32];
   const RhsArgs &a = descs[blockIdx.y];
+  pdl_trigger();   // the control kernel may become resident
+  pdl_wait();      // K rows, partial sums
   if (skipped(a)) return;   // uniform over the block
   if (a.model == FFRG_MODEL_FINITE_T) {
-    const int tiles = (a.n_ext_ang + kMTile - 1) / kMTile, ip = blockIdx.x / tiles;
-    if (ip < a.n_ext_p) ft_contract_tile(a, ip, (blockIdx.x - ip * tiles) * kMTile, red);
+    const int tiles = (a.n_ext_ang + kTile - 1) / kTile, ip = blockIdx.x / tiles;
+    if (ip < a.n_ext_p) ft_contract_tile<kTile>(a, ip, (blockIdx.x - ip * tiles) * kTile, red);
   } else {
     const int e = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (e >= a.n_ext) return;
@@ -1775,9 +1782,16 @@ __global__ void __launch_bounds__(kThreads, 4) batched_finalize_kernel(const Rhs
 // CTA copies the flow's descriptor and angle rules into shared memory (plain
 // loads) and its FP32 tables (one bulk copy, mbarrier phase per segment); its
 // warps then take the segment's warp-sized items.
-__device__ __forceinline__ int item_at_cost(const int *start, const long long *cost, int n_fl, long long x) {
+// Flow boundaries at or below x among v[1 .. n-1] (increasing), by the whole
+// block: a linear search by every thread cost tens of us at 240 descriptors.
+template <typename V>
+__device__ __forceinline__ int flows_below(const V *v, int n, V x) {
   int f = 0;
-  while (f + 1 < n_fl && cost[f + 1] <= x) ++f;
+  for (int i = 1; i < n; i += blockDim.x) f += __syncthreads_count(i + (int)threadIdx.x < n && v[i + threadIdx.x] <= x);
+  return f;
+}
+__device__ __forceinline__ int item_at_cost(const int *start, const long long *cost, int n_fl, long long x) {
+  const int f = flows_below(cost, n_fl, x);
   const int items = start[f + 1] - start[f];
   const long long w = cost[f + 1] - cost[f];
   if (w <= 0) return start[f];
@@ -1796,9 +1810,9 @@ __global__ void __launch_bounds__(kThreadsWide, 1)
   const int g0 = blockIdx.x == 0 ? 0 : item_at_cost(start, cost, n_fl, W * blockIdx.x / gridDim.x);
   const int g1 = blockIdx.x + 1 == gridDim.x ? start[n_fl]
                                              : item_at_cost(start, cost, n_fl, W * (blockIdx.x + 1) / gridDim.x);
-  pdl_wait();   // the precompute kernel's tables, factors and constants
-  int f = 0;
-  while (f < n_fl && start[f + 1] <= g0) ++f;
+  int f = flows_below(start, n_fl, g0);
+  pdl_trigger();   // the finalize kernel may become resident
+  pdl_wait();      // the precompute kernel's tables, factors and constants
   for (; f < n_fl && start[f] < g1; ++f) {
     const int lo = max(g0, start[f]), hi = min(g1, start[f + 1]);
     if (lo >= hi) continue;
@@ -1839,8 +1853,9 @@ int launch_rhs_batched(ffrg_ctx *ctx, const BatchList &bl, cudaStream_t s) {
   const cudaError_t e = launch_dependent(batched_main_kernel, dim3(grid), dim3(kThreadsWide), bl.smem, s, true, bl.descs,
                                          bl.start, bl.cost, bl.n_flows);
   if (e != cudaSuccess) return set_cuda_error(ctx, e, "batched rhs launch");
-  batched_finalize_kernel<<<dim3(std::max(1, bl.max_fin), bl.n_flows), kThreads, 0, s>>>(bl.descs);
-  return set_cuda_error(ctx, cudaGetLastError(), "batched rhs launch");
+  const cudaError_t ef = launch_dependent(bl.fin_few ? batched_finalize_kernel<kMTileFew> : batched_finalize_kernel<kMTile>,
+                                          dim3(std::max(1, bl.max_fin), bl.n_flows), dim3(kThreads), 0, s, true, bl.descs);
+  return set_cuda_error(ctx, ef, "batched rhs launch");
 }
 
 }  // namespace ffrg

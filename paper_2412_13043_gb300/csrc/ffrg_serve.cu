@@ -342,6 +342,7 @@ static int build_set(Server &S, const std::vector<int> &ids, int per, bool first
   // precompute blocks per descriptor: about two waves of the four resident on
   // an SM.  A block is a chain of FP64 functions with little work, so 64 for
   // each of 240 descriptors (25 waves) took 94 us a tick, 52 us so.
+  int fin_few = 0;
   const int pre_cap = std::min(64, std::max(8, 2 * 4 * S.lc.num_sms / n));
   for (int i = 0; i < n; ++i) {
     const Slot &sl = S.slots[ids[i / per]];
@@ -349,7 +350,8 @@ static int build_set(Server &S, const std::vector<int> &ids, int per, bool first
     if (first) hd[i].k_dev = &sl.fa.ctl->k_stage;
     if (i % per == 0) hf[i / per] = sl.fa;
     ls.max_ny = std::max(ls.max_ny, sl.L.ny);
-    bl.max_fin = std::max(bl.max_fin, finalize_blocks(sl.ra[0]));
+    bl.max_fin = std::max(bl.max_fin, finalize_blocks(sl.ra[0], false));
+    fin_few = std::max(fin_few, finalize_blocks(sl.ra[0], true));
     bl.max_pre = std::max(bl.max_pre, precompute_blocks(sl.ra[0], pre_cap));
     bl.smem = std::max(bl.smem, smem32_of(sl.L.pl));
     // estimated cost of one item: rows x (angle nodes per row + per-row work)
@@ -357,6 +359,8 @@ static int build_set(Server &S, const std::vector<int> &ids, int per, bool first
     hs[i + 1] = hs[i] + sl.L.pl.fn_items;
   }
   bl.items = hs[n];
+  bl.fin_few = (long long)fin_few * n <= 4 * S.lc.num_sms;   // one wave of small tiles
+  if (bl.fin_few) bl.max_fin = fin_few;
   // stream order on the tick stream: after every tick that reads the old set
   e = cudaMemcpyAsync(ls.descs, stage, set_bytes_of(cap), cudaMemcpyHostToDevice, S.st);
   if (e == cudaSuccess) e = cudaEventRecord(S.stage_ev[S.stage_i], S.st);
@@ -557,11 +561,15 @@ static void scheduler(Server *Sp) {
     // the control blocks into this tick's host buffer
     const long long id = ++launched;
     const int b = (int)(id % kTickDepth);
-    st = launch_flow_batched_wide_step(&S.lc, S.wide_set.fa, S.wide_set.n, S.wide_set.bl, S.st);
+    FlowCtl *snap = S.ctl_host + (size_t)b * S.slots.size();
+    st = launch_flow_batched_wide_step(&S.lc, S.wide_set.fa, S.wide_set.n, S.wide_set.bl, S.ctl_dev, snap, S.st);
     if (!st) st = launch_flow_batched_step(&S.lc, S.step_set.fa, S.step_set.n, S.step_set.max_ny, S.step_set.bl, S.st);
     if (st) break;
-    cudaError_t e = cudaMemcpyAsync(S.ctl_host + (size_t)b * S.slots.size(), S.ctl_dev,
-                                    sizeof(FlowCtl) * S.slots.size(), cudaMemcpyDeviceToHost, S.st);
+    // the flows' control blocks for the host: the wide step's last kernel
+    // writes its flows' into the pinned buffer; a copy when others are listed
+    cudaError_t e = cudaSuccess;
+    if (S.step_set.n)
+      e = cudaMemcpyAsync(snap, S.ctl_dev, sizeof(FlowCtl) * S.slots.size(), cudaMemcpyDeviceToHost, S.st);
     if (e == cudaSuccess) e = cudaEventRecord(S.tick_ev[b], S.st);
     if (e != cudaSuccess) {
       st = set_cuda_error(&S.lc, e, "serve tick");
