@@ -137,11 +137,6 @@ __device__ __forceinline__ void adj_scatter(double *g, int lc, int j, AdjPos p, 
   }
 }
 
-// regulator form h at y = x
-__device__ __forceinline__ double adj_h(const RhsArgs &a, const KConst<double> &kc, double x) {
-  return a.reg == FFRG_REG_LITIM ? (x < 1.0 ? 1.0 : x) : fx_h(*kc.us, x);
-}
-
 // ---------------------------------------------------------------------------
 // d = 3:  term = F_r w_j G(s); row = (radial node, block of jb angle nodes)
 // ---------------------------------------------------------------------------
@@ -161,7 +156,7 @@ __device__ __forceinline__ void d3_adjoint_rows(const AdjArgs &A, const AdjSmem 
     const int j = on ? j0 + jj : 0;
     const double y = fma(ty, S.c1[j], by);
     const AdjPos ps = adj_pos(a, kc, y, kc.uy1);
-    const double h = adj_h(a, kc, y), G = fx_rcp(fma(adj_val(S.tab, ps), h, kc.m2));
+    const double h = reg_h(a, kc, y), G = fx_rcp(fma(adj_val(S.tab, ps), h, kc.m2));
     const double wG = on ? S.w1[j] * G : 0.0;
     vrow += wG;
     adj_scatter(g, A.lc, 0, ps, -gF * wG * (G * h), on, lane);
@@ -199,7 +194,7 @@ __device__ __forceinline__ void d4_adjoint_rows(const AdjArgs &A, const AdjSmem 
   const double q = a.radq[r], dF = a.radD[r], q2 = q * q, qp = q * p, c1 = S.c1[ia], w1 = S.w1[ia];
   const double A2 = fma(2.0 * qp, c1, q2 + p2), Ay = A2 * sy;
   const AdjPos pA = adj_pos(a, kc, Ay, kc.uy1);
-  const double hA = adj_h(a, kc, Ay), GA = fx_rcp(fma(adj_val(Zt, pA), hA, kc.m2));
+  const double hA = reg_h(a, kc, Ay), GA = fx_rcp(fma(adj_val(Zt, pA), hA, kc.m2));
   const double GPA = -GA * (GA * hA);        // d GA / d Z(A) / k^2
   const double gF = gn * a.radF[r] * w1;     // d(out)/d(row value) x gbar
   double v;                                  // row value (without F w1)
@@ -229,7 +224,7 @@ __device__ __forceinline__ void d4_adjoint_rows(const AdjArgs &A, const AdjSmem 
       const double By = fma(-t2y, cw.x, b0);
       const AdjPos pB = adj_pos(a, kc, By, kc.uy1), pb = adj_pos(a, kc, by + By, kc.uy3),
                    pc = adj_pos(a, kc, sab + By, kc.uy3);
-      const double h = adj_h(a, kc, By), GB = fx_rcp(fma(adj_val(Zt, pB), h, kc.m2));
+      const double h = reg_h(a, kc, By), GB = fx_rcp(fma(adj_val(Zt, pB), h, kc.m2));
       const double lb = adj_val(L3, pb), lc_ = adj_val(L3, pc);
       const double wG = cw.y * GB, t = gFA * wG, cb = t * lc_;
       rs = fma(wG * lb, lc_, rs);

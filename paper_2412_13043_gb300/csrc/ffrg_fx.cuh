@@ -146,7 +146,9 @@ FX_FN void fx_node(const FxGrid &g, int64_t u, int &i, double &w1) {
 FX_FN double fx_h(const FxTables &T, double x) {
   const uint64_t b = fx_bits(x);
   const int E = (int)(b >> 52) - 1023;
-  if (E >= 6) return x <= 0.0 ? 1.0 : x;   // x >= 64, infinity, NaN; a negative x (rounding) counts as 0
+  // x >= 64, infinity, NaN; a negative x (rounding) counts as 0 (comparisons
+  // on the bits: an FP64 one would run on the FP64 pipe, branch taken or not)
+  if (E >= 6) return (b >> 63) && b <= 0xFFF0000000000000ull ? 1.0 : x;
   const uint64_t m = 0x8000000000000000ull | (b << 11);
   // position of x in [0, 1), or of x/2^E - 1, as a 64-bit fraction
   const uint64_t f = E < 0 ? (E < -64 ? 0 : m >> (-E - 1)) : m << 1;
@@ -164,6 +166,12 @@ FX_FN double fx_h(const FxTables &T, double x) {
   const int s = (int)(H >> 63);
   H >>= s;
   return fx_double(((uint64_t)(e + 1022 + s) << 52) + ((H + 512) >> 10));   // the leading bit adds 1 to the exponent
+}
+
+// flat shape: max(1, x), 1 for negative x
+FX_FN double fx_h_flat(double x) {
+  const uint64_t b = fx_bits(x);
+  return b < 0x3FF0000000000000ull || ((b >> 63) && b <= 0xFFF0000000000000ull) ? 1.0 : x;
 }
 
 // 1/d: an FP32 seed (relative error e ~ 2^-22) and 1/d = r (1 + e + e^2) + O(e^3)

@@ -115,14 +115,16 @@ __device__ __forceinline__ void stage_fx(const RhsArgs &a, FxTables *s) {
 
 // Node and weight of the coordinate of y (FP64 lookups): fixed point, or an
 // FP64 logarithm when the grid or k lies outside its range.
-static __device__ __noinline__ void slow_node(const RhsArgs *a, double s2, int c, int &i, double &w1) {
+// (y and 1/sy are passed apart: their product in the caller was computed ahead
+// of the branch, three FP64 multiplications a d=4 term.)
+static __device__ __noinline__ void slow_node(const RhsArgs *a, double y, double isy, int c, int &i, double &w1) {
   double w;
-  lerp_pos(s2, a->u_scale, a->uoc[c - 1], a->n_pts, i, w);
+  lerp_pos(y * isy, a->u_scale, a->uoc[c - 1], a->n_pts, i, w);
   w1 = 1.0 + w;
 }
 __device__ __forceinline__ void node_of(const RhsArgs &a, const KConst<double> &kc, double y, FxOff o, int &i,
                                         double &w1) {
-  if (kc.slow) slow_node(&a, y * kc.isy, o.c, i, w1);   // uniform
+  if (kc.slow) slow_node(&a, y, kc.isy, o.c, i, w1);   // uniform
   else fx_node(a.fg, fx_log(kc.us->log, a.fg, y) + o.v, i, w1);
 }
 __device__ __forceinline__ double line64(double2 t, double w1) { return fma(t.y, w1, t.x); }
@@ -142,18 +144,26 @@ __device__ __forceinline__ double look(const double2 *row, double y, Look64 us, 
   return line64(row[i], w1);
 }
 
-// Inverse propagator from the line-form Z value (times k^2), y = sy s^2 and
-// om2s = omega^2/k^2: Z (s^2 + k^2 r) = Z k^2 h(x), h(x) = x + r(x) = x/(1 -
-// e^{-x}) from the fixed-point tables (flat shape: max(1, x)).
-template <bool POLE = true, typename Pole>
-__device__ __forceinline__ double inv_prop(const RhsArgs &a, double Zk, double y, double om2s,
-                                           const KConst<double> &kc, Pole &&) {
-  const double x = a.model == FFRG_MODEL_D4_FULL ? y * kc.inv_k2 : y;   // sy s^2 = x otherwise
-  double h = a.reg == FFRG_REG_LITIM ? (x < 1.0 ? 1.0 : x) : fx_h(*kc.us, x);
-  if (a.model == FFRG_MODEL_FINITE_T) h += om2s;
-  return fx_rcp(fma(Zk, h, kc.m2));
+// Regulator form h(x) = x + r(x): x/(1 - e^{-x}), flat shape max(1, x).
+__device__ __forceinline__ double reg_h(const RhsArgs &a, const KConst<double> &kc, double x) {
+  if (a.reg == FFRG_REG_LITIM) return fx_h_flat(x);
+  return fx_h(*kc.us, x);
 }
 
+// Inverse propagator from the line-form Z value (times k^2), y = sy s^2 and
+// om2s = omega^2/k^2: Z (s^2 + k^2 r) = Z k^2 h(x).  OM: finite T (om2s
+// counts); FULL: y = s^2.  Template arguments because the compiler computes
+// both sides of such a choice, and each FP64 instruction costs a warp 16
+// clocks: four of them, on the model, the shape and the sign of x, made a d=4
+// term 16.4 FP64 instructions instead of 12.4 (4.05 -> 3.07 ms on the d=4
+// vertex workload).
+template <bool POLE = true, bool OM = false, bool FULL = false, typename Pole>
+__device__ __forceinline__ double inv_prop(const RhsArgs &a, double Zk, double y, double om2s,
+                                           const KConst<double> &kc, Pole &&) {
+  double h = reg_h(a, kc, FULL ? y * kc.inv_k2 : y);
+  if (OM) h += om2s;
+  return fx_rcp(fma(Zk, h, kc.m2));
+}
 // Kinetic part P = k^2 h(x) (= s^2 + k^2 r), regulator derivative rd = k^2
 // rdot(x) and table position of a loop momentum s^2 = x k^2.  FP64 RHS:
 // rdot = 2 h^2 e^{-x} (exact also where e^{-x} is small) and the coordinate

@@ -128,7 +128,7 @@ __device__ __forceinline__ float reg_g(int reg, float y) {
 // Z (omega^2 + s^2 + k^2 r), i.e. P < -2 m^2: close to the convexity pole.
 // `pole` is only evaluated on that rare branch.  POLE = false drops the test;
 // callers use it only when m^2 >= 0 and no Z < 0, where P >= 0 >= -2 m^2.
-template <bool POLE = true, typename Pole>
+template <bool POLE = true, bool OM = false, bool FULL = false, typename Pole>
 __device__ __forceinline__ float inv_prop(const RhsArgs &a, float Zs, float y, float om2s, const KConst<float> &kc,
                                           Pole &&pole) {
   // the denominator is one explicit FMA in both variants and the sum an
@@ -468,9 +468,9 @@ __device__ bool main_prologue(const RhsArgs &a, SmemLayout<T> &S, uint64_t *bar)
 // 2. main kernels.  FP64 (d=4 vertex workload, 1281 x 131072 terms): the FP64
 // pipe bounds a term at 134 instructions (three logarithms, an exponential,
 // two divisions, clamps and conversions), 41.5 ms; with those functions in
-// fixed point on the integer pipe (ffrg_fx.cuh) a term has 11 FP64
-// instructions (arguments, interpolations, products) and about 150 clocks of
-// integer work, which overlap: 4.04 ms.
+// fixed point on the integer pipe (ffrg_fx.cuh) a term has 12.4 FP64
+// instructions (arguments, interpolations, products and its share of a row)
+// and about 150 clocks of integer work, which overlap: 3.07 ms.
 // Work items are warp-sized: external point e x a chunk of
 // `cr` outer rows (d=3: radial nodes; finite T: (Matsubara n, radial node)
 // pairs; d=4: (radial node, first-angle node) pairs).  Lane l takes rows
@@ -749,7 +749,7 @@ __device__ __forceinline__ void ftk_rows(const RhsArgs &a, const RhsArgs *sa, co
       T Z, Lv;
       zl_lookup(S.tab, a, kc, srow, y, Z, Lv);
       auto pole = [&]() { return pole_ftk(sa, ip, jk, r, j); };
-      rs = fma(S.w1[j] * Lv, inv_prop<POLE>(a, Z, y, om2s, kc, pole), rs);
+      rs = fma(S.w1[j] * Lv, inv_prop<POLE, true>(a, Z, y, om2s, kc, pole), rs);
     }
     K[i] = rs;
   }
@@ -1119,7 +1119,7 @@ __device__ __forceinline__ RowAcc<T> d4_witem(const RhsArgs &a, const RhsArgs *s
     const T Ay = A2 * sy;
     const T ZA = look(Zt, Ay, us, kc.uy1, np);
     auto pole_a = [&]() { return pole_d4<FULL ? FFRG_MODEL_D4_FULL : FFRG_MODEL_D4_VERTEX>(sa, e, r, ia, -1); };
-    const T GA = inv_prop<POLE>(a, ZA, Ay, (T)0, kc, pole_a);
+    const T GA = inv_prop<POLE, false, FULL>(a, ZA, Ay, (T)0, kc, pole_a);
     T v;
     if (block == 0) {
       const T l4 = look(L4, (q2 + p2) * sy, us, kc.uy2, np);
@@ -1162,7 +1162,7 @@ __device__ __forceinline__ RowAcc<T> d4_witem(const RhsArgs &a, const RhsArgs *s
         auto pole_b = [&]() { return pole_d4<FULL ? FFRG_MODEL_D4_FULL : FFRG_MODEL_D4_VERTEX>(sa, e, r, ia, b); };
         T GB;
         if constexpr (sizeof(T) == 4 && !POLE) GB = prop1(By, ZB, kc.m2);   // one reciprocal
-        else GB = inv_prop<POLE>(a, ZB, By, (T)0, kc, pole_b);
+        else GB = inv_prop<POLE, false, FULL>(a, ZB, By, (T)0, kc, pole_b);
         T lb, lc;
         if constexpr (FULL) {
           T a_b, a_c, b_b, b_c;

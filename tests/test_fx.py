@@ -22,6 +22,7 @@ static FxTables T;
 extern "C" {
 void init() { fx_build_tables(&T); }
 double h(double x) { return fx_h(T, x); }
+double flat(double x) { return fx_h_flat(x); }
 double rcp(double x) { return fx_rcp(x); }
 int grid(int n, double lo, double hi, FxGrid *g) { return fx_grid(n, lo, hi, g); }
 int node(const FxGrid *g, double y, double *w1) {
@@ -42,7 +43,7 @@ def fx(tmp_path_factory):
     inc = os.path.join(HERE, "..", "paper_2412_13043_gb300", "csrc")
     subprocess.run(["g++", "-O1", "-shared", "-fPIC", "-I", inc, str(d / "fx.cpp"), "-o", str(d / "fx.so")], check=True)
     lib = ctypes.CDLL(str(d / "fx.so"))
-    for f in (lib.h, lib.rcp):
+    for f in (lib.h, lib.rcp, lib.flat):
         f.restype, f.argtypes = ctypes.c_double, [ctypes.c_double]
     lib.grid.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_double, ctypes.c_void_p]
     lib.node.argtypes = [ctypes.c_void_p, ctypes.c_double, ctypes.c_void_p]
@@ -64,7 +65,11 @@ def test_regulator(fx):
         assert abs(fx.h(x) / ref - 1) < 1.5 * 2.0 ** -53, x
     for x in (0.0, -0.0, -1e-18, -1e-300, 5e-324):   # rounding of |q + p|^2 around 0
         assert fx.h(x) == 1.0
-    assert fx.h(float("inf")) == float("inf") and np.isnan(fx.h(float("nan")))
+        assert fx.flat(x) == 1.0
+    for f in (fx.h, fx.flat):
+        assert f(float("inf")) == float("inf") and np.isnan(f(float("nan"))) and np.isnan(f(-float("nan")))
+    for x in (0.3, np.nextafter(1, 0), 1.0, np.nextafter(1, 2), 700.0):
+        assert fx.flat(x) == max(1.0, x)
 
 
 def test_reciprocal(fx):
