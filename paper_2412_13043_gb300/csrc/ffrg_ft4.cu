@@ -176,10 +176,9 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kThreads64 : kThreads)
     kc = load_kconst<double>(a);
     kc.us = fx;
   }
+  ItemQueue items(a.work_ctr);
   for (;;) {
-    int d = 0;
-    if (lane == 0) d = (int)atomicAdd(a.work_ctr, 1u);
-    d = __shfl_sync(0xffffffffu, d, 0);
+    const int d = items.pop(a.n_ext * nc);
     if (d >= a.n_ext * nc) break;
     const int e = d / nc, c0 = d - e * nc, ip = e / nm, m = e - ip * nm;
     const double p = ext_momentum(a, ip);

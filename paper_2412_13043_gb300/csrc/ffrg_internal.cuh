@@ -289,6 +289,38 @@ __device__ __forceinline__ double prop_den(int reg, double Z, double om2, double
   return Z * (om2 + s2 + k2 * reg_r(reg, s2 * inv_k2)) + m2;
 }
 
+// (float)v, rounded to nearest even on the integer pipe: the conversion
+// instruction runs at the FP64 rate (16 clocks a warp).  Results outside the
+// normal floats take the instruction.
+__device__ __forceinline__ float f32_of(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned e = (unsigned)(b >> 52) & 0x7FFu;
+  if (e < 897u || e > 1149u) return (float)v;
+  const unsigned long long m = b + 0x0FFFFFFFull + ((b >> 29) & 1ull);
+  return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | (((unsigned)(m >> 29) - (896u << 23)) & 0x7FFFFFFFu));
+}
+
+// Work items of a persistent kernel: a warp's first by its position in the
+// grid, the next ones from the counter (reset before the launch) when it is
+// free, which a grid with a warp per item never asks.
+struct ItemQueue {
+  unsigned *ctr;
+  int first, warps;
+  __device__ __forceinline__ explicit ItemQueue(unsigned *c)
+      : ctr(c), first((int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x)), warps((int)(gridDim.x * (blockDim.x >> 5))) {}
+  // the warp's next item, or a value >= n_items (uniform over the warp)
+  __device__ __forceinline__ int pop(int n_items) {
+    int d = first;
+    if (d >= 0) {
+      first = -1;
+      return d;
+    }
+    if (warps >= n_items) return n_items;
+    if ((threadIdx.x & 31) == 0) d = (int)atomicAdd(ctr, 1u);
+    return warps + __shfl_sync(0xffffffffu, d, 0);
+  }
+};
+
 // Device-wide status word (sticky bits).
 __device__ __forceinline__ void raise_status(unsigned *status, unsigned bit) {
   if (status) atomicOr(status, bit);

@@ -193,10 +193,9 @@ __global__ void __launch_bounds__(kThreads) ref64_kernel(RhsArgs a) {
   // d=4: the three-point block, with the second-angle loop, first
   const int rot = MODEL == FFRG_MODEL_D3 ? 0 : a.n_ext_p + 1;
   const int rows = ref_rows<MODEL>(a), irows = ref_item_rows<MODEL>(a), nseg = ROWS ? (irows + 31) / 32 : 1;
+  ItemQueue items(a.work_ctr);
   for (;;) {
-    int d = 0;
-    if (lane == 0) d = (int)atomicAdd(a.work_ctr, 1u);
-    d = __shfl_sync(0xffffffffu, d, 0);
+    const int d = items.pop(a.n_items * nseg);
     if (d >= a.n_items * nseg) break;
     const int s = d % nseg, item = d / nseg, c = item % a.n_chunks, e = (item / a.n_chunks + rot) % a.n_ext;
     const int R0 = c * irows, R1 = min(R0 + irows, rows);

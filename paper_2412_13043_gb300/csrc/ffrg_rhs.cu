@@ -442,10 +442,10 @@ __device__ __forceinline__ void stage_angles(const RhsArgs &a, SmemLayout<T> &S)
   }
 }
 
-template <typename T>
+template <typename T, bool S1>
 __device__ bool main_prologue(const RhsArgs &a, SmemLayout<T> &S, uint64_t *bar) {
   bool ok = true;
-  stage_angles<T>(a, S);   // rules of the plan: not written by the precompute kernel
+  stage_angles<T, S1>(a, S);   // rules of the plan: not written by the precompute kernel
   if constexpr (sizeof(T) == 8) {
     // the function tables (logarithms in the grid's units), and line-form
     // tables that the precompute kernel does not write
@@ -1272,10 +1272,18 @@ __device__ __forceinline__ void item_loop(const RhsArgs &a, const RhsArgs *sa, c
                                           const KConst<T> &kc) {
   const int lane = threadIdx.x & 31;
   const int rot = is_d4(MODEL) || MODEL == kModelD4FullCell ? a.n_ext_p + 1 : 0;
+  // every item from the counter in the mixed d=4 vertex kernel: the queue's two
+  // registers are spilled there (213.5 -> 218.7 us)
+  constexpr bool kCounter = MODEL == FFRG_MODEL_D4_VERTEX && sizeof(T) == 4;
+  ItemQueue items(a.work_ctr);
   for (;;) {
     int d = 0;
-    if (lane == 0) d = (int)atomicAdd(a.work_ctr, 1u);
-    d = __shfl_sync(0xffffffffu, d, 0);
+    if constexpr (kCounter) {
+      if (lane == 0) d = (int)atomicAdd(a.work_ctr, 1u);
+      d = __shfl_sync(0xffffffffu, d, 0);
+    } else {
+      d = items.pop(a.n_items);
+    }
     if (d >= a.n_items) break;
     const int c = d % a.n_chunks, e = (d / a.n_chunks + rot) % a.n_ext;
     const double acc = witem<MODEL, T, POLE>(a, sa, S, kc, e, c, lane).item_sum();
@@ -1312,17 +1320,17 @@ __global__ void __launch_bounds__(kMainThreads<T>, MinBlocks<T>::value) rhs_main
   __shared__ RhsArgs sa;  // for the out-of-line near-pole path
   if constexpr (sizeof(T) == 4) copy_args(&sa, a);
   SmemLayout<T> S(smem, a);
-  if (!main_prologue<T>(a, S, &bar)) return;
+  constexpr bool kD4 = MODEL == FFRG_MODEL_D4_VERTEX || MODEL == FFRG_MODEL_D4_FULL;
+  if (!main_prologue<T, kD4>(a, S, &bar)) return;
   KConst<T> kc = load_kconst<T>(a);
   if constexpr (sizeof(T) == 8) kc.us = S.fx;
   const bool pole = pole_possible(a, S, kc);
   if constexpr (MODEL == FFRG_MODEL_FINITE_T) {
     // K rows: items of consecutive rows (stack row, |p|, radial node) from the counter
     const int lane = threadIdx.x & 31;
+    ItemQueue items(a.work_ctr);
     for (;;) {
-      int d = 0;
-      if (lane == 0) d = (int)atomicAdd(a.work_ctr, 1u);
-      d = __shfl_sync(0xffffffffu, d, 0);
+      const int d = items.pop(a.n_items);
       if (d >= a.n_items) break;
       if (sizeof(T) == 4 && pole) ftk_rows<T, true>(a, &sa, S, kc, d, lane);
       else ftk_rows<T, false>(a, &sa, S, kc, d, lane);
@@ -1345,7 +1353,7 @@ __global__ void __launch_bounds__(kThreadsWide, 1) rhs_main_cell(const __grid_co
   __shared__ RhsArgs sa;  // for the out-of-line near-pole path
   copy_args(&sa, a);
   SmemLayout<float> S(smem, a);
-  if (!main_prologue<float>(a, S, &bar)) return;
+  if (!main_prologue<float, true>(a, S, &bar)) return;
   const KConst<float> kc = load_kconst<float>(a);
   const bool pole = pole_possible(a, S, kc);
   if (pole) item_loop<kModelD4FullCell, float, true>(a, &sa, S, kc);
@@ -1439,7 +1447,7 @@ __global__ void __launch_bounds__(kThreadsWide, 1) ft_single_kernel(const __grid
   const int z_count = a.n_stack * a.n_pts;
   int neg = 0;
   for (int i = threadIdx.x; i <= z_count; i += blockDim.x) {
-    const float2 v = i < z_count ? make_float2((float)(kh * a.tab[i]), (float)a.tab[z_count + i])
+    const float2 v = i < z_count ? make_float2(f32_of(kh * a.tab[i]), f32_of(a.tab[z_count + i]))
                                  : make_float2(0.f, 0.f);
     S.tab[i] = v;
     neg |= v.x < 0.0f;
@@ -1456,15 +1464,20 @@ __global__ void __launch_bounds__(kThreadsWide, 1) ft_single_kernel(const __grid
   const bool radial_warp = (threadIdx.x >> 5) == 1 && gridDim.x - 1 - blockIdx.x < (unsigned)radial_units(a);
   if (radial_warp)
     for (int u = gridDim.x - 1 - blockIdx.x; u < radial_units(a); u += gridDim.x) radial_unit(a, u, lane);
-  else
+  else {
+    // first items by position among the warps that take K rows: warp 1 of
+    // every CTA, absent in the last ones, is numbered behind the others
+    const int warp = threadIdx.x >> 5, grid = (int)gridDim.x;
+    ItemQueue items(cnt);
+    items.first = (warp == 1 ? (kThreadsWide / 32 - 1) * grid : (warp - (warp > 1)) * grid) + (int)blockIdx.x;
+    items.warps = kThreadsWide / 32 * grid - min(radial_units(a), grid);
     for (;;) {
-      int d = 0;
-      if (lane == 0) d = (int)atomicAdd(cnt, 1u);
-      d = __shfl_sync(0xffffffffu, d, 0);
+      const int d = items.pop(a.n_items);
       if (d >= a.n_items) break;
       if (pole) ftk_rows<float, true>(a, &sa, S, kc, d, lane, q_loc, p_loc);
       else ftk_rows<float, false>(a, &sa, S, kc, d, lane, q_loc, p_loc);
     }
+  }
   grid_arrive(cnt + 1);
   ok = grid_wait(cnt + 1, base + gridDim.x, a.status, &s_ok) && ok;
   // the outputs by 256-thread groups, four per CTA at once (named barriers
