@@ -12,9 +12,10 @@
 //     largest magnitude is below 1, then cut into kSlices fixed-point slices
 //     of kBits bits, x = sum_i x_i 2^(-kBits (i+1)), x_0 integer in
 //     [-32, 32], x_i in [-16, 16]; the integers are exact in BF16;
-//   - a slice pair (i, j) summed over at most 2^14 K-elements is an integer
-//     below 2^24 in magnitude, exact in the FP32 tensor-memory accumulator
-//     (ffrg_umma.cuh); every pair with i + j < kSlices is one pass;
+//   - up to four slice pairs (i, j) of one level i + j summed over at most 2^13
+//     K-elements are an integer below 2^24 in magnitude, exact in the FP32
+//     tensor-memory accumulator (ffrg_umma.cuh): one pass; the pairs with i + j
+//     < kSlices are kept;
 //   - per output, the passes of one level i + j are added as integers
 //     (exact), the levels in FP64 from the smallest, and the result scaled by
 //     norm 2^(e_row + e_state - 2 kBits).
@@ -39,9 +40,6 @@ struct StatesScratch {
   int *e_row, *e_col;
   int4 *pass_tab;
 };
-
-// BF16 bits of a small integer held in a float (exact: at most 8 significant bits)
-__device__ __forceinline__ uint16_t bf16_int(float v) { return (uint16_t)(__float_as_uint(v) >> 16); }
 
 // |v| as an ordered integer (IEEE bit pattern without the sign)
 __device__ __forceinline__ unsigned long long mag_bits(double v) {
@@ -85,30 +83,35 @@ __device__ __forceinline__ long long fixed50(double v, int e) {
 
 // slices of the 8 values v[0..7] (scale 2^-e) at K-elements 8g .. 8g + 7 of
 // row `row` of a panel with tiles `th` rows high: x = sum_i a_i 2^(-5(i+1)),
-// a_i = round of the remainder at weight 2^(45 - 5i) (shifts of X); one
+// a_0 in [-32, 32], the other digits in [-16, 15]; one
 // 16-byte core-matrix row per slice, slice arrays `slice_elems` apart
 __device__ __forceinline__ void write_slices8(uint16_t *dst, size_t slice_elems, int k_tiles, int row, int th, int g,
                                               const double (&v)[8], int e) {
   const int col = 8 * g;
   const size_t off = ((size_t)(row / th) * k_tiles + col / umma::kBK) * (size_t)(th * umma::kBK) +
                      umma::tile_offset(row % th, col % umma::kBK, th);
+  // Digits by one biased shift: with 16 added at the weight of every slice
+  // but the first, the 5-bit fields of X are the digits plus 16.  The integer
+  // k - 16 in FP32 is (2^23 + k) - (2^23 + 16), its upper half the BF16 bits.
+  constexpr long long kBias = 16ll * (((1ll << (kBits * (kSlices - 1))) - 1) / 31);
   long long X[8];
 #pragma unroll
-  for (int h = 0; h < 8; ++h) X[h] = fixed50(v[h], e);
+  for (int h = 0; h < 8; ++h) X[h] = fixed50(v[h], e) + kBias;
 #pragma unroll
   for (int i = 0; i < kSlices; ++i) {
     const int w = kBits * (kSlices - 1 - i);
     uint32_t pk[4];
 #pragma unroll
-    for (int h = 0; h < 8; ++h) {
-      long long a = X[h];
-      if (w > 0) {
-        a = (X[h] + (1ll << (w - 1))) >> w;
-        X[h] -= a << w;
+    for (int h = 0; h < 8; h += 2) {
+      float lo, hi;
+      if (i == 0) {   // the first slice, in [-32, 32]
+        lo = __uint_as_float(0x4B000000u + (uint32_t)((int)(X[h] >> w) + 64)) - 8388672.0f;
+        hi = __uint_as_float(0x4B000000u + (uint32_t)((int)(X[h + 1] >> w) + 64)) - 8388672.0f;
+      } else {
+        lo = __uint_as_float(0x4B000000u | ((uint32_t)(X[h] >> w) & 31u)) - 8388624.0f;
+        hi = __uint_as_float(0x4B000000u | ((uint32_t)(X[h + 1] >> w) & 31u)) - 8388624.0f;
       }
-      const uint32_t b = (uint32_t)bf16_int((float)(int)a);
-      if (h & 1) pk[h >> 1] |= b << 16;
-      else pk[h >> 1] = b;
+      pk[h >> 1] = __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
     }
     *reinterpret_cast<uint4 *>(dst + (size_t)i * slice_elems + off) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
   }
@@ -124,6 +127,7 @@ struct SplitArgs {
   uint16_t *A, *B;
   int *e_row, *e_col;
   size_t a_slice, b_slice;  // elements per slice array
+  int keep;                 // split_B: shared memory holds a state's values
 };
 
 // one block per row of A (external point e = (p, m); padded rows are zero)
@@ -167,13 +171,18 @@ __global__ void __launch_bounds__(256) split_B_kernel(SplitArgs g) {
   const double q3 = g.qscale * g.qscale * g.qscale;
   for (int r = threadIdx.x; r < g.nr; r += blockDim.x) wq[r] = q3 * g.rad_w[r] * g.rad_x[r] * g.rad_x[r];
   __syncthreads();
+  // the weighted values, kept in shared memory between the two passes when
+  // they fit (one FP64 product and one index modulo per value, not two)
+  double *kept = g.keep ? wq + ((g.nr + 1) & ~1) : nullptr;
   auto val = [&](int col) -> double {
     if (!live || col >= g.kdim) return 0.0;
     return wq[col % g.nr] * g.F[(size_t)s * g.kdim + col];
   };
   unsigned long long mx = 0;
   for (int c = threadIdx.x; c < kpad; c += blockDim.x) {
-    const unsigned long long b = mag_bits(val(c));
+    const double v = val(c);
+    if (kept) kept[c] = v;
+    const unsigned long long b = mag_bits(v);
     mx = b > mx ? b : mx;
   }
   const int e = scale_exp_bits(block_max_bits(mx, red));
@@ -181,7 +190,7 @@ __global__ void __launch_bounds__(256) split_B_kernel(SplitArgs g) {
   for (int q = threadIdx.x; q < kpad / 8; q += blockDim.x) {
     double v[8];
 #pragma unroll
-    for (int h = 0; h < 8; ++h) v[h] = val(8 * q + h);
+    for (int h = 0; h < 8; ++h) v[h] = kept ? kept[8 * q + h] : val(8 * q + h);
     write_slices8(g.B, g.b_slice, g.k_tiles, s, umma::kBN, q, v, e);
   }
 }
@@ -195,35 +204,37 @@ struct CombineArgs {
   int n_rows, n_cols, rows_pad, cols_pad, n_chunks;
 };
 
-// pass index of slice pair (i, j) in level order: level l = i + j holds the
-// pairs (0, l), (1, l - 1), ..., (l, 0)
-__host__ __device__ inline int pair_index(int i, int j) {
-  const int l = i + j;
-  return l * (l + 1) / 2 + i;
+// passes of a level (its l + 1 pairs in groups of at most kGroup) and of the
+// levels before it
+__host__ __device__ constexpr int level_groups(int l) { return (l + umma::kGroup) / umma::kGroup; }
+__host__ __device__ constexpr int groups_before(int l) {
+  int n = 0;
+  for (int k = 0; k < l; ++k) n += level_groups(k);
+  return n;
 }
+constexpr int kGroups = groups_before(kSlices);
 
 // thread per output (state fastest): the passes of a level are exact
-// integers (|sum| < 2^24 each, at most 10 x 12 of them per level: the sum
-// fits a 32-bit integer for n_chunks <= 12); levels 0..6 are combined exactly
-// in a 64-bit integer at weight 2^(30 - 5l), levels 7..9 and the scales in FP64
+// integers (level sums below 3072 x 196608 < 2^31 in all); levels 0..6 are
+// combined exactly in a 64-bit integer at weight 2^(30 - 5l), levels 7..9 and
+// the scales in FP64
 __global__ void __launch_bounds__(256) combine_kernel(CombineArgs g) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)g.n_rows * g.n_cols) return;
   const int e = (int)(t / g.n_cols), s = (int)(t % g.n_cols);
   const size_t plane = (size_t)g.rows_pad * g.cols_pad, at = (size_t)e * g.cols_pad + s;
-  // the passes in pair_index order (level l = 0, 1, ...): all loads independent
-  constexpr int kPairs = kSlices * (kSlices + 1) / 2;
+  // the passes in level order: all loads independent
   int lsum[kSlices];
 #pragma unroll
   for (int l = 0; l < kSlices; ++l) lsum[l] = 0;
   for (int c = 0; c < g.n_chunks; ++c) {
-    float v[kPairs];
+    float v[kGroups];
 #pragma unroll
-    for (int p = 0; p < kPairs; ++p) v[p] = g.part[(size_t)(p * g.n_chunks + c) * plane + at];
+    for (int p = 0; p < kGroups; ++p) v[p] = g.part[(size_t)(p * g.n_chunks + c) * plane + at];
 #pragma unroll
     for (int l = 0, p = 0; l < kSlices; ++l)
 #pragma unroll
-      for (int i = 0; i <= l; ++i, ++p) lsum[l] += __float2int_rn(v[p]);
+      for (int i = 0; i < level_groups(l); ++i, ++p) lsum[l] += __float2int_rn(v[p]);
   }
   long long hi = 0;
   double tail = 0.0;
@@ -263,12 +274,11 @@ extern "C" int ffrg_ft_states(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_
   const int k_tiles = (kdim + umma::kBK - 1) / umma::kBK;
   const int kt_chunk = std::min(k_tiles, umma::kMaxExactK / umma::kBK);
   const int n_chunks = (k_tiles + kt_chunk - 1) / kt_chunk;
-  if (n_chunks > 12) {   // level sums must fit 32-bit integers: nfreq n_rad <= 12 x 16384
+  if (k_tiles > 196608 / umma::kBK) {   // level sums must fit 32-bit integers
     ctx->last_error = "ffrg_ft_states: more than 196608 (loop frequency, radial node) terms";
     return FFRG_EINVAL;
   }
-  const int n_pairs = kSlices * (kSlices + 1) / 2;
-  const int passes = n_pairs * n_chunks;
+  const int passes = kGroups * n_chunks;
   const int rows_pad = m_tiles * umma::kBM, cols_pad = n_tiles * umma::kBN;
   const size_t a_slice = (size_t)rows_pad * k_tiles * umma::kBK, b_slice = (size_t)cols_pad * k_tiles * umma::kBK;
 
@@ -284,9 +294,9 @@ extern "C" int ffrg_ft_states(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_
   if (st) return st;
 
   // scratch, kept by the context and grown on demand (256-byte segments):
-  // pass table (room for 12 K ranges) | A slices | B slices | pass sums | scales
+  // pass table (room for all K ranges) | A slices | B slices | pass sums | scales
   auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-  const size_t o_A = al((size_t)n_pairs * 12 * sizeof(int4));
+  const size_t o_A = al((size_t)kGroups * (196608 / umma::kMaxExactK) * sizeof(int4));
   const size_t o_B = o_A + al(kSlices * a_slice * 2), o_part = o_B + al(kSlices * b_slice * 2);
   const size_t o_er = o_part + al((size_t)passes * rows_pad * cols_pad * 4);
   const size_t o_ec = o_er + al((size_t)rows_pad * 4);
@@ -304,15 +314,21 @@ extern "C" int ffrg_ft_states(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_
   StatesScratch sc{(uint16_t *)(base + o_A), (uint16_t *)(base + o_B), (float *)(base + o_part),
                    (int *)(base + o_er), (int *)(base + o_ec), (int4 *)base};
   if (ctx->states_chunks != n_chunks) {
-    // the pass table, one slot per CTA z: slice pair (i, j), its output pass
-    // (pair_index order, K ranges innermost) and K range.  Slots run in order
-    // of i, so CTAs that run together read the same A slice (uploaded when the
-    // number of K ranges changes)
-    std::vector<int4> ij((size_t)passes);
-    size_t z = 0;
-    for (int i = 0; i < kSlices; ++i)
-      for (int j = 0; i + j < kSlices; ++j)
-        for (int c = 0; c < n_chunks; ++c) ij[z++] = make_int4(i, j, pair_index(i, j) * n_chunks + c, c);
+    // the pass table, one slot per CTA z: first slice pair (i, j) of a group of
+    // a level, output pass (level order, K ranges innermost), K range and
+    // number of pairs; the largest groups first, so that the short ones fill
+    // the last wave (uploaded when the number of K ranges changes)
+    std::vector<int4> ij;
+    for (int n = umma::kGroup; n > 0; --n)
+      for (int l = 0; l < kSlices; ++l)
+        for (int q = 0, i = 0; q < level_groups(l); ++q) {
+          // the level's pairs shared out evenly over its groups
+          const int size = (l + 1) / level_groups(l) + (q < (l + 1) % level_groups(l) ? 1 : 0);
+          if (size == n)
+            for (int c = 0; c < n_chunks; ++c)
+              ij.push_back(make_int4(i, l - i, (groups_before(l) + q) * n_chunks + c, c | size << 16));
+          i += size;
+        }
     st = set_cuda_error(ctx, cudaMemcpyAsync(sc.pass_tab, ij.data(), ij.size() * sizeof(int4),
                                              cudaMemcpyHostToDevice, s), "ffrg_ft_states pass table");
     // from pageable memory: the copy must have read ij before it goes away
@@ -345,7 +361,12 @@ extern "C" int ffrg_ft_states(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_
   sg.a_slice = a_slice;
   sg.b_slice = b_slice;
   split_A_kernel<<<rows_pad, 256, 0, s>>>(sg);
-  split_B_kernel<<<cols_pad, 256, (size_t)pl->nr * sizeof(double), s>>>(sg);
+  size_t b_smem = ((size_t)pl->nr + 1 + (size_t)k_tiles * umma::kBK) * sizeof(double);
+  sg.keep = b_smem <= 56 * 1024;   // four blocks an SM
+  if (!sg.keep) b_smem = (size_t)pl->nr * sizeof(double);
+  st = ensure_smem_limit(ctx, (const void *)split_B_kernel, b_smem);
+  if (st) return st;
+  split_B_kernel<<<cols_pad, 256, b_smem, s>>>(sg);
 
   st = ensure_smem_limit(ctx, (const void *)umma::slice_pair_gemm, umma::kSmemBytes);
   if (st) return st;

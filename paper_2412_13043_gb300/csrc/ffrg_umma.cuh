@@ -1,12 +1,18 @@
 // Tensor-core (tcgen05 / UMMA) pieces of the FP64-faithful sliced contraction
 // used for the finite-T sums over many loop-side states (see ffrg_ozaki.cu).
 //
-// Operands are BF16 slices holding small integers (at most 32 in magnitude),
-// so every product is an integer below 2^10 in magnitude and any sum of up to
-// 2^14 of them is an integer below 2^24: the FP32 accumulator in tensor memory
-// holds it exactly.  One CTA computes one pass: a 128 x 256 output tile of one
-// slice pair over one K range, D = A_i^T-tile x B_j-tile, and writes the exact
-// FP32 sums to global memory.
+// Operands are BF16 slices holding small integers (slice 0 at most 32 in
+// magnitude, the others at most 16), so sums of their products are integers,
+// exact in the FP32 accumulator in tensor memory below 2^24.  One CTA computes
+// one pass: a 128 x 256 output tile of up to kGroup slice pairs (i, j), (i+1,
+// j-1), ... of one level i + j over one K range, D = sum A_i^T-tile x
+// B_j-tile, and writes the exact FP32 sums to global memory.  Per K-element a
+// group adds at most 512 + 256 + 256 + 512, so a range may have 2^24 / 1536
+// elements (kMaxExactK is below that).  Several pairs in one accumulation make
+// a third of the sums to write and to read back (576 x 1024 outputs of 3168
+// terms: 55 passes of one pair 185 us and 54 us to combine them, 18 passes
+// 179 and 39).  What bounds a pass is its operand traffic from L2, 24 KB per
+// 32 K-elements, 14 TB/s over the GPU.
 //
 // Shared-memory operand layout (no swizzle, K-major, the canonical
 // "interleaved" form of the UMMA shared-memory descriptor): a tile of R rows x
@@ -41,7 +47,9 @@ constexpr int kStageBytes = kTileA + kTileB;
 constexpr int kSmemBytes = kStages * kStageBytes;   // 96 KB: two CTAs per SM
 constexpr int kTmemCols = 256;
 constexpr int kThreadsGemm = 128;
-constexpr int kMaxExactK = 16384;  // K-elements whose slice products sum exactly in FP32
+constexpr int kGroup = 4;          // slice pairs of a level in one pass
+constexpr int kMaxExactK = 8192;   // K-elements whose slice products sum exactly in FP32, kGroup pairs at once
+static_assert(kMaxExactK * (2 * 512 + (kGroup - 2) * 256) < (1 << 24), "exact in FP32");
 constexpr unsigned kStatusTimeoutBit = 2u;
 constexpr long long kWaitLimit = 4000000000LL;   // clock cycles (about 2 s)
 
@@ -54,7 +62,7 @@ struct GemmArgs {
   const uint16_t *A;   // BF16 bits, slices [nsl][m_tiles][k_tiles][128 x kBK tile]
   const uint16_t *B;   // BF16 bits, slices [nsl][n_tiles][k_tiles][256 x kBK tile]
   float *part;         // [passes][m_tiles * 128][n_tiles * 256], exact sums per pass
-  const int4 *pass_tab; // per CTA z: slice pair (i, j), output pass, K range
+  const int4 *pass_tab; // per CTA z: first slice pair (i, j), output pass, K range + pairs << 16
   int m_tiles, n_tiles, k_tiles;
   int kt_per_chunk, n_chunks;  // K-tiles per pass and K ranges per slice pair
   unsigned *status;
@@ -147,8 +155,8 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 }
 
 // One pass per CTA: blockIdx.x = output column tile, blockIdx.y = output row
-// tile, blockIdx.z = slot of the pass table (slice pair, its output pass and
-// K range; slots that run together share an A slice).
+// tile, blockIdx.z = slot of the pass table (group of slice pairs, its output
+// pass and K range; the largest groups first).
 __global__ void __launch_bounds__(kThreadsGemm, 1) slice_pair_gemm(GemmArgs g) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[kStages], empty[kStages], done;
@@ -158,9 +166,9 @@ __global__ void __launch_bounds__(kThreadsGemm, 1) slice_pair_gemm(GemmArgs g) {
   const int tn = blockIdx.x, tm = blockIdx.y;
   const int4 pt = g.pass_tab[blockIdx.z];
   const int2 ij = make_int2(pt.x, pt.y);
-  const int pass = pt.z, chunk = pt.w;
+  const int pass = pt.z, chunk = pt.w & 0xFFFF;
   const int kt0 = chunk * g.kt_per_chunk;
-  const int nkt = min(g.kt_per_chunk, g.k_tiles - kt0);
+  const int per_pair = min(g.kt_per_chunk, g.k_tiles - kt0), nkt = per_pair * (pt.w >> 16);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -188,7 +196,9 @@ __global__ void __launch_bounds__(kThreadsGemm, 1) slice_pair_gemm(GemmArgs g) {
   const uint16_t *Bb = g.B + ((size_t)(ij.y * g.n_tiles + tn) * g.k_tiles) * (kBN * kBK);
 
   if (warp == 0 && lane == 0) {
-    // producer: K-tile t goes to stage t % 2; the stage's previous MMAs must have completed
+    // producer: K-tile t goes to stage t % kStages; the stage's previous MMAs must have completed
+    const size_t a_step = (size_t)g.m_tiles * g.k_tiles * (kBM * kBK), b_step = (size_t)g.n_tiles * g.k_tiles * (kBN * kBK);
+    int pr = 0, kt = kt0;   // pair of the group, its K-tile
     for (int t = 0; t < nkt; ++t) {
       const int s = t % kStages;
       const uint32_t ph = (uint32_t)(t / kStages) & 1u;
@@ -199,9 +209,13 @@ __global__ void __launch_bounds__(kThreadsGemm, 1) slice_pair_gemm(GemmArgs g) {
       if (*(volatile int *)&abort_flag) break;
       unsigned char *st = smem + s * kStageBytes;
       bar_expect_tx(&full[s], kStageBytes);
-      bulk_load(st, Ab + (size_t)(kt0 + t) * (kBM * kBK), kTileA, &full[s]);
-      bulk_load(st + kTileA, Bb + (size_t)(kt0 + t) * (kBN * kBK), kTileB, &full[s]);
+      bulk_load(st, Ab + pr * a_step + (size_t)kt * (kBM * kBK), kTileA, &full[s]);
+      bulk_load(st + kTileA, Bb - pr * b_step + (size_t)kt * (kBN * kBK), kTileB, &full[s]);
       issued = t + 1;
+      if (++kt == kt0 + per_pair) {
+        kt = kt0;
+        ++pr;
+      }
     }
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
