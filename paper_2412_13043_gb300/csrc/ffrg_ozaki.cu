@@ -127,7 +127,6 @@ struct SplitArgs {
   uint16_t *A, *B;
   int *e_row, *e_col;
   size_t a_slice, b_slice;  // elements per slice array
-  int keep;                 // split_B: shared memory holds a state's values
 };
 
 // one block per row of A (external point e = (p, m); padded rows are zero)
@@ -160,37 +159,51 @@ __global__ void __launch_bounds__(256) split_A_kernel(SplitArgs g) {
   }
 }
 
-// one block per state (padded states are zero); the state carries the radial
-// weight and measure w_r q_r^2 (from the unit rule, staged per block)
-__global__ void __launch_bounds__(256) split_B_kernel(SplitArgs g) {
-  __shared__ unsigned long long red[8];
+// one block per 8 states (padded states are zero), four warps a state for its
+// largest value, then eight lanes side by side for the eight states' slices of
+// the same K-elements: 128 contiguous bytes of a core matrix (a block per
+// state wrote 16 bytes here and there: 64 us for 1024 states of 3168 terms,
+// 37 so).  Few states leave SMs idle: there the K-elements are shared out over
+// gridDim.y blocks, each of which finds the largest values itself.  The state carries the radial weight and measure w_r q_r^2 (from
+// the unit rule, staged per block).
+constexpr int kStatesPerBlock = 8;
+__global__ void __launch_bounds__(1024) split_B_kernel(SplitArgs g) {
+  __shared__ unsigned long long red[32];
   extern __shared__ double wq[];   // [n_rad]: (k qmax)^3 w_r x_r^2
-  const int s = blockIdx.x;
-  const int kpad = g.k_tiles * umma::kBK;
-  const bool live = s < g.n_cols;
+  const int kpad = g.k_tiles * umma::kBK, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double q3 = g.qscale * g.qscale * g.qscale;
   for (int r = threadIdx.x; r < g.nr; r += blockDim.x) wq[r] = q3 * g.rad_w[r] * g.rad_x[r] * g.rad_x[r];
   __syncthreads();
-  // the weighted values, kept in shared memory between the two passes when
-  // they fit (one FP64 product and one index modulo per value, not two)
-  double *kept = g.keep ? wq + ((g.nr + 1) & ~1) : nullptr;
-  auto val = [&](int col) -> double {
-    if (!live || col >= g.kdim) return 0.0;
-    return wq[col % g.nr] * g.F[(size_t)s * g.kdim + col];
-  };
-  unsigned long long mx = 0;
-  for (int c = threadIdx.x; c < kpad; c += blockDim.x) {
-    const double v = val(c);
-    if (kept) kept[c] = v;
-    const unsigned long long b = mag_bits(v);
-    mx = b > mx ? b : mx;
-  }
-  const int e = scale_exp_bits(block_max_bits(mx, red));
-  if (threadIdx.x == 0) g.e_col[s] = e;
-  for (int q = threadIdx.x; q < kpad / 8; q += blockDim.x) {
-    double v[8];
+  {
+    const int s = blockIdx.x * kStatesPerBlock + (warp >> 2);
+    unsigned long long mx = 0;
+    if (s < g.n_cols)
+      for (int c = (warp & 3) * 32 + lane; c < g.kdim; c += 128) {
+        const unsigned long long b = mag_bits(wq[c % g.nr] * g.F[(size_t)s * g.kdim + c]);
+        mx = b > mx ? b : mx;
+      }
 #pragma unroll
-    for (int h = 0; h < 8; ++h) v[h] = kept ? kept[8 * q + h] : val(8 * q + h);
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long w = __shfl_xor_sync(0xffffffffu, mx, o);
+      mx = w > mx ? w : mx;
+    }
+    if (lane == 0) red[warp] = mx;
+  }
+  __syncthreads();
+  const int row = lane & 7, s = blockIdx.x * kStatesPerBlock + row;
+  unsigned long long mx = 0;
+  for (int w = 0; w < 4; ++w) mx = red[4 * row + w] > mx ? red[4 * row + w] : mx;
+  const int e = scale_exp_bits(mx);
+  if (blockIdx.y == 0 && threadIdx.x < kStatesPerBlock) g.e_col[s] = e;
+  const double *F = g.F + (size_t)s * g.kdim;
+  for (int q = (blockIdx.y * 32 + warp) * 4 + (lane >> 3); q < kpad / 8; q += gridDim.y * 128) {
+    double v[8];
+    int r = 8 * q % g.nr;
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+      v[h] = s < g.n_cols && 8 * q + h < g.kdim ? wq[r] * F[8 * q + h] : 0.0;
+      if (++r == g.nr) r = 0;
+    }
     write_slices8(g.B, g.b_slice, g.k_tiles, s, umma::kBN, q, v, e);
   }
 }
@@ -215,9 +228,10 @@ __host__ __device__ constexpr int groups_before(int l) {
 constexpr int kGroups = groups_before(kSlices);
 
 // thread per output (state fastest): the passes of a level are exact
-// integers (level sums below 3072 x 196608 < 2^31 in all); levels 0..6 are
-// combined exactly in a 64-bit integer at weight 2^(30 - 5l), levels 7..9 and
-// the scales in FP64
+// integers (level sums below 3072 x 196608 < 2^31 in all); levels 0..6 and 7..9
+// are combined exactly in two 64-bit integers, which one FP64 FMA adds; the
+// scale goes into the exponent (FP64 levels and ldexp: 39 us for 576 x 1024
+// outputs, 12 so)
 __global__ void __launch_bounds__(256) combine_kernel(CombineArgs g) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)g.n_rows * g.n_cols) return;
@@ -236,15 +250,19 @@ __global__ void __launch_bounds__(256) combine_kernel(CombineArgs g) {
 #pragma unroll
       for (int i = 0; i < level_groups(l); ++i, ++p) lsum[l] += __float2int_rn(v[p]);
   }
-  long long hi = 0;
-  double tail = 0.0;
+  long long hi = 0, lo = 0;
 #pragma unroll
-  for (int l = kSlices - 1; l >= 0; --l) {
-    if (l > 6) tail += ldexp((double)lsum[l], -kBits * l);
+  for (int l = 0; l < kSlices; ++l) {
+    if (l > 6) lo += (long long)lsum[l] << (kBits * (9 - l));
     else hi += (long long)lsum[l] << (kBits * (6 - l));
   }
-  const double acc = ldexp((double)hi, -30) + tail;
-  const double v = g.norm * ldexp(acc, g.e_row[e] + g.e_col[s] - 2 * kBits);
+  // (hi 2^15 + lo) 2^-45, scaled by its exponent bits while the result is normal
+  const double acc = fma((double)hi, 32768.0, (double)lo);
+  const int x = g.e_row[e] + g.e_col[s] - 2 * kBits - 45;
+  const long long bits = __double_as_longlong(acc);
+  const int be = (int)(bits >> 52) & 0x7FF;
+  const double sc = be > 0 && be + x > 0 && be + x < 0x7FF ? __longlong_as_double(bits + ((long long)x << 52)) : ldexp(acc, x);
+  const double v = g.norm * sc;
   g.out[(size_t)s * g.n_rows + e] = v;
   if (!isfinite(v)) atomicOr(g.status, kStatusNonFinite);
 }
@@ -361,12 +379,8 @@ extern "C" int ffrg_ft_states(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_
   sg.a_slice = a_slice;
   sg.b_slice = b_slice;
   split_A_kernel<<<rows_pad, 256, 0, s>>>(sg);
-  size_t b_smem = ((size_t)pl->nr + 1 + (size_t)k_tiles * umma::kBK) * sizeof(double);
-  sg.keep = b_smem <= 56 * 1024;   // four blocks an SM
-  if (!sg.keep) b_smem = (size_t)pl->nr * sizeof(double);
-  st = ensure_smem_limit(ctx, (const void *)split_B_kernel, b_smem);
-  if (st) return st;
-  split_B_kernel<<<cols_pad, 256, b_smem, s>>>(sg);
+  const int b_blocks = cols_pad / kStatesPerBlock;
+  split_B_kernel<<<dim3(b_blocks, std::max(1, ctx->num_sms / b_blocks)), 1024, (size_t)pl->nr * sizeof(double), s>>>(sg);
 
   st = ensure_smem_limit(ctx, (const void *)umma::slice_pair_gemm, umma::kSmemBytes);
   if (st) return st;
