@@ -295,7 +295,8 @@ FFRG_API int ffrg_rhs_noalloc(const ffrg_problem *pb, const ffrg_table_desc *des
  * FP32 over at most 8192 (n, r) terms per pass, passes combined in FP64
  * (error below ~1e-14 of the sum of the terms' magnitudes).  Scratch is kept
  * by the context (slices of both operands and the exact pass sums: about
- * 20 (n_ext + n_states) nfreq n_rad + 72 n_ext n_states bytes per 8192 terms).
+ * 20 (n_ext + n_states) nfreq n_rad + 72 n_ext n_states bytes per 8192 terms;
+ * few states take up to 16 shorter ranges of terms, without a memory budget).
  * Asynchronous.  FFRG_EINVAL for models other than FFRG_MODEL_FINITE_T and
  * for more than 196608 (loop frequency, radial node) terms. */
 FFRG_API int ffrg_ft_states(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_tables *tables, double k, int n_states,

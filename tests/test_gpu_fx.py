@@ -73,3 +73,25 @@ def test_feedback_flow_does_not_depend_on_where_rows_are_computed(model, n_pts):
         ends.append(y.cpu().numpy())
         c.close()
     assert np.array_equal(ends[0], ends[1])
+
+
+@pytest.mark.parametrize("n_states", [1, 9, 257, 1025])
+def test_states_do_not_depend_on_their_number(ctx, n_states):
+    """The K ranges, and the blocks that share a state's slices, follow the number of states; the pass sums are
+    integers and the scales per state: the same bits as one by one of the whole set, and the oracle's values."""
+    import torch
+
+    import paper_2412_13043_gb300 as ffrg
+    wl = fi.make_finite_t(seed=11, N=15, T=0.01, n_pts=16, n_ext_p=5, n_ext_m=3, n_rad=133, n_ang=3)
+    tabs = ctx.tables(wl.problem, wl.tables)
+    rng = np.random.default_rng(12)
+    F = rng.uniform(-1.0, 2.0, size=(1500, oracle.ft_nfreq(wl.problem), wl.problem.n_rad))
+    dev = torch.from_numpy(F).cuda()
+    whole = ctx.ft_states(wl.problem, tabs, 0.8, dev, precision=ffrg.FP64).cpu().numpy()
+    some = ctx.ft_states(wl.problem, tabs, 0.8, dev[:n_states].contiguous(), precision=ffrg.FP64).cpu().numpy()
+    tabs.free()
+    assert np.array_equal(some, whole[:n_states])
+    at = [0, n_states // 2, n_states - 1]
+    ref = oracle.ft_states(wl.problem, wl.tables, 0.8, F[at])
+    scale = oracle.ft_states(wl.problem, wl.tables, 0.8, np.abs(F[at]))
+    assert np.max(np.abs(some[at] - ref) / scale) < 1e-12
