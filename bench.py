@@ -52,10 +52,9 @@ SFU_PER_CLK_SM = 16      # log2 / reciprocal results per clock per SM
 D4_MAIN_DRAM_BYTES = 83456
 FP32_PER_CLK_SM = 128    # FP32 FMA lanes per SM
 # FP64-pipe thread instructions per integrand term of rhs_main<2, double> (the
-# plain FP64 path), from an ncu capture of the d=4 workload with 16 external
-# momenta: pipe_fp64 86.1 % of 1.077e7 active cycles x 2 per cycle x 152 SMs
-# over 2.11e7 terms
-FP64_OPS_PER_TERM_D4 = 134
+# plain FP64 path), from an ncu capture of the d=4 workload: 5.08e7 warp
+# instructions (pipe_fp64 84.3 % of 6.34e6 active cycles) over 1.68e8 terms
+FP64_OPS_PER_TERM_D4 = 9.7
 FP64_PER_CLK_SM = 2      # FP64 (DFMA) results per clock per SM on this part
 
 

@@ -216,13 +216,14 @@ FFRG_API double ffrg_evals(const ffrg_problem *pb);
  * Eq. FlowGamman): out_dev[e] = k d_k of the target at external point e (raw
  * loop integrals; the D4 Z-block holds the propagator-diagram sum D2(p), see
  * the layout above).  out_dev: caller-owned device array of ffrg_n_ext()
- * doubles.  precision: FFRG_FP64 (all arithmetic FP64) or FFRG_MIXED (FP32
- * integrand and row sums, compensated FP32 accumulation within a work item
+ * doubles.  precision: FFRG_FP64 (all arithmetic FP64, logarithms,
+ * regulators and reciprocals as 64-bit fixed point of the same accuracy) or
+ * FFRG_MIXED (FP32 integrand and row sums, compensated FP32 accumulation within a work item
  * rounded once to FP64, FP64 across work items, FP64 per-radial-node
  * factors, FP64 propagator near the pole).  Asynchronous; non-finite outputs
  * set FFRG_ENONFINITE in the status word.  The kernels stage the tables and
  * rules in the 227 KB of shared memory of a block; FP64 tables that do not fit
- * (8 bytes per value) are read in place from global memory (L2) instead.
+ * (16 bytes per value) are read in place from global memory (L2) instead.
  * Errors: FFRG_EINVAL for a bad problem, tables of another shape, or, in mixed
  * precision, FP32 tables and rules that do not fit in shared memory (8 bytes
  * per table node: one FP32 line-form pair, or the (Z, lambda) pair of finite
@@ -252,8 +253,8 @@ FFRG_API int ffrg_rhs_host(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_tab
  * pool), and a latency-critical loop where cudaMalloc/cudaFree would stall
  * other streams.  It computes exactly what ffrg_rhs computes with the same
  * kernels, but needs no context and calls no cudaMalloc, cudaFree or other
- * allocating routine.  Its scratch is one fixed 4 MiB device array inside
- * this library.  Every GPU that loads the library holds that array until the
+ * allocating routine.  Its scratch is one fixed device array of 4 MiB + 480 KiB
+ * inside this library.  Every GPU that loads the library holds that array until the
  * process exits.
  *   pb, desc: problem and table layout (as for ffrg_rhs / ffrg_tables_upload);
  *   tables_dev: caller-owned device array of n_tables x n_stack x n_pts
@@ -325,8 +326,9 @@ FFRG_API int ffrg_rhs_adjoint(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_
  *       Flow3(p_i, psi_j), d_t lambda4_i = -Flow4(p_i)
  * Feedback requires the external grid to equal the table grid.  k(t) = Lambda
  * exp(-t).  tables: frozen tables (feedback = 0) or the grid/shape template
- * (feedback = 1).  Synchronous: returns when the flow ends; stats (host) may be
- * NULL.  Errors: FFRG_ESTEP_UNDERFLOW, FFRG_EMAXSTEPS, FFRG_ENONFINITE. */
+ * (feedback = 1).  A frozen flow keeps scratch for the stages of a step side
+ * by side (not in a context with a memory budget).  Synchronous: returns when
+ * the flow ends; stats (host) may be NULL.  Errors: FFRG_ESTEP_UNDERFLOW, FFRG_EMAXSTEPS, FFRG_ENONFINITE. */
 FFRG_API int ffrg_flow(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_tables *tables, int feedback, double Lambda,
               double *state_dev, const ffrg_step_opts *opts, int precision, ffrg_flow_stats *stats,
               void *stream);
@@ -379,7 +381,7 @@ FFRG_API int ffrg_profile_read(ffrg_ctx *ctx, double *main_ms, long long *launch
  * A scheduler thread keeps up to max_slots flows resident on the device
  * (tables, DP5(4) state and RHS scratch of each), advances all of them one
  * adaptive step per tick with batched launches (one persistent integrand
- * launch per model over every resident flow's work items), retires finished
+ * launch over the work items of all resident flows and all stages of the step), retires finished
  * flows and admits queued requests as soon as a slot and enough of
  * hbm_budget_bytes are free.  Requests: frozen-background flows
  * (feedback = 0) of FFRG_MODEL_D3 and FFRG_MODEL_FINITE_T, mixed precision

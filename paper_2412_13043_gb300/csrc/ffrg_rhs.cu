@@ -27,9 +27,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <map>
-#include <mutex>
-#include <tuple>
 
 #include "ffrg_internal.cuh"
 #include "ffrg_prop64.cuh"
