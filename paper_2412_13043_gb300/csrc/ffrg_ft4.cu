@@ -58,6 +58,8 @@ __global__ void ft4_freq_kernel(RhsArgs a, int nfreq_max) {
     if (a.fp64) ((KConstPair *)a.kconst)->d = make_kconst<double>(a);
   }
   for (int i = threadIdx.x; i < a.n_ext; i += blockDim.x) a.ext_done[i] = 0u;
+  // external momenta for the items of the main kernel, on the block's last warps
+  for (int i = blockDim.x - 1 - threadIdx.x; i < a.n_ext_p; i += blockDim.x) a.ext_pd[i] = ext_momentum(a, i);
 }
 
 // F(f, r) = w_f w_r q^2 dR(Q) G(Q)^2 L(|Q|), |Q|^2 = q0_f^2 + q_r^2 (FP64; FP32 copy)
@@ -140,7 +142,7 @@ __device__ __forceinline__ float ft4_row32(const RhsArgs &a, const float4 *zl, c
 // quadruples.  Bound: FP64 six FP64 instructions and the integer work of one
 // logarithm, regulator and reciprocal per term.  64 momenta x 9 frequencies,
 // 96 x 48 nodes, k = 1 (25 loop frequencies): FP64 10.60 ms with FP64
-// functions and one block per external point, 1.04 ms so.
+// functions and one block per external point, 0.74 ms so; mixed 0.162, 0.123 ms so.
 template <typename T>
 __global__ void __launch_bounds__(sizeof(T) == 8 ? kThreads64 : kThreads)
     ft4_main_kernel(RhsArgs a, int nfreq_max) {
@@ -167,6 +169,11 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kThreads64 : kThreads)
     }
     for (int c = threadIdx.x; c < a.na1; c += blockDim.x) cw[c] = make_float2((float)a.a1_x[c], (float)a.a1_w[c]);
   }
+  // an FP64 exponential per item held small problems back (15 x 9 external
+  // points, 5 x 96 rows, 12 angles, mixed: 38.9 us, 26.5 so): p0 here and |p| from
+  // the frequency kernel
+  const double p0f = a.stat ? kPi * a.T * exp(-k / (kPi * a.T)) : 0.0;
+  const float k2f = (float)k2, ik2f = (float)(1.0 / k2), m2f = (float)m2;
   __syncthreads();
   pdl_wait();   // the factor kernel's F(f, r) (and through it the frequency set, constants and counters)
   const int rows = (int)kb[2 * nfreq_max] * a.nr, cr = a.cr, nc = max(1, (rows + cr - 1) / cr);
@@ -181,8 +188,8 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kThreads64 : kThreads)
     const int d = items.pop(a.n_ext * nc);
     if (d >= a.n_ext * nc) break;
     const int e = d / nc, c0 = d - e * nc, ip = e / nm, m = e - ip * nm;
-    const double p = ext_momentum(a, ip);
-    const double p0 = a.stat ? kPi * a.T * exp(-k / (kPi * a.T)) : 2.0 * kPi * a.T * m;
+    const double p = a.ext_pd[ip];
+    const double p0 = a.stat ? p0f : 2.0 * kPi * a.T * m;
     double acc = 0.0;
     for (int i = c0 * cr + lane; i < min((c0 + 1) * cr, rows); i += 32) {
       const int f = i / a.nr, r = i - f * a.nr;
@@ -202,8 +209,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kThreads64 : kThreads)
         }
         acc = fma(a.radF[i], rs, acc);
       } else {
-        const float rs = ft4_row32(a, zl, cw, (float)(sh * sh), (float)q, (float)p, (float)k2, (float)(1.0 / k2),
-                                   (float)m2, us, uo);
+        const float rs = ft4_row32(a, zl, cw, (float)(sh * sh), (float)q, (float)p, k2f, ik2f, m2f, us, uo);
         acc = fma(a.radF[i], (double)rs, acc);
       }
     }
