@@ -291,13 +291,14 @@ extern "C" int ffrg_ft_states(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_
   const int n_tiles = (n_states + umma::kBN - 1) / umma::kBN;
   const int k_tiles = (kdim + umma::kBK - 1) / umma::kBK;
   // K ranges: as many as exactness needs, and where the tiles are too few for
-  // two blocks on each SM up to 16, of 256 elements or more (the sums are
+  // two blocks on each SM up to 16, of 128 elements or more (34 states, 725 terms:
+  // 512 69 us, 256 59, 128 57) (the sums are
   // integers: any cut gives the same bits).  576 external points x 3168 terms:
   // 256 states 305 us for the call with one range, 242 with four; 512 states
   // 319, with two 287; 1024 states need no more than one.  Their sums are
   // optional scratch, so one range in a context with a memory budget.
   const int fill = ctx->budget ? 1 : std::min((2 * ctx->num_sms - 1) / (m_tiles * n_tiles * kGroups) + 1, 16);
-  const int kt_chunk = std::min({k_tiles, umma::kMaxExactK / umma::kBK, std::max(8, (k_tiles + fill - 1) / fill)});
+  const int kt_chunk = std::min({k_tiles, umma::kMaxExactK / umma::kBK, std::max(4, (k_tiles + fill - 1) / fill)});
   const int n_chunks = (k_tiles + kt_chunk - 1) / kt_chunk;
   if (k_tiles > 196608 / umma::kBK) {   // level sums must fit 32-bit integers
     ctx->last_error = "ffrg_ft_states: more than 196608 (loop frequency, radial node) terms";
