@@ -266,7 +266,12 @@ inline bool fx_grid(int n_pts, double x_min, double x_max, FxGrid *g) {
   int ex;
   frexpl(us, &ex);              // us in [2^(ex-1), 2^ex)
   g->F = 54 - ex;
-  if (g->F < 16 || g->F > 60) return false;
+  // F >= 32: a coordinate below 2^63 has a node number below 2^31, so fx_node
+  // may cut it to 32 bits before it clamps.  Steeper grids (2^22 nodes an
+  // octave and more, for instance 4096 nodes on [1, 1.0003]) are refused: a
+  // momentum a few octaves away from them would not fit, and no sensible
+  // momentum grid is that narrow.
+  if (g->F < 32 || g->F > 60) return false;
   g->nm1 = n_pts - 1;
   const long double s = ldexpl(us, g->F);
   g->us = (int64_t)roundl(s);

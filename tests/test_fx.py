@@ -105,3 +105,24 @@ def test_grids_outside_fixed_point_are_refused(fx):
     g = ctypes.create_string_buffer(256)
     for n, lo, hi in ((64, 1e-20, 1.0), (64, 1e-3, 1e20), (2, 1.0, 1.0 + 1e-15)):
         assert not fx.grid(n, lo, hi, g)
+
+
+@pytest.mark.parametrize("n,lo,hi", [(128, 1.0, 1.0 + 1e-9), (4096, 1.0, 1.000001), (4096, 1.0, 1.00001),
+                                     (4096, 1.0, 1.0001), (4096, 1.0, 1.001), (4096, 1e-3, 1.001e-3), (64, 1.0, 1.000001),
+                                     (64, 1.0, 1.0001), (2, 1.0, 1.0 + 1e-7), (4096, 2.0 ** 49, 2.0 ** 49.001)])
+def test_nodes_of_narrow_grids_stay_in_the_row(fx, n, lo, hi):
+    """Momenta far outside a narrow grid: the first or the last node, whatever their distance in nodes.  (A grid may
+    be refused: the kernels then take the FP64 logarithm.)"""
+    g, w1 = ctypes.create_string_buffer(256), ctypes.c_double()
+    if not fx.grid(n, lo, hi, g):
+        return
+    for y in list(2.0 ** np.arange(-250.0, 251.0)) + [16.0, 4.0, 1e6, 1e30, 1e300, float("inf"), float("nan")]:
+        assert fx.node(g, y, ctypes.byref(w1)) == (0 if y <= lo * lo else n - 1), y   # lo itself: the first node
+    for y in (0.0, -0.0, -1.0, 5e-324):
+        assert fx.node(g, y, ctypes.byref(w1)) == 0
+
+
+def test_ordinary_grids_take_fixed_point(fx):
+    g = ctypes.create_string_buffer(256)
+    for n, lo, hi in ((4096, 1.0, 1.01), (4096, 1e-3, 10.0), (2, 0.999, 1.001), (256, 0.5, 0.6), (64, 1e-12, 1e12)):
+        assert fx.grid(n, lo, hi, g)

@@ -95,3 +95,25 @@ def test_states_do_not_depend_on_their_number(ctx, n_states):
     ref = oracle.ft_states(wl.problem, wl.tables, 0.8, F[at])
     scale = oracle.ft_states(wl.problem, wl.tables, 0.8, np.abs(F[at]))
     assert np.max(np.abs(some[at] - ref) / scale) < 1e-12
+
+
+@pytest.mark.parametrize("hi", [1.0 + 1e-9, 1.000001, 1.0001, 1.01])
+@pytest.mark.parametrize("model", ["d3", "d4"])
+def test_momenta_far_from_a_narrow_grid(ctx, model, hi):
+    """Values and gradients on grids so narrow that a momentum lies up to 2^40 nodes outside: the end nodes."""
+    import torch
+
+    import paper_2412_13043_gb300 as ffrg
+    wl = (fi.make_d3(seed=15, n_pts=64, n_ext_p=7, n_rad=16, n_ang=8) if model == "d3" else
+          fi.make_d4(seed=15, n_pts=64, n_ext_ang=2, n_rad=5, n_ang1=3, n_ang2=3))
+    wl.problem = dataclasses.replace(wl.problem, x_min=1.0, x_max=hi, p_min=0.01, p_max=3.0, n_ext_p=7)
+    wl.tables = np.random.default_rng(16).uniform(0.5, 1.5, wl.tables.shape)
+    gbar = np.random.default_rng(17).uniform(-1.0, 1.0, wl.problem.n_ext())
+    tabs = ctx.tables(wl.problem, wl.tables)
+    got = ctx.rhs(wl.problem, tabs, 0.3, precision=ffrg.FP64).cpu().numpy()
+    grad = ctx.rhs_adjoint(wl.problem, tabs, 0.3, torch.tensor(gbar, device="cuda")).cpu().numpy().ravel()
+    tabs.free()
+    ref = oracle.rhs(wl.problem, wl.tables, 0.3)
+    gref = oracle.rhs_jacobian(wl.problem, wl.tables, 0.3).T @ gbar
+    assert np.max(np.abs(got - ref) / np.abs(ref)) < 1e-12
+    assert np.max(np.abs(grad - gref)) / np.max(np.abs(gref)) < 1e-12
