@@ -226,6 +226,12 @@ static int upload_rule(ffrg_ctx *ctx, const std::vector<double> &h, double **d) 
   return set_cuda_error(ctx, e, "cudaMemcpy(rule)");
 }
 
+// A copy of less than 64 KB from pageable memory, or a memset, may return
+// before it has reached the device.  Both run on the legacy stream, which a
+// caller's non-blocking stream is not ordered after: wait here, once per plan
+// (and once per device for the function tables).
+static cudaError_t finish_legacy_stream() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 // Scratch of one RHS in flight (the rest of a plan is shared by its stages).
 static int plan_scratch(ffrg_ctx *ctx, Plan *pl, bool want_tab64) {
   const size_t nF = (size_t)pl->nr * pl->nfreq;
@@ -278,7 +284,7 @@ bool stage_plans(ffrg_ctx *ctx, Plan *pl) {
     sp->item_done = nullptr;
     for (Plan *&q : sp->stage) q = nullptr;
     pl->stage[i] = sp;
-    if (plan_scratch(ctx, sp, pl->tab64 != nullptr)) {
+    if (plan_scratch(ctx, sp, pl->tab64 != nullptr) || finish_legacy_stream() != cudaSuccess) {
       cudaGetLastError();
       for (Plan *&q : pl->stage) {
         if (q) plan_scratch_free(ctx, q);
@@ -450,6 +456,7 @@ const FxTables *fx_device_tables(int device) {
   void *p = nullptr;
   if (cudaGetSymbolAddress(&p, g_fx) != cudaSuccess) return nullptr;
   if (cudaMemcpy(p, host.data(), sizeof(FxTables), cudaMemcpyHostToDevice) != cudaSuccess) return nullptr;
+  if (finish_legacy_stream() != cudaSuccess) return nullptr;
   return ptr[device] = (const FxTables *)p;
 }
 
@@ -503,6 +510,7 @@ int get_plan(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc *td, P
   // so that it holds what it would hold without them.
   const bool too_big = pl->smem64 > kMaxDynSmemBytes && pb->model != FFRG_MODEL_FINITE_T_4D;
   if (!st) st = plan_scratch(ctx, pl, (pb->model == FFRG_MODEL_FINITE_T && !ctx->budget) || too_big);
+  if (!st) st = set_cuda_error(ctx, finish_legacy_stream(), "plan uploads");
   if (st) {
     plan_free(ctx, pl);
     return st;
