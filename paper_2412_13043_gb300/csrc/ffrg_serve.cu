@@ -313,10 +313,16 @@ static size_t smem32_of(const Plan &pl) {
   return pl.smem32;
 }
 
-// Launch set layout: descs | fa | cost prefixes (cap + 1) | item prefixes (cap + 1).
-static size_t set_bytes_of(int cap) {
-  return (sizeof(RhsArgs) + sizeof(FlowArgs)) * cap + (sizeof(long long) + sizeof(int)) * (cap + 1);
+// Launch set layout: descs | fa | cost prefixes (cap + 1) | item prefixes (cap
+// + 1), a multiple of 256 bytes: the staging buffers lie one after the other,
+// and each starts with 8-byte aligned descriptors.
+static constexpr size_t set_bytes_of(int cap) {
+  return ((sizeof(RhsArgs) + sizeof(FlowArgs)) * cap + (sizeof(long long) + sizeof(int)) * (cap + 1) + 255) & ~(size_t)255;
 }
+static_assert(alignof(RhsArgs) <= 16 && sizeof(RhsArgs) % alignof(FlowArgs) == 0 &&
+              sizeof(FlowArgs) % alignof(long long) == 0, "segments of a launch set");
+static_assert(set_bytes_of(kStages) % 16 == 0 && set_bytes_of(2 * kStages) % 16 == 0 &&
+              set_bytes_of(63 * kStages) % 16 == 0 && set_bytes_of(256 * kStages) % 16 == 0, "aligned staging buffers");
 
 // Upload the descriptors of the given slots as one compact launch set, `per`
 // descriptors a flow (its stages, or one; first: the first derivative, at
