@@ -463,7 +463,7 @@ const FxTables *fx_device_tables(int device) {
 int get_plan(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc *td, Plan **out) {
   std::vector<long long> key = {pb->model, pb->n_rad, pb->n_ang1, pb->n_ang2, pb->n_ext_p, pb->n_ext_ang,
                                 pb->n_matsubara, pb->include_p0, td->n_tables, td->n_stack, td->n_pts,
-                                pb->model == FFRG_MODEL_FINITE_T ? pb->statistics : 0,
+                                pb->statistics,
                                 pb->model == FFRG_MODEL_D4_FULL ? pb->n_va : 1,
                                 pb->model == FFRG_MODEL_D4_FULL ? pb->n_vb : 1,
                                 pb->model == FFRG_MODEL_FINITE_T_4D ? pb->n_x0 : 0};

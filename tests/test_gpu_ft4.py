@@ -96,3 +96,15 @@ def test_frozen_flow_across_the_branch_switch(ctx):
     assert st["status"] == ffrg.OK
     got = y.cpu().numpy()
     assert np.max(np.abs(got - truth) / np.abs(truth)) < 1e-8
+
+
+@pytest.mark.parametrize("first", [False, True])
+def test_both_statistics_of_one_shape_in_one_context(first):
+    """A bosonic and a fermionic loop of the same sizes, one after the other in one context."""
+    c = gpu_context()
+    for fermionic in (first, not first):
+        wl = fi.make_finite_t_4d(seed=54, N=6, T=0.05, n_pts=16, n_ext_p=5, n_ext_m=1, n_rad=11, n_ang=7, n_x0=13,
+                                 fermionic=fermionic)
+        for k in (0.4, 8.0):
+            _check(c, wl, k)
+    c.close()
