@@ -124,7 +124,8 @@ __device__ __forceinline__ float reg_g(int reg, float y) {
 // The FP32 version switches to FP64 when m^2 cancels more than half of
 // Z (omega^2 + s^2 + k^2 r), i.e. P < -2 m^2: close to the convexity pole.
 // `pole` is only evaluated on that rare branch.  POLE = false drops the test;
-// callers use it only when m^2 >= 0 and no Z < 0, where P >= 0 >= -2 m^2.
+// callers use it only when m^2 >= 0 and no Z < 0, where P >= 0 >= -2 m^2, and
+// not with the flat regulator.
 template <bool POLE = true, bool OM = false, bool FULL = false, typename Pole>
 __device__ __forceinline__ float inv_prop(const RhsArgs &a, float Zs, float y, float om2s, const KConst<float> &kc,
                                           Pole &&pole) {
@@ -551,8 +552,8 @@ __device__ __forceinline__ float2 look2(Row32 r, float2 s2, float us, float uo, 
   return make_float2(line_at(r, {__float_as_uint(t.x) << 3, u.x}), line_at(r, {__float_as_uint(t.y) << 3, u.y}));
 }
 
-// Propagator of two lines as G = N R, R = 1/(Zs D + m2e N), with the regulator
-// form of reg_g: (N, D) = (1 - 2^{-y}, y) for y >= log2(e), (1, series g(y))
+// Propagator of two lines as G = N R, R = 1/(Zs D + m2e N), with the
+// exponential regulator's form in reg_g (the flat one: see pole_possible): (N, D) = (1 - 2^{-y}, y) for y >= log2(e), (1, series g(y))
 // below, and m2e = m^2 (finite T: m^2 + Zs om2s, the frequency part).  One
 // reciprocal instead of two (reg_g's and the propagator's); branch-free
 // (setp / selp).  Only for m^2 >= 0 and Z >= 0 (no near-pole test), where the
@@ -1221,8 +1222,11 @@ __device__ __forceinline__ double warp_sum(double v) {
 // 0, every stack row).  Block-wide: every thread of the CTA must call it.
 // FP32 line rows do not hold node values, so the FP32 d=3 / d=4 kernels take
 // the signs from the FP64 tables, where the Z rows come first (the FP32 value
-// is the FP64 one times k^2 ln 2 > 0, rounded: the same sign).  FP64 kernels
-// have no near-pole path.
+// is the FP64 one times k^2 ln 2 > 0, rounded: the same sign).  The flat
+// regulator takes the tested path as well, whatever the signs: the paths
+// without the test (prop1, prop2) have the exponential shape built in, and a
+// choice of shape there would cost the usual case.  FP64 kernels have no
+// near-pole path, and both shapes on their only one.
 __device__ __forceinline__ bool pole_possible(const RhsArgs &a, const SmemLayout<double> &, const KConst<double> &) {
   return false;
 }
@@ -1233,7 +1237,7 @@ __device__ __forceinline__ bool pole_possible(const RhsArgs &a, const SmemLayout
     for (int i = threadIdx.x; i < nz; i += blockDim.x) neg |= a.tab[i] < 0.0;
   else
     for (int i = threadIdx.x; i < nz; i += blockDim.x) neg |= S.tab[i].x < 0.0f;
-  return __syncthreads_or(neg) || kc.m2 < 0.0f;
+  return __syncthreads_or(neg) || kc.m2 < 0.0f || a.reg == FFRG_REG_LITIM;
 }
 
 // Output of external point e from the sum s of its partials: diagram
@@ -1454,7 +1458,7 @@ __global__ void __launch_bounds__(kThreadsWide, 1) ft_single_kernel(const __grid
   for (int i = threadIdx.x; i < a.n_ext_p; i += blockDim.x) p_loc[i] = (float)ext_momentum(a, i);
   stage_angles<float, false>(a, S);   // finite T: no sqrt(1 - c^2)
   const KConst<float> kc = make_kconst<float>(a);   // the host's copy (plain calls only)
-  const bool pole = __syncthreads_or(neg) || kc.m2 < 0.0f;
+  const bool pole = __syncthreads_or(neg) || kc.m2 < 0.0f || a.reg == FFRG_REG_LITIM;   // as pole_possible
   bool ok = true;
   // The radial factors of the contraction: warp 1 of the last CTAs, one warp
   // unit each (FP64 work spread over SMs) instead of K rows, hidden behind

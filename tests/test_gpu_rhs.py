@@ -515,3 +515,27 @@ def test_back_to_back_calls_equal_synchronised_calls(ctx, case):
             assert np.array_equal(o.cpu().numpy(), ref[key]), (case, prof, key)
     assert ctx.status_read() == ffrg.OK
     tabs.free()
+
+
+FLAT_MIXED = {
+    "d3": lambda: fi.make_d3(seed=91, n_pts=24, n_ext_p=9, n_rad=31, n_ang=11, regulator=fi.REG_LITIM),
+    "d4": lambda: fi.make_d4(seed=92, n_pts=20, n_ext_ang=3, n_rad=14, n_ang1=9, n_ang2=5, regulator=fi.REG_LITIM),
+    "d4 full, cells": lambda: fi.make_d4_full(seed=93, n_pts=12, n_va=3, n_vb=2, n_ext_ang=2, n_rad=8, n_ang1=6, n_ang2=5,
+                                              regulator=fi.REG_LITIM),
+    "d4 full, lines": lambda: fi.make_d4_full(seed=94, n_pts=160, n_va=8, n_vb=7, n_ext_ang=1, n_rad=3, n_ang1=2,
+                                              n_ang2=3, regulator=fi.REG_LITIM),
+    "finite T": lambda: fi.make_finite_t(seed=95, N=5, T=0.05, n_pts=20, n_ext_p=7, n_ext_m=3, n_rad=13, n_ang=9,
+                                         regulator=fi.REG_LITIM),
+    "finite T, one launch": lambda: fi.make_finite_t(seed=96, N=8, T=0.05, n_pts=16, n_ext_p=52, n_ext_m=4, n_rad=64,
+                                                     n_ang=7, regulator=fi.REG_LITIM),
+    "finite T, 4D regulator": lambda: fi.make_finite_t_4d(seed=97, N=6, T=0.05, n_pts=24, n_ext_p=7, n_ext_m=3,
+                                                          n_rad=13, n_ang=9, n_x0=21, regulator=fi.REG_LITIM),
+}
+
+
+@pytest.mark.parametrize("case", FLAT_MIXED)
+def test_flat_regulator_in_mixed_precision(ctx, case):
+    """The flat regulator is an option of every model and precision, whatever the signs of m^2 and Z."""
+    wl = FLAT_MIXED[case]()
+    for k in (0.4, 1.7):
+        _check(ctx, wl, k)

@@ -247,3 +247,21 @@ def test_served_fermionic_flows_match_oracle():
         st, y, _, _ = res[tk]
         assert st == ffrg.OK
         assert np.max(np.abs(y - truth) / np.abs(truth)) < ENDPOINT_TOL
+
+
+@pytest.mark.parametrize("model", ["d3", "ft"])
+def test_served_flow_with_the_flat_regulator(model):
+    import paper_2412_13043_gb300 as ffrg
+    wl = (fi.make_d3(seed=91, n_pts=24, n_ext_p=9, n_rad=24, n_ang=8, regulator=fi.REG_LITIM) if model == "d3" else
+          fi.make_finite_t(seed=92, N=3, T=0.2, n_pts=20, n_ext_p=5, n_ext_m=2, n_rad=16, n_ang=6,
+                           regulator=fi.REG_LITIM))
+    ctx = gpu_context()
+    ctx.serve_start(max_slots=2)
+    tk = _submit(ctx, wl, rtol=SERVE_RTOL)
+    st, y, _, _ = _wait(ctx, [tk], [wl.problem.n_ext()])[tk]
+    ctx.serve_stop()
+    ctx.close()
+    truth, _ = oracle.flow(wl.problem, wl.tables, wl.y0, wl.Lambda, math.log(wl.Lambda / wl.k_end), rtol=1e-13,
+                           atol=1e-16)
+    assert st == ffrg.OK
+    assert np.max(np.abs(y - truth) / np.abs(truth)) < ENDPOINT_TOL
