@@ -253,7 +253,7 @@ FFRG_API int ffrg_rhs_host(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_tab
  * pool), and a latency-critical loop where cudaMalloc/cudaFree would stall
  * other streams.  It computes exactly what ffrg_rhs computes with the same
  * kernels, but needs no context and calls no cudaMalloc, cudaFree or other
- * allocating routine.  Its scratch is one fixed device array of 4 MiB + 480 KiB
+ * allocating routine.  Its scratch is one fixed device array of 4 MiB + 688 KiB
  * inside this library.  Every GPU that loads the library holds that array until the
  * process exits.
  *   pb, desc: problem and table layout (as for ffrg_rhs / ffrg_tables_upload);

@@ -58,7 +58,7 @@ struct AdjSmem {
   __device__ AdjSmem(unsigned char *base, const RhsArgs &a) {
     fx = (FxTables *)base;
     tab = (double2 *)(base + sizeof(FxTables));
-    cw2 = tab + a.tab_count;
+    cw2 = tab + a.tab64_count;
     c1 = (double *)(cw2 + a.na2);
     s1 = c1 + a.na1;
     w1 = s1 + a.na1;
@@ -70,7 +70,7 @@ __device__ __forceinline__ void adj_prologue(const AdjArgs &A, AdjSmem &S) {
   const RhsArgs &a = A.a;
   const double k = scale_k(a), k2 = k * k;
   stage_fx(a, S.fx);
-  for (int i = threadIdx.x; i < a.tab_count; i += blockDim.x) S.tab[i] = tab64_entry(a, i, k2);
+  for (int i = threadIdx.x; i < a.tab64_count; i += blockDim.x) S.tab[i] = tab64_entry(a, i, k2);
   for (int i = threadIdx.x; i < a.na1; i += blockDim.x) {
     double c = a.a1_x[i];
     S.c1[i] = c;
@@ -106,22 +106,22 @@ __device__ __forceinline__ void adj_collect(const AdjArgs &A, AdjSmem &S, double
   __syncthreads();
 }
 
-// A lookup's node, kept inside the row (the last node as weight 1 of the cell
-// before it), and its value
+// A lookup's entry in a line-form row, and its cell of the gradient: the cell's
+// first node (the last node counts as weight 1 of the cell before it) and 1 +
+// weight; and its value
 struct AdjPos {
-  int i;
+  int e, i;
   double w1;
 };
 __device__ __forceinline__ AdjPos adj_pos(const RhsArgs &a, const KConst<double> &kc, double y, FxOff o) {
   AdjPos p;
-  node_of(a, kc, y, o, p.i, p.w1);
-  if (p.i == a.n_pts - 1) {
-    p.i -= 1;
-    p.w1 = 2.0;
-  }
+  node_of(a, kc, y, o, p.e, p.w1);
+  p.i = min(max(p.e - 1, 0), a.n_pts - 2);
+  if (p.e == 0) p.w1 = 1.0;
+  if (p.e == a.n_pts) p.w1 = 2.0;
   return p;
 }
-__device__ __forceinline__ double adj_val(const double2 *row, AdjPos p) { return line64(row[p.i], p.w1); }
+__device__ __forceinline__ double adj_val(const double2 *row, AdjPos p) { return line64(row[p.e], p.w1); }
 
 // add c (1 - w) and c w to entries j + p.i and + 1, in turns of 2^lc lanes
 __device__ __forceinline__ void adj_scatter(double *g, int lc, int j, AdjPos p, double c, bool valid, int lane) {
@@ -172,7 +172,7 @@ __device__ __forceinline__ void d4_adjoint_rows(const AdjArgs &A, const AdjSmem 
                                                 int e, int row, bool valid, int lane) {
   const RhsArgs &a = A.a;
   const int np = a.n_pts, np_ = a.n_ext_p, npsi = a.n_ext_ang, lc = A.lc;
-  const double2 *Zt = S.tab, *L3 = S.tab + np, *L4 = S.tab + 2 * np;
+  const double2 *Zt = S.tab, *L3 = S.tab + (np + 1), *L4 = S.tab + 2 * (np + 1);
   double *g4 = g + (A.n_wide << lc);
   int block, ip, jp = 0;
   if (e <= np_) {
@@ -324,7 +324,7 @@ static int adjoint_setup(ffrg_ctx *ctx, Plan *pl, AdjArgs &A, void (**kern_out)(
     A.lc = pl->adj_lc;
     return FFRG_OK;
   }
-  const size_t fixed = sizeof(FxTables) + (size_t)pl->tab_count * 16 + ((size_t)3 * pl->na1 + 2 * (size_t)pl->na2) * 8;
+  const size_t fixed = sizeof(FxTables) + (size_t)pl->tab64_count * 16 + ((size_t)3 * pl->na1 + 2 * (size_t)pl->na2) * 8;
   int lc = 0, nw = 0;
   double best = 0.0;
   for (int l = 0; l <= 5; ++l) {

@@ -338,12 +338,15 @@ void plan_geometry(Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td) 
   // FP32 layout: (value, difference) node pairs; finite T: (Z, lambda) node
   // pairs per stack row plus one zero pair (same bytes as single values)
   // D4_FULL: compact [Z row 0 | lambda4 row 0 | lambda3 rows] in both precisions
-  // FP64 layout: one double2 per value (finite T: Z and lambda of a node side by side)
+  // FP64 layout: one double2 per value and one in front of each row (finite T: Z and lambda of a node side by side)
   pl->n_va = pb->model == FFRG_MODEL_D4_FULL ? pb->n_va : 1;
   pl->n_vb = pb->model == FFRG_MODEL_D4_FULL ? pb->n_vb : 1;
   const int compact = pb->model == FFRG_MODEL_D4_FULL ? (2 + pl->n_va * pl->n_vb) * td->n_pts : pl->tab_count;
   pl->tab32_count = pb->model == FFRG_MODEL_FINITE_T ? td->n_stack * td->n_pts + 1 : compact;
-  pl->tab64_count = pb->model == FFRG_MODEL_FINITE_T ? 2 * td->n_stack * td->n_pts : compact;
+  const int rows64 = pb->model == FFRG_MODEL_D4_FULL    ? 2 + pl->n_va * pl->n_vb
+                     : pb->model == FFRG_MODEL_FINITE_T ? 2 * td->n_stack
+                                                        : td->n_tables * td->n_stack;
+  pl->tab64_count = rows64 * (td->n_pts + 1);
   int outer_total, rows_per_outer;
   if (is_d4(pb->model)) {
     pl->jb = pl->na2;

@@ -152,12 +152,12 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kThreads64 : kThreads)
   const double k = scale_k(a), k2 = k * k, m2 = mass2(a, k);
   // FP64: function tables | (Z, L) line-form pairs | (node, weight)
   FxTables *fx = (FxTables *)ft4_smem;
-  double2 *zl64 = (double2 *)(ft4_smem + sizeof(FxTables)), *cw64 = zl64 + 2 * a.n_pts;
+  double2 *zl64 = (double2 *)(ft4_smem + sizeof(FxTables)), *cw64 = zl64 + 2 * (a.n_pts + 1);
   float4 *zl = reinterpret_cast<float4 *>(ft4_smem);
   float2 *cw = reinterpret_cast<float2 *>(zl + a.n_pts);
   if constexpr (sizeof(T) == 8) {
     stage_fx(a, fx);
-    for (int i = threadIdx.x; i < 2 * a.n_pts; i += blockDim.x) zl64[i] = tab64_entry(a, i, k2);
+    for (int i = threadIdx.x; i < 2 * (a.n_pts + 1); i += blockDim.x) zl64[i] = tab64_entry(a, i, k2);
     for (int c = threadIdx.x; c < a.na1; c += blockDim.x) cw64[c] = make_double2(a.a1_x[c], a.a1_w[c]);
   } else {
     const double *Zt = a.tab, *Lt = a.tab + a.n_pts;
@@ -245,7 +245,7 @@ int launch_ft4(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int precisi
     ctx->last_error = "plan without the frequency buffer, radial factors or counters";
     return FFRG_EINVAL;
   }
-  const size_t smem = a.fp64 ? sizeof(FxTables) + (size_t)(2 * pl->n_pts + pl->na1) * sizeof(double2)
+  const size_t smem = a.fp64 ? sizeof(FxTables) + (size_t)(2 * (pl->n_pts + 1) + pl->na1) * sizeof(double2)
                              : (size_t)pl->n_pts * sizeof(float4) + (size_t)pl->na1 * sizeof(float2);
   void (*kern)(RhsArgs, int) = a.fp64 ? ft4_main_kernel<double> : ft4_main_kernel<float>;
   const int threads = a.fp64 ? kThreads64 : kThreads;

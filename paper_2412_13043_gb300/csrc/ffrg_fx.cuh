@@ -133,14 +133,15 @@ FX_FN FxLogEntry fx_scaled(FxLogEntry t, const FxGrid &g) {
   return t;
 }
 
-// node and interpolation weight: i in [0, n-1], w1 = 1 + weight in [1, 2); at
+// node and interpolation weight: i in [0, last], w1 = 1 + weight in [1, 2); at
 // the last node the table's difference is 0 and the weight does not matter
-FX_FN void fx_node(const FxGrid &g, int64_t u, int &i, double &w1) {
+FX_FN void fx_node(const FxGrid &g, int64_t u, int last, int &i, double &w1) {
   const uint64_t v = u < 0 ? 0 : (uint64_t)u;
   const int n = (int)(v >> g.F);
-  i = n < g.nm1 ? n : g.nm1;
+  i = n < last ? n : last;
   w1 = fx_double(((v << (64 - g.F)) >> 12) | 0x3FF0000000000000ull);
 }
+FX_FN void fx_node(const FxGrid &g, int64_t u, int &i, double &w1) { fx_node(g, u, g.nm1, i, w1); }
 
 // h(x) = x/(1 - e^{-x}) for x >= 0 (x <= 0 and NaN below: see the callers)
 FX_FN double fx_h(const FxTables &T, double x) {

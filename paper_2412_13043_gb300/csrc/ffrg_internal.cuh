@@ -51,8 +51,9 @@ struct KConst {
   T isy;  // 1/sy
 };
 
-// FP64: table coordinates in fixed point (ffrg_fx.cuh).  FxOff: offset of a
-// coordinate taken in y = sy s^2 of S0^2 = (sum of c squares)/c.
+// FP64: table coordinates in fixed point (ffrg_fx.cuh), counted in entries of
+// the line-form rows.  FxOff: offset of a coordinate taken in y = sy s^2 of
+// S0^2 = (sum of c squares)/c.
 struct FxOff {
   int64_t v;
   int c;

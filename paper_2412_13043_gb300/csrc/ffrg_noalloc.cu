@@ -22,7 +22,10 @@
 namespace ffrg {
 
 constexpr size_t kNoallocScratchBytes = size_t(4) << 20;  // 4 MiB: what the problems may need
-constexpr size_t kNoallocTab64Bytes = size_t(480) << 10;  // and the FP64 line-form tables
+// and the FP64 line-form tables: up to 227 KB of values, 16 bytes each, and a
+// 16-byte entry more per row (two values or more)
+constexpr size_t kNoallocTab64Bytes = size_t(688) << 10;
+static_assert(kNoallocTab64Bytes >= 3 * kMaxDynSmemBytes + 256, "line-form tables behind the scratch");
 constexpr int kNoallocMaxDevices = 64;
 
 // Shared by every call of ffrg_rhs_noalloc on a device; keeps the last call's contents.
@@ -129,8 +132,9 @@ extern "C" int ffrg_rhs_noalloc(const ffrg_problem *pb, const ffrg_table_desc *t
   if (sc.used > kNoallocScratchBytes) return FFRG_EINVAL;  // problem needs more than the 4 MiB scratch
 
   // the tables must fit in shared memory as plain values (FP64 line form: twice as large, in global memory when
-  // it does not fit), so that line-form tables need at most 2 x 227 KB behind the scratch
-  const size_t values = (size_t)(pb->model == FFRG_MODEL_D4_FULL ? pl.tab64_count : pl.tab_count) * sizeof(double);
+  // it does not fit), so that line-form tables need at most 3 x 227 KB behind the scratch
+  const size_t values =
+      (pb->model == FFRG_MODEL_D4_FULL ? (size_t)(2 + pl.n_va * pl.n_vb) * td->n_pts : (size_t)pl.tab_count) * sizeof(double);
   const size_t rules = ((size_t)pl.na1 * 3 + (size_t)pl.na2 * 2) * sizeof(double);
   if (precision == FFRG_MIXED ? pl.smem32 > kMaxDynSmemBytes
                               : ((values + 15) & ~(size_t)15) + ((rules + 15) & ~(size_t)15) > kMaxDynSmemBytes)

@@ -55,6 +55,7 @@ __device__ __forceinline__ KConst<double> make_kconst<double>(const RhsArgs &a) 
     const int hi = fx_clamp_hi(fx_bits(c.k2));
     off += fx_log(fx_scaled(a.fx->log[fx_log_index(hi)], a.fg), a.fg, hi, (uint32_t)fx_bits(c.k2));
   }
+  if (!c.slow) off += (int64_t)1 << a.fg.F;   // entries of the line-form rows (tab64_entry), not nodes
   c.uy1 = {off - a.fg.uc[0], 1};
   c.uy2 = {off - a.fg.uc[1], 2};
   c.uy3 = {off - a.fg.uc[2], 3};
@@ -78,29 +79,32 @@ __device__ __forceinline__ KConst<double> load_kconst<double>(const RhsArgs &a) 
   return c;
 }
 
-// FP64 tables in line form: a node holds (T_i - d_i, d_i), d_i the difference
+// FP64 tables in line form: rows of n_pts + 1 entries, the first (T_0, 0) for
+// arguments below the grid, then (T_i - d_i, d_i) per node, d_i the difference
 // to the next node (0 at a row end), so that the interpolant is one FMA with
-// the weight 1 + w in [1, 2) of fx_node.  Layout: as the tables (D4_FULL: rows
-// Z | lambda4 | lambda3 rows; finite T: [row][node][Z, lambda]).  Z rows carry
-// k^2.  Entry i:
+// the weight 1 + w in [1, 2) of fx_node.  Its rounding, up to |d_i| 2^-53, is
+// below that of the coordinate everywhere on the grid; below the grid, where
+// the coordinate is cut off, the first entry gives T_0 itself (T_0 - d_0 + d_0
+// is 2e-5 off for a T_0 1e-12 of T_1).  A weight in [0, 1), with (T_i, d_i),
+// would do without that entry, but takes 4 % longer to form (d=4 vertex FP64
+// 3.08 -> 3.21 ms).  Layout: as the tables (D4_FULL: rows Z | lambda4 | lambda3
+// rows; finite T: [row][entry][Z, lambda]).  Z rows carry k^2.  Entry i:
 __device__ __forceinline__ double2 tab64_entry(const RhsArgs &a, int i, double k2) {
   const int np = a.n_pts, zn = a.n_stack * np;
-  size_t src;
-  int col;
+  const bool ft = a.model == FFRG_MODEL_FINITE_T || a.model == FFRG_MODEL_FINITE_T_4D;
+  const int j = ft ? i >> 1 : i, row = j / (np + 1), c = j - row * (np + 1), col = max(c - 1, 0);
+  size_t src = (size_t)row * np;
   bool z;
-  if (a.model == FFRG_MODEL_FINITE_T || a.model == FFRG_MODEL_FINITE_T_4D) {
+  if (ft) {
     z = !(i & 1);
-    src = (size_t)(i >> 1) + (z ? 0 : zn);
-    col = (i >> 1) % np;
+    if (!z) src += zn;
   } else {
-    const int row = i / np;
-    col = i - row * np;
     z = row < (a.model == FFRG_MODEL_D4_FULL ? 1 : a.n_stack);
-    src = i;
-    if (a.model == FFRG_MODEL_D4_FULL) src = col + (row == 0 ? (size_t)0 : row == 1 ? (size_t)2 * zn : (size_t)zn + (size_t)(row - 2) * np);
+    if (a.model == FFRG_MODEL_D4_FULL) src = row == 0 ? (size_t)0 : row == 1 ? (size_t)2 * zn : (size_t)zn + (size_t)(row - 2) * np;
   }
+  src += col;
   const double f = z ? k2 : 1.0, v = f * a.tab[src];
-  const double d = col == np - 1 ? 0.0 : f * a.tab[src + 1] - v;
+  const double d = c == 0 || col == np - 1 ? 0.0 : f * a.tab[src + 1] - v;
   return make_double2(v - d, d);
 }
 
@@ -113,19 +117,20 @@ __device__ __forceinline__ void stage_fx(const RhsArgs &a, FxTables *s) {
     ((int4 *)(s->log + kFxLog))[j] = ((const int4 *)(a.fx->log + kFxLog))[j];
 }
 
-// Node and weight of the coordinate of y (FP64 lookups): fixed point, or an
-// FP64 logarithm when the grid or k lies outside its range.
+// Entry of a line-form row and weight for the coordinate of y (FP64 lookups):
+// fixed point, or an FP64 logarithm when the grid or k lies outside its range.
 // (y and 1/sy are passed apart: their product in the caller was computed ahead
 // of the branch, three FP64 multiplications a d=4 term.)
 static __device__ __noinline__ void slow_node(const RhsArgs *a, double y, double isy, int c, int &i, double &w1) {
   double w;
   lerp_pos(y * isy, a->u_scale, a->uoc[c - 1], a->n_pts, i, w);
+  i = i == 0 && w == 0.0 ? 0 : i + 1;
   w1 = 1.0 + w;
 }
 __device__ __forceinline__ void node_of(const RhsArgs &a, const KConst<double> &kc, double y, FxOff o, int &i,
                                         double &w1) {
   if (kc.slow) slow_node(&a, y, kc.isy, o.c, i, w1);   // uniform
-  else fx_node(a.fg, fx_log(kc.us->log, a.fg, y) + o.v, i, w1);
+  else fx_node(a.fg, fx_log(kc.us->log, a.fg, y) + o.v, a.n_pts, i, w1);
 }
 __device__ __forceinline__ double line64(double2 t, double w1) { return fma(t.y, w1, t.x); }
 

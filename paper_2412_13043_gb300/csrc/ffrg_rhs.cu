@@ -273,7 +273,7 @@ __device__ __forceinline__ void precompute_body(const RhsArgs &a) {
   } else if (a.model == FFRG_MODEL_D4_FULL) {
     // compact rows [Z row 0 | lambda4 row 0 | lambda3 rows] (with lambda3 cells: the two line rows only)
     const int np = a.n_pts, ns = a.n_stack;
-    const int n_line = a.l3cell ? 2 * np : a.tab64_count;
+    const int n_line = (a.l3cell ? 2 : 2 + a.n_va * a.n_vb) * np;
     for (int i = tid0; i < n_line; i += stride) {
       const int row = i / np, col = i - row * np;
       const size_t src = row == 0 ? (size_t)col : row == 1 ? (size_t)2 * ns * np + col : ((size_t)ns + row - 2) * np + col;
@@ -687,13 +687,13 @@ __device__ __forceinline__ RowAcc<T> d3_witem(const RhsArgs &a, const RhsArgs *s
 }
 
 // finite-T lookups of Z and lambda at y in stack row srow: FP64 line-form
-// entries [row][pt][Z, lambda]; FP32 (Z, lambda) node pairs [row][pt] (+ one zero pair)
+// entries [row][entry][Z, lambda]; FP32 (Z, lambda) node pairs [row][pt] (+ one zero pair)
 __device__ __forceinline__ void zl_lookup(const double2 *tab, const RhsArgs &a, const KConst<double> &kc, int srow,
                                           double y, double &Z, double &L) {
   int i;
   double w1;
   node_of(a, kc, y, kc.uy1, i, w1);
-  const double2 *e = tab + 2 * ((size_t)srow * a.n_pts + i);
+  const double2 *e = tab + 2 * ((size_t)srow * (a.n_pts + 1) + i);
   Z = line64(e[0], w1);
   L = line64(e[1], w1);
 }
@@ -877,7 +877,7 @@ __device__ __forceinline__ float lam3_full(const RhsArgs &a, Row32 L3, float y3,
 }
 __device__ __forceinline__ double lam3_full(const RhsArgs &a, const double2 *L3, double y3, Look64 us, FxOff uy3,
                                             double va, double vb) {
-  const int np = a.n_pts, na = a.n_va, nb = a.n_vb;
+  const int np = a.n_pts + 1, na = a.n_va, nb = a.n_vb;   // entries of a row
   int i0, ia, ib;
   double w1, wa, wb;
   node_of(us.a, us.kc, y3, uy3, i0, w1);
@@ -1089,7 +1089,8 @@ __device__ __forceinline__ RowAcc<T> d4_witem(const RhsArgs &a, const RhsArgs *s
   const auto us = look_scale(a, kc);
   const T sy = kc.sy;
   const int np = a.n_pts, np_ = a.n_ext_p, npsi = a.n_ext_ang, na1 = a.na1;
-  const auto Zt = tab_row(S, 0), L3 = tab_row(S, (FULL ? 2 : 1) * np), L4 = tab_row(S, (FULL ? 1 : 2) * np);
+  const int rs = sizeof(T) == 8 ? np + 1 : np;   // entries of a row
+  const auto Zt = tab_row(S, 0), L3 = tab_row(S, (FULL ? 2 : 1) * rs), L4 = tab_row(S, (FULL ? 1 : 2) * rs);
   int block, ip, jp = 0;
   if (e <= np_) {
     block = 0;

@@ -117,3 +117,45 @@ def test_momenta_far_from_a_narrow_grid(ctx, model, hi):
     gref = oracle.rhs_jacobian(wl.problem, wl.tables, 0.3).T @ gbar
     assert np.max(np.abs(got - ref) / np.abs(ref)) < 1e-12
     assert np.max(np.abs(grad - gref)) / np.max(np.abs(gref)) < 1e-12
+
+
+def _steep(wl):
+    """Every momentum below the first node, the tables there 1e-12 of the next one."""
+    wl.problem = dataclasses.replace(wl.problem, x_min=1.0, x_max=10.0, p_min=0.01, p_max=0.02, m2_over_k2=0.0,
+                                     m2_shift=0.0)
+    rng = np.random.default_rng(18)
+    wl.tables = rng.uniform(0.5, 1.5, wl.tables.shape)
+    wl.tables[..., 0] *= 1e-12
+    return wl
+
+
+STEEP = {
+    "d3": lambda: fi.make_d3(seed=1, n_pts=12, n_ext_p=5, n_rad=9, n_ang=7),
+    "d4": lambda: fi.make_d4(seed=1, n_pts=12, n_ext_ang=2, n_rad=7, n_ang1=5, n_ang2=3),
+    "d4 full": lambda: fi.make_d4_full(seed=1, n_pts=12, n_va=3, n_vb=2, n_ext_ang=2, n_rad=7, n_ang1=5, n_ang2=3),
+    "finite T": lambda: fi.make_finite_t(seed=1, N=4, T=1e-3, n_pts=12, n_ext_p=5, n_ext_m=2, n_rad=9, n_ang=7),
+    "finite T, 4D regulator": lambda: fi.make_finite_t_4d(seed=1, N=8, T=1e-3, n_pts=12, n_ext_p=5, n_ext_m=2, n_rad=9,
+                                                          n_ang=7, n_x0=9),
+    "tables in global memory": lambda: fi.make_d4(seed=1, n_pts=4000, n_ext_ang=1, n_rad=3, n_ang1=2, n_ang2=2),
+    "grid beyond fixed point": lambda: fi.make_d3(seed=1, n_pts=12, n_ext_p=5, n_rad=9, n_ang=7),
+}
+
+
+@pytest.mark.parametrize("case", STEEP)
+def test_lookups_below_a_steep_first_cell(ctx, case):
+    """Below the grid a table has its first value, however far the second is from it."""
+    import torch
+
+    import paper_2412_13043_gb300 as ffrg
+    wl = _steep(STEEP[case]())
+    wl.problem = dataclasses.replace(wl.problem, n_ext_p=5, x_max=1e17 if case == "grid beyond fixed point" else 10.0)
+    tabs = ctx.tables(wl.problem, wl.tables)
+    got = ctx.rhs(wl.problem, tabs, 0.01, precision=ffrg.FP64).cpu().numpy()
+    ref = oracle.rhs(wl.problem, wl.tables, 0.01)
+    assert np.max(np.abs(got - ref) / np.abs(ref)) < 1e-12
+    if case in ("d3", "d4", "grid beyond fixed point"):
+        gbar = np.random.default_rng(19).uniform(0.5, 1.0, wl.problem.n_ext())
+        grad = ctx.rhs_adjoint(wl.problem, tabs, 0.01, torch.tensor(gbar, device="cuda")).cpu().numpy().ravel()
+        gref = oracle.rhs_jacobian(wl.problem, wl.tables, 0.01).T @ gbar
+        assert np.max(np.abs(grad - gref)) / np.max(np.abs(gref)) < 1e-12
+    tabs.free()
