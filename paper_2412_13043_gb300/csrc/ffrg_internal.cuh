@@ -547,7 +547,6 @@ struct ffrg_ctx {
   // ffrg_ft_states scratch (operand slices, exact pass sums, scales), grown on demand
   void *states_dev = nullptr;
   size_t states_cap = 0;
-  int states_chunks = 0;  // K ranges whose pass table the scratch holds (0: none)
 };
 
 namespace ffrg {

@@ -24,21 +24,21 @@
 #include <math.h>
 
 #include <algorithm>
-#include <vector>
 
 #include "ffrg_internal.cuh"
 #include "ffrg_umma.cuh"
 
 namespace ffrg {
 
-constexpr int kSlices = 10;
+using umma::kGroups;
+using umma::kSlices;
+using umma::level_groups;
 constexpr int kBits = 5;
 
 struct StatesScratch {
   uint16_t *A, *B;
   float *part;
   int *e_row, *e_col;
-  int4 *pass_tab;
 };
 
 // |v| as an ordered integer (IEEE bit pattern without the sign)
@@ -217,16 +217,6 @@ struct CombineArgs {
   int n_rows, n_cols, rows_pad, cols_pad, n_chunks;
 };
 
-// passes of a level (its l + 1 pairs in groups of at most kGroup) and of the
-// levels before it
-__host__ __device__ constexpr int level_groups(int l) { return (l + umma::kGroup) / umma::kGroup; }
-__host__ __device__ constexpr int groups_before(int l) {
-  int n = 0;
-  for (int k = 0; k < l; ++k) n += level_groups(k);
-  return n;
-}
-constexpr int kGroups = groups_before(kSlices);
-
 // thread per output (state fastest): the passes of a level are exact
 // integers (level sums below 3072 x 196608 < 2^31 in all); levels 0..6 and 7..9
 // are combined exactly in two 64-bit integers, which one FP64 FMA adds; the
@@ -320,10 +310,9 @@ extern "C" int ffrg_ft_states(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_
   if (st) return st;
 
   // scratch, kept by the context and grown on demand (256-byte segments):
-  // pass table (room for all K ranges) | A slices | B slices | pass sums | scales
+  // A slices | B slices | pass sums | scales
   auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-  const size_t o_A = al((size_t)kGroups * (196608 / umma::kMaxExactK) * sizeof(int4));
-  const size_t o_B = o_A + al(kSlices * a_slice * 2), o_part = o_B + al(kSlices * b_slice * 2);
+  const size_t o_B = al(kSlices * a_slice * 2), o_part = o_B + al(kSlices * b_slice * 2);
   const size_t o_er = o_part + al((size_t)passes * rows_pad * cols_pad * 4);
   const size_t o_ec = o_er + al((size_t)rows_pad * 4);
   const size_t need = o_ec + al((size_t)cols_pad * 4);
@@ -331,37 +320,13 @@ extern "C" int ffrg_ft_states(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_
     dev_free(ctx, ctx->states_dev, ctx->states_cap);
     ctx->states_dev = nullptr;
     ctx->states_cap = 0;
-    ctx->states_chunks = 0;
     st = dev_alloc(ctx, &ctx->states_dev, need);
     if (st) return st;
     ctx->states_cap = need;
   }
   unsigned char *base = (unsigned char *)ctx->states_dev;
-  StatesScratch sc{(uint16_t *)(base + o_A), (uint16_t *)(base + o_B), (float *)(base + o_part),
-                   (int *)(base + o_er), (int *)(base + o_ec), (int4 *)base};
-  if (ctx->states_chunks != n_chunks) {
-    // the pass table, one slot per CTA z: first slice pair (i, j) of a group of
-    // a level, output pass (level order, K ranges innermost), K range and
-    // number of pairs; the largest groups first, so that the short ones fill
-    // the last wave (uploaded when the number of K ranges changes)
-    std::vector<int4> ij;
-    for (int n = umma::kGroup; n > 0; --n)
-      for (int l = 0; l < kSlices; ++l)
-        for (int q = 0, i = 0; q < level_groups(l); ++q) {
-          // the level's pairs shared out evenly over its groups
-          const int size = (l + 1) / level_groups(l) + (q < (l + 1) % level_groups(l) ? 1 : 0);
-          if (size == n)
-            for (int c = 0; c < n_chunks; ++c)
-              ij.push_back(make_int4(i, l - i, (groups_before(l) + q) * n_chunks + c, c | size << 16));
-          i += size;
-        }
-    st = set_cuda_error(ctx, cudaMemcpyAsync(sc.pass_tab, ij.data(), ij.size() * sizeof(int4),
-                                             cudaMemcpyHostToDevice, s), "ffrg_ft_states pass table");
-    // from pageable memory: the copy must have read ij before it goes away
-    if (!st) st = set_cuda_error(ctx, cudaStreamSynchronize(s), "ffrg_ft_states pass table");
-    if (st) return st;
-    ctx->states_chunks = n_chunks;
-  }
+  StatesScratch sc{(uint16_t *)base, (uint16_t *)(base + o_B), (float *)(base + o_part), (int *)(base + o_er),
+                   (int *)(base + o_ec)};
 
   SplitArgs sg;
   sg.K = pl->kbuf;
@@ -392,8 +357,8 @@ extern "C" int ffrg_ft_states(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_
 
   st = ensure_smem_limit(ctx, (const void *)umma::slice_pair_gemm, umma::kSmemBytes);
   if (st) return st;
-  umma::GemmArgs gg{sc.A, sc.B, sc.part, sc.pass_tab, m_tiles, n_tiles, k_tiles, kt_chunk, n_chunks,
-                    ctx->status_dev};
+  constexpr umma::PairGroups kPairGroups = umma::pair_groups();
+  umma::GemmArgs gg{sc.A, sc.B, sc.part, m_tiles, n_tiles, k_tiles, kt_chunk, n_chunks, ctx->status_dev, kPairGroups};
   const bool prof = ctx->profiling && ctx->prof_used * 2 + 1 < (int)ctx->prof_events.size();
   if (prof) cudaEventRecord(ctx->prof_events[2 * ctx->prof_used], s);
   umma::slice_pair_gemm<<<dim3(n_tiles, m_tiles, passes), umma::kThreadsGemm, umma::kSmemBytes, s>>>(gg);

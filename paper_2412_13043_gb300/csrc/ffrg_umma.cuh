@@ -47,6 +47,7 @@ constexpr int kStageBytes = kTileA + kTileB;
 constexpr int kSmemBytes = kStages * kStageBytes;   // 96 KB: two CTAs per SM
 constexpr int kTmemCols = 256;
 constexpr int kThreadsGemm = 128;
+constexpr int kSlices = 10;        // slices of an operand
 constexpr int kGroup = 4;          // slice pairs of a level in one pass
 constexpr int kMaxExactK = 8192;   // K-elements whose slice products sum exactly in FP32, kGroup pairs at once
 static_assert(kMaxExactK * (2 * 512 + (kGroup - 2) * 256) < (1 << 24), "exact in FP32");
@@ -58,14 +59,47 @@ __host__ __device__ inline int tile_offset(int r, int k, int rows) {
   return (k >> 3) * (rows * 8) + (r >> 3) * 64 + (r & 7) * 8 + (k & 7);
 }
 
+// passes of a level (its l + 1 pairs shared out evenly over groups of at most
+// kGroup) and of the levels before it
+__host__ __device__ constexpr int level_groups(int l) { return (l + kGroup) / kGroup; }
+__host__ __device__ constexpr int groups_before(int l) {
+  int n = 0;
+  for (int k = 0; k < l; ++k) n += level_groups(k);
+  return n;
+}
+constexpr int kGroups = groups_before(kSlices);
+
+// a group: its first slice pair (i, j), its place in level order, its pairs
+struct PairGroup {
+  unsigned char i, j, at, n;
+};
+// the groups in launch order: the largest first, so that the short ones fill
+// the last wave
+struct PairGroups {
+  PairGroup g[kGroups];
+};
+constexpr PairGroups pair_groups() {
+  PairGroups t{};
+  int k = 0;
+  for (int n = kGroup; n > 0; --n)
+    for (int l = 0; l < kSlices; ++l)
+      for (int q = 0, i = 0; q < level_groups(l); ++q) {
+        const int size = (l + 1) / level_groups(l) + (q < (l + 1) % level_groups(l) ? 1 : 0);
+        if (size == n)
+          t.g[k++] = {(unsigned char)i, (unsigned char)(l - i), (unsigned char)(groups_before(l) + q), (unsigned char)n};
+        i += size;
+      }
+  return t;
+}
+
 struct GemmArgs {
   const uint16_t *A;   // BF16 bits, slices [nsl][m_tiles][k_tiles][128 x kBK tile]
   const uint16_t *B;   // BF16 bits, slices [nsl][n_tiles][k_tiles][256 x kBK tile]
   float *part;         // [passes][m_tiles * 128][n_tiles * 256], exact sums per pass
-  const int4 *pass_tab; // per CTA z: first slice pair (i, j), output pass, K range + pairs << 16
   int m_tiles, n_tiles, k_tiles;
   int kt_per_chunk, n_chunks;  // K-tiles per pass and K ranges per slice pair
   unsigned *status;
+  PairGroups groups;   // by value: a table in device memory had to be uploaded again whenever n_chunks changed
 };
 
 __device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -155,8 +189,8 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 }
 
 // One pass per CTA: blockIdx.x = output column tile, blockIdx.y = output row
-// tile, blockIdx.z = slot of the pass table (group of slice pairs, its output
-// pass and K range; the largest groups first).
+// tile, blockIdx.z = group of slice pairs (the largest first) x K range; its
+// output pass is in level order, K ranges innermost.
 __global__ void __launch_bounds__(kThreadsGemm, 1) slice_pair_gemm(GemmArgs g) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[kStages], empty[kStages], done;
@@ -164,11 +198,12 @@ __global__ void __launch_bounds__(kThreadsGemm, 1) slice_pair_gemm(GemmArgs g) {
   __shared__ int abort_flag, issued, consumed;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tn = blockIdx.x, tm = blockIdx.y;
-  const int4 pt = g.pass_tab[blockIdx.z];
-  const int2 ij = make_int2(pt.x, pt.y);
-  const int pass = pt.z, chunk = pt.w & 0xFFFF;
+  const int slot = blockIdx.z / g.n_chunks, chunk = blockIdx.z - slot * g.n_chunks;
+  const PairGroup pg = g.groups.g[slot];
+  const int2 ij = make_int2(pg.i, pg.j);
+  const int pass = pg.at * g.n_chunks + chunk;
   const int kt0 = chunk * g.kt_per_chunk;
-  const int per_pair = min(g.kt_per_chunk, g.k_tiles - kt0), nkt = per_pair * (pt.w >> 16);
+  const int per_pair = min(g.kt_per_chunk, g.k_tiles - kt0), nkt = per_pair * pg.n;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {

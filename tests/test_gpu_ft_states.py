@@ -125,3 +125,28 @@ def test_repeatable_and_rejects_other_models(ctx):
     with pytest.raises(ffrg.FfrgError):
         ctx.ft_states(w3.problem, tabs, 1.0, Fd)
     tabs.free()
+
+
+def test_calls_of_several_sizes_under_capture(ctx):
+    """After a warm-up at the largest size, calls of any number of states are asynchronous: captured in one graph,
+    its replay gives the same bits as the calls themselves."""
+    import torch
+
+    import paper_2412_13043_gb300 as ffrg
+    wl = fi.make_finite_t(seed=21, N=15, T=0.01, n_pts=16, n_ext_p=5, n_ext_m=3, n_rad=133, n_ang=3)
+    tabs = ctx.tables(wl.problem, wl.tables)
+    F = torch.from_numpy(np.random.default_rng(22).uniform(-1.0, 2.0, (1500, oracle.ft_nfreq(wl.problem), 133))).cuda()
+    parts = [F[:n].contiguous() for n in (1500, 40, 700, 1)]
+    want = [ctx.ft_states(wl.problem, tabs, 0.8, p, precision=ffrg.FP64) for p in parts]
+    ctx.ft_states(wl.problem, tabs, 0.8, parts[0], precision=ffrg.FP64)
+    got = [torch.zeros_like(w) for w in want]
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for p, o in zip(parts, got):
+            ctx.ft_states(wl.problem, tabs, 0.8, p, out=o, precision=ffrg.FP64)
+    graph.replay()
+    torch.cuda.synchronize()
+    for g, w in zip(got, want):
+        assert torch.equal(g, w)
+    tabs.free()
