@@ -26,6 +26,7 @@ namespace ffrg {
 // [2 nfreq] the number of frequencies in use
 __global__ void ft4_freq_kernel(RhsArgs a, int nfreq_max) {
   pdl_trigger();   // the factor kernel may start (it waits for these writes)
+  if (skipped(a)) return;
   double *kb = (double *)a.kbuf, *fq = kb, *fw = kb + nfreq_max;
   const double k = scale_k(a), L0 = a.qmax_over_k * k, T = a.T;
   const int cap = 2 * a.N + 1 + (a.stat ? 1 : 0);
@@ -66,6 +67,7 @@ __global__ void ft4_freq_kernel(RhsArgs a, int nfreq_max) {
 __global__ void ft4_factor_kernel(RhsArgs a, int nfreq_max) {
   pdl_trigger();   // the main kernel may start staging its tables
   pdl_wait();      // frequencies, weights and q_r of the frequency kernel
+  if (skipped(a)) return;
   const double *kb = (const double *)a.kbuf;
   const int nf = (int)kb[2 * nfreq_max];
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -146,6 +148,10 @@ __device__ __forceinline__ float ft4_row32(const RhsArgs &a, const float4 *zl, c
 template <typename T>
 __global__ void __launch_bounds__(sizeof(T) == 8 ? kThreads64 : kThreads)
     ft4_main_kernel(RhsArgs a, int nfreq_max) {
+  if (skipped(a)) {   // wait all the same: this kernel completes after the two before it
+    pdl_wait();
+    return;
+  }
   extern __shared__ __align__(16) unsigned char ft4_smem[];
   const int lane = threadIdx.x & 31, nm = a.n_ext_ang;
   const double *kb = (const double *)a.kbuf;

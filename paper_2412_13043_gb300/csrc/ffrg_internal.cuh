@@ -322,6 +322,10 @@ struct ItemQueue {
   }
 };
 
+// True when the flow of this right-hand side has ended (uniform over the grid;
+// the flag does not change while the kernels of a right-hand side run).
+__device__ __forceinline__ bool skipped(const RhsArgs &a) { return a.skip && *(volatile const int *)a.skip; }
+
 // Device-wide status word (sticky bits).
 __device__ __forceinline__ void raise_status(unsigned *status, unsigned bit) {
   if (status) atomicOr(status, bit);

@@ -155,8 +155,6 @@ constexpr int kMainThreads = sizeof(T) == 8 ? kThreads64 : kThreads;
 // ---------------------------------------------------------------------------
 // 1. precompute kernel
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool skipped(const RhsArgs &a) { return a.skip && *(volatile const int *)a.skip; }
-
 // blocks of the per-radial precompute: radial nodes x values of |n|
 constexpr int kPreR = 64, kPreN = 8;
 

@@ -6,6 +6,7 @@ both branches of the frequency integral (Matsubara sum while at most
 both loop statistics, the bench workload on every output, and a frozen flow
 from k = 10 to 0.01 that crosses the branch switch."""
 import math
+import time
 
 import numpy as np
 import pytest
@@ -108,3 +109,37 @@ def test_both_statistics_of_one_shape_in_one_context(first):
         for k in (0.4, 8.0):
             _check(c, wl, k)
     c.close()
+
+
+@pytest.mark.parametrize("budget", [0, 1 << 30])
+def test_steps_past_the_end_of_a_flow_return_at_once(budget):
+    """A flow launches steps past its end; they find it done.  A flow of zero length takes the time of its first
+    derivative, not of the right-hand sides of two more steps; a flow of one step that of its own (five side by side,
+    in a context with a budget six one by one), not of the second step as well; and no right-hand side at a scale
+    that was never set leaves its mark in the status word."""
+    import torch
+
+    import paper_2412_13043_gb300 as ffrg
+    c = ffrg.Context(0, hbm_budget_bytes=budget)
+    wl = fi.make_finite_t_4d(seed=55, n_ext_p=64, n_rad=128, n_ang=96, n_x0=128)
+    tabs = c.tables(wl.problem, wl.tables)
+    y = torch.tensor(wl.y0, dtype=torch.float64, device="cuda")
+
+    def timed(call):
+        call()
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        call()
+        torch.cuda.synchronize()
+        return time.perf_counter() - t
+
+    t_rhs = timed(lambda: c.rhs(wl.problem, tabs, wl.Lambda, precision=ffrg.FP64))
+    t_none = timed(lambda: c.flow(wl.problem, tabs, y, wl.Lambda, 0.0, precision=ffrg.FP64))
+    assert np.array_equal(y.cpu().numpy(), wl.y0)
+    assert c.status_read() == ffrg.OK
+    steps = []
+    t_one = timed(lambda: steps.append(c.flow(wl.problem, tabs, y, wl.Lambda, 1e-3, precision=ffrg.FP64, rtol=1e-6)))
+    assert c.status_read() == ffrg.OK and steps[-1]["steps"] == 1 and steps[-1]["rejects"] == 0
+    c.close()
+    print(f"rhs {t_rhs * 1e3:.2f} ms, flows of no step {t_none * 1e3:.2f} ms and of one {t_one * 1e3:.2f} ms")
+    assert t_none < 3 * t_rhs and t_one < 9 * t_rhs
