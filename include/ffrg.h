@@ -168,7 +168,9 @@ typedef struct {
 } ffrg_step_opts;
 
 typedef struct {
-  long long steps, rejects, rhs_evals;
+  long long steps, rejects;
+  long long rhs_evals;    /* right-hand sides evaluated: six a DP5(4) step (one more at the start), or five where a
+                             frozen flow's stages run side by side (the last two share theirs) */
   double integrand_evals; /* rhs_evals x (external points x quadrature nodes) */
   double t_reached;
   long long jac_evals;    /* Jacobian evaluations (Rosenbrock flows) */

@@ -136,9 +136,10 @@ __global__ void flow_start_kernel(FlowCtl *c) {   // one block
   write_stage_scales(c);
 }
 
-// Accept (returned) or reject the step of error norm err, and the next step
-// size (same controller as the CPU oracle).  One thread.
-__device__ __forceinline__ int step_control(FlowCtl *c, double err, int anybad) {
+// Accept (returned) or reject the step of error norm err, which took `evals`
+// right-hand sides, and the next step size (same controller as the CPU
+// oracle).  One thread.
+__device__ __forceinline__ int step_control(FlowCtl *c, double err, int anybad, int evals) {
   const double h = c->h;
   c->err = err;
   int acc = 0;
@@ -147,6 +148,7 @@ __device__ __forceinline__ int step_control(FlowCtl *c, double err, int anybad) 
     c->done = 1;
   } else if (err <= 1.0) {
     acc = 1;
+    c->stage_evals += evals;
     c->t += h;
     c->steps += 1;
     double fac = (err == 0.0) ? 5.0 : 0.9 * pow(err, -0.2);
@@ -156,6 +158,7 @@ __device__ __forceinline__ int step_control(FlowCtl *c, double err, int anybad) 
     c->dt = h * fac;
   } else {
     c->rejects += 1;
+    c->stage_evals += evals;
     if (h <= c->dt_min) {
       c->status = FFRG_ESTEP_UNDERFLOW;
       c->done = 1;
@@ -206,7 +209,7 @@ __device__ __forceinline__ void flow_control_body(const FlowArgs &f) {
       err = fmax(err, red[w]);
       anybad |= bad_s[w];
     }
-    accept_s = step_control(c, err, anybad);
+    accept_s = step_control(c, err, anybad, 6);
   }
   __syncthreads();
   if (accept_s) {
@@ -272,7 +275,7 @@ __device__ __forceinline__ void flow_frozen_control_body(const FlowArgs &f, cons
   if (warp == 0) {
     double err = lane < (int)(blockDim.x >> 5) ? red[lane] : 0.0;
     for (int o = 16; o > 0; o >>= 1) err = fmax(err, __shfl_xor_sync(0xffffffffu, err, o));
-    if (lane == 0) accept_s = step_control(&c, err, anybad);
+    if (lane == 0) accept_s = step_control(&c, err, anybad, kStages);
   }
   __syncthreads();
   if (accept_s)
@@ -688,7 +691,6 @@ extern "C" int ffrg_flow(ffrg_ctx *ctx, const ffrg_problem *pb_in, const ffrg_ta
   if (a.ref64) ref64_setup(ctx, pl);
 
   const int eb = 256, eg = (ny + eb - 1) / eb;
-  long long attempts_done = 0;
   if (!st) {
     // order after the caller's stream, initialise, first derivative (FSAL stage 0)
     st = set_cuda_error(ctx, cudaEventRecord(ev, user), "cudaEventRecord");
@@ -767,7 +769,6 @@ extern "C" int ffrg_flow(ffrg_ctx *ctx, const ffrg_problem *pb_in, const ffrg_ta
                           "cudaMemcpyAsync(ctl)");
       if (!st) st = set_cuda_error(ctx, cudaStreamSynchronize(fs), "flow sync");
       if (st) break;
-      attempts_done = ctl_host->steps + ctl_host->rejects;
       if (ctl_host->done) break;
       // steps launched past the end return at once, but cost their launches
       batch = std::min(batch * 2, staged ? 8 : 32);
@@ -777,7 +778,7 @@ extern "C" int ffrg_flow(ffrg_ctx *ctx, const ffrg_problem *pb_in, const ffrg_ta
     if (stats) {
       stats->steps = ctl_host->steps;
       stats->rejects = ctl_host->rejects;
-      stats->rhs_evals = 1 + 6 * attempts_done;   // the method's stages (frozen: the last two share one evaluation)
+      stats->rhs_evals = 1 + ctl_host->stage_evals;
       stats->integrand_evals = (double)stats->rhs_evals * ffrg_evals(&pb);
       stats->t_reached = ctl_host->t;
       stats->jac_evals = 0;

@@ -631,7 +631,7 @@ struct FlowCtl {
   double t, dt, h, t0, t1, dt_min, dt_max, atol, rtol, end_tol, Lambda;
   double k_stages[kStages];   // frozen flows: the scales of the next step's stages
   double k_stage, m2_stage, err;
-  long long steps, rejects, max_steps;
+  long long steps, rejects, max_steps, stage_evals;   // stage_evals: right-hand sides of the attempts so far
   int last_rejected, done, status, accepted;
 };
 

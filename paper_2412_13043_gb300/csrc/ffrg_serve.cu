@@ -405,7 +405,7 @@ static int retire(Server &S, int si, const FlowCtl &c, int status) {
     if (e != cudaSuccess) return set_cuda_error(&S.lc, e, "serve result copy");
     r->stats.steps = c.steps;
     r->stats.rejects = c.rejects;
-    r->stats.rhs_evals = 1 + 6 * (c.steps + c.rejects);
+    r->stats.rhs_evals = 1 + c.stage_evals;
     r->stats.integrand_evals = (double)r->stats.rhs_evals * ffrg_evals(&r->pb);
     r->stats.t_reached = c.t;
   }

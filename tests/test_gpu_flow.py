@@ -6,6 +6,7 @@ Endpoint bar (FP64 RHS): 1e-8 relative to the oracle's "truth" run at
 rtol = 1e-13.  The GPU and the oracle may accept/reject differently near the
 tolerance, so each is compared with the truth, not with the other's steps.
 """
+import ctypes
 import math
 
 import numpy as np
@@ -214,3 +215,40 @@ def test_abm_flow_rejects_bad_arguments(ctx):
         with pytest.raises(ffrg.FfrgError):
             ctx.abm_flow(wl.problem, tabs, y, wl.Lambda, 1.0, n, order=order)
     tabs.free()
+
+
+STAGED = {
+    "d3 fp64": (lambda: fi.make_d3(seed=31, n_pts=20, n_ext_p=17, n_rad=19, n_ang=11), "FP64"),
+    "d3 mixed": (lambda: fi.make_d3(seed=31, n_pts=20, n_ext_p=17, n_rad=19, n_ang=11), "MIXED"),
+    "finite T fp64": (lambda: fi.make_finite_t(seed=32, N=4, T=0.05, n_pts=16, n_ext_p=5, n_ext_m=3, n_rad=13, n_ang=7),
+                      "FP64"),
+    "finite T mixed": (lambda: fi.make_finite_t(seed=32, N=4, T=0.05, n_pts=16, n_ext_p=5, n_ext_m=3, n_rad=13, n_ang=7),
+                       "MIXED"),
+    "finite T, 4D regulator": (lambda: fi.make_finite_t_4d(seed=33, N=5, T=0.05, n_pts=16, n_ext_p=4, n_ext_m=2, n_rad=12,
+                                                           n_ang=6, n_x0=16), "FP64"),
+    "d4 full mixed": (lambda: fi.make_d4_full(seed=34, n_pts=9, n_va=3, n_vb=2, n_ext_ang=2, n_rad=8, n_ang1=5, n_ang2=3),
+                      "MIXED"),
+}
+
+
+@pytest.mark.parametrize("case", STAGED)
+def test_frozen_flow_side_by_side_equals_stage_by_stage(case):
+    """The five distinct stage times of a step side by side, or (in a context with a memory budget) its six stages one
+    after the other: the same bits and steps, and the right-hand sides that were evaluated."""
+    import torch
+
+    import paper_2412_13043_gb300 as ffrg
+    make, precision = STAGED[case]
+    wl = make()
+    ends = []
+    for budget, per_step in ((0, 5), (1 << 30, 6)):
+        c = ffrg.Context(0, hbm_budget_bytes=budget)
+        tabs = c.tables(wl.problem, wl.tables)
+        y = torch.tensor(wl.y0, dtype=torch.float64, device="cuda")
+        st = c.flow(wl.problem, tabs, y, wl.Lambda, 3.0, precision=getattr(ffrg, precision), rtol=1e-9, atol=1e-12)
+        c.close()
+        ends.append((y.cpu().numpy(), st["steps"], st["rejects"], st["t_reached"]))
+        assert st["rhs_evals"] == 1 + per_step * (st["steps"] + st["rejects"])
+        assert st["integrand_evals"] == st["rhs_evals"] * float(ffrg.load().ffrg_evals(ctypes.byref(
+            ffrg.to_problem(wl.problem))))
+    assert np.array_equal(ends[0][0], ends[1][0]) and ends[0][1:] == ends[1][1:]

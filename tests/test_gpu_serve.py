@@ -265,3 +265,17 @@ def test_served_flow_with_the_flat_regulator(model):
                            atol=1e-16)
     assert st == ffrg.OK
     assert np.max(np.abs(y - truth) / np.abs(truth)) < ENDPOINT_TOL
+
+
+@pytest.mark.parametrize("slots,per_step", [(2, 5), (64, 6)])
+def test_served_flow_counts_the_right_hand_sides_it_evaluated(slots, per_step):
+    """Five a step with the stages side by side; six in a slot whose share of the budget (256 KB) has no room for it."""
+    import paper_2412_13043_gb300 as ffrg
+    wl = fi.make_d3(seed=93, n_pts=24, n_ext_p=64, n_rad=2048, n_ang=4)
+    ctx = gpu_context()
+    ctx.serve_start(max_slots=slots, hbm_budget_bytes=16 << 20)
+    tk = _submit(ctx, wl, rtol=1e-8)
+    st, _, fst, _ = _wait(ctx, [tk], [wl.problem.n_ext()])[tk]
+    ctx.serve_stop()
+    ctx.close()
+    assert st == ffrg.OK and fst["rhs_evals"] == 1 + per_step * (fst["steps"] + fst["rejects"])
