@@ -281,7 +281,6 @@ bool stage_plans(ffrg_ctx *ctx, Plan *pl) {
     Plan *sp = new Plan(*pl);
     plan_scratch_clear(sp);
     sp->radD = sp->gpart = sp->jrows = sp->rowbuf = nullptr;
-    sp->item_done = nullptr;
     for (Plan *&q : sp->stage) q = nullptr;
     pl->stage[i] = sp;
     if (plan_scratch(ctx, sp, pl->tab64 != nullptr) || finish_legacy_stream() != cudaSuccess) {
@@ -306,7 +305,7 @@ static void plan_free(ffrg_ctx *ctx, Plan *pl) {
     }
   plan_scratch_free(ctx, pl);
   void *arrs[] = {pl->rad_x, pl->rad_w, pl->a1_x, pl->a1_w, pl->a2_x, pl->a2_w, pl->psi_x, pl->psi_w,
-                  pl->radD, pl->gpart, pl->jrows, pl->rowbuf, pl->item_done};
+                  pl->radD, pl->gpart, pl->jrows, pl->rowbuf};
   for (void *p : arrs) dev_free(ctx, p, 0);
   delete pl;
 }
@@ -536,9 +535,7 @@ void fill_args(const Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td
   a.N = pl->N;
   a.stat = pl->stat;
   a.nfreq = pl->nfreq;
-  a.include_p0 = pl->include_p0;
   a.n_ext = pl->n_ext;
-  a.n_tables = td->n_tables;
   a.n_stack = td->n_stack;
   a.n_pts = td->n_pts;
   a.tab_count = pl->tab_count;
@@ -570,7 +567,6 @@ void fill_args(const Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td
   double lr = log(td->x_max / td->x_min);
   a.u_scale = 0.5 * (td->n_pts - 1) / lr;
   a.u_off = -(td->n_pts - 1) * log(td->x_min) / lr;
-  a.x_min2 = td->x_min * td->x_min;
   // k-independent parts of the table coordinates (the kernels add the k-dependent shift)
   const double nm1 = td->n_pts - 1;
   a.us1f = (float)(a.u_scale * 0.6931471805599453094 / nm1);

@@ -59,7 +59,7 @@ struct FxTables {
 // [2^53, 2^54), so that with |e| <= 200, grids within 2^+-50 and scales k
 // within 2^+-30 (coordinates are taken in y = s^2/k^2) no sum leaves 64 bits.
 struct FxGrid {
-  int64_t us, uo, uc[4];   // uc[c-1] = us log2(c): coordinate of y/c
+  int64_t us, uo, uc[3];   // uc[c-2] = us log2(c), c = 2..4: coordinate of y/c
   uint64_t b1, b2;
   uint32_t b3, b4;
   int F, nm1;              // n_pts - 1
@@ -277,7 +277,7 @@ inline bool fx_grid(int n_pts, double x_min, double x_max, FxGrid *g) {
   const long double s = ldexpl(us, g->F);
   g->us = (int64_t)roundl(s);
   g->uo = (int64_t)roundl(-2.0L * log2l((long double)x_min) * s);
-  for (int c = 1; c <= 4; ++c) g->uc[c - 1] = (int64_t)roundl(s * log2l((long double)c));
+  for (int c = 2; c <= 4; ++c) g->uc[c - 2] = (int64_t)roundl(s * log2l((long double)c));
   static const FxLogPoly poly;
   const long double *p = poly.p;
   g->b1 = (uint64_t)roundl(p[0] * s);

@@ -66,47 +66,51 @@ struct KConst<double> {
   const FxTables *us;   // staged tables (logarithms in the grid's units)
 };
 
+// The mixed main kernels hold a copy in static shared memory beside their tables:
+// its size takes away from the largest tables that they accept (kRhsArgsBytes).
 struct RhsArgs {
   int model, reg;
   int nr, na1, na2;
-  int n_ext_p, n_ext_ang, N, include_p0, n_ext;
+  int n_ext_p, n_ext_ang, N, n_ext;
   int stat, nfreq;  // loop statistics (ffrg_statistics) and frequency rows: 2N+1 (bosonic), 2N+2 (fermionic)
-  int n_tables, n_stack, n_pts, tab_count;
+  int n_stack, n_pts, tab_count;
   int tab32_count; // float2 entries of the FP32 table layout
   int tab64_count; // double2 entries of the FP64 table layout
   int n_va, n_vb;  // D4_FULL: vertex nodes in the shape variables a, b
-  int l3cell;      // D4_FULL, mixed: lambda3 as FP32 cell polynomials (one 1024-thread CTA per SM)
   int cr;          // rows per work item (d=4: outer rows)
   int n_chunks;    // work items per external point
   int n_items;     // n_ext * n_chunks
   int jb;          // angle nodes per row (D3 / FINITE_T; rows = outer index x angle block)
-  int tab_global;  // FP64 main kernels: tables read in place from global memory (L2), not staged,
-                   // because they exceed shared memory; only the angle rules are staged
+  unsigned char l3cell;        // D4_FULL, mixed: lambda3 as FP32 cell polynomials (one 1024-thread CTA per SM)
+  unsigned char tab_global;    // FP64 main kernels: tables read in place from global memory (L2), not staged,
+                               // because they exceed shared memory; only the angle rules are staged
+  unsigned char fp64;          // precision of this RHS (what the precompute kernel writes)
+  unsigned char ref64;         // FP64 RHS of an adaptive feedback flow (ffrg_ref64.cu)
+  unsigned char fg_ok;         // fg holds the table grid
+  unsigned char kc_host_ok;    // kc_host is valid
   double k, m2_over_k2, m2_shift, T;
   double p_min, p_ratio_step;  // p_i = p_min * exp(i * p_ratio_step)
   double qmax_over_k;
   double norm;                 // overall factor applied in finalize
   double u_scale, u_off;       // u = u_scale ln(s^2) + u_off
   double uoc[4];               // u_off - u_scale ln c, c = 1..4 (coordinate of S0^2 = sum of c squares / c)
-  float us1f;                  // FP32 coordinate: u_scale ln 2 / (n_pts - 1) (multiplies log2)
   double uoc1[4];              // uoc[c-1] / (n_pts - 1)
   double us1;                  // u_scale / (n_pts - 1)
   double twopiT;               // 2 pi T
-  double x_min2;               // x_min^2 (lookups below x_min return the first node)
   double sum_w2;               // sum of the second-angle weights (D4)
-  KConst<float> kc_host;       // FP32 scale constants from the host (valid when kc_host_ok, k_dev and m2_dev null)
-  int kc_host_ok;
-  int fp64;                    // precision of this RHS (what the precompute kernel writes)
-  int ref64;                   // FP64 RHS of an adaptive feedback flow (ffrg_ref64.cu)
-  double *rowbuf;              // its row values [n_ext][rows], or null: items run whole
-  unsigned *item_done;         // finished row groups per item, reset by the precompute kernel
+  float us1f;                  // FP32 coordinate: u_scale ln 2 / (n_pts - 1) (multiplies log2)
+  KConst<float> kc_host;       // FP32 scale constants from the host (used when kc_host_ok, k_dev and m2_dev null)
   FxGrid fg;                   // the table grid in fixed point (FP64 kernels)
-  int fg_ok;
   const FxTables *fx;          // device tables of the fixed-point functions
   const double *tab;           // FP64 tables [n_tables][n_stack][n_pts]
   double2 *tab64;              // FP64 tables in line form (tab64_entry), written by the precompute kernel; null:
                                // the FP64 main kernels build them in shared memory
-  void *kbuf;                  // FINITE_T: K[j][ip][r], j < N + n_ext_ang, in the kernel precision (main kernel)
+  union {
+    void *kbuf;      // FINITE_T: K[j][ip][r], j < N + n_ext_ang, in the kernel precision (main kernel);
+                     // FINITE_T_4D: the frequency set
+    double *rowbuf;  // ref64 (d=3, d=4): row values [n_ext][rows], then the finished row groups per item (reset by
+                     // the precompute kernel); null: items run whole
+  };
   float2 *tab32;               // FP32 tables (rows in line form, or finite-T (Z, lambda) pairs), precompute kernel
   const double *rad_x, *rad_w; // unit-interval GL rule on [0, 1]
   const double *a1_x, *a1_w;   // first angle rule
@@ -130,6 +134,8 @@ struct RhsArgs {
   double *out;                 // [n_ext]
   unsigned *status;
 };
+constexpr size_t kRhsArgsBytes = 632;   // with an mbarrier: 640 bytes of static shared memory
+static_assert(sizeof(RhsArgs) <= kRhsArgsBytes, "the block of the mixed kernels beside their tables");
 
 // ---------------------------------------------------------------------------
 // Regulator r(x) = R / (Z k^2) and rdot(x) = k d_k R / (Z k^2), x = q^2/k^2.
@@ -325,6 +331,15 @@ struct ItemQueue {
 // True when the flow of this right-hand side has ended (uniform over the grid;
 // the flag does not change while the kernels of a right-hand side run).
 __device__ __forceinline__ bool skipped(const RhsArgs &a) { return a.skip && *(volatile const int *)a.skip; }
+
+// Feedback flows (RhsArgs::ref64): rows of one external point, and the finished
+// row groups per item, which lie behind the row values.
+__host__ __device__ inline int ref64_rows(int model, int nr, int na1, int jb) {
+  return model == FFRG_MODEL_D3 ? nr * ((na1 + jb - 1) / jb) : nr * na1;
+}
+__device__ __forceinline__ unsigned *ref64_item_done(const RhsArgs &a) {
+  return (unsigned *)(a.rowbuf + (size_t)a.n_ext * ref64_rows(a.model, a.nr, a.na1, a.jb));
+}
 
 // Device-wide status word (sticky bits).
 __device__ __forceinline__ void raise_status(unsigned *status, unsigned bit) {
@@ -582,7 +597,6 @@ struct Plan {
   Plan *stage[4];           // frozen flows: the same plan with scratch of its own for further stages (or null)
   int grid_ref;             // feedback flows, FP64
   double *rowbuf;
-  unsigned *item_done;
   int grid_single;          // finite T, mixed: grid of the single-launch RHS (-1: not available)
   size_t smem64, smem32;    // dynamic shared memory bytes
   size_t smem64g;           // FP64 kernels with tables in global memory: the rest

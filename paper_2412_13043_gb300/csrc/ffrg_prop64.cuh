@@ -56,10 +56,10 @@ __device__ __forceinline__ KConst<double> make_kconst<double>(const RhsArgs &a) 
     off += fx_log(fx_scaled(a.fx->log[fx_log_index(hi)], a.fg), a.fg, hi, (uint32_t)fx_bits(c.k2));
   }
   if (!c.slow) off += (int64_t)1 << a.fg.F;   // entries of the line-form rows (tab64_entry), not nodes
-  c.uy1 = {off - a.fg.uc[0], 1};
-  c.uy2 = {off - a.fg.uc[1], 2};
-  c.uy3 = {off - a.fg.uc[2], 3};
-  c.uy4 = {off - a.fg.uc[3], 4};
+  c.uy1 = {off, 1};
+  c.uy2 = {off - a.fg.uc[0], 2};
+  c.uy3 = {off - a.fg.uc[1], 3};
+  c.uy4 = {off - a.fg.uc[2], 4};
   c.us = nullptr;
   c.twopiT = a.twopiT;
   c.sw2 = a.sum_w2;

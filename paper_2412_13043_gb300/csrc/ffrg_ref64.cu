@@ -47,11 +47,7 @@ __device__ __forceinline__ double ref_prop(const RhsArgs &a, double Z, double s2
   return 1.0 / prop_den(a.reg, Z, 0.0, s2, kc.m2, kc.k2, kc.inv_k2);
 }
 
-// rows of one external point, and of one item
-template <int MODEL>
-__device__ __forceinline__ int ref_rows(const RhsArgs &a) {
-  return MODEL == FFRG_MODEL_D3 ? a.nr * ((a.na1 + a.jb - 1) / a.jb) : a.nr * a.na1;
-}
+// rows of one item
 template <int MODEL>
 __device__ __forceinline__ int ref_item_rows(const RhsArgs &a) {
   return MODEL == FFRG_MODEL_D3 ? a.cr : a.cr * a.na1;
@@ -192,7 +188,7 @@ __global__ void __launch_bounds__(kThreads) ref64_kernel(RhsArgs a) {
   const int lane = threadIdx.x & 31;
   // d=4: the three-point block, with the second-angle loop, first
   const int rot = MODEL == FFRG_MODEL_D3 ? 0 : a.n_ext_p + 1;
-  const int rows = ref_rows<MODEL>(a), irows = ref_item_rows<MODEL>(a), nseg = ROWS ? (irows + 31) / 32 : 1;
+  const int rows = ref64_rows(MODEL, a.nr, a.na1, a.jb), irows = ref_item_rows<MODEL>(a), nseg = ROWS ? (irows + 31) / 32 : 1;
   ItemQueue items(a.work_ctr);
   for (;;) {
     const int d = items.pop(a.n_items * nseg);
@@ -220,7 +216,7 @@ __global__ void __launch_bounds__(kThreads) ref64_kernel(RhsArgs a) {
     unsigned done = 0;
     __threadfence();
     __syncwarp();
-    if (lane == 0) done = atomicAdd(a.item_done + (size_t)e * a.n_chunks + c, 1u);
+    if (lane == 0) done = atomicAdd(ref64_item_done(a) + (size_t)e * a.n_chunks + c, 1u);
     done = __shfl_sync(0xffffffffu, done, 0);
     if (done != (unsigned)segs - 1u) continue;
     __threadfence();
@@ -233,18 +229,15 @@ __global__ void __launch_bounds__(kThreads) ref64_kernel(RhsArgs a) {
 
 size_t ref64_smem(const Plan *pl) { return RefSmem::bytes(pl); }
 
-// Row buffer and item counters of a plan whose items are fewer than the
+// Row buffer and item counters (in one allocation) of a plan whose items are fewer than the
 // resident warps (optional, not taken in a context with a memory budget:
 // without them the items run whole).
 void ref64_setup(ffrg_ctx *ctx, Plan *pl) {
   const int items = pl->model == FFRG_MODEL_D3 ? pl->fn_items64 : pl->fn_items;
   if (pl->rowbuf || ctx->budget || items >= 152 * 16) return;
-  const int rows = pl->model == FFRG_MODEL_D3 ? pl->nr * ((pl->na1 + pl->fjb64 - 1) / pl->fjb64) : pl->nr * pl->na1;
-  if (dev_alloc(ctx, (void **)&pl->rowbuf, (size_t)pl->n_ext * rows * sizeof(double))) return;
-  if (dev_alloc(ctx, (void **)&pl->item_done, (size_t)items * sizeof(unsigned))) {
-    dev_free(ctx, pl->rowbuf, (size_t)pl->n_ext * rows * sizeof(double));
+  const int rows = ref64_rows(pl->model, pl->nr, pl->na1, pl->fjb64);
+  if (dev_alloc(ctx, (void **)&pl->rowbuf, (size_t)pl->n_ext * rows * sizeof(double) + (size_t)items * sizeof(unsigned)))
     pl->rowbuf = nullptr;
-  }
 }
 
 // The main kernel after the precompute kernel (which resets the counters).

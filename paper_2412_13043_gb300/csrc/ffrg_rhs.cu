@@ -326,8 +326,10 @@ __device__ __forceinline__ void precompute_body(const RhsArgs &a) {
   }
   if (a.ext_done)
     for (int i = tid0; i < a.n_ext; i += stride) a.ext_done[i] = 0u;
-  if (a.item_done)
-    for (int i = tid0; i < a.n_items; i += stride) a.item_done[i] = 0u;
+  if (a.ref64 && a.rowbuf) {
+    unsigned *item_done = ref64_item_done(a);
+    for (int i = tid0; i < a.n_items; i += stride) item_done[i] = 0u;
+  }
   // per-external-point constants used by every work item of the main kernels
   // one FP64 exp per value: value i on CTA i mod G, thread i / G, so that a
   // large grid spreads them over SMs and a small one keeps them in parallel lanes
@@ -1602,7 +1604,6 @@ int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int 
   a.ref64 = a_in.ref64 && !mixed;
   if (a.ref64) {
     a.rowbuf = pl->rowbuf;
-    a.item_done = pl->item_done;
     a.tab64 = nullptr;
     a.kconst = nullptr;
     if (a.model == FFRG_MODEL_D3) {

@@ -539,3 +539,12 @@ def test_flat_regulator_in_mixed_precision(ctx, case):
     wl = FLAT_MIXED[case]()
     for k in (0.4, 1.7):
         _check(ctx, wl, k)
+
+
+def test_mixed_tables_up_to_the_last_bytes_of_shared_memory(ctx):
+    """Tables and rules of 231,7xx of a block's 232,448 bytes of shared memory, next to the kernel's own block."""
+    ft = fi.make_finite_t(seed=98, N=5, T=0.05, n_pts=4096, n_ext_p=3, n_ext_m=2, n_rad=3, n_ang=198)
+    full = fi.make_d4_full(seed=99, n_pts=499, n_va=8, n_vb=7, n_ext_ang=1, n_rad=2, n_ang1=8, n_ang2=4)
+    full.problem.n_ext_p = 4
+    for wl in (ft, full):
+        _check(ctx, wl, 1.1)

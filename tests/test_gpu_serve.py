@@ -279,3 +279,15 @@ def test_served_flow_counts_the_right_hand_sides_it_evaluated(slots, per_step):
     ctx.serve_stop()
     ctx.close()
     assert st == ffrg.OK and fst["rhs_evals"] == 1 + per_step * (fst["steps"] + fst["rejects"])
+
+
+def test_served_tables_up_to_the_last_bytes_of_shared_memory():
+    import paper_2412_13043_gb300 as ffrg
+    wl = fi.make_finite_t(seed=98, N=5, T=0.05, n_pts=4096, n_ext_p=3, n_ext_m=2, n_rad=3, n_ang=198)
+    ctx = gpu_context()
+    ctx.serve_start(max_slots=2)
+    tk = _submit(ctx, wl, rtol=1e-6)
+    st, _, _, _ = _wait(ctx, [tk], [wl.problem.n_ext()])[tk]
+    ctx.serve_stop()
+    ctx.close()
+    assert st == ffrg.OK
