@@ -3,15 +3,16 @@
 // A scheduler thread owns up to max_slots device-resident flows ("slots").
 // Each slot holds its request's dressing tables, its DP5(4) state and its own
 // RHS scratch.  Every tick advances all resident flows by one adaptive step
-// with batched launches (one precompute, one persistent integrand launch per
-// model over the combined work list, one finalize and one derivative kernel
-// per stage, one control kernel with a CTA per flow).  Flows retire when
-// their control block says done; queued requests are admitted as soon as a
-// slot and enough of the HBM budget are free, so new flows join while others
-// are mid-flight.  Ticks are pipelined two deep: the next tick is queued
-// before the host reads the previous tick's control blocks, retires, admits
-// and rebuilds.  Each flow's reductions and step control depend only on its
-// own data, so its result does not depend on what it is batched with.
+// with batched launches: one precompute, one persistent integrand launch, one
+// finalize over the five distinct stages of every flow's step side by side,
+// and one control kernel with a CTA per flow; for flows without scratch for
+// five stages, the same per stage with a derivative kernel after each.  Flows
+// retire when their control block says done; queued requests are admitted as
+// soon as a slot and enough of the HBM budget are free, so new flows join
+// while others are mid-flight.  Ticks are pipelined two deep: the next tick is
+// queued before the host reads the previous tick's control blocks, retires,
+// admits and rebuilds.  Each flow's reductions and step control depend only on
+// its own data, so its result does not depend on what it is batched with.
 //
 // Requests: frozen-background flows (d_t y = -Flow, Sec. 5.2.2 Eqs. assVar /
 // flowVar) of the d=3 and finite-T models, mixed precision.
@@ -19,7 +20,9 @@
 // Memory: the HBM budget is reserved once, at start, and slot buffers are
 // carved from that reservation on the host (first fit, coalesced on return),
 // so admitting and retiring flows never calls a device allocator: nothing on
-// the tick path synchronises the device.
+// the tick path synchronises the device.  Scratch for the further stages of a
+// step lies in what is left of it (place_extra) and gives way to requests:
+// one that needs the place of such scratch waits for the two ticks in flight.
 #include <math.h>
 #include <string.h>
 
@@ -54,16 +57,18 @@ struct ServeReq {
   ffrg_flow_stats stats{};
   double latency = 0.0;
   Clock::time_point t_submit;
-  size_t need = 0, need_wide = 0;   // device bytes while resident: one set of RHS scratch, and one per stage
+  size_t need = 0, extra = 0;   // device bytes while resident, and optional ones (further stages side by side)
   int ny = 0;
 };
 
-// Geometry and device layout of one resident flow (segments of one buffer).
+// Geometry and device layout of one resident flow: segments of its buffer, the
+// last of them one set of RHS scratch, and of the optional extra block: the
+// outputs of all stages of a step, and scratch for kStages - 1 of them.
 struct SlotLayout {
   Plan pl;
   int ny, npsi;
-  int stages;   // sets of RHS scratch: kStages (a step's stages side by side), or 1
   size_t bytes, stage_bytes;   // stage_bytes: one set of RHS scratch
+  size_t extra_bytes, e_stage;
   size_t o_tab, o_tab32, o_y, o_ys, o_K, o_raw, o_radF, o_radF32, o_radq, o_radq32, o_kc, o_extp, o_psis, o_part;
   size_t o_kbuf, o_stage;
   size_t o_rx, o_rw, o_a1x, o_a1w, o_a2x, o_a2w, o_psx, o_psw;
@@ -75,7 +80,7 @@ static size_t seg(size_t &used, size_t bytes) {
   return off;
 }
 
-static void slot_layout(const ffrg_problem *pb, const ffrg_table_desc *td, int stages, SlotLayout &L) {
+static void slot_layout(const ffrg_problem *pb, const ffrg_table_desc *td, SlotLayout &L) {
   Plan &pl = L.pl;
   pl = Plan();
   plan_geometry(&pl, pb, td);
@@ -84,12 +89,11 @@ static void slot_layout(const ffrg_problem *pb, const ffrg_table_desc *td, int s
   L.npsi = std::max(1, pl.n_ext_ang);
   const size_t d = sizeof(double);
   size_t u = 0;
-  L.stages = stages;
   L.o_tab = seg(u, (size_t)pl.tab_count * d);
   L.o_y = seg(u, (size_t)L.ny * d);
   L.o_ys = seg(u, (size_t)L.ny * d);
   L.o_K = seg(u, (size_t)7 * L.ny * d);
-  L.o_raw = seg(u, (size_t)pl.n_ext * d * stages);
+  L.o_raw = seg(u, (size_t)pl.n_ext * d);
   L.o_rx = seg(u, (size_t)pl.nr * d);
   L.o_rw = seg(u, (size_t)pl.nr * d);
   L.o_a1x = seg(u, (size_t)pl.na1 * d);
@@ -98,7 +102,7 @@ static void slot_layout(const ffrg_problem *pb, const ffrg_table_desc *td, int s
   L.o_a2w = seg(u, d);
   L.o_psx = seg(u, (size_t)L.npsi * d);
   L.o_psw = seg(u, (size_t)L.npsi * d);
-  // RHS scratch, `stages` times
+  // RHS scratch
   L.o_stage = (u + 255) & ~(size_t)255;
   L.o_tab32 = seg(u, (size_t)pl.tab32_count * sizeof(float2));
   L.o_radF = seg(u, (size_t)pl.nr * pl.nfreq * d);
@@ -111,7 +115,9 @@ static void slot_layout(const ffrg_problem *pb, const ffrg_table_desc *td, int s
   L.o_psis = seg(u, (size_t)L.npsi * d);
   L.o_part = seg(u, (size_t)pl.fn_items * d);
   L.stage_bytes = ((u + 255) & ~(size_t)255) - L.o_stage;
-  L.bytes = u + L.stage_bytes * (stages - 1);
+  L.bytes = u;
+  L.e_stage = ((size_t)kStages * L.ny * d + 255) & ~(size_t)255;
+  L.extra_bytes = L.e_stage + (kStages - 1) * L.stage_bytes;
 }
 
 // First-fit allocator over one device reservation; host bookkeeping only.
@@ -164,6 +170,7 @@ struct Slot {
   ServeReq *req = nullptr;
   unsigned char *buf = nullptr;
   size_t cap = 0;
+  unsigned char *extra = nullptr;   // L.extra_bytes in the arena's free ranges, or null: stage by stage
   SlotLayout L;
   RhsArgs ra[kStages];   // ra[0] also takes the first derivative
   FlowArgs fa;
@@ -215,6 +222,35 @@ struct Server {
 }  // namespace ffrg
 
 namespace ffrg {
+
+// A slot's descriptors: one per stage with the extra block, else one.
+static void slot_descriptors(Server &S, Slot &sl) {
+  ServeReq *r = sl.req;
+  SlotLayout &L = sl.L;
+  Plan &pl = L.pl;
+  FlowCtl *ctl = sl.fa.ctl;
+  sl.fa.raw = (double *)(sl.extra ? sl.extra : sl.buf + L.o_raw);
+  for (int q = 0; q < (sl.extra ? kStages : 1); ++q) {
+    RhsArgs &ra = sl.ra[q];
+    unsigned char *bq = q ? sl.extra + L.e_stage + (size_t)(q - 1) * L.stage_bytes - L.o_stage : sl.buf;
+    pl.radF = (double *)(bq + L.o_radF);
+    pl.radq = (double *)(bq + L.o_radq);
+    pl.radq32 = (float *)(bq + L.o_radq32);
+    pl.radF32 = (float *)(bq + L.o_radF32);
+    pl.kconst = bq + L.o_kc;
+    pl.kbuf = pl.kbuf_count ? (double *)(bq + L.o_kbuf) : nullptr;
+    pl.ext_pd = (double *)(bq + L.o_extp);
+    pl.psi_s = (double *)(bq + L.o_psis);
+    pl.partial = (double *)(bq + L.o_part);
+    pl.tab32 = (float2 *)(bq + L.o_tab32);
+    fill_args(&pl, &r->pb, &r->td, (const double *)(sl.buf + L.o_tab), r->Lambda, ra);
+    ra.fused_ctr = nullptr;   // batched kernels only
+    ra.out = sl.fa.raw + (size_t)q * L.ny;
+    ra.status = S.status_dev;
+    ra.k_dev = sl.extra ? &ctl->k_stages[q] : &ctl->k_stage;
+    ra.skip = &ctl->done;
+  }
+}
 
 // Fill a slot's device buffer from its request and build its descriptors.
 static int slot_setup(Server &S, int si) {
@@ -271,26 +307,6 @@ static int slot_setup(Server &S, int si) {
   e = cudaStreamSynchronize(S.io);
   if (e != cudaSuccess) return set_cuda_error(&S.lc, e, "serve upload sync");
   if (!plan_grid(&pl, &r->td, S.lc.device)) return set_cuda_error(&S.lc, cudaGetLastError(), "function tables");
-  for (int q = 0; q < L.stages; ++q) {
-    RhsArgs &ra = sl.ra[q];
-    unsigned char *bq = b + (size_t)q * L.stage_bytes;
-    pl.radF = (double *)(bq + L.o_radF);
-    pl.radq = (double *)(bq + L.o_radq);
-    pl.radq32 = (float *)(bq + L.o_radq32);
-    pl.radF32 = (float *)(bq + L.o_radF32);
-    pl.kconst = bq + L.o_kc;
-    pl.kbuf = pl.kbuf_count ? (double *)(bq + L.o_kbuf) : nullptr;
-    pl.ext_pd = (double *)(bq + L.o_extp);
-    pl.psi_s = (double *)(bq + L.o_psis);
-    pl.partial = (double *)(bq + L.o_part);
-    pl.tab32 = (float2 *)(bq + L.o_tab32);
-    fill_args(&pl, &r->pb, &r->td, (const double *)(b + L.o_tab), r->Lambda, ra);
-    ra.fused_ctr = nullptr;   // batched kernels only
-    ra.out = (double *)(b + L.o_raw) + (size_t)q * L.ny;
-    ra.status = S.status_dev;
-    ra.k_dev = L.stages == kStages ? &ctl->k_stages[q] : &ctl->k_stage;
-    ra.skip = &ctl->done;
-  }
   FlowArgs &f = sl.fa;
   memset(&f, 0, sizeof(f));
   f.ny = L.ny;
@@ -303,8 +319,8 @@ static int slot_setup(Server &S, int si) {
   f.y = (double *)(b + L.o_y);
   f.ys = (double *)(b + L.o_ys);
   f.K = (double *)(b + L.o_K);
-  f.raw = (double *)(b + L.o_raw);
   f.ctl = ctl;
+  slot_descriptors(S, sl);
   sl.fresh = true;
   return FFRG_OK;
 }
@@ -417,14 +433,54 @@ static int retire(Server &S, int si, const FlowCtl &c, int status) {
   return FFRG_OK;
 }
 
+// Extra blocks lie in free ranges of the arena and are not taken from it: the
+// buffers that requests need are placed as if there were none, so that as many
+// flows are resident as without.  The highest free gap that holds `bytes`
+// (buffers are placed from the lowest), or null.
+static unsigned char *place_extra(Server &S, size_t bytes) {
+  for (auto it = S.arena.free_list.rbegin(); it != S.arena.free_list.rend(); ++it) {
+    size_t lo = it->first, end = lo + it->second;
+    for (;;) {   // from the top of the range downwards, below the extra blocks found there
+      if (end < lo + bytes) break;
+      const size_t at = end - bytes;
+      size_t next = end;
+      for (const Slot &sl : S.slots)
+        if (sl.extra) {
+          const size_t b = (size_t)(sl.extra - S.arena.base);
+          if (b < end && b + sl.L.extra_bytes > at) next = std::min(next, b);
+        }
+      if (next == end) return S.arena.base + at;
+      end = next;
+    }
+  }
+  return nullptr;
+}
+
+// Flows whose extra block lies in [p, p + n) go on stage by stage (the same
+// values; a step ends in the same state either way).  Waits for the ticks in
+// flight, which may still use it.
+static int release_extras(Server &S, const unsigned char *p, size_t n) {
+  bool any = false;
+  for (Slot &sl : S.slots)
+    if (sl.extra && sl.extra < p + n && sl.extra + sl.L.extra_bytes > p) {
+      sl.extra = nullptr;
+      if (sl.req) slot_descriptors(S, sl);
+      any = true;
+    }
+  if (!any) return FFRG_OK;
+  return set_cuda_error(&S.lc, cudaStreamSynchronize(S.st), "serve scratch release");
+}
+
 // Admit queued requests (first come, first served) while a slot is free and
 // the reserved HBM budget has a contiguous range for the request's buffers;
 // otherwise the head of the queue waits for retiring flows to return theirs.
-// Host bookkeeping only: no device allocation or free.
+// A flow takes scratch for all stages of a step as well while it stays within a
+// slot's share of the budget and a free range holds it, until a request needs
+// that range.  Host bookkeeping only: no device allocation or free.
 static int admit(Server &S) {
   for (;;) {
     ServeReq *r = nullptr;
-    int si = -1, stages = 1;
+    int si = -1;
     {
       std::lock_guard<std::mutex> lock(S.mu);
       while (!S.queue.empty() && S.queue.front()->cancel) {
@@ -437,23 +493,21 @@ static int admit(Server &S) {
       for (int i = 0; i < (int)S.slots.size() && si < 0; ++i)
         if (!S.slots[i].req && !S.slots[i].cooling) si = i;
       if (si < 0) return FFRG_OK;
-      // scratch for all stages of a step while it stays within a slot's
-      // share of the budget, so that as many flows are resident as without
-      const size_t wide = Arena::round(r->need_wide);
-      unsigned char *buf = wide <= S.arena.size / S.slots.size() ? S.arena.take(wide) : nullptr;
-      stages = buf ? kStages : 1;
-      if (!buf) buf = S.arena.take(r->need);
+      unsigned char *buf = S.arena.take(r->need);
       if (!buf) return FFRG_OK;
       S.queue.pop_front();
       r->state = kResident;
       Slot &sl = S.slots[si];
       sl.req = r;
       sl.buf = buf;
-      sl.cap = stages == kStages ? r->need_wide : r->need;
+      sl.cap = r->need;
     }
     Slot &sl = S.slots[si];
-    slot_layout(&r->pb, &r->td, stages, sl.L);
-    int st = slot_setup(S, si);
+    slot_layout(&r->pb, &r->td, sl.L);
+    int st = release_extras(S, sl.buf, Arena::round(sl.cap));
+    if (st) return st;
+    if (Arena::round(r->need) + r->extra <= S.arena.size / S.slots.size()) sl.extra = place_extra(S, r->extra);
+    st = slot_setup(S, si);
     if (st) return st;
     std::lock_guard<std::mutex> lock(S.mu);
     S.stats.admitted++;
@@ -497,6 +551,8 @@ static void scheduler(Server *Sp) {
         S.stats.resident = (int)T.live.size();
         S.stats.peak_resident = std::max(S.stats.peak_resident, (int)T.live.size());
         S.stats.hbm_in_use = S.arena.used;
+        for (const Slot &sl : S.slots)
+          if (sl.extra) S.stats.hbm_in_use += sl.L.extra_bytes;
       }
       const FlowCtl *ctl = S.ctl_host + (size_t)b * S.slots.size();
       for (int i : T.live) {
@@ -523,6 +579,7 @@ static void scheduler(Server *Sp) {
           S.arena.give(cs.buf, cs.cap);
           cs.buf = nullptr;
           cs.cap = 0;
+          cs.extra = nullptr;
           cooling[k] = cooling.back();
           cooling.pop_back();
         } else {
@@ -557,7 +614,7 @@ static void scheduler(Server *Sp) {
     }
     if (changed) {
       std::vector<int> narrow, wide;
-      for (int i : live) (S.slots[i].L.stages == kStages ? wide : narrow).push_back(i);
+      for (int i : live) (S.slots[i].extra ? wide : narrow).push_back(i);
       st = build_set(S, narrow, 1, false, S.step_set);
       if (!st) st = build_set(S, wide, kStages, false, S.wide_set);
       if (st) break;
@@ -689,9 +746,7 @@ extern "C" int ffrg_serve_submit(ffrg_ctx *ctx, const ffrg_problem *pb, const ff
       o->max_steps < 1)
     return FFRG_EINVAL;
   SlotLayout L;
-  slot_layout(pb, desc, kStages, L);
-  const size_t need_wide = L.bytes;
-  slot_layout(pb, desc, 1, L);
+  slot_layout(pb, desc, L);
   if (smem32_of(L.pl) > 227 * 1024) return FFRG_EINVAL;
   ServeReq *r = new ServeReq();
   r->pb = *pb;
@@ -701,7 +756,7 @@ extern "C" int ffrg_serve_submit(ffrg_ctx *ctx, const ffrg_problem *pb, const ff
   r->tab.assign(tables_host, tables_host + (size_t)L.pl.tab_count);
   r->y0.assign(y0_host, y0_host + L.ny);
   r->need = L.bytes;
-  r->need_wide = need_wide;
+  r->extra = L.extra_bytes;
   r->ny = L.ny;
   std::lock_guard<std::mutex> lock(S->mu);
   if (S->stop) {

@@ -291,3 +291,59 @@ def test_served_tables_up_to_the_last_bytes_of_shared_memory():
     ctx.serve_stop()
     ctx.close()
     assert st == ffrg.OK
+
+
+def test_a_large_request_joins_many_small_ones():
+    """Fifteen small flows and a large one fit the budget together with one set of scratch each.  The small ones may
+    take more while nobody else wants it; the large one is resident beside all of them all the same."""
+    import paper_2412_13043_gb300 as ffrg
+    small = [fi.make_finite_t(seed=100 + i, N=4, T=0.1, n_pts=16, n_ext_p=200, n_ext_m=2, n_rad=150, n_ang=4)
+             for i in range(15)]
+    large = fi.make_finite_t(seed=120, N=6, T=0.1, n_pts=16, n_ext_p=2000, n_ext_m=2, n_rad=400, n_ang=4)
+    budget, need = 64 << 20, []
+    alone = []
+    for wl in (small[0], large):
+        ctx = gpu_context()
+        ctx.serve_start(max_slots=1)
+        tk = _submit(ctx, wl, rtol=1e-12)
+        alone.append(_wait(ctx, [tk], [wl.problem.n_ext()])[tk])
+        ctx.serve_stop()
+        ctx.close()
+    ctx = gpu_context()
+    ctx.serve_start(max_slots=16, hbm_budget_bytes=budget)
+    tks = [_submit(ctx, wl, rtol=1e-12) for wl in small + [large]]
+    res = _wait(ctx, tks, [wl.problem.n_ext() for wl in small + [large]])
+    stats = ctx.serve_stats()
+    assert ctx.serve_stop() == ffrg.OK
+    ctx.close()
+    assert stats["peak_resident"] == 16, stats
+    for tk, (st, y, fst, _) in ((tks[0], alone[0]), (tks[-1], alone[1])):
+        assert res[tk][0] == st == ffrg.OK
+        assert np.array_equal(res[tk][1], y) and res[tk][2]["steps"] == fst["steps"]
+
+
+@pytest.mark.parametrize("n_ext_m", [1, 2, 4, 9, 10, 20])
+def test_external_frequencies_of_any_number(n_ext_m):
+    """Outputs come in tiles of nine external frequencies, or of three where few flows are resident: a request alone
+    (small tiles) and among many (large ones) has the same bits, and the single-flow path's values."""
+    import torch
+
+    import paper_2412_13043_gb300 as ffrg
+    wl = fi.make_finite_t(seed=130 + n_ext_m, N=3, T=0.2, n_pts=20, n_ext_p=31, n_ext_m=n_ext_m, n_rad=18, n_ang=6)
+    n, ctx = wl.problem.n_ext(), gpu_context()
+    ctx.serve_start(max_slots=32)
+    tk = _submit(ctx, wl)
+    alone = _wait(ctx, [tk], [n])[tk]
+    tks = [_submit(ctx, wl) for _ in range(24)]
+    mix = _wait(ctx, tks, [n] * 24)
+    assert ctx.serve_stats()["peak_resident"] > 1
+    ctx.serve_stop()
+    for tk in tks:
+        assert mix[tk][0] == alone[0] == ffrg.OK and np.array_equal(mix[tk][1], alone[1])
+    tabs = ctx.tables(wl.problem, wl.tables)
+    y = torch.tensor(wl.y0, dtype=torch.float64, device="cuda")
+    ctx.flow(wl.problem, tabs, y, wl.Lambda, math.log(wl.Lambda / wl.k_end), precision=ffrg.MIXED, rtol=1e-10,
+             atol=1e-13)
+    ctx.close()
+    ref = y.cpu().numpy()
+    assert np.max(np.abs(alone[1] - ref) / np.abs(ref)) < 1e-9
