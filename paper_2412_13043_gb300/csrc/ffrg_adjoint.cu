@@ -261,8 +261,18 @@ __global__ void __launch_bounds__(32 * kAdjMaxWarps) adjoint_kernel(AdjArgs A) {
   };
   if (!A.jrows) {
     const int per = (rows + 31) / 32, rot = MODEL == FFRG_MODEL_D3 ? 0 : a.n_ext_p + 1;
-    for (int u = warp * gridDim.x + blockIdx.x; u < a.n_ext * per; u += nw * gridDim.x)
-      unit((u / per + rot) % a.n_ext, (u % per) * 32 + lane, rows);
+    // unit u = e per + j, kept as (e, j): u itself exceeds 32 bits for problems
+    // whose 512-row items fit
+    const int u0 = warp * gridDim.x + blockIdx.x, step = nw * gridDim.x, de = step / per, dj = step % per;
+    for (int e = u0 / per, j = u0 % per; e < a.n_ext;) {
+      unit((e + rot) % a.n_ext, j * 32 + lane, rows);
+      e += de;
+      j += dj;
+      if (j >= per) {
+        j -= per;
+        ++e;
+      }
+    }
     adj_collect(A, S, kc.k2, A.gpart + (size_t)blockIdx.x * a.tab_count);
     return;
   }
