@@ -251,8 +251,7 @@ static int plan_scratch(ffrg_ctx *ctx, Plan *pl, bool want_tab64) {
   if (!st) st = dev_alloc(ctx, (void **)&pl->psi_s, (size_t)std::max(1, pl->n_ext_ang) * sizeof(double));
   if (!st)
     st = dev_alloc(ctx, (void **)&pl->partial, (size_t)std::max(pl->fn_items, pl->fn_items64) * sizeof(double));
-  if (!st) st = dev_alloc(ctx, (void **)&pl->tab32,
-                          (size_t)std::max(pl->tab_count, pl->tab32_count) * sizeof(float2));
+  if (!st) st = dev_alloc(ctx, (void **)&pl->tab32, (size_t)pl->tab32_count * sizeof(float2));
   return st;
 }
 static void plan_scratch_free(ffrg_ctx *ctx, Plan *pl) {
@@ -344,7 +343,7 @@ void plan_geometry(Plan *pl, const ffrg_problem *pb, const ffrg_table_desc *td) 
   pl->tab32_count = pb->model == FFRG_MODEL_FINITE_T ? td->n_stack * td->n_pts + 1 : compact;
   const int rows64 = pb->model == FFRG_MODEL_D4_FULL    ? 2 + pl->n_va * pl->n_vb
                      : pb->model == FFRG_MODEL_FINITE_T ? 2 * td->n_stack
-                                                        : td->n_tables * td->n_stack;
+                                                        : tables_needed(pb->model);   // one stack row each
   pl->tab64_count = rows64 * (td->n_pts + 1);
   int outer_total, rows_per_outer;
   if (is_d4(pb->model)) {
@@ -507,11 +506,14 @@ int get_plan(ffrg_ctx *ctx, const ffrg_problem *pb, const ffrg_table_desc *td, P
     pl->fn_items64 = pl->fn_items;
   }
   // FP64 line-form tables in global memory: finite T (long to build in every
-  // CTA), and tables that do not fit in shared memory.  The former can do
-  // without: optional buffers are left out in a context with a memory budget,
-  // so that it holds what it would hold without them.
+  // CTA), and tables that do not fit in shared memory.  Optional buffers are
+  // left out in a context with a memory budget, so that it holds what it would
+  // hold without them: finite T then builds them in shared memory, and large
+  // tables are read in place (not those of the full vertex, whose line form
+  // takes the place of a copy that was always made).
   const bool too_big = pl->smem64 > kMaxDynSmemBytes && pb->model != FFRG_MODEL_FINITE_T_4D;
-  if (!st) st = plan_scratch(ctx, pl, (pb->model == FFRG_MODEL_FINITE_T && !ctx->budget) || too_big);
+  const bool want = pb->model == FFRG_MODEL_D4_FULL ? too_big : (pb->model == FFRG_MODEL_FINITE_T || too_big) && !ctx->budget;
+  if (!st) st = plan_scratch(ctx, pl, want);
   if (!st) st = set_cuda_error(ctx, finish_legacy_stream(), "plan uploads");
   if (st) {
     plan_free(ctx, pl);

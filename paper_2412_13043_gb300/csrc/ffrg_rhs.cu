@@ -408,10 +408,50 @@ struct SmemLayout {
   }
 };
 
+// FP64 kernels without line-form tables in global memory either (a context with
+// a memory budget): the tables themselves, read in place.
+struct Smem64Plain : SmemLayout<double> {
+  const RhsArgs &args;
+  double k2;
+  __device__ Smem64Plain(unsigned char *base, const RhsArgs &a) : SmemLayout<double>(base, a), args(a) {
+    const double k = scale_k(a);
+    k2 = k * k;
+  }
+};
+template <typename T, bool PLAIN>
+struct LayoutOf {
+  using type = SmemLayout<T>;
+};
+template <>
+struct LayoutOf<double, true> {
+  using type = Smem64Plain;
+};
+
 // handle of the table row that starts `off` entries into the staged tables:
 // an FP64 line row, or an FP32 one (Row32)
 __device__ __forceinline__ const double2 *tab_row(const SmemLayout<double> &S, int off) { return S.tab + off; }
 __device__ __forceinline__ Row32 tab_row(const SmemLayout<float> &S, int off) { return row32(S.tab + off); }
+// or the row of the tables in place (d=4 vertex: rows of n_pts + 1 entries), and the factor of its values
+struct Plain64 {
+  const double *t;
+  double f;
+};
+__device__ __forceinline__ Plain64 tab_row(const Smem64Plain &S, int off) {
+  const int row = off / (S.args.n_pts + 1);
+  return {S.args.tab + (size_t)row * S.args.n_pts, row ? 1.0 : S.k2};
+}
+// cell and weight in [0, 1] of the tables for entry i and weight w1 of the line form
+__device__ __forceinline__ void plain_cell(int n, int i, double w1, int &i0, double &w) {
+  i0 = min(max(i - 1, 0), n - 2);
+  w = i == 0 ? 0.0 : i == n ? 1.0 : w1 - 1.0;
+}
+__device__ __forceinline__ double look(Plain64 row, double y, Look64 us, FxOff o, int n) {
+  int i, i0;
+  double w1, w;
+  node_of(us.a, us.kc, y, o, i, w1);
+  plain_cell(n, i, w1, i0, w);
+  return row.f * lerp_at(row.t, i0, w);
+}
 
 // angle rules into shared memory in the kernel precision.  S1 = false skips
 // sqrt(1 - c^2), which only the d=4 models read (FP64, slow on this part);
@@ -448,7 +488,7 @@ __device__ bool main_prologue(const RhsArgs &a, SmemLayout<T> &S, uint64_t *bar)
     // the function tables (logarithms in the grid's units), and line-form
     // tables that the precompute kernel does not write
     stage_fx(a, S.fx);
-    if (!a.tab64) {
+    if (!a.tab64 && !SmemLayout<T>::in_global(a)) {
       const double k = scale_k(a), k2 = k * k;
       for (int i = threadIdx.x; i < SmemLayout<T>::entries(a); i += blockDim.x) S.tab[i] = tab64_entry(a, i, k2);
     }
@@ -688,21 +728,31 @@ __device__ __forceinline__ RowAcc<T> d3_witem(const RhsArgs &a, const RhsArgs *s
 
 // finite-T lookups of Z and lambda at y in stack row srow: FP64 line-form
 // entries [row][entry][Z, lambda]; FP32 (Z, lambda) node pairs [row][pt] (+ one zero pair)
-__device__ __forceinline__ void zl_lookup(const double2 *tab, const RhsArgs &a, const KConst<double> &kc, int srow,
+__device__ __forceinline__ void zl_lookup(const Smem64Plain &S, const RhsArgs &a, const KConst<double> &kc, int srow,
+                                          double y, double &Z, double &L) {
+  int i, i0;
+  double w1, w;
+  node_of(a, kc, y, kc.uy1, i, w1);
+  plain_cell(a.n_pts, i, w1, i0, w);
+  const double *t = a.tab + (size_t)srow * a.n_pts;
+  Z = S.k2 * lerp_at(t, i0, w);
+  L = lerp_at(t + (size_t)a.n_stack * a.n_pts, i0, w);
+}
+__device__ __forceinline__ void zl_lookup(const SmemLayout<double> &S, const RhsArgs &a, const KConst<double> &kc, int srow,
                                           double y, double &Z, double &L) {
   int i;
   double w1;
   node_of(a, kc, y, kc.uy1, i, w1);
-  const double2 *e = tab + 2 * ((size_t)srow * (a.n_pts + 1) + i);
+  const double2 *e = S.tab + 2 * ((size_t)srow * (a.n_pts + 1) + i);
   Z = line64(e[0], w1);
   L = line64(e[1], w1);
 }
-__device__ __forceinline__ void zl_lookup(const float2 *tab, const RhsArgs &a, const KConst<float> &kc, int srow,
+__device__ __forceinline__ void zl_lookup(const SmemLayout<float> &S, const RhsArgs &a, const KConst<float> &kc, int srow,
                                           float y, float &Z, float &L) {
   int i0;
   float w;
   lerp_pos(y, kc.us, kc.uy1, a.n_pts, i0, w);
-  const float2 *row = tab + (size_t)srow * a.n_pts;
+  const float2 *row = S.tab + (size_t)srow * a.n_pts;
   const float2 v0 = row[i0], v1 = row[i0 + 1];
   Z = fmaf(w, v1.x - v0.x, v0.x);
   L = fmaf(w, v1.y - v0.y, v0.y);
@@ -718,8 +768,8 @@ __device__ __forceinline__ void zl_lookup(const float2 *tab, const RhsArgs &a, c
 // is a contraction over loop frequencies and radial nodes (ft_contract).
 // The same discrete sum as the direct loop over (m, n, r, c), with (N+M)
 // instead of (2N+1) M angular sums per (p, r).
-template <typename T, bool POLE>
-__device__ __forceinline__ void ftk_rows(const RhsArgs &a, const RhsArgs *sa, const SmemLayout<T> &S,
+template <typename T, bool POLE, typename SL>
+__device__ __forceinline__ void ftk_rows(const RhsArgs &a, const RhsArgs *sa, const SL &S,
                                          const KConst<T> &kc, int item, int lane, const T *q_loc = nullptr,
                                          const T *p_loc = nullptr) {
   const T sy = kc.sy;
@@ -745,7 +795,7 @@ __device__ __forceinline__ void ftk_rows(const RhsArgs &a, const RhsArgs *sa, co
     else for (int j = 0; j < na1; ++j) {
       const T y = fma(ty, S.c1[j], by);
       T Z, Lv;
-      zl_lookup(S.tab, a, kc, srow, y, Z, Lv);
+      zl_lookup(S, a, kc, srow, y, Z, Lv);
       auto pole = [&]() { return pole_ftk(sa, ip, jk, r, j); };
       rs = fma(S.w1[j] * Lv, inv_prop<POLE, true>(a, Z, y, om2s, kc, pole), rs);
     }
@@ -1083,8 +1133,8 @@ __device__ __forceinline__ float tp_full_cell_x2(const RhsArgs &a, const SmemLay
 // d=4 vertex expansion: row = (radial node r, first-angle node ia), inner loop
 // over the second-angle nodes for the three-point block.  FULL: the D4_FULL
 // model (lambda3 on (S0, a, b); compact tables Z | lambda4 | lambda3 rows).
-template <typename T, bool POLE, bool FULL = false, bool CELL = false>
-__device__ __forceinline__ RowAcc<T> d4_witem(const RhsArgs &a, const RhsArgs *sa, const SmemLayout<T> &S,
+template <typename T, bool POLE, bool FULL = false, bool CELL = false, typename SL>
+__device__ __forceinline__ RowAcc<T> d4_witem(const RhsArgs &a, const RhsArgs *sa, const SL &S,
                                            const KConst<T> &kc, int e, int c, int lane) {
   const auto us = look_scale(a, kc);
   const T sy = kc.sy;
@@ -1202,8 +1252,8 @@ __device__ __forceinline__ RowAcc<T> d4_witem(const RhsArgs &a, const RhsArgs *s
   return acc;
 }
 
-template <int MODEL, typename T, bool POLE>
-__device__ __forceinline__ RowAcc<T> witem(const RhsArgs &a, const RhsArgs *sa, const SmemLayout<T> &S,
+template <int MODEL, typename T, bool POLE, typename SL>
+__device__ __forceinline__ RowAcc<T> witem(const RhsArgs &a, const RhsArgs *sa, const SL &S,
                                         const KConst<T> &kc, int e, int c, int lane) {
   if constexpr (MODEL == FFRG_MODEL_D3) return d3_witem<T, POLE>(a, sa, S, kc, e, c, lane);
   else if constexpr (MODEL == FFRG_MODEL_D4_VERTEX) return d4_witem<T, POLE>(a, sa, S, kc, e, c, lane);
@@ -1269,8 +1319,8 @@ __device__ __forceinline__ double sum_partials(const RhsArgs &a, int e, int lane
 // Single-flow work loop: items from the device counter (d=4: the three-point
 // block, 16x more work per item, first), outputs by the warp that completes
 // an external point (fixed-order sum of its partials).
-template <int MODEL, typename T, bool POLE>
-__device__ __forceinline__ void item_loop(const RhsArgs &a, const RhsArgs *sa, const SmemLayout<T> &S,
+template <int MODEL, typename T, bool POLE, typename SL>
+__device__ __forceinline__ void item_loop(const RhsArgs &a, const RhsArgs *sa, const SL &S,
                                           const KConst<T> &kc) {
   const int lane = threadIdx.x & 31;
   const int rot = is_d4(MODEL) || MODEL == kModelD4FullCell ? a.n_ext_p + 1 : 0;
@@ -1311,7 +1361,8 @@ __device__ __forceinline__ void copy_args(RhsArgs *dst, const RhsArgs &a) {
   for (int i = threadIdx.x; i < (int)(sizeof(RhsArgs) / 4); i += blockDim.x) ((int *)dst)[i] = ((const int *)&a)[i];
 }
 
-template <int MODEL, typename T>
+// PLAIN (FP64, finite T and the d=4 vertex model): tables read in place.
+template <int MODEL, typename T, bool PLAIN = false>
 __global__ void __launch_bounds__(kMainThreads<T>, MinBlocks<T>::value) rhs_main(const __grid_constant__ RhsArgs a) {
   if (skipped(a)) {   // wait all the same: this kernel completes after its precompute
     pdl_wait();
@@ -1322,7 +1373,7 @@ __global__ void __launch_bounds__(kMainThreads<T>, MinBlocks<T>::value) rhs_main
   __shared__ RhsArgs sa;  // for the out-of-line near-pole path
   // one thread's copy: it runs while the precompute kernel does (d=4 213.1 us, by all threads 213.3)
   if (sizeof(T) == 4 && threadIdx.x == 0) sa = a;
-  SmemLayout<T> S(smem, a);
+  typename LayoutOf<T, PLAIN>::type S(smem, a);
   constexpr bool kD4 = MODEL == FFRG_MODEL_D4_VERTEX || MODEL == FFRG_MODEL_D4_FULL;
   if (!main_prologue<T, kD4>(a, S, &bar)) return;
   KConst<T> kc = load_kconst<T>(a);
@@ -1628,7 +1679,7 @@ int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int 
   if (!mixed && smem > kMaxDynSmem) {   // FP64 tables beyond shared memory: read from L2
     a.tab_global = 1;
     smem = pl->smem64g;
-    if (!a.tab64) {
+    if (!a.tab64 && a.model == FFRG_MODEL_D4_FULL) {
       ctx->last_error = "plan without FP64 line-form tables";
       return FFRG_ENOMEM;
     }
@@ -1644,6 +1695,9 @@ int launch_rhs_stages(ffrg_ctx *ctx, const Plan *pl_c, const RhsArgs &a_in, int 
     break;
   default: kern = mixed ? rhs_main<FFRG_MODEL_FINITE_T, float> : rhs_main<FFRG_MODEL_FINITE_T, double>; break;
   }
+  if (a.tab_global && !a.tab64)
+    kern = a.model == FFRG_MODEL_D4_VERTEX ? rhs_main<FFRG_MODEL_D4_VERTEX, double, true>
+                                           : rhs_main<FFRG_MODEL_FINITE_T, double, true>;
   int threads = mixed ? kThreads : kThreads64;
   if (mixed && a.model == FFRG_MODEL_D4_FULL && a.l3cell) {
     kern = rhs_main_cell;

@@ -159,3 +159,26 @@ def test_lookups_below_a_steep_first_cell(ctx, case):
         gref = oracle.rhs_jacobian(wl.problem, wl.tables, 0.01).T @ gbar
         assert np.max(np.abs(grad - gref)) / np.max(np.abs(gref)) < 1e-12
     tabs.free()
+
+
+@pytest.mark.parametrize("case", ["d4", "finite T", "d4, below the grid", "finite T, below the grid"])
+def test_large_tables_in_a_context_with_a_tight_budget(case):
+    """Tables beyond shared memory need no more device memory than themselves, their FP32 copy and a plan's small
+    buffers: read in place, without the line form (192 KB and 251 KB here) that a context without a budget keeps."""
+    import paper_2412_13043_gb300 as ffrg
+    if case.startswith("d4"):
+        wl = fi.make_d4(seed=5, n_pts=4000, n_ext_ang=1, n_rad=5, n_ang1=4, n_ang2=3)
+    else:
+        wl = fi.make_finite_t(seed=6, N=40, T=0.02, n_pts=160, n_ext_p=2, n_rad=8, n_ang=5)
+    k = 0.7
+    if case.endswith("grid"):
+        wl, k = _steep(wl), 0.01
+        wl.problem = dataclasses.replace(wl.problem, T=1e-4)
+    wl.problem = dataclasses.replace(wl.problem, n_ext_p=5)
+    c = ffrg.Context(0, hbm_budget_bytes=2 * wl.tables.nbytes + (64 << 10))
+    tabs = c.tables(wl.problem, wl.tables)
+    ref = oracle.rhs(wl.problem, wl.tables, k)
+    for precision, tol in ((ffrg.FP64, 1e-12),) + (((ffrg.MIXED, 1e-6),) if case in ("d4", "finite T") else ()):
+        got = c.rhs(wl.problem, tabs, k, precision=precision).cpu().numpy()
+        assert np.max(np.abs(got - ref) / np.abs(ref)) < tol
+    c.close()
