@@ -25,8 +25,12 @@ int ensure_smem_limit(ffrg_ctx *ctx, const void *func, size_t bytes) {
   return FFRG_OK;
 }
 
+// Status and message of a CUDA error, which is taken off the runtime's record:
+// the launch checks of a later call must not find it again (an optional buffer
+// that could not be had, a launch that was refused).
 int set_cuda_error(ffrg_ctx *ctx, cudaError_t e, const char *what) {
   if (e == cudaSuccess) return FFRG_OK;
+  (void)cudaGetLastError();
   if (ctx) {
     char buf[256];
     snprintf(buf, sizeof(buf), "%s: %s (%d)", what, cudaGetErrorString(e), (int)e);
@@ -283,7 +287,6 @@ bool stage_plans(ffrg_ctx *ctx, Plan *pl) {
     for (Plan *&q : sp->stage) q = nullptr;
     pl->stage[i] = sp;
     if (plan_scratch(ctx, sp, pl->tab64 != nullptr) || finish_legacy_stream() != cudaSuccess) {
-      cudaGetLastError();
       for (Plan *&q : pl->stage) {
         if (q) plan_scratch_free(ctx, q);
         delete q;

@@ -548,3 +548,28 @@ def test_mixed_tables_up_to_the_last_bytes_of_shared_memory(ctx):
     full.problem.n_ext_p = 4
     for wl in (ft, full):
         _check(ctx, wl, 1.1)
+
+
+def test_a_refused_call_does_not_fail_the_next(ctx):
+    """Tables of 232,176 bytes and the kernel's own block exceed a block's shared memory: the call reports it, and the
+    next ones, of any kind and with kernels that have run before, run."""
+    import torch
+
+    import paper_2412_13043_gb300 as ffrg
+    big = fi.make_finite_t(seed=98, N=5, T=0.05, n_pts=4096, n_ext_p=3, n_ext_m=2, n_rad=3, n_ang=230)
+    ft4 = fi.make_finite_t_4d(seed=97, N=6, T=0.05, n_pts=24, n_ext_p=7, n_ext_m=3, n_rad=13, n_ang=9, n_x0=21)
+    ft = fi.make_finite_t(seed=95, N=5, T=0.05, n_pts=20, n_ext_p=7, n_ext_m=3, n_rad=13, n_ang=9)
+    d3 = fi.make_d3(seed=95, n_pts=20, n_ext_p=7, n_rad=13, n_ang=9)
+    tabs = ctx.tables(d3.problem, d3.tables)
+    gbar = torch.ones(d3.problem.n_ext(), dtype=torch.float64, device="cuda")
+    y = torch.tensor(d3.y0, dtype=torch.float64, device="cuda")
+    for call in (lambda: _check(ctx, ft4, 1.1), lambda: _check(ctx, ft, 1.1),
+                 lambda: ctx.rhs_adjoint(d3.problem, tabs, 1.1, gbar),
+                 lambda: ctx.flow(d3.problem, tabs, y, d3.Lambda, 0.1, precision=ffrg.FP64, rtol=1e-6)):
+        call()
+        large = ctx.tables(big.problem, big.tables)
+        with pytest.raises(ffrg.FfrgError):
+            ctx.rhs(big.problem, large, 1.1, precision=ffrg.MIXED)
+        large.free()
+        call()
+    tabs.free()
