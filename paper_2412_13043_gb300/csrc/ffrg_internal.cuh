@@ -134,7 +134,7 @@ struct RhsArgs {
   double *out;                 // [n_ext]
   unsigned *status;
 };
-constexpr size_t kRhsArgsBytes = 632;   // with an mbarrier: 640 bytes of static shared memory
+constexpr size_t kRhsArgsBytes = 632, kMixedStaticSmemBytes = 640;   // with an mbarrier
 static_assert(sizeof(RhsArgs) <= kRhsArgsBytes, "the block of the mixed kernels beside their tables");
 
 // ---------------------------------------------------------------------------

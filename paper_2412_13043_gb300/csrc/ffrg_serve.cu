@@ -747,7 +747,8 @@ extern "C" int ffrg_serve_submit(ffrg_ctx *ctx, const ffrg_problem *pb, const ff
     return FFRG_EINVAL;
   SlotLayout L;
   slot_layout(pb, desc, L);
-  if (smem32_of(L.pl) > 227 * 1024) return FFRG_EINVAL;
+  // beside the main kernel's own block: a launch that the device refuses would end the server
+  if (smem32_of(L.pl) > kMaxDynSmemBytes - kMixedStaticSmemBytes) return FFRG_EINVAL;
   ServeReq *r = new ServeReq();
   r->pb = *pb;
   r->td = *desc;

@@ -347,3 +347,18 @@ def test_external_frequencies_of_any_number(n_ext_m):
     ctx.close()
     ref = y.cpu().numpy()
     assert np.max(np.abs(alone[1] - ref) / np.abs(ref)) < 1e-9
+
+
+def test_a_request_beyond_shared_memory_is_refused_and_the_server_goes_on():
+    """Tables of 232,176 bytes leave no room for the kernel's own block."""
+    import paper_2412_13043_gb300 as ffrg
+    big = fi.make_finite_t(seed=98, N=5, T=0.05, n_pts=4096, n_ext_p=3, n_ext_m=2, n_rad=3, n_ang=230)
+    good = fi.make_d3(seed=93, n_pts=24, n_ext_p=9, n_rad=16, n_ang=4)
+    ctx = gpu_context()
+    ctx.serve_start(max_slots=2)
+    with pytest.raises(ffrg.FfrgError):
+        _submit(ctx, big)
+    tk = _submit(ctx, good, rtol=1e-8)
+    assert _wait(ctx, [tk], [good.problem.n_ext()])[tk][0] == ffrg.OK
+    assert ctx.serve_stop() == ffrg.OK
+    ctx.close()
