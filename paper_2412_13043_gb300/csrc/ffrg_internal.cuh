@@ -712,8 +712,8 @@ const FxTables *fx_device_tables(int device);
 // grid of a persistent kernel: resident CTAs, at most one warp per item
 int persistent_grid(ffrg_ctx *ctx, const void *kernel, size_t smem, int items, int *grid, int threads);
 int launch_rhs(ffrg_ctx *ctx, const Plan *pl, const RhsArgs &a, int precision, cudaStream_t s);
-// the finite-T model with a 4D regulator (frequency set, loop factors, one
-// block per external point); launch_rhs dispatches to it
+// the finite-T model with a 4D regulator (frequency set, loop factors, then
+// warp items of external points x rows); launch_rhs dispatches to it
 int launch_ft4(ffrg_ctx *ctx, const Plan *pl, const RhsArgs &a, int precision, cudaStream_t s);
 // the FP64 RHS of adaptive feedback flows (RhsArgs::ref64): buffers (before
 // any capture) and main kernel

@@ -1371,7 +1371,7 @@ __global__ void __launch_bounds__(kMainThreads<T>, MinBlocks<T>::value) rhs_main
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t bar;
   __shared__ RhsArgs sa;  // for the out-of-line near-pole path
-  // one thread's copy: it runs while the precompute kernel does (d=4 213.1 us, by all threads 213.3)
+  // one thread's copy, which runs while the precompute kernel does (by all threads: no difference beyond noise)
   if (sizeof(T) == 4 && threadIdx.x == 0) sa = a;
   typename LayoutOf<T, PLAIN>::type S(smem, a);
   constexpr bool kD4 = MODEL == FFRG_MODEL_D4_VERTEX || MODEL == FFRG_MODEL_D4_FULL;
@@ -1765,7 +1765,11 @@ __global__ void __launch_bounds__(kThreads) batched_precompute_kernel(const RhsA
 // once.  One output at a time read 2 x (2N+1) n_rad values each from L2, which
 // bounded the kernel (48 flows x 5 stages of the serving mix: 300 us, so 136).
 // kMTile frequencies a block; fewer (kMTileFew) when the blocks of all flows
-// do not fill the GPU, where the length of a block's chain counts.
+// do not fill the GPU, where the length of a block's chain counts.  Any number
+// of frequencies works, the last tile is ragged.  Nine accumulators are about
+// what 64 registers hold; 40 flows of 180 external points in 1, 5, 9, 10, 20
+// frequencies take 54.8, 18.6, 15.9, 16.3, 14.1 ms so, 56.7, 18.8, 16.7, 16.2,
+// 14.3 with tiles of five and 54.2, 18.5, 16.0, 15.6, 13.9 with thirteen.
 constexpr int kMTile = 9, kMTileFew = 3;
 template <int kMTile>
 __device__ __forceinline__ void ft_contract_tile(const RhsArgs &a, int ip, int m0, double (*red)[kThreads / 32]) {
